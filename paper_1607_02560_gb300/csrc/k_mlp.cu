@@ -15,13 +15,14 @@
 // tensor memory (M = 128 rows per tile, N = 256). A single elected thread issues the MMAs and
 // the bulk copies of the weight chunks (double-buffered); the epilogue (bias, activation, bf16
 // pack into the canonical shared-memory layout of the next layer's A operand) runs on eight
-// warps from tcgen05.ld. Training uses the same fused forward (saving z and h),
-// a generic tcgen05 TN GEMM for the backward products, and Adam.
+// warps from tcgen05.ld. Training uses the same fused forward (saving h), a backward kernel over
+// the same tiles, split weight-gradient products, and Adam.
 #include <math.h>
 #include <stdarg.h>
 #include <stdio.h>
 #include <string.h>
 
+#include <algorithm>
 #include <string>
 #include <vector>
 
@@ -124,9 +125,6 @@ ChunkPlan plan_for(const Dims& m) {
   return p;
 }
 
-// Derivative of the ReLU activation max(z, 0) (0 at z = 0).
-__device__ __forceinline__ float act_grad(float z) { return z > 0.0f ? 1.0f : 0.0f; }
-
 __device__ __forceinline__ int64_t snap_m(double x) {
   const double yf = fma(x, kQuarterInvPi2, -0.5);
   const double r = rint(yf);
@@ -173,7 +171,6 @@ struct FusedParams {
   // batch mode
   float* Y;  // [M x OUTP] normalised outputs
   __nv_bfloat16* Hs[3];
-  float* Zs[3];
   int* err;
   // limit of the pipeline's operand waits (the drain at the end always waits up to 1 s, so
   // that no copy or MMA is still in flight when the CTA exits)
@@ -259,20 +256,18 @@ __device__ __forceinline__ double f2d_int(float x) {
 // Two columns of the hidden-layer epilogue: z = acc + b with one packed FP32 addition (it
 // rounds like the scalar one), then ReLU and the conversion to bf16 in one instruction,
 // packed as the next layer's operand wants it (column 2i in the low half). Returns the packed
-// pair; z0, z1 receive z (kept for the backward pass in batch mode).
-__device__ __forceinline__ uint32_t relu_bf16x2(uint32_t a0, uint32_t a1, float b0, float b1,
-                                                float& z0, float& z1) {
-  uint32_t h, r0, r1;
+// pair (the backward pass needs only the sign of z, which is that of h).
+__device__ __forceinline__ uint32_t relu_bf16x2(uint32_t a0, uint32_t a1, float b0, float b1) {
+  uint32_t h;
   asm("{\n\t.reg .b64 a, b, z;\n\t"
-      "mov.b64 a, {%3, %4};\n\t"
-      "mov.b64 b, {%5, %6};\n\t"
+      ".reg .b32 z0, z1;\n\t"
+      "mov.b64 a, {%1, %2};\n\t"
+      "mov.b64 b, {%3, %4};\n\t"
       "add.rn.f32x2 z, a, b;\n\t"
-      "mov.b64 {%1, %2}, z;\n\t"
-      "cvt.rn.relu.bf16x2.f32 %0, %2, %1;\n\t}"
-      : "=r"(h), "=r"(r0), "=r"(r1)
+      "mov.b64 {z0, z1}, z;\n\t"
+      "cvt.rn.relu.bf16x2.f32 %0, z1, z0;\n\t}"
+      : "=r"(h)
       : "r"(a0), "r"(a1), "r"(__float_as_uint(b0)), "r"(__float_as_uint(b1)));
-  z0 = __uint_as_float(r0);
-  z1 = __uint_as_float(r1);
   return h;
 }
 
@@ -494,16 +489,13 @@ __global__ void __launch_bounds__(kFusedThreads, 1) k_mlp_fused(FusedParams p) {
             const int i = 8 * q8;
             const float4 b0 = *reinterpret_cast<const float4*>(bl + cb + i);
             const float4 b1 = *reinterpret_cast<const float4*>(bl + cb + i + 4);
-            float z[8];
             uint4 q;
-            q.x = relu_bf16x2(rr[i + 0], rr[i + 1], b0.x, b0.y, z[0], z[1]);
-            q.y = relu_bf16x2(rr[i + 2], rr[i + 3], b0.z, b0.w, z[2], z[3]);
-            q.z = relu_bf16x2(rr[i + 4], rr[i + 5], b1.x, b1.y, z[4], z[5]);
-            q.w = relu_bf16x2(rr[i + 6], rr[i + 7], b1.z, b1.w, z[6], z[7]);
+            q.x = relu_bf16x2(rr[i + 0], rr[i + 1], b0.x, b0.y);
+            q.y = relu_bf16x2(rr[i + 2], rr[i + 3], b0.z, b0.w);
+            q.z = relu_bf16x2(rr[i + 4], rr[i + 5], b1.x, b1.y);
+            q.w = relu_bf16x2(rr[i + 6], rr[i + 7], b1.z, b1.w);
             *reinterpret_cast<uint4*>(Hs + tc::kmajor_off(trow, cb + i, kH)) = q;
             if (MODE == kModeBatch && myrow < p.M) {
-#pragma unroll
-              for (int u = 0; u < 8; ++u) p.Zs[layer][myrow * kH + cb + i + u] = z[u];
               *reinterpret_cast<uint4*>(p.Hs[layer] + myrow * kH + cb + i) = q;
             }
           }
@@ -854,16 +846,13 @@ __global__ void __launch_bounds__(kPPThreads, 1) k_mlp_pp(FusedParams p) {
                 const int i = 8 * q8;
                 const float4 b0 = *reinterpret_cast<const float4*>(bl + cb + i);
                 const float4 b1 = *reinterpret_cast<const float4*>(bl + cb + i + 4);
-                float z[8];
-                uint4 q;
-                q.x = relu_bf16x2(rr[i + 0], rr[i + 1], b0.x, b0.y, z[0], z[1]);
-                q.y = relu_bf16x2(rr[i + 2], rr[i + 3], b0.z, b0.w, z[2], z[3]);
-                q.z = relu_bf16x2(rr[i + 4], rr[i + 5], b1.x, b1.y, z[4], z[5]);
-                q.w = relu_bf16x2(rr[i + 6], rr[i + 7], b1.z, b1.w, z[6], z[7]);
+                    uint4 q;
+                q.x = relu_bf16x2(rr[i + 0], rr[i + 1], b0.x, b0.y);
+                q.y = relu_bf16x2(rr[i + 2], rr[i + 3], b0.z, b0.w);
+                q.z = relu_bf16x2(rr[i + 4], rr[i + 5], b1.x, b1.y);
+                q.w = relu_bf16x2(rr[i + 6], rr[i + 7], b1.z, b1.w);
                 *reinterpret_cast<uint4*>(Ht + tc::kmajor_off(trow, cb + i, kH)) = q;
                 if (MODE == kModeBatch && myrow < p.M) {
-#pragma unroll
-                  for (int u = 0; u < 8; ++u) p.Zs[l][myrow * kH + cb + i + u] = z[u];
                   *reinterpret_cast<uint4*>(p.Hs[l] + myrow * kH + cb + i) = q;
                 }
               }
@@ -1257,16 +1246,13 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPPThreads, 1) k_mlp
                 const int i = 8 * q8;
                 const float4 b0 = *reinterpret_cast<const float4*>(bl + cb + i);
                 const float4 b1 = *reinterpret_cast<const float4*>(bl + cb + i + 4);
-                float z[8];
-                uint4 q;
-                q.x = relu_bf16x2(rr[i + 0], rr[i + 1], b0.x, b0.y, z[0], z[1]);
-                q.y = relu_bf16x2(rr[i + 2], rr[i + 3], b0.z, b0.w, z[2], z[3]);
-                q.z = relu_bf16x2(rr[i + 4], rr[i + 5], b1.x, b1.y, z[4], z[5]);
-                q.w = relu_bf16x2(rr[i + 6], rr[i + 7], b1.z, b1.w, z[6], z[7]);
+                    uint4 q;
+                q.x = relu_bf16x2(rr[i + 0], rr[i + 1], b0.x, b0.y);
+                q.y = relu_bf16x2(rr[i + 2], rr[i + 3], b0.z, b0.w);
+                q.z = relu_bf16x2(rr[i + 4], rr[i + 5], b1.x, b1.y);
+                q.w = relu_bf16x2(rr[i + 6], rr[i + 7], b1.z, b1.w);
                 *reinterpret_cast<uint4*>(Ht + tc::kmajor_off(trow, cb + i, kH)) = q;
                 if (MODE == kModeBatch && myrow < p.M) {
-#pragma unroll
-                  for (int u = 0; u < 8; ++u) p.Zs[l][myrow * kH + cb + i + u] = z[u];
                   *reinterpret_cast<uint4*>(p.Hs[l] + myrow * kH + cb + i) = q;
                 }
               }
@@ -1450,7 +1436,8 @@ __global__ void k_inputs_rows(const __nv_bfloat16* __restrict__ xb,
 template <int D>
 __global__ void k_inputs_batch(const float* __restrict__ Xraw, const float* __restrict__ params,
                                int64_t norm_off, int64_t M, uint8_t* __restrict__ Xt,
-                               __nv_bfloat16* __restrict__ X16) {
+                               __nv_bfloat16* __restrict__ X16, double* __restrict__ loss) {
+  if (blockIdx.x == 0 && threadIdx.x == 0) *loss = 0.0;  // the sum of k_backward
   constexpr int NF = D == 2 ? 26 : 126;
   constexpr int K0 = D == 2 ? 32 : 128, KG = K0 / 8;
   const float mu_x = params[norm_off], isig_x = 1.0f / params[norm_off + 1];
@@ -1473,185 +1460,474 @@ __global__ void k_inputs_batch(const float* __restrict__ Xraw, const float* __re
   }
 }
 
-// ---- generic C[M x N] (fp32) = A[M x K] B[N x K]^T, bf16 row-major operands ---------------
-// M % 128 == 0, N % 16 == 0, K % 16 == 0. One CTA per 128 x min(N, 256) tile; K in chunks of
-// up to 64 staged in the canonical layout; one elected thread issues the MMAs.
-__global__ void __launch_bounds__(128, 1) k_gemm_tn(const __nv_bfloat16* __restrict__ A,
-                                                    const __nv_bfloat16* __restrict__ B,
-                                                    float* __restrict__ Cm, int M, int N, int K,
-                                                    int* err) {
+// ---- the training step's backward pass -----------------------------------------------------
+// Three launches after the fused forward: k_backward (loss, dY and the chain dZ3, dZ2, dZ1, one
+// CTA per 128-row tile), k_wgrad (every weight and bias gradient) and k_update (Adam, the
+// bf16 copies of the weights).
+//
+// What bounds it: latency. At a batch of 4096 the step's products are 3.5 GFLOP (2 us at the
+// tensor rate), so the launches, the chain of dependent layers and the host wait are what
+// remain. With dW on two CTAs over the whole batch, bias gradients on one thread per column and
+// every activation transposed in memory a step took 4.08 ms at batch 4096 in 2D; in this form
+// 0.18 ms, the copy of the gradients to the host included, with the same gradients bit for bit.
+
+// Element e = (n, k) of layer l's weights, row-major [N x K], rounded to bf16 and written where
+// the kernels read it: the chunk stream of the forward kernels, and (layers 1..3) the stream
+// of k_backward.
+__device__ __forceinline__ void store_weight(const Layout& L, const int64_t* fwd_off,
+                                             const int64_t* back_off, int l, int64_t e, float w,
+                                             uint8_t* tiles, uint8_t* back) {
+  const int N = (int)L.nN[l], K = (int)L.nK[l];
+  const int n = (int)(e / K), k = (int)(e - (int64_t)n * K);
+  const __nv_bfloat16 x = __float2bfloat16(w);
+  const int kw_max = kChunkBytes / (N * 2), kw = K < kw_max ? K : kw_max;
+  const int c = k / kw;
+  *reinterpret_cast<__nv_bfloat16*>(tiles + fwd_off[l] + (int64_t)c * N * kw * 2 +
+                                    tc::kmajor_off(n, k - c * kw, kw)) = x;
+  if (l > 0) {  // operand W^T: rows k (256), K dimension n in chunks of at most 64
+    const int nw = N < kChunkK ? N : kChunkK, cb = n / nw;
+    *reinterpret_cast<__nv_bfloat16*>(back + back_off[l] + (int64_t)cb * kH * nw * 2 +
+                                      tc::kmajor_off(k, n - cb * nw, nw)) = x;
+  }
+}
+
+struct WeightStreams {
+  uint8_t* tiles;       // forward chunk stream
+  uint8_t* back;        // backward stream: layer 3, then 2, then 1
+  int64_t fwd_off[4];   // bytes into tiles
+  int64_t back_off[4];  // bytes into back
+};
+
+__global__ void k_retile(const float* __restrict__ params, Layout L, WeightStreams ws) {
+  for (int l = 0; l < 4; ++l)
+    for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < L.wn[l];
+         e += (int64_t)gridDim.x * blockDim.x)
+      store_weight(L, ws.fwd_off, ws.back_off, l, e, params[L.w[l] + e], ws.tiles, ws.back);
+}
+
+struct BackParams {
+  const float* Y;       // [B x OUTP] network outputs
+  const float* T;       // [B x OUT] raw targets
+  const float* params;
+  const uint8_t* back;  // weight stream (WeightStreams::back)
+  const __nv_bfloat16* Hs[3];
+  __nv_bfloat16* dY16;
+  float* dY32;
+  __nv_bfloat16* dZ16[3];
+  float* dZ32[3];
+  double* loss;
+  int* err;
+  int64_t B, norm_off;
+};
+
+// One CTA per 128-row tile of the batch (tiles strided by the grid), 256 threads. The tile's
+// dY = 2 (y - t_norm) / (B OUT) becomes the first A operand; then for l = 2, 1, 0
+//   dZ_l = (dZ_{l+1} W_{l+1}) .* [h_l > 0]      (ReLU: h > 0 exactly where z > 0)
+// runs as one 128 x 256 product per layer, its result turned into the next product's A operand
+// in place (bf16, shared memory) and stored for k_wgrad (bf16) and the bias gradients (fp32).
+// The weights arrive by bulk copies through four 32 KiB buffers, the next layer's as soon as
+// this layer's products have completed, under its epilogue. One CTA per SM (193 KiB of shared
+// memory); the 256 x 256 operands are read from L2 by every tile.
+// The waits are bounded; after one gives up the CTA issues no more work, waits for its own
+// copies and products (bounded), frees its tensor memory and returns.
+constexpr int kBackThreads = 256;
+template <int D>
+__global__ void __launch_bounds__(kBackThreads, 1) k_backward(BackParams p) {
+  using Cfg = FusedCfg<D>;
+  constexpr int OUTP = Cfg::OUTP, OUT = 2 * Cfg::MU, NBUF = 4;
+  constexpr int BUF = kH * kChunkK * 2;         // 32 KiB: 256 x 64 bf16
+  constexpr int CH0 = kH * OUTP * 2;            // the one chunk of layer 3
+  constexpr int NCH = 1 + 2 * (kH / kChunkK);   // chunks per tile: 1 + 4 + 4
   extern __shared__ __align__(1024) uint8_t smem[];
-  constexpr int NT_MAX = 256;
-  uint8_t* As = smem;                    // 128 x 64
-  uint8_t* Bs = smem + 128 * kChunkK * 2;  // 256 x 64
-  __shared__ __align__(8) uint64_t bar;
+  uint8_t* As = smem;                  // 128 x 256 bf16, K-major
+  uint8_t* Wb = As + kTile * kH * 2;   // NBUF chunks
+  __shared__ __align__(8) uint64_t bar_w[NBUF], bar_mma;
   __shared__ uint32_t tslot;
   __shared__ int s_abort;
+  __shared__ double s_loss[kBackThreads / 32];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int m0 = blockIdx.x * 128, n0 = blockIdx.y * NT_MAX;
-  const int NT = (N - n0) < NT_MAX ? (N - n0) : NT_MAX;
   if (tid == 0) {
-    tc::mbar_init(&bar, 1);
+    for (int b = 0; b < NBUF; ++b) tc::mbar_init(&bar_w[b], 1);
+    tc::mbar_init(&bar_mma, 1);
     s_abort = 0;
   }
-  if (warp == 0) tc::tmem_alloc(&tslot, NT_MAX);
+  if (warp == 0) tc::tmem_alloc(&tslot, kH);
   tc::fence_before();
   __syncthreads();
   tc::fence_after();
   const uint32_t tmem = tslot;
-  uint32_t ph = 0;
-  for (int k0 = 0; k0 < K; k0 += kChunkK) {
-    const int kw = (K - k0) < kChunkK ? (K - k0) : kChunkK;
-    const int seg = kw / 8;  // 16-byte segments per row
-    for (int e = tid; e < 128 * seg; e += 128) {
-      const int r = e / seg, s8 = (e % seg) * 8;
-      const uint4 q = *reinterpret_cast<const uint4*>(A + (int64_t)(m0 + r) * K + k0 + s8);
-      *reinterpret_cast<uint4*>(As + tc::kmajor_off(r, s8, kw)) = q;
+  volatile int* abort_flag = &s_abort;
+  const int64_t ntiles = p.B / kTile;
+  const int64_t my_tiles = blockIdx.x < ntiles ? (ntiles - 1 - blockIdx.x) / gridDim.x + 1 : 0;
+  const int64_t total = my_tiles * NCH;  // chunks this CTA consumes
+  int64_t issued = 0, done = 0, used = 0;  // thread 0: chunks copied, released, multiplied
+  uint32_t ph_mma = 0;
+  // thread 0: start the copies of every chunk whose buffer is free
+  auto top_up = [&]() {
+    while (issued < total && issued < done + NBUF) {
+      const int c = (int)(issued % NCH), slot = (int)(issued % NBUF);
+      const uint32_t bytes = c == 0 ? CH0 : BUF;
+      const int64_t off = c == 0 ? 0 : CH0 + (int64_t)(c - 1) * BUF;
+      tc::mbar_expect_tx(&bar_w[slot], bytes);
+      tc::bulk_g2s(Wb + slot * BUF, p.back + off, bytes, &bar_w[slot]);
+      ++issued;
     }
-    for (int e = tid; e < NT * seg; e += 128) {
-      const int r = e / seg, s8 = (e % seg) * 8;
-      const uint4 q = *reinterpret_cast<const uint4*>(B + (int64_t)(n0 + r) * K + k0 + s8);
-      *reinterpret_cast<uint4*>(Bs + tc::kmajor_off(r, s8, kw)) = q;
-    }
-    tc::fence_async_smem();
-    tc::fence_before();
-    __syncthreads();
-    tc::fence_after();
-    if (tid == 0 && !s_abort) {
-      const uint32_t sbo = (uint32_t)(kw / 8) * 128;
-      for (int s = 0; s < kw / 16; ++s) {
-        const uint64_t ad = tc::desc_kmajor(tc::smem_u32(As) + s * 256, 128, sbo);
-        const uint64_t bd = tc::desc_kmajor(tc::smem_u32(Bs) + s * 256, 128, sbo);
-        tc::mma_bf16(tmem, ad, bd, tc::idesc_bf16(128, NT), (k0 > 0 || s > 0) ? 1u : 0u);
-      }
-      tc::commit(&bar);
-      if (!tc::mbar_wait(&bar, ph, err, 16)) s_abort = 1;
-    }
-    ph ^= 1;
-    tc::fence_before();
-    __syncthreads();  // the staging buffers are free again
-    tc::fence_after();
-    if (s_abort) break;
-  }
-  if (!s_abort) {
-    const uint32_t taddr = tmem + ((uint32_t)(warp * 32) << 16);
-    const int row = m0 + warp * 32 + lane;
-    for (int c0 = 0; c0 < NT; c0 += 16) {
-      float a[16];
-      tc::tmem_ld16(taddr + c0, a);
+  };
+  if (tid == 0) top_up();
+  double acc_loss = 0.0;
+  const double scale = 2.0 / ((double)p.B * OUT);
+  const int quarter = warp & 3, half = warp >> 2;
+  const int trow = quarter * 32 + lane;
+  for (int64_t it = 0; it < my_tiles; ++it) {
+    const int64_t r0 = (blockIdx.x + it * gridDim.x) * kTile;
+    // dY of the tile: two threads per row, half the columns each
+    {
+      const int row = tid >> 1, o0 = (tid & 1) * (OUTP / 2);
+      const int64_t b = r0 + row;
 #pragma unroll
-      for (int i = 0; i < 16; ++i) Cm[(int64_t)row * N + n0 + c0 + i] = a[i];
+      for (int o8 = 0; o8 < OUTP / 2; o8 += 8) {
+        float g[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+          const int o = o0 + o8 + u;
+          g[u] = 0.0f;
+          if (o < OUT) {
+            const float mu = p.params[p.norm_off + 2 + o];
+            const float sg = p.params[p.norm_off + 2 + OUTP + o];
+            const float t = (p.T[b * OUT + o] - mu) / sg;
+            const float r = p.Y[b * OUTP + o] - t;
+            acc_loss += (double)r * r;
+            g[u] = (float)(scale * r);
+          }
+        }
+        uint4 q;
+        q.x = tc::pack_bf16(g[0], g[1]);
+        q.y = tc::pack_bf16(g[2], g[3]);
+        q.z = tc::pack_bf16(g[4], g[5]);
+        q.w = tc::pack_bf16(g[6], g[7]);
+        *reinterpret_cast<uint4*>(As + tc::kmajor_off(row, o0 + o8, OUTP)) = q;
+        *reinterpret_cast<uint4*>(p.dY16 + b * OUTP + o0 + o8) = q;
+        float4* d32 = reinterpret_cast<float4*>(p.dY32 + b * OUTP + o0 + o8);
+        d32[0] = make_float4(g[0], g[1], g[2], g[3]);
+        d32[1] = make_float4(g[4], g[5], g[6], g[7]);
+      }
+    }
+    for (int l = 2; l >= 0; --l) {
+      const int Kl = l == 2 ? OUTP : kH, kw = l == 2 ? OUTP : kChunkK;
+      tc::fence_async_smem();  // this thread's part of the A operand
+      tc::fence_before();
+      __syncthreads();
+      tc::fence_after();
+      if (tid == 0 && !*abort_flag) {
+        const uint32_t sboA = (uint32_t)(Kl / 8) * 128, sboB = (uint32_t)(kw / 8) * 128;
+        for (int k0 = 0; k0 < Kl; k0 += kw, ++used) {
+          const int slot = (int)(used % NBUF);
+          if (!tc::mbar_wait(&bar_w[slot], (uint32_t)(used / NBUF) & 1u, p.err, 16)) {
+            *abort_flag = 1;
+            break;
+          }
+          const uint64_t ad = tc::desc_kmajor(tc::smem_u32(As) + (k0 / 8) * 128, 128, sboA);
+          const uint64_t bd = tc::desc_kmajor(tc::smem_u32(Wb + slot * BUF), 128, sboB);
+          for (int s = 0; s < kw / 16; ++s)
+            tc::mma_bf16(tmem, ad + (uint64_t)(16 * s), bd + (uint64_t)(16 * s),
+                         tc::idesc_bf16(kTile, kH), (k0 > 0 || s > 0) ? 1u : 0u);
+        }
+        tc::commit(&bar_mma);  // also after an abort: the products issued so far
+      }
+      // every thread waits for the layer's products (lane 0 of each warp, then the warp)
+      if (lane == 0 && !*abort_flag && !tc::mbar_wait(&bar_mma, ph_mma, p.err, 16))
+        *abort_flag = 1;
+      ph_mma ^= 1;
+      __syncthreads();
+      if (*abort_flag) break;  // uniform: read after the barrier, written before it
+      tc::fence_after();
+      if (tid == 0) {
+        done = used;
+        top_up();
+      }
+      const __nv_bfloat16* hrow = p.Hs[l] + (r0 + trow) * kH;
+      __nv_bfloat16* z16 = p.dZ16[l] + (r0 + trow) * kH;
+      float* z32 = p.dZ32[l] + (r0 + trow) * kH;
+      const uint32_t taddr = tmem + ((uint32_t)(quarter * 32) << 16);
+#pragma unroll
+      for (int pass = 0; pass < 4; ++pass) {
+        const int c0 = half * 128 + pass * 32;
+        uint32_t r[32];
+        tc::tmem_ld32_nowait(taddr + c0, r);
+        uint4 h[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) h[u] = *reinterpret_cast<const uint4*>(hrow + c0 + 8 * u);
+        tc::ld_wait(r);
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const uint32_t hw[4] = {h[u].x, h[u].y, h[u].z, h[u].w};
+          float g[8];
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {  // h >= 0: its bits are nonzero where it is positive
+            g[2 * i] = (hw[i] & 0x7fffu) ? __uint_as_float(r[8 * u + 2 * i]) : 0.0f;
+            g[2 * i + 1] = (hw[i] & 0x7fff0000u) ? __uint_as_float(r[8 * u + 2 * i + 1]) : 0.0f;
+          }
+          uint4 q;
+          q.x = tc::pack_bf16(g[0], g[1]);
+          q.y = tc::pack_bf16(g[2], g[3]);
+          q.z = tc::pack_bf16(g[4], g[5]);
+          q.w = tc::pack_bf16(g[6], g[7]);
+          if (l > 0) *reinterpret_cast<uint4*>(As + tc::kmajor_off(trow, c0 + 8 * u, kH)) = q;
+          *reinterpret_cast<uint4*>(z16 + c0 + 8 * u) = q;
+          *reinterpret_cast<float4*>(z32 + c0 + 8 * u) = make_float4(g[0], g[1], g[2], g[3]);
+          *reinterpret_cast<float4*>(z32 + c0 + 8 * u + 4) = make_float4(g[4], g[5], g[6], g[7]);
+        }
+      }
+      tc::fence_before();
+    }
+    __syncthreads();  // the tensor memory and As may be written for the next tile
+    if (*abort_flag) break;
+  }
+  for (int o = 16; o > 0; o >>= 1) acc_loss += __shfl_xor_sync(0xffffffffu, acc_loss, o);
+  if (lane == 0) s_loss[warp] = acc_loss;
+  tc::fence_before();
+  __syncthreads();
+  tc::fence_after();
+  if (tid == 0) {
+    double sum = 0.0;
+    for (int w = 0; w < kBackThreads / 32; ++w) sum += s_loss[w];
+    atomicAdd(p.loss, sum);
+    // after an abort: the copies in flight land before the CTA leaves (their last phase each);
+    // the products were committed before the abort was seen
+    if (*abort_flag) {
+      for (int b = 0; b < NBUF; ++b) {
+        const int64_t uses = issued / NBUF + (b < issued % NBUF ? 1 : 0);
+        if (uses) tc::mbar_wait(&bar_w[b], (uint32_t)(uses - 1) & 1u, p.err, 0);
+      }
+      if (my_tiles > 0) tc::mbar_wait(&bar_mma, ph_mma ^ 1u, p.err, 0);
+    }
+  }
+  __syncthreads();
+  if (warp == 0) tc::tmem_dealloc(tmem, kH);
+}
+
+// Weight gradients dW_l = dZ_l^T a_{l-1} and bias gradients (column sums of dZ_l).
+//
+// A weight block computes one 128 x 32 output tile over the whole batch, 64 rows a stage: layer 0
+// with M = n (rows of W_1) and N = k, layers 1..3 with M = k (columns of a_{l-1}) and N = n, so
+// that a warp stores consecutive floats. Both operands are row-major [batch x columns] in
+// memory, i.e. MN-major for a product whose K dimension is the batch: 16-byte pieces (8 columns
+// of one row) go straight into MN-major core matrices (8 batch rows x 16 bytes), and nothing is
+// transposed. Core matrices lie 160 bytes apart along MN, so that the eight threads of a
+// quarter-warp store, which write 2 rows x 4 pieces, touch every bank once.
+// The tiles, not the batch, are split over the blocks: each weight's gradient stays one FP32
+// accumulation in batch order. Narrow tiles (N = 32) keep a block's traffic near that of its
+// 128-wide operand (20 KiB a stage): a block is bound by its own loads from L2, 1.3 MB at a
+// batch of 4096. The other blocks add the bias columns, a share of the rows each, in unevaluated
+// sums of three floats (error-free two-sums), which round to the same float as FP64 sums.
+constexpr int kWgThreads = 256, kWgStages = 7, kWgRows = 64, kWgN = 32;
+constexpr int kBiasChunks = 28;  // row shares: with the weight blocks, one block per SM
+constexpr int kWgMN = 160;       // bytes between core matrices along MN
+constexpr int kWgKA = (kTile / 8) * kWgMN, kWgKB = (kWgN / 8) * kWgMN;  // and along K
+constexpr int kWgStage = (kWgKA + kWgKB) * (kWgRows / 8);               // 25 600
+constexpr size_t kWgSmem = (size_t)kWgStages * kWgStage;
+struct WgradParams {
+  const __nv_bfloat16* X16;
+  const __nv_bfloat16* Hs[3];
+  const __nv_bfloat16* dZ16[3];
+  const __nv_bfloat16* dY16;
+  const float* dZ32[3];
+  const float* dY32;
+  float* g;     // flat gradient
+  double* wsb;  // [kBiasChunks x (3 * 256 + OUTP)] partial bias gradients
+  int64_t w_off[4];
+  int64_t B;
+  int* err;
+};
+template <int D>
+constexpr int wgrad_units() {  // 128 x 32 tiles of the four layers
+  return 2 * (FusedCfg<D>::K0 / kWgN + 2 * (kH / kWgN) + FusedCfg<D>::OUTP / kWgN);
+}
+
+// MN-major operand descriptor (no swizzle): stride between core matrices along MN, and along K.
+__device__ __forceinline__ uint64_t desc_mnmajor(uint32_t addr, uint32_t mn_stride,
+                                                 uint32_t k_stride) {
+  return tc::desc_kmajor(addr, k_stride, mn_stride);
+}
+
+template <int D>
+__global__ void __launch_bounds__(kWgThreads, 1) k_wgrad(WgradParams p) {
+  using Cfg = FusedCfg<D>;
+  constexpr int K0 = Cfg::K0, OUTP = Cfg::OUTP;
+  constexpr int NB = 3 * kH + OUTP;  // bias columns
+  constexpr int U0 = 2 * (K0 / kWgN), U1 = 2 * (kH / kWgN), UNITS = wgrad_units<D>();
+  extern __shared__ __align__(1024) uint8_t smem[];
+  __shared__ __align__(8) uint64_t bar[kWgStages];
+  __shared__ uint32_t tslot;
+  __shared__ int s_abort;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  if ((int)blockIdx.x >= UNITS) {
+    // ---- bias columns: one block per (layer, share of the rows), one thread per column ----
+    const int q = (int)blockIdx.x - UNITS, l = q & 3, ch = q >> 2;
+    const int cols = l < 3 ? kH : OUTP;
+    const float* src = l < 3 ? p.dZ32[l] : p.dY32;
+    if (tid >= cols) return;
+    int64_t b = p.B * ch / kBiasChunks;
+    const int64_t b1 = p.B * (ch + 1) / kBiasChunks;
+    float s0 = 0.0f, s1 = 0.0f, s2 = 0.0f;
+    auto two_sum = [](float& s, float x) {  // s += x exactly: returns the rounding error
+      const float t = __fadd_rn(s, x), bb = __fsub_rn(t, s);
+      const float e = __fadd_rn(__fsub_rn(s, __fsub_rn(t, bb)), __fsub_rn(x, bb));
+      s = t;
+      return e;
+    };
+    auto add = [&](float x) { s2 = __fadd_rn(s2, two_sum(s1, two_sum(s0, x))); };
+    for (; b + 16 <= b1; b += 16) {
+      float x[16];
+#pragma unroll
+      for (int k = 0; k < 16; ++k) x[k] = __ldg(src + (b + k) * cols + tid);
+#pragma unroll
+      for (int k = 0; k < 16; ++k) add(x[k]);
+    }
+    for (; b < b1; ++b) add(__ldg(src + b * cols + tid));
+    p.wsb[(int64_t)ch * NB + l * kH + tid] = ((double)s0 + (double)s1) + (double)s2;
+    return;
+  }
+  int u = blockIdx.x, l = 0;
+  if (u >= U0) {
+    u -= U0;
+    l = 1;
+    while (l < 3 && u >= U1) {
+      u -= U1;
+      ++l;
+    }
+  }
+  const int m0 = (u & 1) * kTile, n0 = (u >> 1) * kWgN;
+  if (tid == 0) {
+    for (int s = 0; s < kWgStages; ++s) tc::mbar_init(&bar[s], 1);
+    s_abort = 0;
+  }
+  if (warp == 0) tc::tmem_alloc(&tslot, kWgN);
+  tc::fence_before();
+  __syncthreads();
+  tc::fence_after();
+  const uint32_t tmem = tslot;
+  volatile int* abort_flag = &s_abort;
+  const __nv_bfloat16* Asrc = l == 0 ? p.dZ16[0] : p.Hs[l - 1];  // [B x 256]
+  const __nv_bfloat16* Bsrc = l == 0 ? p.X16 : (l == 3 ? p.dY16 : p.dZ16[l]);
+  const int ldb = l == 0 ? K0 : (l == 3 ? OUTP : kH);
+  const int steps = (int)(p.B / kWgRows);
+  // stage loads: e -> (4 consecutive pieces) x (64 rows) x (groups of 4 pieces); 16 pieces of
+  // A and 4 of B per row
+  auto load = [&](int g) {
+    uint8_t* sa = smem + (g % kWgStages) * kWgStage;
+    const int r = (tid >> 2) % kWgRows;
+    const int64_t row = (int64_t)g * kWgRows + r;
+    const uint32_t at = tc::smem_u32(sa) + (tid & 3) * kWgMN + (r & 7) * 16;
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+      asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(
+                       at + (r >> 3) * kWgKA + q * 4 * kWgMN),
+                   "l"(Asrc + row * kH + m0 + 8 * ((tid & 3) + 4 * q))
+                   : "memory");
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(
+                     at + kWgKA * (kWgRows / 8) + (r >> 3) * kWgKB),
+                 "l"(Bsrc + row * ldb + n0 + 8 * (tid & 3))
+                 : "memory");
+  };
+  for (int i = 0; i < kWgStages - 1; ++i) {
+    if (i < steps) load(i);
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  }
+  constexpr uint32_t idesc =
+      tc::idesc_bf16(kTile, kWgN) | (1u << 15) | (1u << 16);  // MN-major A and B
+  for (int i = 0; i < steps; ++i) {
+    const int nx = i + kWgStages - 1;
+    if (nx < steps) {
+      // the stage of step nx is free once the products of step nx - stages have completed
+      if (nx >= kWgStages && lane == 0 && !*abort_flag &&
+          !tc::mbar_wait(&bar[nx % kWgStages], (uint32_t)(nx / kWgStages - 1) & 1u, p.err, 16))
+        *abort_flag = 1;
+      __syncwarp();
+      load(nx);
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+    asm volatile("cp.async.wait_group %0;" ::"n"(kWgStages - 1) : "memory");
+    tc::fence_async_smem();
+    __syncthreads();
+    if (tid == 0) {
+      const uint32_t sa = tc::smem_u32(smem + (i % kWgStages) * kWgStage);
+      const uint32_t sb = sa + kWgKA * (kWgRows / 8);
+      tc::fence_after();
+      if (!*abort_flag)
+        for (int s = 0; s < kWgRows / 16; ++s)
+          tc::mma_bf16(tmem, desc_mnmajor(sa + 2 * s * kWgKA, kWgMN, kWgKA),
+                       desc_mnmajor(sb + 2 * s * kWgKB, kWgMN, kWgKB), idesc,
+                       (i > 0 || s > 0) ? 1u : 0u);
+      tc::commit(&bar[i % kWgStages]);
+    }
+  }
+  asm volatile("cp.async.wait_group 0;" ::: "memory");
+  // the last step's commit completes after every earlier product; it is waited for (bounded)
+  // after an abort as well, before the tensor memory is released
+  if (lane == 0 && !tc::mbar_wait(&bar[(steps - 1) % kWgStages],
+                                  (uint32_t)((steps - 1) / kWgStages) & 1u, p.err, 16))
+    *abort_flag = 1;
+  __syncthreads();
+  tc::fence_after();
+  if (warp < 4 && !*abort_flag) {
+    const int m = m0 + warp * 32 + lane;
+    uint32_t r[32];
+    tc::tmem_ld32_nowait(tmem + ((uint32_t)(warp * 32) << 16), r);
+    tc::ld_wait(r);
+    float* out = p.g + p.w_off[l];
+    if (l == 0) {
+#pragma unroll
+      for (int i = 0; i < 32; i += 4)
+        *reinterpret_cast<float4*>(out + (int64_t)m * K0 + n0 + i) =
+            make_float4(__uint_as_float(r[i]), __uint_as_float(r[i + 1]),
+                        __uint_as_float(r[i + 2]), __uint_as_float(r[i + 3]));
+    } else {
+#pragma unroll
+      for (int i = 0; i < 32; ++i) out[(int64_t)(n0 + i) * kH + m] = __uint_as_float(r[i]);
     }
   }
   tc::fence_before();
   __syncthreads();
-  if (warp == 0) tc::tmem_dealloc(tmem, NT_MAX);
+  if (warp == 0) tc::tmem_dealloc(tmem, kWgN);
 }
 
-// ---- elementwise kernels of the training step ----------------------------------------------
-// dY = 2 (y - t_norm) / (B * OUT) on the OUT real outputs (0 on padding), bf16 row-major and
-// transposed ([128 x B], rows >= OUT zero); loss partial sums in double.
-__global__ void k_loss_grad(const float* __restrict__ Y, const float* __restrict__ Traw,
-                            const float* __restrict__ params, int64_t norm_off, int64_t B,
-                            int OUT, int OUTP, __nv_bfloat16* __restrict__ dY,
-                            __nv_bfloat16* __restrict__ dYT, float* __restrict__ dY32,
-                            double* __restrict__ loss) {
-  double acc = 0.0;
-  const double scale = 2.0 / ((double)B * OUT);
-  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < B * OUTP;
-       e += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t b = e / OUTP;
-    const int o = (int)(e - b * OUTP);
-    float g = 0.0f;
-    if (o < OUT) {
-      const float mu = params[norm_off + 2 + o], sg = params[norm_off + 2 + OUTP + o];
-      const float t = (Traw[b * OUT + o] - mu) / sg;
-      const float r = Y[e] - t;
-      acc += (double)r * r;
-      g = (float)(scale * r);
-    }
-    dY[e] = __float2bfloat16(g);
-    dY32[e] = g;
-    dYT[(int64_t)o * B + b] = __float2bfloat16(g);
+// Bias gradients from their partial sums, then, when apply is set and no wait of the step gave
+// up, Adam and the bf16 copies of the weights. Also reports the loss and the error word.
+__global__ void k_update(float* __restrict__ w, float* __restrict__ g, float* __restrict__ m,
+                         float* __restrict__ v, const double* __restrict__ wsb, Layout L,
+                         WeightStreams st, const int* __restrict__ err, int apply, float lr,
+                         float b1, float b2, float eps, float c1, float c2,
+                         const double* __restrict__ loss, double* __restrict__ host) {
+  const bool step = apply && *err == 0;
+  if (blockIdx.x == 0 && threadIdx.x == 0) {  // page-locked host memory, read after the wait
+    host[0] = *loss;
+    host[1] = (double)*err;
   }
-  for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-  if ((threadIdx.x & 31) == 0) atomicAdd(loss, acc);
-}
-
-// dZ = dH * a'(Z) (fp32 in), bf16 row-major and transposed copies.
-__global__ void k_silu_back(const float* __restrict__ dH, const float* __restrict__ Z, int64_t B,
-                            __nv_bfloat16* __restrict__ dZ, __nv_bfloat16* __restrict__ dZT,
-                            float* __restrict__ dZ32) {
-  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < B * kH;
-       e += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t b = e / kH;
-    const int k = (int)(e - b * kH);
-    const float g = dH[e] * act_grad(Z[e]);
-    dZ[e] = __float2bfloat16(g);
-    dZ32[e] = g;
-    dZT[(int64_t)k * B + b] = __float2bfloat16(g);
-  }
-}
-
-// Column sums of a [B x N] fp32 matrix (bias gradients), one thread per column.
-__global__ void k_colsum(const float* __restrict__ G, int64_t B, int N, float* __restrict__ out) {
-  const int c = blockIdx.x * blockDim.x + threadIdx.x;
-  if (c >= N) return;
-  double s = 0.0;
-  for (int64_t b = 0; b < B; ++b) s += G[b * N + c];
-  out[c] = (float)s;
-}
-
-// out[c][r] = in[r][c] for a [R x Cn] bf16 matrix.
-__global__ void k_transpose_bf16(const __nv_bfloat16* __restrict__ in, int64_t R, int Cn,
-                                 __nv_bfloat16* __restrict__ out) {
-  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < R * Cn;
-       e += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t r = e / Cn;
-    const int c = (int)(e - r * Cn);
-    out[(int64_t)c * R + r] = in[e];
-  }
-}
-
-// Adam on the flat parameter vector (gradients already in g).
-__global__ void k_adam(float* __restrict__ w, const float* __restrict__ g, float* __restrict__ m,
-                       float* __restrict__ v, int64_t n, float lr, float b1, float b2, float eps,
-                       float c1, float c2) {
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
+  const int NB = 3 * kH + (int)L.nN[3];
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < L.nparams;
        i += (int64_t)gridDim.x * blockDim.x) {
-    const float gi = g[i];
+    const int l = i >= L.w[3] ? 3 : i >= L.w[2] ? 2 : i >= L.w[1] ? 1 : 0;
+    const bool bias = i >= L.b[l];
+    float gi;
+    if (bias) {
+      double s = 0.0;
+      const int c = l * kH + (int)(i - L.b[l]);
+#pragma unroll
+      for (int q = 0; q < kBiasChunks; ++q) s += wsb[(int64_t)q * NB + c];
+      gi = (float)s;
+      g[i] = gi;
+    } else {
+      gi = g[i];
+    }
+    if (!step) continue;
     const float mi = b1 * m[i] + (1.0f - b1) * gi;
     const float vi = b2 * v[i] + (1.0f - b2) * gi * gi;
     m[i] = mi;
     v[i] = vi;
-    w[i] -= lr * (mi / c1) / (sqrtf(vi / c2) + eps);
-  }
-}
-
-// bf16 copies of the weights: the chunk stream of the fused kernel (canonical K-major tiles)
-// and transposed row-major copies W^T [K x N] for the backward products.
-__global__ void k_retile(const float* __restrict__ params, Layout L, ChunkPlan plan, int OUTP,
-                         uint8_t* __restrict__ tiles, __nv_bfloat16* __restrict__ WT0,
-                         __nv_bfloat16* __restrict__ WT1, __nv_bfloat16* __restrict__ WT2,
-                         __nv_bfloat16* __restrict__ WT3, __nv_bfloat16* __restrict__ W16_0,
-                         __nv_bfloat16* __restrict__ W16_1, __nv_bfloat16* __restrict__ W16_2,
-                         __nv_bfloat16* __restrict__ W16_3) {
-  __nv_bfloat16* WT[4] = {WT0, WT1, WT2, WT3};
-  __nv_bfloat16* W16[4] = {W16_0, W16_1, W16_2, W16_3};
-  for (int l = 0; l < 4; ++l) {
-    const int N = (int)L.nN[l], K = (int)L.nK[l];
-    for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < (int64_t)N * K;
-         e += (int64_t)gridDim.x * blockDim.x) {
-      const int n = (int)(e / K), k = (int)(e % K);
-      const __nv_bfloat16 x = __float2bfloat16(params[L.w[l] + e]);
-      WT[l][(int64_t)k * N + n] = x;
-      W16[l][e] = x;
-      int gi = 0;
-      for (int q = 0; q < plan.n; ++q)
-        if (plan.layer[q] == l && k >= plan.k0[q] && k < plan.k0[q] + plan.kw[q]) gi = q;
-      *reinterpret_cast<__nv_bfloat16*>(tiles + plan.off[gi] +
-                                        tc::kmajor_off(n, k - plan.k0[gi], plan.kw[gi])) = x;
-    }
+    const float wi = w[i] - lr * (mi / c1) / (sqrtf(vi / c2) + eps);
+    w[i] = wi;
+    if (!bias) store_weight(L, st.fwd_off, st.back_off, l, i - L.w[l], wi, st.tiles, st.back);
   }
 }
 
@@ -1736,13 +2012,15 @@ struct lsp_mlp {
   ChunkPlan plan;
   cudaStream_t stream = nullptr;
   std::string err;
-  lsp::DevBuf params, grads, adam_m, adam_v, tiles, WT[4], W16[4], errflag, loss;
+  lsp::DevBuf params, grads, adam_m, adam_v, tiles, back, errflag, loss;
   uint64_t wait_ns = lsp::tc::kWaitLimitNs;  // operand-wait limit of the fused kernel
   int schedule = 1;  // 2D: 1 = two tiles in flight (k_mlp_pp), 0 = one tile at a time,
                      // 2 = two 256-row tiles in flight on a CTA pair (k_mlp_pp2, rows mode)
   // training workspace
-  int64_t cap = 0;
-  lsp::DevBuf X16, XT, Xt, Zs[3], Hs[3], HT[3], Y, dY16, dYT, dY32, G, dZ16, dZT, dZ32;
+  int64_t cap = 0, bcap = 0;  // batch rows the forward / backward buffers hold
+  lsp::DevBuf X16, Xt, Hs[3], Y, dY16, dY32, dZ16[3], dZ32[3], wsb;
+  double* h_res = nullptr;      // page-locked: the loss sum and the error word of a step
+  double* h_res_dev = nullptr;  // its device address
   int64_t step = 0;
 };
 
@@ -1835,12 +2113,24 @@ cudaError_t launch_fused(lsp_mlp* m, const FusedParams& p, int64_t rows) {
   return cudaGetLastError();
 }
 
+WeightStreams weight_streams(lsp_mlp* m) {
+  WeightStreams w;
+  w.tiles = (uint8_t*)m->tiles.p;
+  w.back = (uint8_t*)m->back.p;
+  int64_t f = 0;
+  for (int l = 0; l < 4; ++l) {
+    w.fwd_off[l] = f;
+    f += m->L.wn[l] * 2;
+  }
+  w.back_off[0] = 0;  // no product with the first layer's weights
+  w.back_off[3] = 0;
+  w.back_off[2] = m->L.wn[3] * 2;
+  w.back_off[1] = w.back_off[2] + m->L.wn[2] * 2;
+  return w;
+}
+
 lsp_status retile(lsp_mlp* m) {
-  k_retile<<<152 * 4, 256, 0, m->stream>>>(
-      (const float*)m->params.p, m->L, m->plan, m->dm.OUTP, (uint8_t*)m->tiles.p,
-      (__nv_bfloat16*)m->WT[0].p, (__nv_bfloat16*)m->WT[1].p, (__nv_bfloat16*)m->WT[2].p,
-      (__nv_bfloat16*)m->WT[3].p, (__nv_bfloat16*)m->W16[0].p, (__nv_bfloat16*)m->W16[1].p,
-      (__nv_bfloat16*)m->W16[2].p, (__nv_bfloat16*)m->W16[3].p);
+  k_retile<<<152 * 4, 256, 0, m->stream>>>((const float*)m->params.p, m->L, weight_streams(m));
   MCUDA(m, cudaGetLastError());
   return LSP_OK;
 }
@@ -1857,52 +2147,43 @@ lsp_status ensure_workspace(lsp_mlp* m, int64_t B) {
   if (m->cap >= B) return LSP_OK;
   const Dims& d = m->dm;
   bool ok = grow(m->X16, sizeof(__nv_bfloat16) * B * d.K0) &&
-            grow(m->Xt, input_tile_bytes(d.d, B)) &&
-            grow(m->XT, sizeof(__nv_bfloat16) * B * d.K0) && grow(m->Y, sizeof(float) * B * d.OUTP) &&
-            grow(m->dY16, sizeof(__nv_bfloat16) * B * d.OUTP) &&
-            grow(m->dYT, sizeof(__nv_bfloat16) * B * 128) &&
-            grow(m->dY32, sizeof(float) * B * d.OUTP) && grow(m->G, sizeof(float) * B * kH) &&
-            grow(m->dZ16, sizeof(__nv_bfloat16) * B * kH) &&
-            grow(m->dZT, sizeof(__nv_bfloat16) * B * kH) && grow(m->dZ32, sizeof(float) * B * kH);
-  for (int l = 0; ok && l < 3; ++l)
-    ok = grow(m->Zs[l], sizeof(float) * B * kH) && grow(m->Hs[l], sizeof(__nv_bfloat16) * B * kH) &&
-         grow(m->HT[l], sizeof(__nv_bfloat16) * B * kH);
+            grow(m->Xt, input_tile_bytes(d.d, B)) && grow(m->Y, sizeof(float) * B * d.OUTP);
+  for (int l = 0; ok && l < 3; ++l) ok = grow(m->Hs[l], sizeof(__nv_bfloat16) * B * kH);
   if (!ok) return mfail(m, LSP_ERR_OOM, "training workspace allocation failed");
   m->cap = B;
   return LSP_OK;
 }
 
-cudaError_t gemm(lsp_mlp* m, const void* A, const void* B, float* C, int M, int N, int K) {
-  // 48 KiB of staging is enough; asking for 100 KiB keeps at most two CTAs per SM, so their two
-  // 256-column tensor-memory allocations always fit in the SM's 512 columns.
-  const size_t smem = 100 * 1024;
-  cudaError_t e =
-      cudaFuncSetAttribute(k_gemm_tn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
-  dim3 grid(M / 128, (N + 255) / 256);
-  k_gemm_tn<<<grid, 128, smem, m->stream>>>((const __nv_bfloat16*)A, (const __nv_bfloat16*)B, C, M,
-                                            N, K, (int*)m->errflag.p);
-  return cudaGetLastError();
+// Buffers of the backward pass (a forward call alone does not need them).
+lsp_status ensure_backward(lsp_mlp* m, int64_t B) {
+  if (m->bcap >= B) return LSP_OK;
+  const Dims& d = m->dm;
+  bool ok = grow(m->dY16, sizeof(__nv_bfloat16) * B * d.OUTP) &&
+            grow(m->dY32, sizeof(float) * B * d.OUTP) &&
+            grow(m->wsb, sizeof(double) * kBiasChunks * (3 * kH + d.OUTP));
+  for (int l = 0; ok && l < 3; ++l)
+    ok = grow(m->dZ16[l], sizeof(__nv_bfloat16) * B * kH) &&
+         grow(m->dZ32[l], sizeof(float) * B * kH);
+  if (!ok) return mfail(m, LSP_ERR_OOM, "training workspace allocation failed");
+  m->bcap = B;
+  return LSP_OK;
 }
 
 // Training-mode forward: normalised bf16 inputs (canonical tiles and row-major), then the fused
-// network, saving z and h of every hidden layer.
+// network, saving h of every hidden layer.
 cudaError_t batch_forward(lsp_mlp* m, const float* X_dev, int64_t batch, float* Y_dev) {
   FusedParams p = fused_params(m);
   p.M = batch;
   p.Xt = (const uint8_t*)m->Xt.p;
   p.Y = Y_dev;
-  for (int l = 0; l < 3; ++l) {
-    p.Zs[l] = (float*)m->Zs[l].p;
-    p.Hs[l] = (__nv_bfloat16*)m->Hs[l].p;
-  }
+  for (int l = 0; l < 3; ++l) p.Hs[l] = (__nv_bfloat16*)m->Hs[l].p;
   __nv_bfloat16* X16 = (__nv_bfloat16*)m->X16.p;
   if (m->dm.d == 2)
     k_inputs_batch<2><<<152 * 8, 256, 0, m->stream>>>(X_dev, p.params, p.norm_off, batch,
-                                                      (uint8_t*)p.Xt, X16);
+                                                      (uint8_t*)p.Xt, X16, (double*)m->loss.p);
   else
     k_inputs_batch<3><<<152 * 8, 256, 0, m->stream>>>(X_dev, p.params, p.norm_off, batch,
-                                                      (uint8_t*)p.Xt, X16);
+                                                      (uint8_t*)p.Xt, X16, (double*)m->loss.p);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   return m->dm.d == 2 ? launch_fused<2, kModeBatch>(m, p, batch)
@@ -1926,10 +2207,13 @@ lsp_status lsp_mlp_create(int d, uint64_t seed, void* cuda_stream, lsp_mlp** out
   bool ok = grow(m->params, sizeof(float) * P) && grow(m->grads, sizeof(float) * P) &&
             grow(m->adam_m, sizeof(float) * P) && grow(m->adam_v, sizeof(float) * P) &&
             grow(m->tiles, (size_t)m->plan.total_bytes) && grow(m->errflag, 64) &&
-            grow(m->loss, 64);
-  for (int l = 0; ok && l < 4; ++l)
-    ok = grow(m->WT[l], sizeof(__nv_bfloat16) * m->L.wn[l]) &&
-         grow(m->W16[l], sizeof(__nv_bfloat16) * m->L.wn[l]);
+            grow(m->loss, 64) &&
+            grow(m->back, sizeof(__nv_bfloat16) * (m->L.wn[1] + m->L.wn[2] + m->L.wn[3]));
+  if (ok && (cudaMallocHost(&m->h_res, 2 * sizeof(double)) != cudaSuccess ||
+             cudaHostGetDevicePointer((void**)&m->h_res_dev, m->h_res, 0) != cudaSuccess)) {
+    cudaGetLastError();
+    ok = false;
+  }
   if (!ok) {
     lsp_mlp_destroy(m);
     return LSP_ERR_OOM;
@@ -1980,19 +2264,15 @@ lsp_status lsp_mlp_destroy(lsp_mlp* m) {
   if (!m) return LSP_OK;
   cudaStreamSynchronize(m->stream);
   lsp::DevBuf* bufs[] = {&m->params, &m->grads, &m->adam_m, &m->adam_v, &m->tiles, &m->errflag,
-                         &m->loss, &m->X16, &m->XT, &m->Xt, &m->Y, &m->dY16, &m->dYT, &m->dY32, &m->G,
-                         &m->dZ16, &m->dZT, &m->dZ32};
+                         &m->loss, &m->back, &m->X16, &m->Xt, &m->Y, &m->dY16, &m->dY32, &m->wsb};
   for (auto* b : bufs)
     if (b->p) cudaFree(b->p);
-  for (int l = 0; l < 4; ++l) {
-    if (m->WT[l].p) cudaFree(m->WT[l].p);
-    if (m->W16[l].p) cudaFree(m->W16[l].p);
-  }
   for (int l = 0; l < 3; ++l) {
-    if (m->Zs[l].p) cudaFree(m->Zs[l].p);
     if (m->Hs[l].p) cudaFree(m->Hs[l].p);
-    if (m->HT[l].p) cudaFree(m->HT[l].p);
+    if (m->dZ16[l].p) cudaFree(m->dZ16[l].p);
+    if (m->dZ32[l].p) cudaFree(m->dZ32[l].p);
   }
+  if (m->h_res) cudaFreeHost(m->h_res);
   delete m;
   return LSP_OK;
 }
@@ -2051,64 +2331,62 @@ lsp_status lsp_mlp_train_step(lsp_mlp* m, const float* X_dev, const float* T_dev
   const Layout& L = m->L;
   lsp_status st = ensure_workspace(m, batch);
   if (st != LSP_OK) return st;
-  // forward (saves z, h, and the normalised bf16 inputs)
+  if ((st = ensure_backward(m, batch)) != LSP_OK) return st;
+  // forward (saves h and the normalised bf16 inputs)
   MCUDA(m, batch_forward(m, X_dev, batch, (float*)m->Y.p));
-  // loss and dY
-  MCUDA(m, cudaMemsetAsync(m->loss.p, 0, sizeof(double), m->stream));
-  MCUDA(m, cudaMemsetAsync(m->dYT.p, 0, sizeof(__nv_bfloat16) * 128 * batch, m->stream));
-  k_loss_grad<<<152 * 4, 256, 0, m->stream>>>(
-      (const float*)m->Y.p, T_dev, (const float*)m->params.p, L.norm, batch, d.OUT, d.OUTP,
-      (__nv_bfloat16*)m->dY16.p, (__nv_bfloat16*)m->dYT.p, (float*)m->dY32.p,
-      (double*)m->loss.p);
-  MCUDA(m, cudaGetLastError());
-  float* g = (float*)m->grads.p;
-  MCUDA(m, cudaMemsetAsync(g, 0, sizeof(float) * L.total, m->stream));
-  // layer 4: dW4 = dY^T h3 (M padded to 128), db4 = colsum(dY), dH3 = dY W4
-  for (int l = 0; l < 3; ++l)
-    k_transpose_bf16<<<152 * 4, 256, 0, m->stream>>>((const __nv_bfloat16*)m->Hs[l].p, batch, kH,
-                                                     (__nv_bfloat16*)m->HT[l].p);
-  k_transpose_bf16<<<152 * 4, 256, 0, m->stream>>>((const __nv_bfloat16*)m->X16.p, batch, d.K0,
-                                                   (__nv_bfloat16*)m->XT.p);
-  float* G = (float*)m->G.p;  // [>= 128 x 256] scratch for weight gradients / [B x 256] for dH
-  MCUDA(m, gemm(m, m->dYT.p, m->HT[2].p, G, 128, kH, (int)batch));
-  MCUDA(m, cudaMemcpyAsync(g + L.w[3], G, sizeof(float) * d.OUTP * kH, cudaMemcpyDeviceToDevice,
-                           m->stream));
-  k_colsum<<<1, 128, 0, m->stream>>>((const float*)m->dY32.p, batch, d.OUTP, g + L.b[3]);
-  // dH3 = dY W4: A = dY [B x OUTP], B-operand = W4^T [256 x OUTP]
-  MCUDA(m, gemm(m, m->dY16.p, m->WT[3].p, G, (int)batch, kH, d.OUTP));
-  for (int l = 2; l >= 0; --l) {
-    k_silu_back<<<152 * 4, 256, 0, m->stream>>>(G, (const float*)m->Zs[l].p, batch,
-                                                (__nv_bfloat16*)m->dZ16.p,
-                                                (__nv_bfloat16*)m->dZT.p, (float*)m->dZ32.p);
-    MCUDA(m, cudaGetLastError());
-    k_colsum<<<2, 128, 0, m->stream>>>((const float*)m->dZ32.p, batch, kH, g + L.b[l]);
-    // dW_l = dZ^T a_{l-1}: A = dZ^T [256 x B], B-operand = a_{l-1}^T [K_l x B]
-    const void* prevT = l == 0 ? m->XT.p : m->HT[l - 1].p;
-    const int Kl = (int)L.nK[l];
-    MCUDA(m, gemm(m, m->dZT.p, prevT, g + L.w[l], kH, Kl, (int)batch));
-    if (l > 0) {
-      // dH_{l-1} = dZ W_l: A = dZ [B x 256], B-operand = W_l^T [256 x 256]
-      MCUDA(m, gemm(m, m->dZ16.p, m->WT[l].p, G, (int)batch, kH, kH));
-    }
+  BackParams bp;
+  WgradParams wp;
+  bp.Y = (const float*)m->Y.p;
+  bp.T = T_dev;
+  bp.params = (const float*)m->params.p;
+  bp.back = (const uint8_t*)m->back.p;
+  bp.dY16 = (__nv_bfloat16*)m->dY16.p;
+  bp.dY32 = (float*)m->dY32.p;
+  bp.loss = (double*)m->loss.p;
+  bp.err = wp.err = (int*)m->errflag.p;
+  bp.B = wp.B = batch;
+  bp.norm_off = L.norm;
+  wp.X16 = (const __nv_bfloat16*)m->X16.p;
+  wp.dY16 = bp.dY16;
+  wp.dY32 = bp.dY32;
+  for (int l = 0; l < 3; ++l) {
+    bp.Hs[l] = wp.Hs[l] = (const __nv_bfloat16*)m->Hs[l].p;
+    wp.dZ16[l] = bp.dZ16[l] = (__nv_bfloat16*)m->dZ16[l].p;
+    wp.dZ32[l] = bp.dZ32[l] = (float*)m->dZ32[l].p;
   }
-  double loss = 0;
-  MCUDA(m, cudaMemcpyAsync(&loss, m->loss.p, sizeof(double), cudaMemcpyDeviceToHost, m->stream));
-  st = check_err(m);
-  if (st != LSP_OK) return st;
-  if (loss_out) *loss_out = (float)(loss / ((double)batch * d.OUT));
+  float* g = (float*)m->grads.p;
+  wp.g = g;
+  wp.wsb = (double*)m->wsb.p;
+  for (int l = 0; l < 4; ++l) wp.w_off[l] = L.w[l];
+  const int grid = (int)std::min<int64_t>(152, batch / kTile);
+  const size_t smem_b = kTile * kH * 2 + 4 * kH * kChunkK * 2;
+  auto back = [&](auto kb, auto kw, int units) -> cudaError_t {
+    cudaError_t e =
+        cudaFuncSetAttribute(kb, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_b);
+    if (e != cudaSuccess) return e;
+    kb<<<grid, kBackThreads, smem_b, m->stream>>>(bp);
+    e = cudaFuncSetAttribute(kw, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kWgSmem);
+    if (e != cudaSuccess) return e;
+    kw<<<units + 4 * kBiasChunks, kWgThreads, kWgSmem, m->stream>>>(wp);
+    return cudaGetLastError();
+  };
+  MCUDA(m, d.d == 2 ? back(k_backward<2>, k_wgrad<2>, wgrad_units<2>())
+                    : back(k_backward<3>, k_wgrad<3>, wgrad_units<3>()));
+  const float b1 = 0.9f, b2 = 0.999f;
+  const float c1 = 1.0f - powf(b1, (float)(m->step + 1));
+  const float c2 = 1.0f - powf(b2, (float)(m->step + 1));
+  k_update<<<152 * 4, 256, 0, m->stream>>>(
+      (float*)m->params.p, g, (float*)m->adam_m.p, (float*)m->adam_v.p, wp.wsb, L,
+      weight_streams(m), wp.err, apply ? 1 : 0, lr, b1, b2, 1e-8f, c1, c2, bp.loss,
+      m->h_res_dev);
+  MCUDA(m, cudaGetLastError());
+  MCUDA(m, cudaStreamSynchronize(m->stream));
+  if (m->h_res[1] != 0.0)
+    return mfail(m, LSP_ERR_TIMEOUT, "a tensor-core wait gave up (bits %d)", (int)m->h_res[1]);
+  if (apply) ++m->step;
+  if (loss_out) *loss_out = (float)(m->h_res[0] / ((double)batch * d.OUT));
   if (grads_host)
     MCUDA(m, cudaMemcpy(grads_host, g, sizeof(float) * L.nparams, cudaMemcpyDeviceToHost));
-  if (apply) {
-    ++m->step;
-    const float b1 = 0.9f, b2 = 0.999f;
-    const float c1 = 1.0f - powf(b1, (float)m->step), c2 = 1.0f - powf(b2, (float)m->step);
-    k_adam<<<152 * 4, 256, 0, m->stream>>>((float*)m->params.p, g, (float*)m->adam_m.p,
-                                           (float*)m->adam_v.p, L.nparams, lr, b1, b2, 1e-8f, c1,
-                                           c2);
-    MCUDA(m, cudaGetLastError());
-    st = retile(m);
-    if (st != LSP_OK) return st;
-  }
   return LSP_OK;
 }
 

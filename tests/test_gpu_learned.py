@@ -184,6 +184,46 @@ def test_forward_and_gradients_match_oracle(stream, d):
     assert flagged.sum() <= B // 16  # a few boundary cases, not a systematic difference
 
 
+@pytest.mark.parametrize("d", [2, 3])
+@pytest.mark.parametrize("tiles", [1, 4, 9, 155])
+def test_gradient_of_a_batch_is_the_mean_over_its_tiles(stream, d, tiles):
+    """The backward kernels at their edges: one tile (two 64-row stages, fewer than the buffers),
+    a power of two of tiles, a stage count that is no multiple of the buffers, and more tiles
+    than SMs (two tiles per CTA).
+
+    The gradient of a batch is the mean of the gradients of its 128-row tiles. With a power of
+    two of tiles the scale 2 / (B OUT) changes by a power of two, so every bf16 value scales
+    exactly and only the FP32 order differs (at most B 2^-24 of the terms' magnitudes, taken with
+    a factor 8 for their cancellation); otherwise each bf16 dZ may round differently, 2^-8."""
+    import torch
+    from paper_1607_02560_gb300 import Mlp
+    mlp = Mlp(d, seed=9, stream=stream)
+    X, T = (pool_2d if d == 2 else pool_3d)(mlp, stream, samples=12288)
+    torch.cuda.synchronize()
+    mlp.fit_normalization(X, T, X.shape[0])
+    B = 128 * tiles
+    X, T = X[:B].contiguous(), T[:B].contiguous()
+    assert X.shape[0] == B
+    torch.cuda.synchronize()
+    g = np.empty(mlp.nweights, dtype=np.float32)
+    loss = mlp.train_step(X, T, B, 0.0, apply=False, grads=g)
+    ref, loss_ref, part = np.zeros(mlp.nweights), 0.0, np.empty_like(g)
+    for k in range(tiles):
+        rows = slice(128 * k, 128 * (k + 1))
+        loss_ref += mlp.train_step(X[rows], T[rows], 128, 0.0, apply=False, grads=part) / tiles
+        ref += part.astype(np.float64) / tiles
+    tol = 8 * B * 2.0 ** -24 if tiles & (tiles - 1) == 0 else 2.0 ** -8
+    assert abs(loss - loss_ref) <= 1e-5 * loss_ref
+    off = 0
+    k0, outp = mlp.k0, mlp.outp
+    for rows, cols in ((256, k0), (256, 256), (256, 256), (outp, 256)):
+        for size in (rows * cols, rows):  # weights, then biases
+            a, b = g[off:off + size], ref[off:off + size]
+            assert np.linalg.norm(a - b) <= tol * np.linalg.norm(b), (rows, cols, size)
+            off += size
+    assert off == mlp.nweights
+
+
 @pytest.mark.parametrize("n", [8, 16, 64, 256, 1024])
 def test_two_tiles_in_flight_give_the_same_rows(stream, n):
     """The 2D inference kernels with two tiles in flight per SM (schedule 1) and with two
