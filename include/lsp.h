@@ -325,9 +325,8 @@ void lsp_inject_alloc_failure(int after);
  * pool or framework allocator that must not see extra allocations or device-wide syncs.
  * The paper has no counterpart; this is a deployment variant of the same operator.
  *
- * Nothing is allocated: the transform's complex work array is a fixed array inside the
- * library (16 MiB plus 32 KiB of twiddles, held on every GPU that loads the library until the
- * process exits). The caller passes all inputs and outputs as device pointers to n^d float64
+ * Nothing is allocated: the operator's scratch is a fixed array inside the library (8 MiB plus
+ * 24 KiB of tables, held on every GPU that loads the library until the process exits). The caller passes all inputs and outputs as device pointers to n^d float64
  * values: the potential v, the input u and the output y (y may alias u). d in {2, 3}, n a power
  * of two >= 8, and n^d <= LSP_NOALLOC_MAX_POINTS; larger grids return LSP_ERR_ARG (use a
  * context). The work is issued on cuda_stream (a cudaStream_t; NULL = legacy default stream).

@@ -586,12 +586,15 @@ lsp_status lsp_create(int d, int n, void* cuda_stream, lsp_ctx** out) {
         const long double wgt = (p == 0 || p == n / 2) ? 1.0L : 2.0L;
         X[a * P + p] = (double)(wgt * cos_r(a * p));
       }
-    // twiddles exp(-2 pi i j / n), j < n/2
-    std::vector<double> tw(n);
-    for (int j = 0; j < n / 2; ++j) {
-      const long double ang = two_pi * (long double)j / (long double)n;
-      tw[2 * j] = (double)cosl(ang);
-      tw[2 * j + 1] = (double)(-sinl(ang));
+    // the axis table of the operator: exp(-2 pi i j / n), j < n, then 4 pi^2 k^2 / n, k < n in
+    // FFT order (the sine is the cosine a quarter period later, so both have the exact
+    // symmetries of cos_r)
+    std::vector<double> tw(3 * (size_t)n);
+    for (int j = 0; j < n; ++j) {
+      tw[2 * j] = (double)cos_r(j);
+      tw[2 * j + 1] = (double)cos_r(j + n / 4);  // -sin(t) = cos(t + pi / 2)
+      const double k = j < n / 2 ? (double)j : (double)(j - n);
+      tw[2 * (size_t)n + j] = 4.0 * kPi2 * (k * k) / (double)n;
     }
     std::vector<float> X32(X.begin(), X.end());
     // double words of the same values, split from the extended-precision cosines
@@ -986,7 +989,7 @@ lsp_status lsp_apply_operator(lsp_ctx* c, const double* u, double* y) {
   cudaGetLastError();
   if (!u || !y) return fail(c, LSP_ERR_ARG, "u or y is NULL");
   if (!c->have_v) return fail(c, LSP_ERR_STATE, "apply_operator before set_potential");
-  if (!ensure(c, c->fftbuf, sizeof(double) * 2 * c->geo.N)) return LSP_ERR_OOM;
+  if (!ensure(c, c->fftbuf, sizeof(double) * c->geo.N)) return LSP_ERR_OOM;
   CUDA_OK(c, launch_apply(c, u, y));
   return LSP_OK;
 }

@@ -293,7 +293,7 @@ lsp_status lsp_gmres(lsp_ctx* c, const lsp_gmres_opts* opts, const double* f, do
       !ensure(c, S.b, sizeof(double) * N) || !ensure(c, S.x, sizeof(double) * N) ||
       !ensure(c, S.tmp, sizeof(double) * N) || !ensure(c, S.fvec, sizeof(double) * N) ||
       !ensure(c, S.gs, sizeof(double) * gs_n) ||
-      !ensure(c, c->fftbuf, sizeof(double) * 2 * N))
+      !ensure(c, c->fftbuf, sizeof(double) * N))
     return sfail(c, LSP_ERR_OOM, "gmres workspace: %s", c->err.c_str());
   if (!S.h_gs && cudaMallocHost(&S.h_gs, sizeof(double) * kGsPartial) != cudaSuccess) {
     S.h_gs = nullptr;
