@@ -63,9 +63,6 @@ FP64_FLOP_PER_SM_CLK, FP32_FLOP_PER_SM_CLK = 4, 256
 # dram__bytes_write.sum), keyed by (kernel, workload, mode); null where no capture of the
 # current kernel exists. The profile named beside each figure holds the command.
 TRAFFIC = {
-    # profiles/stencil_build_fp64_helm2d_n1024.md: k_stage<1, 3, double, double, 1>, four
-    # launches at 2D n = 1024 (per-point shifts): 11.1-11.3 MB read, 0 written
-    ("stage1", "helm2d_n1024", "fp64"): 11.2e6,
 }
 
 
@@ -181,9 +178,47 @@ def lattice_domain_sizes(m_list: np.ndarray, n: int, d: int) -> list[int]:
     return sizes  # [|E_d| = shifts, |E_{d-1}|, ..., |E_1|]
 
 
-def kernel_work(name: str, n: int, d: int, N: int, mu: int, sizes: list[int],
-                mode: str = "fp64"):
-    """Algorithmic (amount, kind) of one launch of a kernel, or None.
+def fmm_flops(m_list: np.ndarray, n: int, d: int) -> dict:
+    """FP64 flops of the fast multipole evaluation of the kernel vectors (t = 1, 2D and 3D): 20
+    nodes per box of 128 integers, classes x 2 functions; "stage1" the node-to-node products of
+    every box that holds a shift (up to three sources each) and one interpolation from its
+    parent, "stage2" the interpolation to the shifts and their near sources (three boxes)."""
+    half, nq, box = n // 2, 20, 128
+    fc = 2 * {2: 6, 3: 10}[d]
+    p2 = np.arange(half + 1, dtype=np.int64) ** 2
+    r = np.unique(p2[:, None] + p2[None, :])
+    if d == 3:
+        r = np.unique(r[:, None] + p2[None, :])
+    x = -np.asarray(m_list, dtype=np.int64)
+    lo, hi = min(int(x.min()), 0), max(int(x.max()), int(r.max()))
+    prods = 0
+    level = 0
+    while True:
+        width = box << level
+        j = np.unique(x // width)
+        top = (hi // (2 * width)) - (lo // (2 * width)) <= 1
+        for odd, offs in ((0, (-2, 2, 3)), (1, (-3, -2, 2))):
+            sel = j[j % 2 == odd]
+            prods += sum(int(((sel + o >= 0) & (sel + o <= r.max() // width)).sum()) for o in offs)
+        prods += 0 if top else len(j)
+        if top:
+            break
+        level += 1
+    start = np.searchsorted(r, np.maximum(x // box - 1, 0) * box)
+    end = np.searchsorted(r, (x // box + 2) * box)
+    near = int(np.maximum(end - start, 0).sum())
+    return {"stage1": 2.0 * prods * nq * nq * fc, "stage2": 2.0 * fc * (near + nq * len(x))}
+
+
+def stage_work(m_list: np.ndarray, n: int, d: int, mode: str):
+    """What kernel_work needs for the stages of a t = 1 build in this mode."""
+    return (fmm_flops(m_list, n, d) if mode in ("fp64", "dword") and d > 1
+            else lattice_domain_sizes(m_list, n, d))
+
+
+def kernel_work(name: str, n: int, d: int, N: int, mu: int, sizes, mode: str = "fp64"):
+    """Algorithmic (amount, kind) of one launch of a kernel, or None. sizes: the stage domains
+    (lattice_domain_sizes), or the flops of the multipole passes (fmm_flops).
 
     kind: "flop" (FP64 ALU), "tensor_flop" (BF16 tensor cores), "byte" (HBM) or "l2_byte"
     (gathers served by L2: the FP32 stages of the mixed mode)."""
@@ -192,17 +227,11 @@ def kernel_work(name: str, n: int, d: int, N: int, mu: int, sizes: list[int],
     if name.startswith("stage"):
         if not sizes:
             return None
+        if isinstance(sizes, dict):
+            return (sizes[name], "flop") if name in sizes else None
         k = int(name[-1])
         # stage k runs over E_k; sizes lists E_d, E_{d-1}, ..., so E_k = sizes[d - k]
         count = sizes[d - k]
-        if mode == "dword":
-            # double-word stages: FP32 operations as written (a double-word multiply-add is
-            # 10, a double-word add or subtract 11, a renormalisation 3, every fourth step)
-            if k == 1:
-                per = (n // 4) * (4 * 11 + 6 * 10 + 6 * 3 / 4) + 2 * 3 * 10
-                return count * per, "fp32_op"
-            ncls_k = ncls[k]
-            return count * P * ncls_k * 2 * (10 + 3 / 4), "fp32_op"
         if mode == "mixed":
             # FP32 stages, counted in FP32 operations as written: stage 1 per mirror pair two
             # squarings, four additions and six fused multiply-adds; later stages one fused
@@ -436,7 +465,7 @@ def run_ours(args):
     value = job_throughput(N, args.steps, ws, total_ms)
     peaks, peak_src = load_peaks()
     peaks = dict(peaks, l2_gbs=measure_l2_gbs(torch))
-    sizes = lattice_domain_sizes(m_list, n, d) if m_list is not None else []
+    sizes = [] if m_list is None else stage_work(m_list, n, d, args.mode)
     launches = int(sum(c for _, c in ktimes.values()))
     kern = {}
     for name, (ms, cnt) in ktimes.items():
@@ -658,7 +687,7 @@ def time_config(torch, workload: str, policy: str, mode: str, steps: int, warmup
     mu = (2 * t + 1) ** d
     out["kernel_ms_per_launch"] = {k: round(ms / max(cnt, 1), 4) for k, (ms, cnt) in kt.items()}
     if peaks is not None and t == 1:
-        sizes = lattice_domain_sizes(m_list, n, d) if m_list is not None else []
+        sizes = [] if m_list is None else stage_work(m_list, n, d, used)
         out["roofline"] = dominant_roofline(kt, n, d, N, mu, sizes, used, peaks, workload)
     return out
 

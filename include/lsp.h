@@ -48,10 +48,12 @@ typedef enum {
 /*
  * LSP_FP64: every step in FP64. LSP_MIXED: the a3 contractions and the Gram blocks in FP32,
  * the near-null solve in FP64. LSP_LEARNED: a trained network gives alpha and c (see lsp_mlp).
- * LSP_DWORD: the a3 contractions in double words (pairs of FP32 values, about 48 significant
- * bits, formed with exact two-sum and fused-multiply-add product errors on the FP32 pipe), the
- * rest in FP64; the stencils meet the FP64 path's tolerance. Double words serve t = 1 builds
- * in 1D and 2D; elsewhere a LSP_DWORD build runs the FP64 stages (lsp_get_mode_used says so).
+ * LSP_DWORD: t = 1 builds whose a3 contractions need only double-word accuracy (pairs of FP32
+ * values, about 48 significant bits), the rest in FP64; the stencils meet the FP64 path's
+ * tolerance. In 1D the contractions run in double words (exact two-sum and fused-multiply-add
+ * product errors on the FP32 pipe); in 2D the FP64 evaluation is faster than double words and
+ * serves this mode as well; in 3D and for t = 2 a LSP_DWORD build is an LSP_FP64 build
+ * (lsp_get_mode_used says so).
  */
 typedef enum { LSP_FP64 = 0, LSP_MIXED = 1, LSP_LEARNED = 2, LSP_DWORD = 3 } lsp_mode;
 

@@ -238,28 +238,13 @@ __global__ void __launch_bounds__(1024) k_compact_scan(int32_t* __restrict__ til
   if (threadIdx.x == 1023) *count = part[1023];
 }
 
-// Compaction pass 3: write list[pos] = lo + r for every set flag r (in increasing r), and
-// idx_of[r] = pos (or -1) when idx_of is given.
-__global__ void __launch_bounds__(kThreads) k_compact_write(const uint8_t* __restrict__ flag,
-                                                            const int32_t* __restrict__ tileoff,
-                                                            int64_t lo, int64_t range,
-                                                            int32_t* __restrict__ list,
-                                                            int32_t* __restrict__ idx_of) {
-  const int64_t base = (int64_t)blockIdx.x * kTileFlags + (int64_t)threadIdx.x * 16;
-  const uint4 q = reinterpret_cast<const uint4*>(flag)[(int64_t)blockIdx.x * kThreads + threadIdx.x];
-  const int c = count16(q);
-  int incl = c;
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  for (int o = 1; o < 32; o <<= 1) {
-    int y = __shfl_up_sync(0xffffffffu, incl, o);
-    if (lane >= o) incl += y;
-  }
-  __shared__ int wsum[kThreads / 32];
-  if (lane == 31) wsum[w] = incl;
-  __syncthreads();
-  int woff = 0;
-  for (int i = 0; i < w; ++i) woff += wsum[i];
-  int pos = tileoff[blockIdx.x] + woff + incl - c;
+// The list entries of this thread's 16 flags (those of range indices base..), from position pos
+// on: list[pos] = lo + r for every set flag r (in increasing r), idx_of[r] = pos (or -1) when
+// idx_of is given; with used, the boxes of tree that hold the entry are marked.
+__device__ __forceinline__ void write16(uint4 q, int64_t base, int64_t lo, int64_t range, int pos,
+                                        int32_t* __restrict__ list, int32_t* __restrict__ idx_of,
+                                        const FmmTree& tree, uint8_t* __restrict__ used,
+                                        int32_t* __restrict__ err) {
   const uint32_t words[4] = {q.x, q.y, q.z, q.w};
 #pragma unroll
   for (int k = 0; k < 16; ++k) {
@@ -275,6 +260,78 @@ __global__ void __launch_bounds__(kThreads) k_compact_write(const uint8_t* __res
       }
     }
   }
+  // an aligned group of 16 indices lies in at most two boxes of a level; its set ends mark them
+  if (used && (q.x | q.y | q.z | q.w)) {
+    int first = 16, last = 0;
+#pragma unroll
+    for (int k = 0; k < 16; ++k)
+      if ((words[k >> 2] >> (8 * (k & 3))) & 1u) {
+        first = min(first, k);
+        last = k;
+      }
+    if (base + last < range) fmm_mark(tree, lo + base + last, used, err);
+    fmm_mark(tree, lo + base + first, used, err);
+  }
+}
+
+// Inclusive sum of c over the block (at most 32 warps); part holds 32 ints.
+__device__ __forceinline__ int block_scan(int c, int* part) {
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  int incl = c;
+  for (int o = 1; o < 32; o <<= 1) {
+    const int y = __shfl_up_sync(0xffffffffu, incl, o);
+    if (lane >= o) incl += y;
+  }
+  if (lane == 31) part[w] = incl;
+  __syncthreads();
+  int woff = 0;
+  for (int i = 0; i < w; ++i) woff += part[i];
+  return woff + incl;
+}
+
+// Compaction pass 3: the list entries of every tile.
+__global__ void __launch_bounds__(kThreads) k_compact_write(const uint8_t* __restrict__ flag,
+                                                            const int32_t* __restrict__ tileoff,
+                                                            int64_t lo, int64_t range,
+                                                            int32_t* __restrict__ list,
+                                                            int32_t* __restrict__ idx_of,
+                                                            const __grid_constant__ FmmTree tree,
+                                                            uint8_t* __restrict__ used,
+                                                            int32_t* __restrict__ err) {
+  __shared__ int part[32];
+  const int64_t base = (int64_t)blockIdx.x * kTileFlags + (int64_t)threadIdx.x * 16;
+  const uint4 q = reinterpret_cast<const uint4*>(flag)[(int64_t)blockIdx.x * kThreads + threadIdx.x];
+  const int c = count16(q);
+  const int pos = tileoff[blockIdx.x] + block_scan(c, part) - c;
+  write16(q, base, lo, range, pos, list, idx_of, tree, used, err);
+}
+
+// A few tiles: the three passes in one block of 1024 threads (16 384 flags a step), two launches
+// fewer in a chain of short kernels.
+constexpr int kSmallSteps = 3;
+__global__ void __launch_bounds__(1024) k_compact_small(const uint8_t* __restrict__ flag,
+                                                        int64_t ngroups, int64_t lo, int64_t range,
+                                                        int32_t* __restrict__ list,
+                                                        int32_t* __restrict__ count,
+                                                        int32_t* __restrict__ idx_of,
+                                                        const __grid_constant__ FmmTree tree,
+                                                        uint8_t* __restrict__ used,
+                                                        int32_t* __restrict__ err) {
+  __shared__ int part[32];
+  __shared__ int total;
+  int done = 0;  // entries of the earlier steps
+  for (int64_t g0 = 0; g0 < ngroups; g0 += 1024) {
+    const int64_t g = g0 + threadIdx.x;
+    const uint4 q = g < ngroups ? reinterpret_cast<const uint4*>(flag)[g] : make_uint4(0, 0, 0, 0);
+    const int c = count16(q), incl = block_scan(c, part);
+    if (threadIdx.x == 1023) total = incl;
+    if (g < ngroups)
+      write16(q, g * 16, lo, range, done + incl - c, list, idx_of, tree, used, err);
+    __syncthreads();
+    done += total;
+    __syncthreads();  // total and part are free again
+  }
+  if (threadIdx.x == 0) *count = done;
 }
 
 // w(l) = 1 / (pi^2 (4 l + 2)): FP64 interleaved with w^2, or w alone rounded to FP32.
@@ -324,6 +381,20 @@ __global__ void __launch_bounds__(kThreads) k_zero_u32(uint32_t* __restrict__ p,
     p[i] = 0u;
 }
 
+__global__ void __launch_bounds__(kThreads) k_zero3_u32(uint32_t* __restrict__ a, int64_t na,
+                                                        uint32_t* __restrict__ b, int64_t nb,
+                                                        uint32_t* __restrict__ d, int64_t nd) {
+  for (int64_t i = (int64_t)blockIdx.x * kThreads + threadIdx.x; i < na + nb + nd;
+       i += (int64_t)gridDim.x * kThreads) {
+    if (i < na)
+      a[i] = 0u;
+    else if (i < na + nb)
+      b[i - na] = 0u;
+    else
+      d[i - na - nb] = 0u;
+  }
+}
+
 // dst[0, n) = src[0, n) (doubles; both 16-byte aligned): pairs by every thread, an odd last
 // element by thread 0.
 __global__ void __launch_bounds__(kThreads) k_copy_f64(const double* __restrict__ src,
@@ -357,6 +428,16 @@ cudaError_t launch_zero(lsp_ctx* c, void* p, size_t bytes) {
   return cudaGetLastError();
 }
 
+cudaError_t launch_zero3(lsp_ctx* c, ZeroRange a, ZeroRange b, ZeroRange d) {
+  const int64_t na = (int64_t)(a.bytes / 4), nb = (int64_t)(b.bytes / 4);
+  const int64_t nd = (int64_t)(d.bytes / 4);
+  int t = timer_begin(c, "zero");
+  k_zero3_u32<<<grid_for(na + nb + nd), kThreads, 0, c->stream>>>(
+      (uint32_t*)a.p, na, (uint32_t*)b.p, nb, (uint32_t*)d.p, nd);
+  timer_end(c, t);
+  return cudaGetLastError();
+}
+
 cudaError_t launch_copy_f64(lsp_ctx* c, const double* src, double* dst, int64_t n) {
   int t = timer_begin(c, "copy_rows");
   k_copy_f64<<<grid_for((n + 1) / 2), kThreads, 0, c->stream>>>(src, dst, n);
@@ -376,14 +457,24 @@ cudaError_t launch_mark_local(lsp_ctx* c) {
 // flags must hold a multiple of kTileFlags bytes (zero beyond `range`); tile scratch lives in
 // the context's `counts` buffer after its first 16 entries.
 cudaError_t launch_compact(lsp_ctx* c, const uint8_t* flags, int64_t lo, int64_t range,
-                           int32_t* list, int32_t* count, int32_t* idx_of) {
+                           int32_t* list, int32_t* count, int32_t* idx_of, const FmmTree* tree,
+                           uint8_t* used) {
+  int32_t* err = (int32_t*)c->counts.p + kErrWord;
+  const FmmTree t = tree ? *tree : FmmTree{};
+  if (!tree) used = nullptr;
   const int ntiles = (int)((range + kTileFlags - 1) / kTileFlags);
   int32_t* tiles = (int32_t*)c->counts.p + 16;
-  int t = timer_begin(c, "compact");
-  k_compact_count<<<ntiles, kThreads, 0, c->stream>>>(flags, tiles);
-  k_compact_scan<<<1, 1024, 0, c->stream>>>(tiles, ntiles, count);
-  k_compact_write<<<ntiles, kThreads, 0, c->stream>>>(flags, tiles, lo, range, list, idx_of);
-  timer_end(c, t);
+  int tm = timer_begin(c, "compact");
+  if (range <= kSmallSteps * 16 * 1024) {
+    k_compact_small<<<1, 1024, 0, c->stream>>>(flags, (int64_t)ntiles * kThreads, lo, range, list,
+                                               count, idx_of, t, used, err);
+  } else {
+    k_compact_count<<<ntiles, kThreads, 0, c->stream>>>(flags, tiles);
+    k_compact_scan<<<1, 1024, 0, c->stream>>>(tiles, ntiles, count);
+    k_compact_write<<<ntiles, kThreads, 0, c->stream>>>(flags, tiles, lo, range, list, idx_of, t,
+                                                        used, err);
+  }
+  timer_end(c, tm);
   return cudaGetLastError();
 }
 

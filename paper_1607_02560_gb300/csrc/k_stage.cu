@@ -15,6 +15,8 @@
 //   g_f[a_1..a_d](m) = N^-1 T_d,f[a_1..a_d](m)          (E_d = the shift list).
 // T_k is symmetric in its class tuple, so only sorted tuples (a <= rest) are formed. This is
 // the exact sum of the definition with the terms grouped by axis; no approximation is made.
+// These stages serve the FP32 sums of the mixed mode, t = 2 builds and 1D; FP64 sums of t = 1
+// builds in 2D and 3D run through k_fmm.cu.
 #include <type_traits>
 
 #include "lsp_internal.h"
@@ -162,85 +164,46 @@ __device__ __forceinline__ void store_out(double* p, float v, double scale) { *p
 __device__ __forceinline__ void store_out(double* p, dword v, double scale) {
   *p = ((double)v.h + (double)v.l) * scale;
 }
-__device__ __forceinline__ void store_out(dword* p, dword v, double) {
-  dw_norm(v);
-  *p = v;
-}
-
-// Double-word form of stage_accumulate (below): the same sums in the same order, with the
-// w table holding (w, w^2) as two double words per l (16 bytes, one load) and the stage tables
-// holding double words. The accumulators are renormalised every four frequencies.
+// Double-word form of the first stage of stage_accumulate (below; 1D has no other): the same sums
+// in the same order, with the w table holding (w, w^2) as two double words per l (16 bytes, one
+// load). The accumulators are renormalised every four frequencies.
 template <int K, int A>
 __device__ __forceinline__ void stage_accumulate_dw(const dword* __restrict__ xs, int P,
                                                     int64_t l, const dword* __restrict__ Tprev,
-                                                    int64_t lo_prev, int64_t stride_prev,
-                                                    int first, int step,
+                                                    int64_t lo_prev, int first, int step,
                                                     dword (&acc)[StageMap<K, A>::NCO][2]) {
-  using M = StageMap<K, A>;
   const int half = P - 1;  // n/2
-  if (K == 1) {
-    const float4* tab = reinterpret_cast<const float4*>(Tprev) + (l - lo_prev);
-    const int quarter = half / 2;  // n/4
-    int cnt = 0;
+  const float4* tab = reinterpret_cast<const float4*>(Tprev) + (l - lo_prev);
+  const int quarter = half / 2;  // n/4
+  int cnt = 0;
 #pragma unroll 4
-    for (int p = first; p < quarter; p += step) {
-      const int q = half - p;
-      const float4 wa = __ldg(tab + (int64_t)p * p);
-      const float4 wb = __ldg(tab + (int64_t)q * q);
-      const dword a1 = {wa.x, wa.y}, b1 = {wb.x, wb.y}, a2 = {wa.z, wa.w}, b2 = {wb.z, wb.w};
-      const dword s1 = dw_add(a1, b1), d1 = dw_sub(a1, b1);
-      const dword s2 = dw_add(a2, b2), d2 = dw_sub(a2, b2);
+  for (int p = first; p < quarter; p += step) {
+    const int q = half - p;
+    const float4 wa = __ldg(tab + (int64_t)p * p);
+    const float4 wb = __ldg(tab + (int64_t)q * q);
+    const dword a1 = {wa.x, wa.y}, b1 = {wb.x, wb.y}, a2 = {wa.z, wa.w}, b2 = {wb.z, wb.w};
+    const dword s1 = dw_add(a1, b1), d1 = dw_sub(a1, b1);
+    const dword s2 = dw_add(a2, b2), d2 = dw_sub(a2, b2);
 #pragma unroll
-      for (int a = 0; a < A; ++a) {  // even a: X_a(q) = X_a(p); odd a: X_a(q) = -X_a(p)
-        const dword xa = xs[a * P + p];
-        dw_mac(acc[a][0], xa, (a & 1) ? d1 : s1);
-        dw_mac(acc[a][1], xa, (a & 1) ? d2 : s2);
-      }
-      if ((++cnt & 3) == 0) {
+    for (int a = 0; a < A; ++a) {  // even a: X_a(q) = X_a(p); odd a: X_a(q) = -X_a(p)
+      const dword xa = xs[a * P + p];
+      dw_mac(acc[a][0], xa, (a & 1) ? d1 : s1);
+      dw_mac(acc[a][1], xa, (a & 1) ? d2 : s2);
+    }
+    if ((++cnt & 3) == 0) {
 #pragma unroll
-        for (int a = 0; a < A; ++a) {
-          dw_norm(acc[a][0]);
-          dw_norm(acc[a][1]);
-        }
+      for (int a = 0; a < A; ++a) {
+        dw_norm(acc[a][0]);
+        dw_norm(acc[a][1]);
       }
     }
-    if (first == 0) {
-      const float4 wm = __ldg(tab + (int64_t)quarter * quarter);
+  }
+  if (first == 0) {
+    const float4 wm = __ldg(tab + (int64_t)quarter * quarter);
 #pragma unroll
-      for (int c = 0; c < A; ++c) {
-        dw_mac(acc[c][0], xs[c * P + quarter], dword{wm.x, wm.y});
-        dw_mac(acc[c][1], xs[c * P + quarter], dword{wm.z, wm.w});
-      }
-    }
-  } else {
-    const dword* base = Tprev + (l - lo_prev);
-    int cnt = 0;
-#pragma unroll 4
-    for (int p = first; p < P; p += step) {
-      const int64_t off = (int64_t)p * p;
-      dword in[M::NCP][2];
-#pragma unroll
-      for (int c = 0; c < M::NCP; ++c) {
-        const float2 v0 = __ldg(reinterpret_cast<const float2*>(base + (2 * c + 0) * stride_prev + off));
-        const float2 v1 = __ldg(reinterpret_cast<const float2*>(base + (2 * c + 1) * stride_prev + off));
-        in[c][0] = {v0.x, v0.y};
-        in[c][1] = {v1.x, v1.y};
-      }
-      dword x[A];
-#pragma unroll
-      for (int a = 0; a < A; ++a) x[a] = xs[a * P + p];
-#pragma unroll
-      for (int c = 0; c < M::NCO; ++c) {
-        dw_mac(acc[c][0], x[M::a(c)], in[M::r(c)][0]);
-        dw_mac(acc[c][1], x[M::a(c)], in[M::r(c)][1]);
-      }
-      if ((++cnt & 3) == 0) {
-#pragma unroll
-        for (int c = 0; c < M::NCO; ++c) {
-          dw_norm(acc[c][0]);
-          dw_norm(acc[c][1]);
-        }
-      }
+    for (int c = 0; c < A; ++c) {
+      dw_mac(acc[c][0], xs[c * P + quarter], dword{wm.x, wm.y});
+      dw_mac(acc[c][1], xs[c * P + quarter], dword{wm.z, wm.w});
     }
   }
 }
@@ -368,7 +331,7 @@ __device__ __forceinline__ void stage_body(const int32_t* __restrict__ list,
 #pragma unroll
     for (int c = 0; c < M::NCO; ++c) acc[c][0] = acc[c][1] = zero_of<R>();
     if constexpr (std::is_same<R, dword>::value)
-      stage_accumulate_dw<K, A>(xs, P, l, Tprev, lo_prev, stride_prev, lane, LANES, acc);
+      stage_accumulate_dw<K, A>(xs, P, l, Tprev, lo_prev, lane, LANES, acc);
     else
       stage_accumulate<K, A, R>(xs, P, l, Tprev, lo_prev, stride_prev, lane, LANES, acc);
     if (LANES > 1) {
@@ -407,9 +370,8 @@ __device__ __forceinline__ void stage_body(const int32_t* __restrict__ list,
 
 // Register budgets, measured at 2D n = 1024 and 3D n = 64. Four resident blocks of 256 threads
 // (at most 64 registers) suit the stages whose gathers the unrolled loops keep in flight:
-// FP32 stage 2 0.165 -> 0.159 ms, FP32 stage 1 -3%, double-word stages 1 and 2 -4% and -3%,
-// the FP64 3D stage 3 0.020 -> 0.014 ms. The FP64 stage 1 (no gather: consecutive reads, FP64
-// pipe bound) is 2% faster with the compiler's own choice (48 registers, five blocks).
+// FP32 stage 2 0.165 -> 0.159 ms, FP32 stage 1 -3%. The FP64 stage 1 (no gather: consecutive
+// reads, FP64 pipe bound) is 2% faster with the compiler's own choice (48 registers, five blocks).
 template <int K, int A, typename R, typename OUT, int LANES>
 __global__ void __launch_bounds__(kThreads) k_stage(LSP_STAGE_PARAMS) {
   stage_body<K, A, R, OUT, LANES>(LSP_STAGE_ARGS);
@@ -481,38 +443,39 @@ cudaError_t launch_typed(lsp_ctx* c, int d, int k, int t, const int32_t* list,
                          int64_t stride_prev, void* Tout, int64_t lo_out, int64_t stride_out,
                          bool by_index, double scale, const R* X) {
   const R* prev = (const R*)Tprev;
-  if constexpr (std::is_same<R, dword>::value) {
-    if (t == 2) return cudaErrorInvalidValue;  // double-word stages serve t = 1 builds only
-  } else if (t == 2) {  // five cosine rows (2D and 3D)
+  if constexpr (!std::is_same<R, dword>::value) {
+    if (t == 2) {  // five cosine rows (2D and 3D)
+      if (k == 1)
+        return launch_k<1, 5, R, R>(c, list, count, cap, X, prev, lo_prev, stride_prev, (R*)Tout,
+                                    lo_out, stride_out, by_index, scale);
+      if (k == 2 && d == 3)
+        return launch_k<2, 5, R, R>(c, list, count, cap, X, prev, lo_prev, stride_prev, (R*)Tout,
+                                    lo_out, stride_out, by_index, scale);
+      if (k == 2)
+        return launch_k<2, 5, R, double>(c, list, count, cap, X, prev, lo_prev, stride_prev,
+                                         (double*)Tout, lo_out, stride_out, by_index, scale);
+      return launch_k<3, 5, R, double>(c, list, count, cap, X, prev, lo_prev, stride_prev,
+                                       (double*)Tout, lo_out, stride_out, by_index, scale);
+    }
+  }
+  double* out = (double*)Tout;
+  if (d == 1)  // 1D: the single stage, double g values for the eigen step
+    return launch_k<1, 3, R, double>(c, list, count, cap, X, prev, lo_prev, stride_prev, out,
+                                     lo_out, stride_out, by_index, scale);
+  if constexpr (std::is_same<R, float>::value) {  // FP64 t = 1 builds run k_fmm.cu
     if (k == 1)
-      return launch_k<1, 5, R, R>(c, list, count, cap, X, prev, lo_prev, stride_prev, (R*)Tout,
+      return launch_k<1, 3, R, R>(c, list, count, cap, X, prev, lo_prev, stride_prev, (R*)Tout,
                                   lo_out, stride_out, by_index, scale);
     if (k == 2 && d == 3)
-      return launch_k<2, 5, R, R>(c, list, count, cap, X, prev, lo_prev, stride_prev, (R*)Tout,
+      return launch_k<2, 3, R, R>(c, list, count, cap, X, prev, lo_prev, stride_prev, (R*)Tout,
                                   lo_out, stride_out, by_index, scale);
-    if (k == 2)
-      return launch_k<2, 5, R, double>(c, list, count, cap, X, prev, lo_prev, stride_prev,
-                                       (double*)Tout, lo_out, stride_out, by_index, scale);
-    return launch_k<3, 5, R, double>(c, list, count, cap, X, prev, lo_prev, stride_prev,
-                                     (double*)Tout, lo_out, stride_out, by_index, scale);
-  }
-  if (k == d) {  // last stage: double g values for the eigen step
-    double* out = (double*)Tout;
-    if (k == 1)  // 1D: the single stage
-      return launch_k<1, 3, R, double>(c, list, count, cap, X, prev, lo_prev, stride_prev, out,
-                                       lo_out, stride_out, by_index, scale);
     if (k == 2)
       return launch_k<2, 3, R, double>(c, list, count, cap, X, prev, lo_prev, stride_prev, out,
                                        lo_out, stride_out, by_index, scale);
     return launch_k<3, 3, R, double>(c, list, count, cap, X, prev, lo_prev, stride_prev, out,
                                      lo_out, stride_out, by_index, scale);
   }
-  R* out = (R*)Tout;
-  if (k == 1)
-    return launch_k<1, 3, R, R>(c, list, count, cap, X, prev, lo_prev, stride_prev, out, lo_out,
-                                stride_out, by_index, scale);
-  return launch_k<2, 3, R, R>(c, list, count, cap, X, prev, lo_prev, stride_prev, out, lo_out,
-                              stride_out, by_index, scale);
+  return cudaErrorInvalidValue;
 }
 
 }  // namespace

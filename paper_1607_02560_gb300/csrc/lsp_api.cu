@@ -416,38 +416,52 @@ lsp_status flush_timers(lsp_ctx* c) {
   return LSP_OK;
 }
 
-// The launch sequence of steps a2-a7 for the sizes already prepared in the context.
-// Arithmetic of the a3 stages for a build: FP32 in the mixed mode; double words in the dword
-// mode for t = 1 in 1D and 2D (in 3D the stages are a small part of the build and the
-// tolerance, set by the spectral gap, is tight, so they stay FP64); FP64 otherwise.
+// Accuracy of the a3 sums of a build: FP32 in the mixed mode; double words in the dword mode for
+// t = 1 in 1D and 2D (in 3D the tolerance, set by the spectral gap, is too tight); FP64 otherwise.
 int stage_prec(const lsp_ctx* c, const lsp_stencil_opts& o) {
   if (o.mode == LSP_MIXED) return kPrecFP32;
   if (o.mode == LSP_DWORD && o.t == 1 && c->geo.d <= 2) return kPrecDword;
   return kPrecFP64;
 }
 
+// The FP64 sums of t = 1 builds in 2D and 3D run through the fast multipole evaluation, the
+// double-word mode's too (more accurate than double words, and faster); FP32 sums (mixed), 1D and
+// t = 2 builds go stage by stage.
+bool uses_fmm(const lsp_ctx* c, const lsp_stencil_opts& o) {
+  return o.t == 1 && c->geo.d >= 2 && stage_prec(c, o) != kPrecFP32;
+}
+
+// The launch sequence of steps a2-a7 for the sizes already prepared in the context.
 lsp_status issue_build(lsp_ctx* c, const lsp_stencil_opts& o, int64_t cap_s, bool upload,
                        bool rows = true) {
   const int d = c->geo.d;
   int32_t* counts = (int32_t*)c->counts.p;
-  // zeroing by kernels: a memset may be queued behind host copies on the copy engines
-  CUDA_OK(c, launch_zero(c, counts + kErrWord, sizeof(int32_t)));
-  if (o.policy == LSP_SHIFT_LOCAL) {
-    const int64_t R = c->mrange.size();
-    CUDA_OK(c, launch_zero(c, c->shift_flag.p, round_up(R, 4096)));
+  const bool fmm = uses_fmm(c, o), local = o.policy == LSP_SHIFT_LOCAL;
+  // zeroing by a kernel: a memset may be queued behind host copies on the copy engines
+  const int64_t R = c->mrange.size();
+  CUDA_OK(c, launch_zero3(c, {counts + kErrWord, sizeof(int32_t)},
+                          {c->shift_flag.p, local ? round_up(R, 4096) : 0},
+                          {c->fmm.used.p, fmm ? c->fmm.used_bytes : 0}));
+  if (local) {
     CUDA_OK(c, launch_mark_local(c));
+    const FmmTree tree = fmm ? fmm_tree(c) : FmmTree{};
     CUDA_OK(c, launch_compact(c, (const uint8_t*)c->shift_flag.p, c->mrange.lo, R,
-                              (int32_t*)c->shift_m.p, counts + 0, (int32_t*)c->idx_of.p));
-  } else if (upload) {
-    CUDA_OK(c, cudaMemcpyAsync(c->shift_m.p, c->h_list, sizeof(int32_t) * cap_s,
-                               cudaMemcpyHostToDevice, c->stream));
-    CUDA_OK(c, cudaMemcpyAsync(counts, c->h_list + cap_s, sizeof(int32_t),
-                               cudaMemcpyHostToDevice, c->stream));
+                              (int32_t*)c->shift_m.p, counts + 0, (int32_t*)c->idx_of.p,
+                              fmm ? &tree : nullptr, (uint8_t*)c->fmm.used.p));
+  } else {
+    if (upload) {
+      CUDA_OK(c, cudaMemcpyAsync(c->shift_m.p, c->h_list, sizeof(int32_t) * cap_s,
+                                 cudaMemcpyHostToDevice, c->stream));
+      CUDA_OK(c, cudaMemcpyAsync(counts, c->h_list + cap_s, sizeof(int32_t),
+                                 cudaMemcpyHostToDevice, c->stream));
+    }
+    if (fmm) CUDA_OK(c, launch_fmm_mark(c, (const int32_t*)c->shift_m.p, counts + 0, cap_s));
   }
   const int32_t* list = (const int32_t*)c->shift_m.p;
   const int32_t* count = counts + 0;
   int64_t cap = cap_s;
-  for (int k = d - 1; k >= 1; --k) {
+  if (fmm) CUDA_OK(c, launch_fmm(c, list, count, cap_s));
+  for (int k = fmm ? 0 : d - 1; k >= 1; --k) {
     const int64_t sz = c->erange[k].size();
     if (c->edense[k]) {
       // every l of the range is evaluated: no marking or compaction needed
@@ -466,7 +480,7 @@ lsp_status issue_build(lsp_ctx* c, const lsp_stencil_opts& o, int64_t cap_s, boo
   }
   const int prec = stage_prec(c, o);  // the w table is refreshed by the caller
   const bool fp32 = prec == kPrecFP32;
-  for (int k = 1; k <= d; ++k) {
+  for (int k = fmm ? d + 1 : 1; k <= d; ++k) {
     const void* prev = k == 1 ? c->wtab.p : c->T[k - 1].p;
     const int64_t lo_prev = c->erange[k - 1].lo, stride_prev = c->erange[k - 1].size();
     if (k < d) {
@@ -671,6 +685,7 @@ lsp_status lsp_destroy(lsp_ctx* c) {
   for (cudaEvent_t e : c->ev_pool) cudaEventDestroy(e);
   if (c->graph) cudaGraphExecDestroy(c->graph);
   nd_free(c->nd);
+  fmm_free(c->fmm);
   delete c;
   return LSP_OK;
 }
@@ -859,6 +874,13 @@ lsp_status lsp_build_stencils(lsp_ctx* c, const lsp_stencil_opts* opts) {
 
   // ---- buffers (all allocation happens before any capture) ----
   const int64_t R = c->mrange.size();
+  const bool fmm = uses_fmm(c, o);
+  if (fmm) {
+    const cudaError_t e = fmm_plan(c);
+    if (e != cudaSuccess)
+      return fail(c, e == cudaErrorMemoryAllocation ? LSP_ERR_OOM : LSP_ERR_CUDA,
+                  "plan of the kernel vectors: %s", cudaGetErrorString(e));
+  }
   bool ok = ensure(c, c->shift_m, sizeof(int32_t) * cap_s) &&
             ensure(c, c->counts, sizeof(int32_t) * (16 + 2 + c->erange[0].size() / 4096 + 16)) &&
             ensure(c, c->gvals, sizeof(double) * 2 * G.ncls * cap_s) &&
@@ -871,12 +893,14 @@ lsp_status lsp_build_stencils(lsp_ctx* c, const lsp_stencil_opts* opts) {
                           ensure(c, c->cst2, sizeof(double) * mu * cap_s) &&
                           ensure(c, c->lam2, sizeof(double) * 2 * cap_s) &&
                           ensure(c, c->sflags2, sizeof(int32_t) * cap_s))) &&
-            ensure_tracked(c, c->wtab, sizeof(double) * 2 * c->erange[0].size(), &c->wtab_size) &&
+            (fmm || ensure_tracked(c, c->wtab, sizeof(double) * 2 * c->erange[0].size(),
+                                   &c->wtab_size)) &&
             ensure(c, c->Q, sizeof(double) * mu * N) && ensure(c, c->C, sizeof(double) * mu * N) &&
             ensure(c, c->P, sizeof(double) * mu * N);
   if (ok && o.policy == LSP_SHIFT_LOCAL)
     ok = ensure(c, c->shift_flag, round_up(R, 4096)) && ensure(c, c->idx_of, sizeof(int32_t) * R);
-  for (int k = 1; ok && k < d; ++k) {
+  if (ok && fmm) ok = fmm_buffers(c);
+  for (int k = 1; ok && !fmm && k < d; ++k) {
     const int64_t sz = c->erange[k].size();
     ok = ensure(c, c->eflag[k], round_up(sz, 4096)) && ensure(c, c->elist[k], sizeof(int32_t) * sz) &&
          ensure(c, c->T[k], sizeof(double) * 2 * ncls_stage(k, o.t) * sz);
@@ -904,7 +928,7 @@ lsp_status lsp_build_stencils(lsp_ctx* c, const lsp_stencil_opts* opts) {
 
   // w depends only on its index range and precision: refreshed (outside any graph) only when
   // those change, so a replayed graph always finds the table it was recorded with.
-  {
+  if (!fmm) {
     const int prec = stage_prec(c, o);
     if (!(c->wtab_lo == c->erange[0].lo && c->wtab_size == c->erange[0].size() &&
           c->wtab_prec == prec)) {

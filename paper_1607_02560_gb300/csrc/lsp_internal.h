@@ -111,6 +111,38 @@ struct DevBuf {
   size_t bytes = 0;
 };
 
+// Plan and workspace of the fast multipole evaluation of a3 (k_fmm.cu): charges, leaf lists and
+// moments depend on the grid only and are made once per context; used and loc belong to a build.
+constexpr int kFmmLevels = 24;  // boxes of 128 * 2^23 integers hold any shift range and |p|^2
+// Shifts at most (a bound known on the host) for one block per shift, and for eight lanes a shift
+// instead of two.
+constexpr int64_t kFmmBlockShifts = 152 * 8, kFmmLaneShifts = 152 * 256;
+struct FmmPlan {
+  bool ready = false;
+  int32_t ns = 0;                 // sources: distinct |p|^2
+  int64_t nsb[kFmmLevels] = {0};  // source boxes of a level
+  int64_t qoff[kFmmLevels] = {0}; // boxes of the levels below it in q
+  DevBuf tab, pos, wgt, start, q, used, loc;
+  size_t used_bytes = 0;  // of the last build's tree, a multiple of 4
+};
+// Boxes of the tree over the points -m - 1/2 of a shift range, level 0 the leaves: box j of level l
+// covers the integers [128 2^l j, 128 2^l (j + 1)) of -m (points half an integer below).
+constexpr int kFmmLog = 7;
+struct FmmTree {
+  int L;                          // top level: its parents are all neighbours
+  int64_t jlo[kFmmLevels];        // first box of a level
+  int64_t off[kFmmLevels + 1];    // boxes of the levels below, off[L + 1] = all
+  int64_t nsb[kFmmLevels];        // source boxes [0, nsb) of a level
+  int64_t qoff[kFmmLevels];       // their moments: boxes before the level
+};
+#ifdef __CUDACC__
+// used[box] = 1 for the boxes that hold lattice index m, at every level.
+__device__ __forceinline__ void fmm_mark(const FmmTree& t, int64_t m, uint8_t* used, int32_t* err) {
+  for (int l = 0; l <= t.L; ++l)
+    used[checked(t.off[l] + (-m >> (kFmmLog + l)) - t.jlo[l], t.off[t.L + 1], err)] = 1;
+}
+#endif
+
 struct KernelTimer {
   std::string name;
   double ms = 0;
@@ -161,6 +193,8 @@ struct lsp_ctx {
   int64_t wtab_lo = 0, wtab_size = -1;  // range held by wtab (-1: none)
   int wtab_prec = -1;
   int64_t alloc_gen = 0;  // bumped whenever a device buffer is (re)allocated
+
+  lsp::FmmPlan fmm;  // FP64 kernel vectors of t = 1 builds in 2D and 3D
 
   // per-shift results (a3-a6); *2: the t = 2 stencils
   lsp::DevBuf gvals, alpha, cst, lam, sflags, alpha2, cst2, lam2, sflags2;
@@ -227,11 +261,19 @@ void timer_end(lsp_ctx* ctx, int slot);
 cudaError_t launch_stats(lsp_ctx* c, int nblocks, const double* src);
 // bytes / 4 words of p set to zero (bytes a multiple of 4, p 4-byte aligned)
 cudaError_t launch_zero(lsp_ctx* c, void* p, size_t bytes);
+// the same for up to three ranges in one launch
+struct ZeroRange {
+  void* p;
+  size_t bytes;
+};
+cudaError_t launch_zero3(lsp_ctx* c, ZeroRange a, ZeroRange b, ZeroRange d);
 // n doubles from src to dst (device, 16-byte aligned)
 cudaError_t launch_copy_f64(lsp_ctx* c, const double* src, double* dst, int64_t n);
 cudaError_t launch_mark_local(lsp_ctx* c);
+// tree (optional): also marks the tree's boxes that hold an index of the list in used.
 cudaError_t launch_compact(lsp_ctx* c, const uint8_t* flags, int64_t lo, int64_t range,
-                           int32_t* list, int32_t* count, int32_t* idx_of);
+                           int32_t* list, int32_t* count, int32_t* idx_of,
+                           const FmmTree* tree = nullptr, uint8_t* used = nullptr);
 cudaError_t launch_mark_stage(lsp_ctx* c, const int32_t* list, const int32_t* count,
                               int64_t cap, int64_t lo_prev, uint8_t* flag_prev);
 cudaError_t launch_wtable(lsp_ctx* c, int64_t lo, int64_t range, void* w, int prec);
@@ -239,6 +281,14 @@ cudaError_t launch_stage(lsp_ctx* c, int d, int k, int t, const int32_t* list,
                          const int32_t* count, int64_t cap, const void* Tprev, int64_t lo_prev,
                          int64_t stride_prev, void* Tout, int64_t lo_out, int64_t stride_out,
                          bool by_index, int prec);
+// Fast multipole evaluation of a3 (t = 1, 2D and 3D): plan of a context (synchronises; not under
+// capture), buffers of a build (needs c->mrange), and the launches that fill c->gvals.
+cudaError_t fmm_plan(lsp_ctx* c);
+bool fmm_buffers(lsp_ctx* c);
+FmmTree fmm_tree(const lsp_ctx* c);
+cudaError_t launch_fmm_mark(lsp_ctx* c, const int32_t* list, const int32_t* count, int64_t cap);
+cudaError_t launch_fmm(lsp_ctx* c, const int32_t* list, const int32_t* count, int64_t cap);
+void fmm_free(FmmPlan& p);
 cudaError_t launch_eig_t2(lsp_ctx* c, const int32_t* count, int64_t cap);
 cudaError_t launch_eig_dense3(lsp_ctx* c, const int32_t* count, int64_t cap);
 cudaError_t upload_cls125(const Geometry& g);
