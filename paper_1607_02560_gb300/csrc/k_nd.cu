@@ -649,199 +649,216 @@ __global__ void __launch_bounds__(256) k_nd_update(double* __restrict__ fronts, 
 }
 
 // ---- solve ----
-// Going up: w = [y_E; 0] + children's u (through the ring maps), w'_E = w_E[perm];
-// z = A^-1 w_E = F[E, E] w'_E; u = w_R + F[R, E] w'_E. 64 rows of one front per CTA.
-__global__ void __launch_bounds__(256) k_nd_fwd(const double* __restrict__ F, int f, int s, int r,
-                                                const int32_t* __restrict__ E,
-                                                const int32_t* __restrict__ perm,
-                                                const int32_t* __restrict__ inv, int nchild,
-                                                const double* __restrict__ uc, int rc,
-                                                const double* __restrict__ y,
-                                                double* __restrict__ z, double* __restrict__ u,
-                                                int rows) {
-  extern __shared__ double wE[];
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+// After the factorisation the blocks that a solve reads are stored once more, transposed and
+// contiguous per front: FT[m][i] = F[i][m] (m < s, i < f) for the way up, BT[m][i] = F[i][s + m]
+// (m < r, i < s) for the way down. Threads that own consecutive rows i then read consecutive
+// doubles for every m: no staging, no shuffles, one FMA per element, at every front size. (From
+// the row-major fronts a solve at 2D n = 1024 took 1.2 ms: blocks staged in shared memory for
+// small fronts, a warp per row with a shuffle reduction for large ones; now 0.66 ms, and 0.14 ms
+// instead of 0.23 ms at n = 256.) What bounds it now: the FP64 pipe (2e8 products at n = 1024,
+// 0.32 ms; the bytes would take 0.24 ms) and, at the depths above the leaves, the chain of
+// launches and gathers; a depth's kernel loads its first matrix values and its indices before it
+// waits for the depth before (programmatic dependent launch).
+//
+// Also stored per eliminated position: where its right-hand side entry comes from (the grid
+// point and the children's ring entries of the pivoted row), so that the gather on the way up is
+// two loads deep.
+constexpr int kTile = 32;
+__global__ void __launch_bounds__(256) k_nd_store(const double* __restrict__ fronts, int f, int s,
+                                                  int r, const int32_t* __restrict__ E,
+                                                  const int32_t* __restrict__ perm,
+                                                  const int32_t* __restrict__ inv, int nchild,
+                                                  int rc, double* __restrict__ FT,
+                                                  double* __restrict__ BT,
+                                                  int32_t* __restrict__ gsrc) {
+  __shared__ double t[kTile][kTile + 1];
   const int64_t p = blockIdx.y;
-  const double* Fp = F + p * f * f;
-  const int32_t* iv = nchild ? inv + p * f * 2 : nullptr;
-  auto wsum = [&](int i) -> double {
-    double v = i < s ? y[E[p * s + i]] : 0.0;
-    for (int c = 0; c < nchild; ++c) {
-      const int a = iv[i * 2 + c];
-      if (a >= 0) v += uc[(nchild == 1 ? p : 2 * p + c) * rc + a];
-    }
-    return v;
-  };
-  for (int m = tid; m < s; m += blockDim.x) wE[m] = wsum(perm[p * s + m]);
-  __syncthreads();
-  const int row0 = blockIdx.x * rows;
-  for (int rr = warp; rr < rows; rr += blockDim.x / 32) {
-    const int i = row0 + rr;
-    if (i >= f) break;
-    const double* Fi = Fp + (int64_t)i * f;
-    double acc = 0.0;
-    for (int m = lane; m < s; m += 32) acc = fma(Fi[m], wE[m], acc);
-    for (int off = 16; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
-    if (lane == 0) {
-      if (i < s)
-        z[p * s + i] = acc;
-      else
-        u[p * r + (i - s)] = wsum(i) + acc;
+  const double* F = fronts + p * f * f;
+  const int ti = (f + kTile - 1) / kTile, tm = (s + kTile - 1) / kTile;  // tiles of FT
+  const int bi = (s + kTile - 1) / kTile, bm = (r + kTile - 1) / kTile;  // tiles of BT
+  int q = blockIdx.x;
+  const int x = threadIdx.x & 31, y = threadIdx.x >> 5;
+  if (q < ti * tm || (q -= ti * tm) < bi * bm) {
+    const bool fwd = (int)blockIdx.x < ti * tm;
+    const int nr = fwd ? f : s, nm = fwd ? s : r, c0 = fwd ? 0 : s, tr = fwd ? ti : bi;
+    const int i0 = (q % tr) * kTile, m0 = (q / tr) * kTile;
+    for (int k = y; k < kTile; k += 8)
+      if (i0 + k < nr && m0 + x < nm) t[k][x] = F[(int64_t)(i0 + k) * f + c0 + m0 + x];
+    __syncthreads();
+    double* out = fwd ? FT + p * s * f : BT + p * r * s;
+    for (int k = y; k < kTile; k += 8)
+      if (m0 + k < nm && i0 + x < nr) out[(int64_t)(m0 + k) * nr + i0 + x] = t[x][k];
+    return;
+  }
+  // gsrc[(p s + m) 3 ..]: grid point, then the children's entries (or -1) of position perm[m]
+  for (int m = threadIdx.x; m < s; m += blockDim.x) {
+    const int pm = perm[p * s + m];
+    int32_t* g = gsrc + (p * s + m) * 3;
+    g[0] = E[p * s + pm];
+    for (int c = 0; c < 2; ++c) {
+      const int a = c < nchild ? inv[(p * f + pm) * 2 + c] : -1;
+      g[1 + c] = a < 0 ? -1 : (int32_t)((nchild == 1 ? p : 2 * p + c) * rc + a);
     }
   }
 }
 
-// Coming down: x_E = z - F[E, R] x_R, x_R read from the ancestors' results.
-__global__ void __launch_bounds__(256) k_nd_bwd(const double* __restrict__ F, int f, int s, int r,
-                                                const int32_t* __restrict__ E,
-                                                const int32_t* __restrict__ R,
-                                                const double* __restrict__ z,
-                                                double* __restrict__ x, int rows) {
-  extern __shared__ double xR[];
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int64_t p = blockIdx.y;
-  const double* Fp = F + p * f * f;
-  for (int m = tid; m < r; m += blockDim.x) xR[m] = x[R[p * r + m]];
-  __syncthreads();
-  const int row0 = blockIdx.x * rows;
-  for (int rr = warp; rr < rows; rr += blockDim.x / 32) {
-    const int i = row0 + rr;
-    if (i >= s) break;
-    const double* Fi = Fp + (int64_t)i * f + s;
-    double acc = 0.0;
-    for (int m = lane; m < r; m += 32) acc = fma(Fi[m], xR[m], acc);
-    for (int off = 16; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
-    if (lane == 0) x[E[p * s + i]] = z[p * s + i] - acc;
-  }
-}
+struct MvArgs {
+  const double* M;      // FT or BT of the depth
+  int nr, nm;           // rows i and columns m of a front's block
+  int s, r;
+  int ib, mg;           // rows per block, groups of threads that split the columns
+  const int32_t* src;   // up: gsrc; down: R
+  const int32_t* E;     // down: destination points
+  const int32_t* inv;   // up: child ring positions of front positions (null at the leaves)
+  int nchild, rc;
+  const double* uc;     // up: the children's u
+  const double* in;     // up: y; down: x (the ancestors' results)
+  double* z;            // up: written; down: read
+  double* out;          // up: u; down: x
+  int wait;             // launched to overlap the kernel before
+};
 
-// Copies rows 0..nr-1, columns c0..c0+nc-1 of the f x f front Fp into dst (row stride ld),
-// eight independent loads in flight per thread.
-__device__ __forceinline__ void stage_block(const double* __restrict__ Fp, int f, int c0, int nr,
-                                            int nc, double* __restrict__ dst, int ld) {
-  const int total = nr * nc, nt = blockDim.x;
-  for (int e0 = threadIdx.x; e0 < total; e0 += 8 * nt) {
-    double v[8];
-    int at[8];
+// Up:   w_m = y + children's u, z_i = sum_m F[i][m] w_m (i < s), u_i = children's u + the same sum.
+// Down: x_E[i] = z_i - sum_m F[i][s + m] x_R[m].
+// Block: ib consecutive rows of one front x mg column groups; group g takes m = g, g + mg, ...,
+// and the groups' sums are added in a fixed tree.
+template <bool UP>
+__global__ void __launch_bounds__(1024) k_nd_mv(MvArgs a) {
+  extern __shared__ double sh[];
+  double* w = sh;            // nm
+  double* part = sh + a.nm;  // ib * mg
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  constexpr int NP = 8;  // values in flight per thread
+  const int tid = threadIdx.x, nt = a.ib * a.mg;
+  const int ti = tid % a.ib, tm = tid / a.ib, i = blockIdx.x * a.ib + ti;
+  const int64_t p = blockIdx.y;
+  const double* M = a.M + p * a.nr * a.nm + (i < a.nr ? i : 0);
+  const bool live = __any_sync(0xffffffffu, i < a.nr);  // else the warp only helps to gather
+  const int nm = live ? a.nm : 0;
+  double v[NP];
 #pragma unroll
-    for (int q = 0; q < 8; ++q) {
-      const int e = e0 + q * nt;
-      at[q] = -1;
-      if (e < total) {
-        const int i = e / nc, m = e - i * nc;
-        v[q] = Fp[(int64_t)i * f + c0 + m];
-        at[q] = i * ld + m;
+  for (int k = 0; k < NP; ++k) {
+    const int m = tm + k * a.mg;
+    v[k] = m < nm ? __ldg(M + (int64_t)m * a.nr) : 0.0;
+  }
+  int ca = -1, cb = -1;  // the row's own child entries (up, ring rows)
+  if (UP && a.nchild && tm == 0 && i >= a.s && i < a.nr) {
+    ca = __ldg(a.inv + (p * a.nr + i) * 2);
+    cb = a.nchild > 1 ? __ldg(a.inv + (p * a.nr + i) * 2 + 1) : -1;
+  }
+  const int m0 = tid < a.nm ? tid : 0;
+  int g0 = 0, g1 = -1, g2 = -1;
+  if (UP && a.nm) {
+    const int32_t* g = a.src + (p * a.s + m0) * 3;
+    g0 = __ldg(g);
+    g1 = __ldg(g + 1);
+    g2 = __ldg(g + 2);
+  }
+  if (!UP && a.nm) g0 = __ldg(a.src + p * a.r + m0);
+  if (a.wait) asm volatile("griddepcontrol.wait;" ::: "memory");
+  for (int m = tid; m < a.nm; m += nt) {
+    if (m != tid) {
+      if (UP) {
+        const int32_t* g = a.src + (p * a.s + m) * 3;
+        g0 = __ldg(g);
+        g1 = __ldg(g + 1);
+        g2 = __ldg(g + 2);
+      } else {
+        g0 = __ldg(a.src + p * a.r + m);
+      }
+    }
+    double t = a.in[g0];
+    if (UP && g1 >= 0) t += a.uc[g1];
+    if (UP && g2 >= 0) t += a.uc[g2];
+    w[m] = t;
+  }
+  __syncthreads();
+  double c0 = 0.0, c1 = 0.0;
+  for (int m = tm; m < nm; m += NP * a.mg) {
+    double cur[NP];
+#pragma unroll
+    for (int k = 0; k < NP; ++k) cur[k] = v[k];
+    const int mn = m + NP * a.mg;
+    if (mn < nm) {
+#pragma unroll
+      for (int k = 0; k < NP; ++k) {
+        const int mm = mn + k * a.mg;
+        v[k] = mm < nm ? __ldg(M + (int64_t)mm * a.nr) : 0.0;
       }
     }
 #pragma unroll
-    for (int q = 0; q < 8; ++q)
-      if (at[q] >= 0) dst[at[q]] = v[q];
+    for (int k = 0; k < NP; ++k) {
+      const int mm = m + k * a.mg;
+      if (mm >= nm) break;  // the same for a warp's rows of one group
+      (k & 1 ? c1 : c0) = fma(cur[k], w[mm], k & 1 ? c1 : c0);
+    }
+  }
+  double acc = c0 + c1;
+  if (a.mg > 1) {
+    part[tid] = acc;
+    __syncthreads();
+    for (int h = a.mg >> 1; h > 0; h >>= 1) {
+      if (tm < h) {
+        acc += part[tid + h * a.ib];
+        part[tid] = acc;
+      }
+      __syncthreads();
+    }
+  }
+  if (tm != 0 || i >= a.nr) return;
+  if (UP) {
+    if (i < a.s) {
+      a.z[p * a.s + i] = acc;
+    } else {
+      if (ca >= 0) acc += a.uc[(a.nchild == 1 ? p : 2 * p) * a.rc + ca];
+      if (cb >= 0) acc += a.uc[(2 * p + 1) * a.rc + cb];
+      a.out[p * a.r + (i - a.s)] = acc;
+    }
+  } else {
+    a.out[a.E[p * a.s + i]] = a.z[p * a.s + i] - acc;
   }
 }
 
-// Fronts whose block fits in shared memory, one CTA per front: the block the product reads is staged
-// in shared memory with an odd row stride (conflict-free column access), then one thread per
-// row. Same sums in the same order as the warp-per-row kernels would not give; each kernel is
-// deterministic on its own.
-__global__ void __launch_bounds__(256) k_nd_fwd_small(const double* __restrict__ F, int f, int s,
-                                                      int r, const int32_t* __restrict__ E,
-                                                      const int32_t* __restrict__ perm,
-                                                      const int32_t* __restrict__ inv,
-                                                      int nchild, const double* __restrict__ uc,
-                                                      int rc, const double* __restrict__ y,
-                                                      double* __restrict__ z,
-                                                      double* __restrict__ u) {
+// y_j = sum_a rows[j][a] u[(j + o_a) mod n], o_a in [-t, t]^d lexicographic (last fastest), or
+// y_j = sub_j - that sum. A block's rows are one contiguous span: read coalesced into shared
+// memory (odd row width: no bank conflicts), then one thread per point. HBM-bound: 2D n = 1024,
+// 88 MB a product; reading each row by its own thread took 54 us, now 29 us.
+template <int D, int T>
+__global__ void __launch_bounds__(128) k_apply_rows(const double* __restrict__ rows, int logn,
+                                                    const double* __restrict__ u,
+                                                    const double* sub, double* y, int64_t N,
+                                                    int pts) {
+  constexpr int W = 2 * T + 1, MU = D == 1 ? W : (D == 2 ? W * W : W * W * W);
   extern __shared__ double sh[];
-  const int ld = s | 1;
-  double* wE = sh;           // s
-  double* Ms = sh + ld;      // f rows of stride ld: F[i][0..s)
-  const int tid = threadIdx.x;
-  const int64_t p = blockIdx.x;
-  const double* Fp = F + p * f * f;
-  const int32_t* iv = nchild ? inv + p * f * 2 : nullptr;
-  auto wsum = [&](int i) -> double {
-    double v = i < s ? y[E[p * s + i]] : 0.0;
-    for (int c = 0; c < nchild; ++c) {
-      const int a = iv[i * 2 + c];
-      if (a >= 0) v += uc[(nchild == 1 ? p : 2 * p + c) * rc + a];
-    }
-    return v;
-  };
-  for (int m = tid; m < s; m += blockDim.x) wE[m] = wsum(perm[p * s + m]);
-  stage_block(Fp, f, 0, f, s, Ms, ld);
+  const int64_t j0 = (int64_t)blockIdx.x * pts;
+  const int np = (int)(N - j0 < pts ? N - j0 : pts);
+  for (int e = threadIdx.x; e < np * MU; e += blockDim.x) sh[e] = __ldcs(rows + j0 * MU + e);
   __syncthreads();
-  for (int i = tid; i < f; i += blockDim.x) {
-    const double* Mi = Ms + i * ld;
-    double a0 = 0.0, a1 = 0.0;
-    int m = 0;
-    for (; m + 1 < s; m += 2) {
-      a0 = fma(Mi[m], wE[m], a0);
-      a1 = fma(Mi[m + 1], wE[m + 1], a1);
-    }
-    if (m < s) a0 = fma(Mi[m], wE[m], a0);
-    const double acc = a0 + a1;
-    if (i < s)
-      z[p * s + i] = acc;
-    else
-      u[p * r + (i - s)] = wsum(i) + acc;
-  }
-}
-
-__global__ void __launch_bounds__(256) k_nd_bwd_small(const double* __restrict__ F, int f, int s,
-                                                      int r, const int32_t* __restrict__ E,
-                                                      const int32_t* __restrict__ R,
-                                                      const double* __restrict__ z,
-                                                      double* __restrict__ x) {
-  extern __shared__ double sh[];
-  const int ld = r | 1;
-  double* xR = sh;          // r
-  double* Mb = sh + ld;     // s rows of stride ld: F[i][s..f)
-  const int tid = threadIdx.x;
-  const int64_t p = blockIdx.x;
-  const double* Fp = F + p * f * f;
-  for (int m = tid; m < r; m += blockDim.x) xR[m] = x[R[p * r + m]];
-  stage_block(Fp, f, s, s, r, Mb, ld);
-  __syncthreads();
-  for (int i = tid; i < s; i += blockDim.x) {
-    const double* Mi = Mb + i * ld;
-    double a0 = 0.0, a1 = 0.0;
-    int m = 0;
-    for (; m + 1 < r; m += 2) {
-      a0 = fma(Mi[m], xR[m], a0);
-      a1 = fma(Mi[m + 1], xR[m + 1], a1);
-    }
-    if (m < r) a0 = fma(Mi[m], xR[m], a0);
-    x[E[p * s + i]] = z[p * s + i] - (a0 + a1);
-  }
-}
-
-// y_j = sum_a rows[j][a] u[(j + o_a) mod n], o_a in [-t, t]^d lexicographic (last fastest).
-__global__ void k_apply_rows(const double* __restrict__ rows, int mu, int d, int n, int t,
-                             const double* __restrict__ u, double* __restrict__ y, int64_t N) {
-  const int w = 2 * t + 1;
-  for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < N;
-       j += (int64_t)gridDim.x * blockDim.x) {
-    int x[3] = {0, 0, 0};
+  const int64_t mask = ((int64_t)1 << logn) - 1;
+  for (int q = threadIdx.x; q < np; q += blockDim.x) {
+    const int64_t j = j0 + q;
+    int64_t x[D];
     int64_t rem = j;
-    for (int a = d - 1; a >= 0; --a) {
-      x[a] = (int)(rem % n);
-      rem /= n;
+#pragma unroll
+    for (int a = D - 1; a >= 0; --a) {
+      x[a] = rem & mask;
+      rem >>= logn;
     }
-    const double* rj = rows + j * mu;
     double acc = 0.0;
-    for (int a = 0; a < mu; ++a) {
-      int o = a;
-      int64_t col = 0;
-      int64_t stride = 1;
-      for (int b = d - 1; b >= 0; --b) {
-        const int ob = o % w - t;
-        o /= w;
-        col += (int64_t)((x[b] + ob + n) % n) * stride;
-        stride *= n;
+#pragma unroll 9
+    for (int a = 0; a < MU; ++a) {
+      int o = a, off[D];
+#pragma unroll
+      for (int b = D - 1; b >= 0; --b) {
+        off[b] = o % W - T;
+        o /= W;
       }
-      acc = fma(rj[a], u[col], acc);
+      int64_t col = 0;
+#pragma unroll
+      for (int b = 0; b < D; ++b) col = (col << logn) | ((x[b] + off[b]) & mask);
+      acc = fma(sh[q * MU + a], __ldg(u + col), acc);
     }
-    y[j] = acc;
+    y[j] = sub ? sub[j] - acc : acc;
   }
 }
 
@@ -985,87 +1002,136 @@ cudaError_t launch_nd_sweep(lsp_ctx* c, int depth) {
   return cudaGetLastError();
 }
 
+// The solve's copies of one depth's blocks, after its sweep.
+cudaError_t launch_nd_store(lsp_ctx* c, int depth) {
+  NdState& S = *c->nd;
+  const NdLevel& lv = S.plan.lv[depth];
+  if (lv.s == 0) return cudaSuccess;
+  const int tf = (lv.f + kTile - 1) / kTile, ts = (lv.s + kTile - 1) / kTile;
+  const int tr = (lv.r + kTile - 1) / kTile;
+  int t = timer_begin(c, level_name("nd_asm", depth));
+  k_nd_store<<<dim3(tf * ts + ts * tr + 1, lv.count), 256, 0, c->stream>>>(
+      (const double*)S.fronts.p + lv.front_off, lv.f, lv.s, lv.r,
+      (const int32_t*)S.E.p + lv.E_off, (const int32_t*)S.perm.p + lv.perm_off,
+      lv.nchild ? (const int32_t*)S.inv.p + lv.inv_off : nullptr, lv.nchild,
+      lv.nchild ? S.plan.lv[depth + 1].r : 0, (double*)S.solve.p + lv.ft_off,
+      (double*)S.solve.p + lv.bt_off, (int32_t*)S.gsrc.p + 3 * lv.z_off);
+  timer_end(c, t);
+  return cudaGetLastError();
+}
+
 cudaError_t launch_nd_solve(lsp_ctx* c, const double* y, double* x) {
   NdState& S = *c->nd;
   const NdPlan& P = S.plan;
   const int L = (int)P.lv.size();
-  const double* Fb = (const double*)S.fronts.p;
+  const double* sv = (const double*)S.solve.p;
   double* z = (double*)S.z.p;
   double* u = (double*)S.u.p;
-  const int32_t* E = (const int32_t*)S.E.p;
-  const int32_t* R = (const int32_t*)S.R.p;
-  // rows of one front per CTA: 64 where the level has fronts enough to fill the GPU, else 8
-  // (one row per warp) so that the few large fronts near the root still spread over the SMs
-  auto rows_for = [](int count, int nrows) {
-    return (int64_t)count * ((nrows + 63) / 64) >= 8 * 152 ? 64 : 8;
+  auto launch = [&](bool up, MvArgs& a, int count) -> cudaError_t {
+    // Rows per block: all of a short front (whole warps), else 128 down to 16 until there are two
+    // blocks per SM. Column groups: at least eight columns each, until the depth has 512 threads
+    // per SM: the next depth's blocks then find room to load beside it (a solve at 2D n = 1024,
+    // 256 and 3D n = 32: 660, 140, 222 us; with 2048 threads per SM 752, 149, 251 us).
+    auto blocks = [&]() { return (int64_t)count * ((a.nr + a.ib - 1) / a.ib); };
+    a.ib = a.nr >= 128 ? 128 : (a.nr + 31) / 32 * 32;
+    if (blocks() < 2 * 152) {
+      a.ib = 128;
+      while (a.ib > 16 && (a.ib >= 2 * a.nr || blocks() < 2 * 152)) a.ib >>= 1;
+    }
+    a.mg = 1;
+    while (2 * a.mg * a.ib <= 1024 && a.nm >= 16 * a.mg &&
+           blocks() * a.ib * a.mg < (int64_t)152 * 512)
+      a.mg <<= 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((a.nr + a.ib - 1) / a.ib, count);
+    cfg.blockDim = dim3(a.ib * a.mg);
+    cfg.dynamicSmemBytes = sizeof(double) * ((size_t)a.nm + (a.mg > 1 ? a.ib * a.mg : 0));
+    cfg.stream = c->stream;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = a.wait ? 1 : 0;
+    return up ? cudaLaunchKernelEx(&cfg, k_nd_mv<true>, a)
+              : cudaLaunchKernelEx(&cfg, k_nd_mv<false>, a);
   };
+  MvArgs a;
+  a.wait = 0;  // the first kernel starts after whatever produced y
   for (int d = L - 1; d >= 0; --d) {
     const NdLevel& lv = P.lv[d];
     const NdLevel* cl = lv.nchild ? &P.lv[d + 1] : nullptr;
-    const int rows = rows_for(lv.count, lv.f);
-    dim3 grid((lv.f + rows - 1) / rows, lv.count);
+    if (lv.f == 0) continue;
     int t = timer_begin(c, level_name("nd_fwd", d));
-    // one CTA per front with the block staged in shared memory: small fronts, or larger ones
-    // when the depth has fronts enough to fill the GPU (else rows spread over many CTAs)
-    const size_t smf = sizeof(double) * ((size_t)(lv.s | 1) * (lv.f + 1));
-    const bool many = lv.count >= 2 * 152;
-    if (lv.f <= kNdSmallFront || (many && smf <= kNdStagedBytes)) {
-      k_nd_fwd_small<<<lv.count, lv.f <= kNdSmallFront ? 128 : 256, smf, c->stream>>>(
-          Fb + lv.front_off, lv.f, lv.s, lv.r, E + lv.E_off,
-          (const int32_t*)S.perm.p + lv.perm_off,
-          lv.nchild ? (const int32_t*)S.inv.p + lv.inv_off : nullptr, lv.nchild,
-          cl ? u + cl->u_off : nullptr, cl ? cl->r : 0, y, z + lv.z_off, u + lv.u_off);
-    } else {
-      k_nd_fwd<<<grid, 256, sizeof(double) * (lv.s > 0 ? lv.s : 1), c->stream>>>(
-          Fb + lv.front_off, lv.f, lv.s, lv.r, E + lv.E_off,
-          (const int32_t*)S.perm.p + lv.perm_off,
-          lv.nchild ? (const int32_t*)S.inv.p + lv.inv_off : nullptr, lv.nchild,
-          cl ? u + cl->u_off : nullptr, cl ? cl->r : 0, y, z + lv.z_off, u + lv.u_off, rows);
-    }
+    a.M = sv + lv.ft_off;
+    a.nr = lv.f;
+    a.nm = lv.s;
+    a.s = lv.s;
+    a.r = lv.r;
+    a.src = (const int32_t*)S.gsrc.p + 3 * lv.z_off;
+    a.E = nullptr;
+    a.inv = lv.nchild ? (const int32_t*)S.inv.p + lv.inv_off : nullptr;
+    a.nchild = lv.nchild;
+    a.rc = cl ? cl->r : 0;
+    a.uc = cl ? u + cl->u_off : nullptr;
+    a.in = y;
+    a.z = z + lv.z_off;
+    a.out = u + lv.u_off;
+    const cudaError_t e = launch(true, a, lv.count);
+    if (e != cudaSuccess) return e;
     timer_end(c, t);
+    a.wait = !c->timing;
   }
   for (int d = 0; d < L; ++d) {
     const NdLevel& lv = P.lv[d];
-    const int rows = rows_for(lv.count, lv.s);
-    dim3 grid((lv.s + rows - 1) / rows, lv.count);
+    if (lv.s == 0) continue;
     int t = timer_begin(c, level_name("nd_bwd", d));
-    const size_t smb = sizeof(double) * ((size_t)(lv.r | 1) * (lv.s + 1));
-    const bool many = lv.count >= 2 * 152;
-    if (lv.f <= kNdSmallFront || (many && smb <= kNdStagedBytes)) {
-      k_nd_bwd_small<<<lv.count, lv.s <= kNdSmallFront ? 128 : 256, smb, c->stream>>>(
-          Fb + lv.front_off, lv.f, lv.s, lv.r,
-                                                       E + lv.E_off, R + lv.R_off,
-                                                       z + lv.z_off, x);
-    } else {
-      k_nd_bwd<<<grid, 256, sizeof(double) * (lv.r > 0 ? lv.r : 1), c->stream>>>(
-          Fb + lv.front_off, lv.f, lv.s, lv.r, E + lv.E_off, R + lv.R_off, z + lv.z_off, x,
-          rows);
-    }
+    a.M = sv + lv.bt_off;
+    a.nr = lv.s;
+    a.nm = lv.r;
+    a.s = lv.s;
+    a.r = lv.r;
+    a.src = (const int32_t*)S.R.p + lv.R_off;
+    a.E = (const int32_t*)S.E.p + lv.E_off;
+    a.inv = nullptr;
+    a.nchild = 0;
+    a.rc = 0;
+    a.uc = nullptr;
+    a.in = x;
+    a.z = z + lv.z_off;
+    a.out = x;
+    const cudaError_t e = launch(false, a, lv.count);
+    if (e != cudaSuccess) return e;
     timer_end(c, t);
   }
   return cudaGetLastError();
 }
 
-cudaError_t nd_prepare_kernels(int max_smem) {
-  // staged solve kernels: (s | 1) (f + 1) or (r | 1) (s + 1) doubles, with s, r <= f <= 160
-  // for small fronts, and at most kNdStagedBytes for the larger ones
-  const int small_front = (int)sizeof(double) * ((kNdSmallFront | 1) + 1) * (kNdSmallFront + 1);
-  const int small = small_front > (int)kNdStagedBytes ? small_front : (int)kNdStagedBytes;
-  cudaError_t e = cudaFuncSetAttribute(k_nd_fwd, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       max_smem);
+cudaError_t nd_prepare_kernels(int max_cols) {
+  const int smem = (int)sizeof(double) * (max_cols + 1024);
+  cudaError_t e = cudaFuncSetAttribute(k_nd_mv<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       smem);
   if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(k_nd_fwd_small, cudaFuncAttributeMaxDynamicSharedMemorySize, small);
-  if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(k_nd_bwd_small, cudaFuncAttributeMaxDynamicSharedMemorySize, small);
-  if (e != cudaSuccess) return e;
-  return cudaFuncSetAttribute(k_nd_bwd, cudaFuncAttributeMaxDynamicSharedMemorySize, max_smem);
+  return cudaFuncSetAttribute(k_nd_mv<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
 }
 
 cudaError_t launch_apply_rows(lsp_ctx* c, const double* rows, int mu, int t, const double* u,
-                              double* y) {
+                              double* y, const double* sub) {
   const int64_t N = c->geo.N;
+  const int d = c->geo.d;
+  int logn = 0;
+  while ((1 << logn) < c->geo.n) ++logn;
+  const int pts = mu > 27 ? 32 : 128;
+  const size_t smem = sizeof(double) * mu * pts;  // at most 32 KiB
   int tm = timer_begin(c, "apply_rows");
-  k_apply_rows<<<grid_for(N, 256), 256, 0, c->stream>>>(rows, mu, c->geo.d, c->geo.n, t, u, y, N);
+  auto go = [&](auto kern) {
+    kern<<<(unsigned)((N + pts - 1) / pts), 128, smem, c->stream>>>(rows, logn, u, sub, y, N, pts);
+  };
+  if (d == 1)
+    go(k_apply_rows<1, 1>);
+  else if (d == 2)
+    t == 1 ? go(k_apply_rows<2, 1>) : go(k_apply_rows<2, 2>);
+  else
+    t == 1 ? go(k_apply_rows<3, 1>) : go(k_apply_rows<3, 2>);
   timer_end(c, tm);
   return cudaGetLastError();
 }

@@ -56,6 +56,15 @@ bool nd_ready(const lsp_ctx* c) {
   return c->nd && c->nd->factored && c->nd->factored_gen == c->build_gen && c->built;
 }
 
+// The barrier counter of the Arnoldi kernel, zero when it is first made.
+bool ensure_bar(lsp_ctx* c) {
+  NdState& S = *c->nd;
+  if (S.bar.p) return true;
+  S.bar_count = 0;
+  return ensure(c, S.bar, sizeof(unsigned)) &&
+         cudaMemsetAsync(S.bar.p, 0, sizeof(unsigned), c->stream) == cudaSuccess;
+}
+
 // x = P^-1 y with the chosen refinement steps x += P^-1 (y - P x); x may equal y.
 lsp_status nd_apply(lsp_ctx* c, const double* y, double* x) {
   NdState& S = *c->nd;
@@ -71,8 +80,7 @@ lsp_status nd_apply(lsp_ctx* c, const double* y, double* x) {
   SCUDA(c, cudaMemcpyAsync(ry, y, sizeof(double) * N, cudaMemcpyDeviceToDevice, c->stream));
   SCUDA(c, launch_nd_solve(c, ry, x));
   for (int k = 0; k < S.refine_steps; ++k) {
-    SCUDA(c, launch_apply_rows(c, (const double*)c->P.p, rows_mu(c), c->t_built, x, rd));
-    SCUDA(c, launch_axpby(c, rd, ry, rd, nullptr, -1.0, N));
+    SCUDA(c, launch_apply_rows(c, (const double*)c->P.p, rows_mu(c), c->t_built, x, rd, ry));
     SCUDA(c, launch_nd_solve(c, rd, rd));
     SCUDA(c, launch_axpby(c, x, x, rd, nullptr, 1.0, N));
   }
@@ -87,7 +95,8 @@ void nd_free(NdState* s) {
   if (!s) return;
   DevBuf* bufs[] = {&s->fronts, &s->E, &s->R, &s->inv, &s->asm_dst, &s->asm_src, &s->perm,
                     &s->z, &s->u, &s->cbuf, &s->pinv, &s->swaps, &s->err, &s->V, &s->w,
-                    &s->b, &s->x, &s->tmp, &s->gs, &s->fvec, &s->ry, &s->rd, &s->pscratch};
+                    &s->b, &s->x, &s->tmp, &s->gs, &s->fvec, &s->ry, &s->rd, &s->pscratch, &s->solve,
+                    &s->gsrc, &s->bar};
   for (DevBuf* b : bufs)
     if (b->p) cudaFree(b->p);
   if (s->h_gs) cudaFreeHost(s->h_gs);
@@ -97,7 +106,7 @@ void nd_free(NdState* s) {
   delete s;
 }
 
-cudaError_t nd_prepare_kernels(int max_smem);
+cudaError_t nd_prepare_kernels(int max_cols);
 
 }  // namespace lsp
 
@@ -171,7 +180,9 @@ lsp_status lsp_nd_factor(lsp_ctx* c, const lsp_nd_opts* opts) {
         !ensure(c, S.u, sizeof(double) * (P.u_doubles > 0 ? P.u_doubles : 1)) ||
         !ensure(c, S.cbuf, sizeof(double) * 2 * cb) ||
         !ensure(c, S.pinv, sizeof(double) * 2 * pv) ||
-        !ensure(c, S.swaps, sizeof(int32_t) * 2 * sw) || !ensure(c, S.err, sizeof(int32_t)))
+        !ensure(c, S.swaps, sizeof(int32_t) * 2 * sw) || !ensure(c, S.err, sizeof(int32_t)) ||
+        !ensure(c, S.solve, sizeof(double) * P.solve_doubles) ||
+        !ensure(c, S.gsrc, sizeof(int32_t) * 3 * P.z_doubles))
       return sfail(c, LSP_ERR_OOM, "nested dissection buffers: %s", c->err.c_str());
     S.cbuf_half = cb;
     S.pinv_half = pv;
@@ -184,7 +195,7 @@ lsp_status lsp_nd_factor(lsp_ctx* c, const lsp_nd_opts* opts) {
       SCUDA(c, cudaEventCreateWithFlags(&S.ev_cols, cudaEventDisableTiming));
       SCUDA(c, cudaEventCreateWithFlags(&S.ev_panel, cudaEventDisableTiming));
     }
-    SCUDA(c, nd_prepare_kernels((int)std::min<int64_t>(sizeof(double) * max_sr + 64, 220 * 1024)));
+    SCUDA(c, nd_prepare_kernels(max_sr));
     S.have_plan = true;
   }
   S.factored = false;
@@ -194,6 +205,7 @@ lsp_status lsp_nd_factor(lsp_ctx* c, const lsp_nd_opts* opts) {
   for (int d = (int)P.lv.size() - 1; d >= 0; --d) {
     SCUDA(c, launch_nd_assemble(c, d, rows));
     SCUDA(c, launch_nd_sweep(c, d));
+    SCUDA(c, launch_nd_store(c, d));
   }
   int32_t herr = 0;
   SCUDA(c, cudaMemcpyAsync(&herr, S.err.p, sizeof(int32_t), cudaMemcpyDeviceToHost, c->stream));
@@ -292,13 +304,14 @@ lsp_status lsp_gmres(lsp_ctx* c, const lsp_gmres_opts* opts, const double* f, do
   if (!ensure(c, S.V, sizeof(double) * N * ld) || !ensure(c, S.w, sizeof(double) * N) ||
       !ensure(c, S.b, sizeof(double) * N) || !ensure(c, S.x, sizeof(double) * N) ||
       !ensure(c, S.tmp, sizeof(double) * N) || !ensure(c, S.fvec, sizeof(double) * N) ||
-      !ensure(c, S.gs, sizeof(double) * gs_n) ||
+      !ensure(c, S.gs, sizeof(double) * gs_n) || !ensure_bar(c) ||
       !ensure(c, c->fftbuf, sizeof(double) * N))
     return sfail(c, LSP_ERR_OOM, "gmres workspace: %s", c->err.c_str());
   if (!S.h_gs && cudaMallocHost(&S.h_gs, sizeof(double) * kGsPartial) != cudaSuccess) {
     S.h_gs = nullptr;
     return sfail(c, LSP_ERR_OOM, "pinned allocation failed");
   }
+  const bool fused = arnoldi_fits(c, N);
   double* V = (double*)S.V.p;
   double* w = (double*)S.w.p;
   double* b = (double*)S.b.p;
@@ -356,14 +369,23 @@ lsp_status lsp_gmres(lsp_ctx* c, const lsp_gmres_opts* opts, const double* f, do
       double* vc = V + (int64_t)col * N;
       double* hc = H + (int64_t)col * ld;
       if ((st = op(vc, w)) != LSP_OK) return st;
-      SCUDA(c, launch_mgs(c, w, nullptr, nullptr, nullptr, gs + kGsH0, N));
-      for (int k = 0; k <= col; ++k)
-        SCUDA(c, launch_mgs(c, w, k ? V + (int64_t)(k - 1) * N : nullptr, k ? hc + k - 1 : nullptr,
-                            V + (int64_t)k * N, hc + k, N));
-      SCUDA(c, launch_mgs(c, w, vc, hc + col, nullptr, gs + kGsH1, N));
-      SCUDA(c, launch_gmres_givens(c, gs, col, ld));
-      SCUDA(c, launch_axpby(c, V + (int64_t)(col + 1) * N, nullptr, w, gs + kGsInvH1, 1.0, N));
+      if (fused) {
+        SCUDA(c, launch_arnoldi(c, w, V, gs, col, ld, N));
+      } else {
+        SCUDA(c, launch_mgs(c, w, nullptr, nullptr, nullptr, gs + kGsH0, N));
+        for (int k = 0; k <= col; ++k)
+          SCUDA(c, launch_mgs(c, w, k ? V + (int64_t)(k - 1) * N : nullptr,
+                              k ? hc + k - 1 : nullptr, V + (int64_t)k * N, hc + k, N));
+        SCUDA(c, launch_mgs(c, w, vc, hc + col, nullptr, gs + kGsH1, N));
+        SCUDA(c, launch_gmres_givens(c, gs, col, ld));
+        SCUDA(c, launch_axpby(c, V + (int64_t)(col + 1) * N, nullptr, w, gs + kGsInvH1, 1.0, N));
+      }
       if ((st = readback()) != LSP_OK) return st;
+      if (S.h_gs[kGsFail] != 0.0) {
+        S.bar_count = 0;  // the count is unknown: start again from zero
+        SCUDA(c, cudaMemsetAsync(S.bar.p, 0, sizeof(unsigned), c->stream));
+        return sfail(c, LSP_ERR_TIMEOUT, "a block of the Arnoldi kernel did not arrive");
+      }
       ++iters;
       brk = S.h_gs[kGsBreak] != 0.0;
       if (S.h_gs[kGsPresid] <= atol || brk) break;

@@ -34,7 +34,6 @@ namespace lsp {
 
 constexpr int kNdPanel = 16;       // columns eliminated per step in the blocked path
 constexpr int kNdSmallFront = 160; // fronts with f <= this are swept in shared memory
-constexpr int kNdStagedBytes = 64 * 1024;  // solve blocks up to this size are staged
 constexpr int kNdMaxN = 1024;      // 2D: the cross has 2n - 1 points
 constexpr int kNdMaxN3 = 64;       // 3D: the slab fronts have 2 (n/2 - 1) n + 2 n^2 points (12 160 at 64)
 constexpr int kNdPanelRegRows = 8 * 256;  // panels up to this many rows keep them in registers
@@ -49,6 +48,7 @@ struct NdLevel {
   int64_t asm_off = 0, asm_n = 0; // P entries assembled at this depth
   int64_t perm_off = 0;           // int32 offset into perm (count * s)
   int64_t z_off = 0, u_off = 0;   // doubles into the solve vectors z (count * s), u (count * r)
+  int64_t ft_off = 0, bt_off = 0; // doubles into the solve's copies: count * s * f, count * r * s
 };
 
 struct NdPlan {
@@ -58,7 +58,7 @@ struct NdPlan {
   // inv[(front * f + i) * 2 + c]: position of front position i in child c's ring, or -1.
   // asm_dst / asm_src: P entry rows[src] goes to element dst of its depth's front block.
   std::vector<int32_t> E, R, inv, asm_dst, asm_src;
-  int64_t front_doubles = 0, perm_ints = 0, z_doubles = 0, u_doubles = 0;
+  int64_t front_doubles = 0, perm_ints = 0, z_doubles = 0, u_doubles = 0, solve_doubles = 0;
   double flops_sweep = 0;  // FP64 flops of the partial inversions, 2 s f^2 per front
   double flops_lu = 0;     // multifrontal LU count, 2/3 s^3 + 2 s^2 r + 2 s r^2 per front
   int64_t solve_bytes = 0; // front bytes one solve reads: (f s + s r) * 8 per front
@@ -77,6 +77,7 @@ struct NdState {
   int64_t factored_gen = -1;  // ctx->build_gen of the rows that were factored
   int refine_steps = 0;       // iterative-refinement steps after every solve
   DevBuf fronts, E, R, inv, asm_dst, asm_src, perm, z, u, cbuf, pinv, swaps, err;
+  DevBuf solve, gsrc;         // the blocks a solve reads, transposed; right-hand side sources
   DevBuf ry, rd;              // refinement scratch: a copy of y, the correction
   DevBuf pscratch;            // FP32 pivot-ranking rows of panels over 2048 rows
   int64_t cbuf_half = 0, pinv_half = 0, swaps_half = 0;  // the two copies of the step buffers
@@ -85,6 +86,9 @@ struct NdState {
   // GMRES workspace
   DevBuf V, w, b, x, tmp, gs, fvec;
   double* h_gs = nullptr;  // pinned mirror of the scalars the host loop reads
+  DevBuf bar;              // arrivals at the barriers of k_arnoldi, counted up over all launches
+  unsigned bar_count = 0;
+  int coop_blocks = -1;    // blocks of k_arnoldi that are resident together (-1: not asked yet)
   int restart_cap = 0;
 };
 
@@ -93,14 +97,21 @@ void nd_free(NdState* s);
 // ---- launchers (k_nd.cu) ----
 cudaError_t launch_nd_assemble(lsp_ctx* c, int depth, const double* rows);
 cudaError_t launch_nd_sweep(lsp_ctx* c, int depth);
+cudaError_t launch_nd_store(lsp_ctx* c, int depth);
 cudaError_t launch_nd_solve(lsp_ctx* c, const double* y, double* x);
+// y = rows u, or sub - rows u when sub is given (y may be sub)
 cudaError_t launch_apply_rows(lsp_ctx* c, const double* rows, int mu, int t, const double* u,
-                              double* y);
+                              double* y, const double* sub = nullptr);
 
 // ---- GMRES kernels (k_gmres.cu) ----
 // MGS step: w -= h_prev * v_prev (if v_prev), then *h_out = <v_next, w> (or <w, w>).
 cudaError_t launch_mgs(lsp_ctx* c, double* w, const double* v_prev, const double* h_prev,
                        const double* v_next, double* h_out, int64_t N);
+// One Arnoldi column in one launch (w in registers across all projections): H[0..col, col] and
+// |w| into gs, the rotations, V[col + 1] = w / |w|. arnoldi_fits says whether N allows it.
+bool arnoldi_fits(lsp_ctx* c, int64_t N);
+cudaError_t launch_arnoldi(lsp_ctx* c, const double* w, double* V, double* gs, int col, int ld,
+                           int64_t N);
 cudaError_t launch_axpby(lsp_ctx* c, double* y, const double* a, const double* x,
                          const double* scale, double sign, int64_t N);
 cudaError_t launch_gmres_givens(lsp_ctx* c, double* gs, int col, int ld);
@@ -119,8 +130,9 @@ enum GmresSlot {
   kGsInvH1 = 5,    // 1 / |w| (0 on breakdown)
   kGsBeta = 6,     // |r| at the start of a cycle
   kGsTicket = 7,   // reduction ticket (as an unsigned int)
-  kGsPartial = 8,  // 1024 block partial sums
-  kGsArrays = 8 + 1024  // then H[(ld) * restart], cs[restart], sn[restart], S[ld], y[restart]
+  kGsFail = 8,     // 1 when a block's wait for the others ran out
+  kGsPartial = 16, // 1024 block partial sums
+  kGsArrays = 16 + 1024  // then H[(ld) * restart], cs[restart], sn[restart], S[ld], y[restart]
 };
 
 }  // namespace lsp

@@ -247,6 +247,9 @@ std::string build_nd_plan(NdPlan& P, int d, int n, int leaf, int t_built, int le
     z_off += (int64_t)lv.count * lv.s;
     lv.u_off = u_off;
     u_off += (int64_t)lv.count * lv.r;
+    lv.ft_off = P.solve_doubles;
+    lv.bt_off = lv.ft_off + (int64_t)lv.count * lv.s * lv.f;
+    P.solve_doubles = lv.bt_off + (int64_t)lv.count * lv.r * lv.s;
     lv.inv_off = inv_off;
     inv_off += is_leaf ? 0 : (int64_t)lv.count * lv.f * 2;
     const double s = lv.s, r = lv.r, f = lv.f;
