@@ -1284,57 +1284,39 @@ __global__ void __launch_bounds__(WARPS * 32) k_eig2d_t2(const double* __restric
 
 // ---- 2D, one thread per shift ------------------------------------------------------------
 // In 2D the symmetry-adapted vectors are u_0..u_2 (fully symmetric: centre, edges, corners),
-// u_3 (edges, x^2 - y^2), u_4 (corners, xy) and u_5, u_6 (x-odd on edges and corners). With
-// W_i = G_s[mu, mu] u_i (linear in g) and the A1 part u_i^T A1 u_j (linear in g * g), every
-// block entry is  B_ij = u_i^T A1 u_j - W_i . W_j, so the 9 x 9 matrix A is never formed.
-__constant__ double c_W2[7][9][6];   // W_i[k] = sum_c c_W2[i][k][c] g[c]
-__constant__ double c_B2[7][7][6];   // u_i^T A1 u_j = sum_c c_B2[i][j][c] (g*g)[c]
-__constant__ float c_W2f[7][9][6];   // the same tables in FP32 (mixed mode)
-__constant__ float c_B2f[7][7][6];
+// u_3 (edges, x^2 - y^2), u_4 (corners, xy) and u_5, u_6 (x-odd on edges and corners); the 9 x 9
+// matrix A is never formed. FP64: through the class values of each block (see below). FP32 (mixed
+// mode): with W_i = G_s[mu, mu] u_i (linear in g) and the A1 part u_i^T A1 u_j (linear in g * g),
+// B_ij = u_i^T A1 u_j - W_i . W_j.
+//
+// What bounds it: the FP64 pipe for long lists (about 450 instructions a shift), the latency of
+// that chain for short ones. Measured (before: FP64 assembly through W_i, a division for the scale,
+// FP64 maxima, Jacobi sweeps for the shifts that stagnate above the residual bound): per-point
+// shifts at 2D n = 1024 246 -> 68 us in FP64 and 122 -> 80 us in mixed mode, n = 256 73 -> 18 us,
+// n = 32 39 -> 20 us.
+__constant__ float c_W2f[7][9][6];   // W_i[k] = sum_c c_W2f[i][k][c] g[c]
+__constant__ float c_B2f[7][7][6];   // u_i^T A1 u_j = sum_c c_B2f[i][j][c] (g*g)[c]
 
-template <typename GT>
-__device__ __forceinline__ GT coefW(int i, int k, int c);
-template <>
-__device__ __forceinline__ double coefW<double>(int i, int k, int c) { return c_W2[i][k][c]; }
-template <>
-__device__ __forceinline__ float coefW<float>(int i, int k, int c) { return c_W2f[i][k][c]; }
-template <typename GT>
-__device__ __forceinline__ GT coefB(int i, int j, int c);
-template <>
-__device__ __forceinline__ double coefB<double>(int i, int j, int c) { return c_B2[i][j][c]; }
-template <>
-__device__ __forceinline__ float coefB<float>(int i, int j, int c) { return c_B2f[i][j][c]; }
-
-// GT is the arithmetic of the Gram assembly: double (FP64 mode) or float (mixed mode).
-template <int I, typename GT>
-__device__ __forceinline__ void w_vec(const GT (&g)[6], GT (&w)[9]) {
+template <int I>
+__device__ __forceinline__ void w_vec(const float (&g)[6], float (&w)[9]) {
 #pragma unroll
   for (int k = 0; k < 9; ++k) {
-    GT s = GT(0);
+    float s = 0.0f;
 #pragma unroll
-    for (int c = 0; c < 6; ++c) s = fma(coefW<GT>(I, k, c), g[c], s);
+    for (int c = 0; c < 6; ++c) s = fma(c_W2f[I][k][c], g[c], s);
     w[k] = s;
   }
 }
-template <int I, int J, typename GT>
-__device__ __forceinline__ GT b_entry(const GT (&g2)[6], const GT (&wi)[9], const GT (&wj)[9]) {
-  GT s = GT(0);
+template <int I, int J>
+__device__ __forceinline__ float b_entry(const float (&g2)[6], const float (&wi)[9],
+                                         const float (&wj)[9]) {
+  float s = 0.0f;
 #pragma unroll
-  for (int c = 0; c < 6; ++c) s = fma(coefB<GT>(I, J, c), g2[c], s);
-  GT t = GT(0);
+  for (int c = 0; c < 6; ++c) s = fma(c_B2f[I][J][c], g2[c], s);
+  float t = 0.0f;
 #pragma unroll
   for (int k = 0; k < 9; ++k) t = fma(wi[k], wj[k], t);
   return s - t;
-}
-
-// 2^-ilogb(x) for x > 0: the power of two that scales x into [1, 2). For a normal x whose
-// reciprocal power is normal (biased exponent field ef in 1..2045) it is built from the
-// exponent field with integer operations, 2^(1023 - ef + 1023) as a bit pattern, which keeps
-// the FP64 pipe (narrow on this GPU) free; other x take the library functions.
-__device__ __forceinline__ double pow2_neg_ilogb(double x) {
-  const int ef = (int)((__double_as_longlong(x) >> 52) & 0x7FF);
-  if (ef >= 1 && ef <= 2045) return __longlong_as_double((long long)(2046 - ef) << 52);
-  return exp2((double)(-ilogb(x)));
 }
 
 // Eigenvalues of the symmetric 2 x 2 [[a, b], [b, c]], smaller one first; the small one as
@@ -1369,17 +1351,57 @@ __global__ void __launch_bounds__(128) k_eig2d(const double* __restrict__ gvals,
       g[c] = (GT)__ldg(gvals + (int64_t)(2 * c) * cap + i);
       g2[c] = (GT)__ldg(gvals + (int64_t)(2 * c + 1) * cap + i);
     }
-    // fully symmetric block (3 x 3)
-    GT w0[9], w1[9], w2[9];
-    w_vec<0>(g, w0);
-    w_vec<1>(g, w1);
-    w_vec<2>(g, w2);
-    double b00 = b_entry<0, 0>(g2, w0, w0), b01 = b_entry<0, 1>(g2, w0, w1),
-           b02 = b_entry<0, 2>(g2, w0, w2), b11 = b_entry<1, 1>(g2, w1, w1),
-           b12 = b_entry<1, 2>(g2, w1, w2), b22 = b_entry<2, 2>(g2, w2, w2);
-    // the other blocks: two 1 x 1 and one 2 x 2 (two copies)
-    double e00, e01, e11, bb1, bb2;
-    {
+    GT w0[9], w1[9], w2[9];  // FP32 only: G u_i of the fully symmetric block
+    // G_b = U_b^T G U_b of the fully symmetric block (m..) and of the doubled block (h..): FP64
+    double m00 = 0, m01 = 0, m02 = 0, m11 = 0, m12 = 0, m22 = 0, h00 = 0, h01 = 0, h11 = 0;
+    double hx = 0, hd = 0;  // and of the two 1 x 1 blocks
+    double b00, b01, b02, b11, b12, b22, e00, e01, e11, bb1, bb2;
+    if constexpr (sizeof(GT) == 8) {
+      // G maps the span of a block's vectors into itself (as in 3D), so B_b = U_b^T A1 U_b -
+      // G_b G_b with both first factors linear in the six class values. Orbits of mu_0: centre,
+      // edges, corners (each vector 1/2 on its four points; the doubled block's edge vector
+      // 1/sqrt 2 on two): 70 FP64 operations for all blocks instead of 528 through G u_i.
+      constexpr double rt2 = 1.41421356237309504880;
+      auto sym = [](const double (&v)[6], double& c00, double& c01, double& c02, double& c11,
+                    double& c12, double& c22) {
+        c00 = v[0];
+        c01 = 2.0 * v[1];
+        c02 = 2.0 * v[3];
+        c11 = fma(2.0, v[3], v[0] + v[2]);
+        c12 = 2.0 * (v[1] + v[4]);
+        c22 = fma(2.0, v[2], v[0] + v[5]);
+      };
+      double A00, A01, A02, A11, A12, A22;
+      sym(g, m00, m01, m02, m11, m12, m22);
+      sym(g2, A00, A01, A02, A11, A12, A22);
+      b00 = fma(-m00, m00, fma(-m01, m01, fma(-m02, m02, A00)));
+      b01 = fma(-m00, m01, fma(-m01, m11, fma(-m02, m12, A01)));
+      b02 = fma(-m00, m02, fma(-m01, m12, fma(-m02, m22, A02)));
+      b11 = fma(-m01, m01, fma(-m11, m11, fma(-m12, m12, A11)));
+      b12 = fma(-m01, m02, fma(-m11, m12, fma(-m12, m22, A12)));
+      b22 = fma(-m02, m02, fma(-m12, m12, fma(-m22, m22, A22)));
+      hx = fma(-2.0, g[3], g[0] + g[2]);
+      bb1 = fma(-hx, hx, fma(-2.0, g2[3], g2[0] + g2[2]));
+      hd = fma(-2.0, g[2], g[0] + g[5]);
+      bb2 = fma(-hd, hd, fma(-2.0, g2[2], g2[0] + g2[5]));
+      h00 = g[0] - g[2];
+      h01 = rt2 * (g[1] - g[4]);
+      h11 = g[0] - g[5];
+      e00 = fma(-h00, h00, fma(-h01, h01, g2[0] - g2[2]));
+      e01 = fma(-h00, h01, fma(-h01, h11, rt2 * (g2[1] - g2[4])));
+      e11 = fma(-h01, h01, fma(-h11, h11, g2[0] - g2[5]));
+    } else {
+      // fully symmetric block (3 x 3)
+      w_vec<0>(g, w0);
+      w_vec<1>(g, w1);
+      w_vec<2>(g, w2);
+      b00 = b_entry<0, 0>(g2, w0, w0);
+      b01 = b_entry<0, 1>(g2, w0, w1);
+      b02 = b_entry<0, 2>(g2, w0, w2);
+      b11 = b_entry<1, 1>(g2, w1, w1);
+      b12 = b_entry<1, 2>(g2, w1, w2);
+      b22 = b_entry<2, 2>(g2, w2, w2);
+      // the other blocks: two 1 x 1 and one 2 x 2 (two copies)
       GT u[9], v[9];
       w_vec<3>(g, u);
       bb1 = b_entry<3, 3>(g2, u, u);
@@ -1391,17 +1413,30 @@ __global__ void __launch_bounds__(128) k_eig2d(const double* __restrict__ gvals,
       e01 = b_entry<5, 6>(g2, u, v);
       e11 = b_entry<6, 6>(g2, v, v);
     }
-    // smallest eigenpair of the 3 x 3 block: scale to unit max entry, then repeated products
-    // with the adjugate (= det * inverse: inverse iteration without divisions), starting from
-    // the adjugate column with the largest diagonal entry.
-    const double sc = fmax(fmax(fmax(fabs(b00), fabs(b01)), fmax(fabs(b02), fabs(b11))),
-                           fmax(fabs(b12), fabs(b22)));
-    const double isc = sc > 0 ? 1.0 / sc : 0.0;
+    // smallest eigenpair of the 3 x 3 block: scale the largest entry into [1, 2) by a power of two
+    // (exact; found on the integer pipe), then repeated products with the adjugate (= det *
+    // inverse: inverse iteration without divisions), starting from the adjugate column with the
+    // largest diagonal entry.
+    auto mag = [](double x) { return __double2hiint(x) & 0x7fffffff; };
+    const int top = max(max(max(mag(b00), mag(b01)), max(mag(b02), mag(b11))),
+                        max(mag(b12), mag(b22)));
+    const int ef = top >> 20;
+    const bool normal = ef >= 1 && ef <= 2045;
+    const double isc = normal ? __longlong_as_double((long long)(2046 - ef) << 52) : 1.0;
+    const double sc = normal ? __longlong_as_double((long long)ef << 52) : 1.0;
+    const double unit = __hiloint2double((top & 0xfffff) | 0x3ff00000, 0);  // the largest, scaled
     const double s00 = b00 * isc, s01 = b01 * isc, s02 = b02 * isc, s11 = b11 * isc,
                  s12 = b12 * isc, s22 = b22 * isc;
-    const double a00 = s11 * s22 - s12 * s12, a01 = s02 * s12 - s01 * s22,
-                 a02 = s01 * s12 - s02 * s11, a11 = s00 * s22 - s02 * s02,
-                 a12 = s01 * s02 - s00 * s12, a22 = s00 * s11 - s01 * s01;
+    // a d - b c with the rounding error of b c put back (Kahan): the minors cancel to the size of
+    // the small eigenvalues, and without it one shift in twelve missed the residual test below
+    // and took Jacobi
+    auto det2 = [](double a, double d, double b, double c) {
+      const double w = b * c;
+      return fma(a, d, -w) + fma(-b, c, w);
+    };
+    const double a00 = det2(s11, s22, s12, s12), a01 = det2(s02, s12, s01, s22),
+                 a02 = det2(s01, s12, s02, s11), a11 = det2(s00, s22, s02, s02),
+                 a12 = det2(s01, s02, s00, s12), a22 = det2(s00, s11, s01, s01);
     double x0, x1, x2;
     if (a00 >= a11 && a00 >= a22) {
       x0 = a00; x1 = a01; x2 = a02;
@@ -1410,45 +1445,62 @@ __global__ void __launch_bounds__(128) k_eig2d(const double* __restrict__ gvals,
     } else {
       x0 = a02; x1 = a12; x2 = a22;
     }
-#pragma unroll
-    for (int it = 0; it < 5; ++it) {
+    auto times = [&](bool norm) {
       const double y0 = a00 * x0 + a01 * x1 + a02 * x2;
       const double y1 = a01 * x0 + a11 * x1 + a12 * x2;
       const double y2 = a02 * x0 + a12 * x1 + a22 * x2;
-      // renormalise by a power of two (exact) to stay clear of under/overflow
-      const double mx = fmax(fabs(y0), fmax(fabs(y1), fabs(y2)));
-      const double p2 = mx > 0 ? pow2_neg_ilogb(mx) : 1.0;
-      x0 = y0 * p2;
-      x1 = y1 * p2;
-      x2 = y2 * p2;
-    }
-    const double inrm = rsqrt(x0 * x0 + x1 * x1 + x2 * x2);
-    double y[3] = {x0 * inrm, x1 * inrm, x2 * inrm};
-    // one Newton correction of the normalisation (rsqrt is approximate)
-    {
+      // renormalise by a power of two (exact) every other time, to stay clear of under/overflow
+      const int ey = max(mag(y0), max(mag(y1), mag(y2))) >> 20;
+      const double p2 = norm && ey >= 1 && ey <= 2045
+                            ? __longlong_as_double((long long)(2046 - ey) << 52) : 1.0;
+      x0 = norm ? y0 * p2 : y0;
+      x1 = norm ? y1 * p2 : y1;
+      x2 = norm ? y2 * p2 : y2;
+    };
+    double y[3], ls, res, l1s, S, Pp, disc, l3s, l2s;
+    const double tr = s00 + s11 + s22, m2 = a00 + a11 + a22;
+    int flags = 0;
+    // The error of the vector falls by lambda_1 / lambda_2 a product: six (the starting column is
+    // one) suffice where that is below 2e-3; elsewhere five more a round until the power of the
+    // ratio is below the rounding level. The residual alone would accept a vector too early where
+    // lambda_2 is small as well.
+    float left = 1.0f;
+    for (int round = 0; round < 10; ++round) {
+      times(false);
+      times(true);
+      times(false);
+      times(true);
+      times(false);
+      const double inrm = rsqrt(x0 * x0 + x1 * x1 + x2 * x2);
+      y[0] = x0 * inrm;
+      y[1] = x1 * inrm;
+      y[2] = x2 * inrm;
+      // one Newton correction of the normalisation (rsqrt is approximate)
       const double n2 = y[0] * y[0] + y[1] * y[1] + y[2] * y[2];
       const double f = 1.5 - 0.5 * n2;
       y[0] *= f;
       y[1] *= f;
       y[2] *= f;
+      const double r0 = s00 * y[0] + s01 * y[1] + s02 * y[2];
+      const double r1 = s01 * y[0] + s11 * y[1] + s12 * y[2];
+      const double r2 = s02 * y[0] + s12 * y[1] + s22 * y[2];
+      ls = y[0] * r0 + y[1] * r1 + y[2] * r2;  // Rayleigh quotient (scaled)
+      res = fmax(fabs(r0 - ls * y[0]), fmax(fabs(r1 - ls * y[1]), fabs(r2 - ls * y[2])));
+      l1s = ls;
+      // remaining eigenvalues of the 3 x 3 block from its trace and principal minors
+      S = tr - l1s;
+      Pp = m2 - l1s * S;
+      disc = fmax(0.25 * S * S - Pp, 0.0);
+      l3s = 0.5 * S + sqrt(disc);
+      l2s = l3s > 0 ? Pp / l3s : 0.0;
+      const float ratio = fabsf((float)l1s / (float)l2s), r2f = ratio * ratio;
+      left *= r2f * r2f * (round == 0 ? r2f : ratio);
+      if (!(left > 1.1e-16f)) break;  // converged (or NaN: the residual test decides)
     }
-    const double r0 = s00 * y[0] + s01 * y[1] + s02 * y[2];
-    const double r1 = s01 * y[0] + s11 * y[1] + s12 * y[2];
-    const double r2 = s02 * y[0] + s12 * y[1] + s22 * y[2];
-    const double ls = y[0] * r0 + y[1] * r1 + y[2] * r2;  // Rayleigh quotient (scaled)
-    const double res = fmax(fabs(r0 - ls * y[0]), fmax(fabs(r1 - ls * y[1]), fabs(r2 - ls * y[2])));
-    int flags = 0;
-    double l1s = ls;
-    // remaining eigenvalues of the 3 x 3 block from its trace and principal minors
-    const double tr = s00 + s11 + s22, m2 = a00 + a11 + a22;
-    double S = tr - l1s, Pp = m2 - l1s * S;
-    double disc = fmax(0.25 * S * S - Pp, 0.0);
-    double l3s = 0.5 * S + sqrt(disc);
-    double l2s = l3s > 0 ? Pp / l3s : 0.0;
     // The adjugate iteration converges to the eigenvalue of smallest magnitude. Accept it when
     // the residual is at rounding level and it is also the algebraically smallest (it can be
     // slightly negative when the block was assembled in FP32); otherwise run cyclic Jacobi.
-    if (!(res <= 64 * 2.2e-16) || !(l1s <= l2s)) {
+    if (!(res <= 64 * 2.2e-16 * unit) || !(l1s <= l2s) || left > 1.1e-16f) {
       double a[4][4] = {{s00, s01, s02, 0}, {s01, s11, s12, 0}, {s02, s12, s22, 0}, {0, 0, 0, 0}};
       double vv[4][4];
       if (!jacobi_small(a, vv, 3)) flags |= LSP_FLAG_NOT_CONVERGED;
@@ -1486,19 +1538,37 @@ __global__ void __launch_bounds__(128) k_eig2d(const double* __restrict__ gvals,
     if (win != 0) flags |= LSP_FLAG_NONSYMMETRIC;
     double al[9], cv[9];
     if (win == 0) {
+      if constexpr (sizeof(GT) == 4) {
 #pragma unroll
-      for (int a = 0; a < 9; ++a) {
-        al[a] = y[0] * c_sym.u[0][a] + y[1] * c_sym.u[1][a] + y[2] * c_sym.u[2][a];
-        cv[a] = y[0] * w0[a] + y[1] * w1[a] + y[2] * w2[a];
+        for (int a = 0; a < 9; ++a) {
+          al[a] = y[0] * c_sym.u[0][a] + y[1] * c_sym.u[1][a] + y[2] * c_sym.u[2][a];
+          cv[a] = y[0] * w0[a] + y[1] * w1[a] + y[2] * w2[a];
+        }
+      } else {  // c = U_b (G_b y): one value per orbit
+        const double z0 = fma(m00, y[0], fma(m01, y[1], m02 * y[2]));
+        const double z1 = fma(m01, y[0], fma(m11, y[1], m12 * y[2]));
+        const double z2 = fma(m02, y[0], fma(m12, y[1], m22 * y[2]));
+        const double yo[3] = {y[0], 0.5 * y[1], 0.5 * y[2]}, zo[3] = {z0, 0.5 * z1, 0.5 * z2};
+#pragma unroll
+        for (int a = 0; a < 9; ++a) {
+          const int orb = (a / 3 != 1) + (a % 3 != 1);
+          al[a] = yo[orb];
+          cv[a] = zo[orb];
+        }
       }
     } else if (win == 1 || win == 2) {
       const int vi = win == 1 ? 3 : 4;
-      GT u[9];
-      if (win == 1) w_vec<3>(g, u); else w_vec<4>(g, u);
 #pragma unroll
-      for (int a = 0; a < 9; ++a) {
-        al[a] = c_sym.u[vi][a];
-        cv[a] = u[a];
+      for (int a = 0; a < 9; ++a) al[a] = c_sym.u[vi][a];
+      if constexpr (sizeof(GT) == 4) {
+        GT u[9];
+        if (win == 1) w_vec<3>(g, u); else w_vec<4>(g, u);
+#pragma unroll
+        for (int a = 0; a < 9; ++a) cv[a] = u[a];
+      } else {
+        const double hv = win == 1 ? hx : hd;
+#pragma unroll
+        for (int a = 0; a < 9; ++a) cv[a] = hv * al[a];
       }
     } else {
       // eigenvector of the 2 x 2 block for eLo
@@ -1511,13 +1581,18 @@ __global__ void __launch_bounds__(128) k_eig2d(const double* __restrict__ gvals,
       if (nr == 0) { p = 1; q = 0; nr = 1; }
       p /= nr;
       q /= nr;
-      GT u[9], v[9];
-      w_vec<5>(g, u);
-      w_vec<6>(g, v);
 #pragma unroll
-      for (int a = 0; a < 9; ++a) {
-        al[a] = p * c_sym.u[5][a] + q * c_sym.u[6][a];
-        cv[a] = p * u[a] + q * v[a];
+      for (int a = 0; a < 9; ++a) al[a] = p * c_sym.u[5][a] + q * c_sym.u[6][a];
+      if constexpr (sizeof(GT) == 4) {
+        GT u[9], v[9];
+        w_vec<5>(g, u);
+        w_vec<6>(g, v);
+#pragma unroll
+        for (int a = 0; a < 9; ++a) cv[a] = p * u[a] + q * v[a];
+      } else {
+        const double zp = fma(h00, p, h01 * q), zq = fma(h01, p, h11 * q);
+#pragma unroll
+        for (int a = 0; a < 9; ++a) cv[a] = zp * c_sym.u[5][a] + zq * c_sym.u[6][a];
       }
     }
     // sign: alpha[centre] > 0, else the first entry above 1e-12 in magnitude
@@ -1620,8 +1695,6 @@ cudaError_t upload_sym(lsp_ctx* c) {
   for (int i = 0; i < 7; ++i)
     for (int j = 0; j < 7; ++j)
       for (int q = 0; q < 6; ++q) B2f[i][j][q] = (float)B2[i][j][q];
-  e = cudaMemcpyToSymbol(c_W2, W2, sizeof W2);
-  if (e != cudaSuccess) return e;
   {
     // t = 2 (2D): block entries (b, i <= j) of mu_0^2 and their class coefficients
     const SymBasis& s2 = c->sym2;
@@ -1653,9 +1726,7 @@ cudaError_t upload_sym(lsp_ctx* c) {
   }
   e = cudaMemcpyToSymbol(c_W2f, W2f, sizeof W2f);
   if (e != cudaSuccess) return e;
-  e = cudaMemcpyToSymbol(c_B2f, B2f, sizeof B2f);
-  if (e != cudaSuccess) return e;
-  return cudaMemcpyToSymbol(c_B2, B2, sizeof B2);
+  return cudaMemcpyToSymbol(c_B2f, B2f, sizeof B2f);
 }
 
 cudaError_t launch_eig_t2(lsp_ctx* c, const int32_t* count, int64_t cap) {
