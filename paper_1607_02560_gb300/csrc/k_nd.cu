@@ -3,8 +3,8 @@
 //  - assembly: a front = its children's Schur complements (extend-add through the ring maps)
 //    plus P's entries listed for it;
 //  - partial inversion of each front on its eliminated set E with row pivoting inside E
-//    (Gauss-Jordan sweep): in shared memory for small fronts, else in blocked steps of
-//    kNdPanel pivots (panel choice, row block, rank-kNdPanel update of the whole front);
+//    (Gauss-Jordan sweep): in shared memory for small fronts, else in blocked steps (the panels
+//    here, the steps and their rank-kNdStep update on the tensor cores in k_nd_tc.cu);
 //  - the solve: one matrix-vector product per front going up the tree, one coming down.
 // Every reduction runs in a fixed order, so a factorisation and a solve are deterministic.
 #include <math.h>
@@ -148,10 +148,12 @@ __global__ void __launch_bounds__(256) k_nd_sweep_small(double* __restrict__ fro
   for (int e = tid; e < s; e += nt) perm[(int64_t)blockIdx.x * s + e] = sperm[e];
 }
 
-// ---- blocked partial inversion: one step eliminates the pivot columns K = [k, k + nb) ----
+// ---- blocked partial inversion (k_nd_tc.cu): panels of the sub-steps K = [k, k + nb) of a step
+// with the columns [k0, k0 + sb) ----
 // swaps layout per front: [0] = number of entries q, then dst[q] at 1 + q, src[q] at
-// 1 + 2 NP + q: after the step, position dst holds the row that was at position src.
-constexpr int kSwapInts = 1 + 4 * NP;
+// 1 + 2 NP + q: after the sub-step, position dst holds the row that was at position src; the
+// first nb entries are the pivot rows.
+constexpr int kSwapInts = kNdSwapInts, SB = kNdStep;
 
 // FP32 value of x for ranking pivot candidates, from the high word of the IEEE double: sign,
 // exponent rebased from 1023 to 127, the top 20 fraction bits (relative error < 2^-20);
@@ -165,20 +167,29 @@ __device__ __forceinline__ float rank_f32(double x) {
   return __uint_as_float(sign | ((unsigned)e << 23) | (((unsigned)hi & 0xfffffu) << 3));
 }
 
-// Part 1, one CTA per front: choose nb pivot rows among positions k..s-1 by partial pivoting
-// on the panel F[k.., K]; record the row exchanges, update perm, write the column block
-// cbuf[x][c] = F[src(x)][k + c] of the exchanged rows x, and the inverse of the pivot block.
-// The pivot rows come from a trial elimination of the panel in FP32: it only ranks candidate
-// rows by magnitude, while every value the factorisation keeps is FP64, computed from the
-// original entries (the pivot-block inverse here, the row block and the update in parts 2 and
-// 3). Each thread keeps its panel rows (row tid + t * 256, t < kPanelRows) in registers and
-// publishes its best candidate row to shared memory, so a pivot costs one block barrier.
-// Common end of part 1 (after the pivot rows sel[0..nb) are known, block-synchronised):
-// row exchanges, the column block of the exchanged rows, the FP64 pivot-block inverse.
+// 1 / x to within an ulp: the reciprocal of the mantissa in FP32, one third-order step
+// r (1 + e + e^2) with e = 1 - m r in FP64, the exponent by integers. Three FP64 operations where
+// the FP64 division takes several times that, on a pipe that is serial for one warp.
+__device__ __forceinline__ double recip_f64(double x) {
+  const int hi = __double2hiint(x), lo = __double2loint(x);
+  const int ef = (hi >> 20) & 0x7ff;
+  const double m = __hiloint2double((hi & 0xfffff) | 0x3ff00000, lo);  // in [1, 2)
+  const unsigned rb = __float_as_uint(
+      1.0f / __uint_as_float(0x3f800000u | ((unsigned)(hi & 0xfffff) << 3) | ((unsigned)lo >> 29)));
+  const double r0 = __hiloint2double((int)((rb >> 3) + (896u << 20)), (int)(rb << 29));
+  const double e = fma(-m, r0, 1.0);
+  const double r = fma(r0, fma(e, e, e), r0);  // in [1/2, 1]
+  const int rh = __double2hiint(r), fld = (rh >> 20) - (ef - 1023);
+  if (ef == 0 || ef == 0x7ff || fld < 1 || fld > 2046) return 1.0 / x;
+  return __hiloint2double((hi & 0x80000000) | (fld << 20) | (rh & 0xfffff), __double2loint(r));
+}
+
+// Common end (after the pivot rows sel[0..nb) are known, block-synchronised): row exchanges, the
+// exchanged rows' columns of the step, the FP64 pivot-block inverse.
 __device__ __forceinline__ void panel_tail(const double* __restrict__ F, int f, int s, int k,
-                                           int nb, int64_t fid, const int* sel,
-                                           int32_t* __restrict__ perm, double* __restrict__ cbuf,
-                                           double* __restrict__ pinv,
+                                           int nb, int k0, int sb, int64_t fid, const int* sel,
+                                           int32_t* __restrict__ perm, int32_t* __restrict__ cur,
+                                           double* __restrict__ xrow, double* __restrict__ pinv,
                                            int32_t* __restrict__ swaps, int32_t* __restrict__ err) {
   constexpr int NT = 256;
   __shared__ int nq;
@@ -204,19 +215,22 @@ __device__ __forceinline__ void panel_tail(const double* __restrict__ F, int f, 
     }
     const int nout = __popc(outb);
     int32_t* pf = perm + fid * s;
+    int32_t* cf = cur + fid * s;
     int32_t* sw = swaps + fid * kSwapInts;
-    const int old_sel = act ? pf[ps] : 0;
-    const int old_dis = dpos >= 0 ? pf[dpos] : 0;
+    const int old_sel = act ? pf[ps] : 0, cur_sel = act ? cf[ps] : 0;
+    const int old_dis = dpos >= 0 ? pf[dpos] : 0, cur_dis = dpos >= 0 ? cf[dpos] : 0;
     __syncwarp();
     if (act) {
       dstp[lane] = k + lane;
       srcp[lane] = ps;
       pf[k + lane] = old_sel;
+      cf[k + lane] = cur_sel;
     }
     if (dpos >= 0) {
       dstp[nb + rank] = ps;
       srcp[nb + rank] = dpos;
       pf[ps] = old_dis;
+      cf[ps] = cur_dis;
     }
     __syncwarp();
     const int qq = nb + nout;
@@ -231,104 +245,128 @@ __device__ __forceinline__ void panel_tail(const double* __restrict__ F, int f, 
   }
   __syncthreads();
   const int q = nq;
-  // the column block of the exchanged rows (the other rows are read in place by part 2)
-  double* cb = cbuf + fid * (int64_t)f * NP;
-  for (int e = tid; e < q * NP; e += NT) {
-    const int a = e / NP, c = e % NP;
-    cb[(int64_t)dstp[a] * NP + c] = c < nb ? F[(int64_t)srcp[a] * f + k + c] : 0.0;
+  // the step's columns of the exchanged rows (the other rows are read in place by k_nd_sub): loaded
+  // here, stored after the inversion, which covers the latency
+  double* xr = xrow + fid * (2 * NP * SB);
+  double keep[2 * NP * SB / NT];
+#pragma unroll
+  for (int u = 0; u < 2 * NP * SB / NT; ++u) {
+    const int e = tid + u * NT, a = e / SB, c = e % SB;
+    keep[u] = a < q && c < sb ? F[(int64_t)srcp[a] * f + k0 + c] : 0.0;
   }
-  // inverse of the pivot block A (FP64): Gauss-Jordan on [A | I], one element per thread in
-  // each half (rows r = tid / 16, columns c and c + 16), no row exchanges: pivot j is taken in
-  // the unpivoted row p_j of largest |a_pj,j| (integer comparison of magnitude bits), row p_j
-  // is scaled by one reciprocal, column j is eliminated from the other rows. The left block
-  // ends as a permutation with a 1 at (p_j, j), so row j of A^-1 is the right block's row p_j.
-  __shared__ double aug[NP][2 * NP + 1];
-  __shared__ double gd;
-  __shared__ int gp, rowpiv[NP];
-  const int gr = tid / NP, gc = tid % NP;  // 256 threads = 16 rows x 16 column pairs
+  // Inverse of the pivot block A (FP64): Gauss-Jordan in place, one element per thread, no row
+  // exchanges: pivot j is taken in the unpivoted row p_j of largest |a_pj,j| (by the upper 32 bits),
+  // row p_j is scaled by one reciprocal, column j is eliminated from the other rows. Row p_j,
+  // column c of the result is element (j, p_c) of A^-1.
+  __shared__ double A[2][NP][NP + 1];
+  __shared__ double trow[NP];
+  __shared__ int piv_row[NP], row_piv[NP];  // p_j, and the j of a row
+  const int gr = tid / NP, gc = tid % NP;  // 256 threads = 16 x 16
   {
     int src = k + gr;
     for (int e = 0; e < q; ++e)
       if (dstp[e] == k + gr) src = srcp[e];
-    aug[gr][gc] = (gr < nb && gc < nb) ? F[(int64_t)src * f + k + gc] : 0.0;
-    aug[gr][NP + gc] = (gr < nb && gc == gr) ? 1.0 : 0.0;
-    if (gc == 0) rowpiv[gr] = gr < nb ? -1 : NP;  // pivot index of the row, -1 while unpivoted
+    A[0][gr][gc] = (gr < nb && gc < nb) ? F[(int64_t)src * f + k + gc] : 0.0;
   }
   __syncthreads();
+  bool open = lane < nb;  // warp 0: the lane's row has not been a pivot row
   for (int j = 0; j < nb; ++j) {
+    const double(*Aj)[NP + 1] = A[j & 1];
+    double(*An)[NP + 1] = A[~j & 1];
     if (warp == 0) {
-      const bool cand_ok = lane < nb && rowpiv[lane] < 0;
-      unsigned long long key =
-          cand_ok ? ((unsigned long long)__double_as_longlong(aug[lane][j]) & 0x7fffffffffffffffull)
-                  : 0ull;
-      int p = lane;
-      for (int off = 16; off > 0; off >>= 1) {
-        const unsigned long long ok = __shfl_xor_sync(0xffffffffu, key, off);
-        const int op = __shfl_xor_sync(0xffffffffu, p, off);
-        if (ok > key || (ok == key && op < p)) {
-          key = ok;
-          p = op;
-        }
+      const unsigned key =
+          open ? ((unsigned)__double2hiint(Aj[lane & (NP - 1)][j]) & 0x7fffffffu) + 1u : 0u;
+      const unsigned top = __reduce_max_sync(0xffffffffu, key);
+      const int p = __ffs(__ballot_sync(0xffffffffu, key == top)) - 1;
+      const double x = Aj[p][j];
+      if (lane == p) {
+        open = false;
+        if (x == 0.0 || top - 1u >= 0x7ff00000u) atomicOr(err, 4);  // zero, Inf or NaN
+        piv_row[j] = p;
+        row_piv[p] = j;
       }
-      if (lane == 0) {
-        if (key == 0ull || key >= 0x7ff0000000000000ull) atomicOr(err, 4);  // zero, Inf or NaN
-        gp = p;
-        rowpiv[p] = j;
-        gd = 1.0 / aug[p][j];  // the one FP64 division of this pivot
-      }
+      const double d = recip_f64(x);
+      if (lane < NP) trow[lane] = lane == j ? d : Aj[p][lane] * d;
     }
     __syncthreads();
-    const int p = gp;
-    const double d = gd;
-    const double lr = gr == p ? 0.0 : aug[gr][j];  // multipliers, read before any update
-    const double p0 = aug[p][gc] * d, p1 = aug[p][NP + gc] * d;
-    __syncthreads();
-    if (gr == p) {
-      aug[gr][gc] = p0;
-      aug[gr][NP + gc] = p1;
-    } else {
-      aug[gr][gc] = fma(-lr, p0, aug[gr][gc]);
-      aug[gr][NP + gc] = fma(-lr, p1, aug[gr][NP + gc]);
-    }
+    const double t = trow[gc];
+    An[gr][gc] = gr == piv_row[j] ? t : fma(-Aj[gr][j], t, gc == j ? 0.0 : Aj[gr][gc]);
     __syncthreads();
   }
-  {
-    const int jr = rowpiv[gr];
-    if (jr >= 0 && jr < NP) pinv[fid * NP * NP + jr * NP + gc] = gc < nb ? aug[gr][NP + gc] : 0.0;
-    else if (gr >= nb) pinv[fid * NP * NP + gr * NP + gc] = 0.0;
-  }
+  const bool in = gr < nb && gc < nb;
+  pinv[fid * NP * NP + (in ? row_piv[gr] * NP + piv_row[gc] : tid)] = in ? A[nb & 1][gr][gc] : 0.0;
+#pragma unroll
+  for (int u = 0; u < 2 * NP * SB / NT; ++u)
+    if (tid + u * NT < q * SB) xr[tid + u * NT] = keep[u];
 }
 
 constexpr int kPanelRows = 8;  // rows per thread: panels of up to 2048 rows (the cross, n = 1024)
+// A step's first panel: no row has moved yet.
+__device__ __forceinline__ void start_cur(int32_t* __restrict__ cur, int64_t fid, int s, int k,
+                                          int k0) {
+  if (k == k0)
+    for (int p = k0 + threadIdx.x; p < s; p += blockDim.x) cur[fid * s + p] = p;
+}
+// A kernel of a chain launched to overlap the one before: its blocks wait here.
+__device__ __forceinline__ void chain_start() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+// One CTA per front: choose nb pivot rows among positions k..s-1 by partial pivoting on the panel
+// F[k.., K16]; record the row exchanges, update perm and cur (the position before the step of the
+// row now at a position), copy the step's columns of the exchanged rows into xrow, and write the
+// inverse of the pivot block. The pivot rows come from a trial elimination of the panel in FP32:
+// it only ranks candidate rows by magnitude, while every value the factorisation keeps is computed
+// from the FP64 entries. Each thread keeps its panel rows (row tid + t * 256, t < ROWS) in
+// registers and each warp publishes its best candidate row to shared memory, so a pivot costs one
+// block barrier. Bound by the latency of the 16 pivots, once here and once in the inversion.
+// Measured at the root of 2D n = 512 (1023 rows): 40 -> 24 us a panel (before: rows read 128 bytes
+// apart by neighbouring lanes, every thread publishing its row, shuffles for the maxima, an FP64
+// division and both halves of [A | I] per pivot of the inversion).
+template <int ROWS>
 __global__ void __launch_bounds__(256) k_nd_panel(const double* __restrict__ fronts, int f, int s,
-                                                  int k, int nb, int32_t* __restrict__ perm,
-                                                  double* __restrict__ cbuf,
+                                                  int k, int nb, int k0, int sb,
+                                                  int32_t* __restrict__ perm,
+                                                  int32_t* __restrict__ cur,
+                                                  double* __restrict__ xrow,
                                                   double* __restrict__ pinv,
                                                   int32_t* __restrict__ swaps,
                                                   int32_t* __restrict__ err) {
-  constexpr int NT = 256;
-  __shared__ float cand[2][NT][NP + 1];  // each thread's best remaining row, double-buffered
-  __shared__ float wbest[2][8];
-  __shared__ int wbi[2][8];
+  constexpr int NT = 256, NW = NT / 32;
+  __shared__ float st[NT][NP + 1];                     // 256 panel rows on their way to registers
+  __shared__ __align__(16) float cand[2][NW][NP + 4];  // each warp's best row, double-buffered
+  __shared__ __align__(16) uint2 wb[2][NW];            // its magnitude (bits + 1) and index
   __shared__ int sel[NP];
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int tid = threadIdx.x, warp = tid >> 5;
   const int m = s - k;
   const int64_t fid = blockIdx.x;
   const double* F = fronts + fid * f * f;
-  float rv[kPanelRows][NP];
+  chain_start();
+  start_cur(cur, fid, s, k, k0);
+  float rv[ROWS][NP];
+  double v[NP];
+  const int hr = tid / NP, hc = tid % NP;  // half a warp reads one row of the panel
+  auto fetch = [&](int t) {
 #pragma unroll
-  for (int t = 0; t < kPanelRows; ++t) {
-    const int i = tid + t * NT;
-    const double* Fi = F + (int64_t)(k + (i < m ? i : 0)) * f + k;
-    double v[NP];
+    for (int u = 0; u < NP; ++u) {
+      const int row = t * NT + hr + u * (NT / NP);
+      v[u] = row < m && hc < nb ? F[(int64_t)(k + row) * f + k + hc] : 0.0;
+    }
+  };
+  fetch(0);
 #pragma unroll
-    for (int c = 0; c < NP; ++c) v[c] = (i < m && c < nb) ? Fi[c] : 0.0;
+  for (int t = 0; t < ROWS; ++t) {
+    if (t) __syncthreads();
 #pragma unroll
-    for (int c = 0; c < NP; ++c) rv[t][c] = rank_f32(v[c]);
+    for (int u = 0; u < NP; ++u) st[hr + u * (NT / NP)][hc] = rank_f32(v[u]);
+    __syncthreads();
+    if (t + 1 < ROWS) fetch(t + 1);
+#pragma unroll
+    for (int c = 0; c < NP; ++c) rv[t][c] = st[tid][c];
   }
   unsigned used = 0;  // bit t: row tid + t NT is a pivot row (or does not exist)
 #pragma unroll
-  for (int t = 0; t < kPanelRows; ++t)
+  for (int t = 0; t < ROWS; ++t)
     if (tid + t * NT >= m) used |= 1u << t;
 #pragma unroll
   for (int j = 0; j < NP; ++j) {
@@ -337,56 +375,57 @@ __global__ void __launch_bounds__(256) k_nd_panel(const double* __restrict__ fro
     float best = -1.0f;
     int bt = 0;
 #pragma unroll
-    for (int t = 0; t < kPanelRows; ++t) {
+    for (int t = 0; t < ROWS; ++t) {
       const float a = fabsf(rv[t][j]);
       if (!(used >> t & 1u) && a > best) {
         best = a;
         bt = t;
       }
     }
-    int bi = best >= 0.0f ? tid + bt * NT : m;
+    // the warp's: the largest magnitude, ties to the smaller index
+    const unsigned key = best >= 0.0f ? __float_as_uint(best) + 1u : 0u;
+    const unsigned top = __reduce_max_sync(0xffffffffu, key);
+    const unsigned bi = (unsigned)(tid + bt * NT);
+    const unsigned wi = __reduce_min_sync(0xffffffffu, key == top ? bi : 0xffffffffu);
+    if (bi == wi) {
 #pragma unroll
-    for (int c = 0; c < NP; ++c) {
-      if (c < j) continue;
-      float val = rv[0][c];
+      for (int c = 0; c < NP; ++c) {
+        if (c < j) continue;
+        float val = rv[0][c];
 #pragma unroll
-      for (int t = 1; t < kPanelRows; ++t)
-        if (t == bt) val = rv[t][c];
-      cand[j & 1][tid][c] = val;
-    }
-    warp_argmax_f(best, bi);
-    if (lane == 0) {
-      wbest[j & 1][warp] = best;
-      wbi[j & 1][warp] = bi;
+        for (int t = 1; t < ROWS; ++t)
+          if (t == bt) val = rv[t][c];
+        cand[j & 1][warp][c] = val;
+      }
+      wb[j & 1][warp] = make_uint2(top, wi);
     }
     __syncthreads();
-    float b = wbest[j & 1][0];
-    int pr = wbi[j & 1][0];
+    unsigned bk = 0, pr = 0xffffffffu;
+    int bw = 0;
 #pragma unroll
-    for (int w = 1; w < NT / 32; ++w) {
-      const float bw = wbest[j & 1][w];
-      const int iw = wbi[j & 1][w];
-      if (bw > b || (bw == b && iw < pr)) {
-        b = bw;
-        pr = iw;
+    for (int w = 0; w < NW; ++w) {
+      const uint2 x = wb[j & 1][w];
+      if (x.x > bk || (x.x == bk && x.y < pr)) {
+        bk = x.x;
+        pr = x.y;
+        bw = w;
       }
     }
-    if (!(b > 0.0f) || !isfinite(b) || pr >= m) {  // uniform: every thread read the same values
+    if (bk < 2u || bk > 0x7f800000u || pr >= (unsigned)m) {  // zero, Inf: uniform over the block
       if (tid == 0) {
         atomicOr(err, 2);
         swaps[fid * kSwapInts] = 0;  // the next kernels of the step then exchange nothing
       }
       return;
     }
-    if (tid == 0) sel[j] = pr;
-    const int owner = pr % NT, ot = pr / NT;
+    if (tid == 0) sel[j] = (int)pr;
+    if ((int)(pr % NT) == tid) used |= 1u << (pr / NT);
     float pv[NP];  // the pivot row from column j on
 #pragma unroll
-    for (int c = 0; c < NP; ++c) pv[c] = c >= j ? cand[j & 1][owner][c] : 0.0f;
-    if (owner == tid) used |= 1u << ot;
+    for (int c = 0; c < NP; ++c) pv[c] = c >= j ? cand[j & 1][bw][c] : 0.0f;
     const float ipv = 1.0f / pv[j];
 #pragma unroll
-    for (int t = 0; t < kPanelRows; ++t) {
+    for (int t = 0; t < ROWS; ++t) {
       if (used >> t & 1u) continue;
       const float l = rv[t][j] * ipv;
 #pragma unroll
@@ -395,16 +434,17 @@ __global__ void __launch_bounds__(256) k_nd_panel(const double* __restrict__ fro
     }
   }
   __syncthreads();  // sel complete
-  panel_tail(F, f, s, k, nb, fid, sel, perm, cbuf, pinv, swaps, err);
+  panel_tail(F, f, s, k, nb, k0, sb, fid, sel, perm, cur, xrow, pinv, swaps, err);
 }
 
-// Part 1 for panels of more than kPanelRows * 256 rows (the root planes of 3D grids): the same
+// The same for panels of more than kPanelRows * 256 rows (the root planes of 3D grids): the same
 // FP32 trial elimination with the ranking rows in a global scratch (L2-resident) instead of
 // registers; each thread handles rows tid + t * 256, t < 64 (up to 16 384 rows).
 __global__ void __launch_bounds__(256) k_nd_panel_big(const double* __restrict__ fronts, int f,
-                                                      int s, int k, int nb,
+                                                      int s, int k, int nb, int k0, int sb,
                                                       int32_t* __restrict__ perm,
-                                                      double* __restrict__ cbuf,
+                                                      int32_t* __restrict__ cur,
+                                                      double* __restrict__ xrow,
                                                       double* __restrict__ pinv,
                                                       int32_t* __restrict__ swaps,
                                                       int32_t* __restrict__ err,
@@ -418,6 +458,8 @@ __global__ void __launch_bounds__(256) k_nd_panel_big(const double* __restrict__
   const int m = s - k;
   const int64_t fid = blockIdx.x;
   const double* F = fronts + fid * f * f;
+  chain_start();
+  start_cur(cur, fid, s, k, k0);
   float* pan = scratch + fid * (int64_t)s * PS;
   const int nrows = (m - tid + NT - 1) / NT;  // rows of this thread (<= 64)
   float best = -1.0f;
@@ -504,148 +546,7 @@ __global__ void __launch_bounds__(256) k_nd_panel_big(const double* __restrict__
     }
   }
   __syncthreads();  // sel complete
-  panel_tail(F, f, s, k, nb, fid, sel, perm, cbuf, pinv, swaps, err);
-}
-
-// Part 2: rows K become A_KK^-1 F[K, j] for the columns j outside K (after applying the row
-// exchanges to those columns), and the column block becomes [A_KK^-1 on K; -cbuf A_KK^-1 off K];
-// the column tiles also complete cbuf with the rows that the exchanges did not move.
-constexpr int kRowThreads = 64;  // one column (or row) per thread; small CTAs spread the step
-__global__ void __launch_bounds__(kRowThreads) k_nd_rowblock(double* __restrict__ fronts, int f, int k,
-                                                     int nb, int tiles_w,
-                                                     double* __restrict__ cbuf,
-                                                     const double* __restrict__ pinv,
-                                                     const int32_t* __restrict__ swaps) {
-  __shared__ double pi[NP][NP];
-  __shared__ int dstp[2 * NP], srcp[2 * NP], kq[NP];
-  __shared__ int nq;
-  const int tid = threadIdx.x;
-  const int64_t fid = blockIdx.y;
-  double* F = fronts + fid * f * f;
-  const int32_t* sw = swaps + fid * kSwapInts;
-  for (int e = tid; e < NP * NP; e += blockDim.x) pi[e / NP][e % NP] = pinv[fid * NP * NP + e];
-  if (tid == 0) {
-    int q0 = sw[0];
-    q0 = q0 < 0 || q0 > 2 * NP ? 0 : q0;
-    for (int a = 0; a < q0; ++a) {
-      const int dp = sw[1 + a], sp = sw[1 + 2 * NP + a];
-      if (dp < 0 || dp >= f || sp < 0 || sp >= f) q0 = 0;
-    }
-    nq = q0;
-  }
-  __syncthreads();
-  const int q = nq;
-  if (tid < q) {
-    dstp[tid] = sw[1 + tid];
-    srcp[tid] = sw[1 + 2 * NP + tid];
-  }
-  __syncthreads();
-  if (tid < nb) {
-    int a0 = -1;
-    for (int a = 0; a < q; ++a)
-      if (dstp[a] == k + tid) a0 = a;
-    kq[tid] = a0;
-  }
-  __syncthreads();
-  if ((int)blockIdx.x < tiles_w) {
-    const int j = blockIdx.x * blockDim.x + tid;
-    if (j >= f || (j >= k && j < k + nb)) return;
-    double val[2 * NP];
-    for (int a = 0; a < 2 * NP; ++a)
-      if (a < q) val[a] = F[(int64_t)srcp[a] * f + j];
-    double rv[NP];
-    for (int c = 0; c < NP; ++c) {
-      double v = 0.0;
-      if (c < nb) {
-        v = F[(int64_t)(k + c) * f + j];
-        for (int a = 0; a < 2 * NP; ++a)
-          if (a == kq[c]) v = val[a];
-      }
-      rv[c] = v;
-    }
-    for (int c = 0; c < nb; ++c) {
-      double w = 0.0;
-      for (int mm = 0; mm < NP; ++mm) w = fma(pi[c][mm], rv[mm], w);
-      F[(int64_t)(k + c) * f + j] = w;
-    }
-    for (int a = 0; a < 2 * NP; ++a)
-      if (a < q && (dstp[a] < k || dstp[a] >= k + nb)) F[(int64_t)dstp[a] * f + j] = val[a];
-  } else {
-    const int x = (blockIdx.x - tiles_w) * blockDim.x + tid;
-    if (x >= f) return;
-    bool moved = false;
-    for (int a = 0; a < q; ++a)
-      if (dstp[a] == x) moved = true;
-    double* cx = cbuf + fid * (int64_t)f * NP + (int64_t)x * NP;
-    double* Fx = F + (int64_t)x * f + k;
-    double cr[NP];
-    if (moved) {  // written by part 1 from the row's source position
-#pragma unroll
-      for (int mm = 0; mm < NP; ++mm) cr[mm] = cx[mm];
-    } else {      // still in place: this thread is the only reader and writer of F[x][K]
-#pragma unroll
-      for (int mm = 0; mm < NP; ++mm) cr[mm] = mm < nb ? Fx[mm] : 0.0;
-#pragma unroll
-      for (int mm = 0; mm < NP; ++mm) cx[mm] = cr[mm];
-    }
-    if (x >= k && x < k + nb) {
-      for (int c = 0; c < nb; ++c) Fx[c] = pi[x - k][c];
-    } else {
-      for (int c = 0; c < nb; ++c) {
-        double acc = 0.0;
-#pragma unroll
-        for (int mm = 0; mm < NP; ++mm) acc = fma(cr[mm], pi[mm][c], acc);
-        Fx[c] = -acc;
-      }
-    }
-  }
-}
-
-// Part 3: F[i][j] -= cbuf[i][:] . F[K][j] for every i, j outside K (64 x 64 tiles).
-constexpr int kUT = 64;
-// Columns updated: [col_lo, col_hi) without [skip_lo, skip_hi) (which holds K); the tiles
-// start at col_lo. With look-ahead a step is split into the next panel's columns and the rest.
-__global__ void __launch_bounds__(256) k_nd_update(double* __restrict__ fronts, int f, int k,
-                                                   int nb, int tiles_j, int col_lo, int col_hi,
-                                                   int skip_lo, int skip_hi,
-                                                   const double* __restrict__ cbuf) {
-  __shared__ double cs[kUT][NP + 1];
-  __shared__ double ws[NP][kUT];
-  const int tid = threadIdx.x;
-  const int64_t fid = blockIdx.y;
-  double* F = fronts + fid * f * f;
-  const int ti = blockIdx.x / tiles_j, tj = blockIdx.x % tiles_j;
-  const int i0 = ti * kUT, j0 = col_lo + tj * kUT;
-  const double* cb = cbuf + fid * (int64_t)f * NP;
-  for (int e = tid; e < kUT * NP; e += blockDim.x) {
-    const int r = e / NP, c = e % NP;
-    cs[r][c] = (i0 + r < f) ? cb[(int64_t)(i0 + r) * NP + c] : 0.0;
-    const int c2 = e / kUT, col = e % kUT;
-    ws[c2][col] = (c2 < nb && j0 + col < col_hi) ? F[(int64_t)(k + c2) * f + j0 + col] : 0.0;
-  }
-  __syncthreads();
-  const int ty = tid / 16, tx = tid % 16;
-  double acc[4][4];
-  bool rok[4], cok[4];
-  for (int a = 0; a < 4; ++a) {
-    const int i = i0 + ty + 16 * a, j = j0 + tx + 16 * a;
-    rok[a] = i < f && (i < k || i >= k + nb);
-    cok[a] = j < col_hi && (j < skip_lo || j >= skip_hi);
-  }
-  for (int a = 0; a < 4; ++a)
-    for (int b = 0; b < 4; ++b)
-      acc[a][b] = (rok[a] && cok[b]) ? F[(int64_t)(i0 + ty + 16 * a) * f + j0 + tx + 16 * b] : 0.0;
-#pragma unroll
-  for (int c = 0; c < NP; ++c) {
-    double cr[4], wr[4];
-    for (int a = 0; a < 4; ++a) cr[a] = cs[ty + 16 * a][c];
-    for (int b = 0; b < 4; ++b) wr[b] = ws[c][tx + 16 * b];
-    for (int a = 0; a < 4; ++a)
-      for (int b = 0; b < 4; ++b) acc[a][b] = fma(-cr[a], wr[b], acc[a][b]);
-  }
-  for (int a = 0; a < 4; ++a)
-    for (int b = 0; b < 4; ++b)
-      if (rok[a] && cok[b]) F[(int64_t)(i0 + ty + 16 * a) * f + j0 + tx + 16 * b] = acc[a][b];
+  panel_tail(F, f, s, k, nb, k0, sb, fid, sel, perm, cur, xrow, pinv, swaps, err);
 }
 
 // ---- solve ----
@@ -928,78 +829,48 @@ cudaError_t launch_nd_sweep(lsp_ctx* c, int depth) {
   }
   // blocked steps; perm starts as the identity
   k_nd_iota<<<grid_for((int64_t)lv.count * lv.s, 256), 256, 0, c->stream>>>(perm, lv.count, lv.s);
+  cudaError_t e = cudaGetLastError();
+  if (e == cudaSuccess) e = launch_nd_blocked(c, depth);
+  timer_end(c, t);
+  return e;
+}
+
+const char* nd_timer_name(int kind, int depth) {
+  return level_name(kind == 4 ? "nd_row" : "nd_upd", depth);
+}
+
+cudaError_t launch_nd_panel(lsp_ctx* c, int depth, int k, int nb, int k0, int sb) {
+  NdState& S = *c->nd;
+  const NdLevel& lv = S.plan.lv[depth];
+  const double* F = (const double*)S.fronts.p + lv.front_off;
+  int32_t* perm = (int32_t*)S.perm.p + lv.perm_off;
   const bool big = lv.s > kPanelRows * 256;
   if (big && !S.pscratch.p) return cudaErrorInvalidValue;
-  const int tiles_w = (lv.f + kRowThreads - 1) / kRowThreads;
-  const int tiles_c = (lv.f + kRowThreads - 1) / kRowThreads;
-  const int tiles_u = (lv.f + kUT - 1) / kUT;
-  // Look-ahead: once a step's update has reached the next panel's columns, that panel runs on
-  // the side stream while the rest of the update runs here (disjoint columns). The step
-  // buffers (cbuf, pinv, swaps) alternate between two copies. Per-kernel timing keeps one
-  // stream so that every launch is bracketed by its own events.
-  const bool ahead = S.side != nullptr && !c->timing;
-  auto buf = [&](int par, double** cb, double** pv, int32_t** sw) {
-    *cb = (double*)S.cbuf.p + (int64_t)par * S.cbuf_half;
-    *pv = (double*)S.pinv.p + (int64_t)par * S.pinv_half;
-    *sw = (int32_t*)S.swaps.p + (int64_t)par * S.swaps_half;
-  };
-  auto panel = [&](int k, int par, cudaStream_t st) {
-    double *cb, *pv;
-    int32_t* sw;
-    buf(par, &cb, &pv, &sw);
-    const int nb = lv.s - k < NP ? lv.s - k : NP;
-    const int t1 = c->timing ? timer_begin(c, level_name("nd_pnl", depth)) : -1;
-    if (big)
-      k_nd_panel_big<<<lv.count, 256, 0, st>>>(F, lv.f, lv.s, k, nb, perm, cb, pv, sw, err,
-                                               (float*)S.pscratch.p);
-    else
-      k_nd_panel<<<lv.count, 256, 0, st>>>(F, lv.f, lv.s, k, nb, perm, cb, pv, sw, err);
-    timer_end(c, t1);
-  };
-  auto update = [&](int k, int nb, const double* cb, int col_lo, int col_hi, int skip_lo,
-                    int skip_hi) {
-    const int tj = (col_hi - col_lo + kUT - 1) / kUT;
-    const int t3 = c->timing ? timer_begin(c, level_name("nd_upd", depth)) : -1;
-    k_nd_update<<<dim3(tiles_u * tj, lv.count), 256, 0, c->stream>>>(
-        F, lv.f, k, nb, tj, col_lo, col_hi, skip_lo, skip_hi, cb);
-    timer_end(c, t3);
-  };
-  panel(0, 0, c->stream);
-  for (int k = 0, step = 0; k < lv.s; k += NP, ++step) {
-    const int nb = lv.s - k < NP ? lv.s - k : NP;
-    const int par = step & 1;
-    double *cb, *pv;
-    int32_t* sw;
-    buf(par, &cb, &pv, &sw);
-    if (ahead && step > 0) {
-      cudaError_t e = cudaStreamWaitEvent(c->stream, S.ev_panel, 0);
-      if (e != cudaSuccess) return e;
-    }
-    const int t2 = c->timing ? timer_begin(c, level_name("nd_row", depth)) : -1;
-    k_nd_rowblock<<<dim3(tiles_w + tiles_c, lv.count), kRowThreads, 0, c->stream>>>(
-        F, lv.f, k, nb, tiles_w, cb, pv, sw);
-    timer_end(c, t2);
-    const int kn = k + nb;
-    if (kn >= lv.s) {  // last step: the whole update
-      update(k, nb, cb, 0, lv.f, k, kn);
-    } else if (ahead) {
-      const int nbn = lv.s - kn < NP ? lv.s - kn : NP;
-      update(k, nb, cb, kn, kn + nbn, k, kn);  // the next panel's columns first
-      cudaError_t e = cudaEventRecord(S.ev_cols, c->stream);
-      if (e != cudaSuccess) return e;
-      e = cudaStreamWaitEvent(S.side, S.ev_cols, 0);
-      if (e != cudaSuccess) return e;
-      panel(kn, par ^ 1, S.side);
-      e = cudaEventRecord(S.ev_panel, S.side);
-      if (e != cudaSuccess) return e;
-      update(k, nb, cb, 0, lv.f, k, kn + nbn);  // the rest, beside the panel
-    } else {
-      update(k, nb, cb, 0, lv.f, k, kn);
-      panel(kn, par ^ 1, c->stream);
-    }
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(lv.count);
+  cfg.blockDim = dim3(256);
+  cfg.stream = c->stream;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = c->timing ? 0 : 1;
+  const int t = timer_begin(c, level_name("nd_pnl", depth));
+  cudaError_t e;
+  if (big)
+    e = cudaLaunchKernelEx(&cfg, k_nd_panel_big, F, lv.f, lv.s, k, nb, k0, sb, perm,
+                           (int32_t*)S.cur.p, (double*)S.xrow.p, (double*)S.pinv.p,
+                           (int32_t*)S.swaps.p, (int32_t*)S.err.p, (float*)S.pscratch.p);
+  else {  // rows per thread: as few as cover the rows that are left
+    const int per = (lv.s - k + 255) / 256;
+    auto kern = per <= 1 ? k_nd_panel<1> : per <= 2 ? k_nd_panel<2>
+                : per <= 4 ? k_nd_panel<4> : k_nd_panel<kPanelRows>;
+    e = cudaLaunchKernelEx(&cfg, kern, F, lv.f, lv.s, k, nb, k0, sb, perm, (int32_t*)S.cur.p,
+                           (double*)S.xrow.p, (double*)S.pinv.p, (int32_t*)S.swaps.p,
+                           (int32_t*)S.err.p);
   }
   timer_end(c, t);
-  return cudaGetLastError();
+  return e;
 }
 
 // The solve's copies of one depth's blocks, after its sweep.

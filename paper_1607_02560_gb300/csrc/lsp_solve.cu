@@ -94,15 +94,13 @@ namespace lsp {
 void nd_free(NdState* s) {
   if (!s) return;
   DevBuf* bufs[] = {&s->fronts, &s->E, &s->R, &s->inv, &s->asm_dst, &s->asm_src, &s->perm,
-                    &s->z, &s->u, &s->cbuf, &s->pinv, &s->swaps, &s->err, &s->V, &s->w,
+                    &s->z, &s->u, &s->cur, &s->xrow, &s->pinv, &s->swaps, &s->err, &s->vst, &s->digits,
+                    &s->expo, &s->V, &s->w,
                     &s->b, &s->x, &s->tmp, &s->gs, &s->fvec, &s->ry, &s->rd, &s->pscratch, &s->solve,
                     &s->gsrc, &s->bar};
   for (DevBuf* b : bufs)
     if (b->p) cudaFree(b->p);
   if (s->h_gs) cudaFreeHost(s->h_gs);
-  if (s->ev_cols) cudaEventDestroy(s->ev_cols);
-  if (s->ev_panel) cudaEventDestroy(s->ev_panel);
-  if (s->side) cudaStreamDestroy(s->side);
   delete s;
 }
 
@@ -161,13 +159,15 @@ lsp_status lsp_nd_factor(lsp_ctx* c, const lsp_nd_opts* opts) {
     if ((st = upload(c, S.asm_dst, S.plan.asm_dst)) != LSP_OK) return st;
     if ((st = upload(c, S.asm_src, S.plan.asm_src)) != LSP_OK) return st;
     const NdPlan& P = S.plan;
-    int64_t cb = 1, pv = 1, sw = 1, ps = 0;
+    int64_t nf = 1, cu = 1, dg = 16, ex = 1, vs = 1, ps = 0;
     int max_sr = 1;
     for (const NdLevel& lv : P.lv) {
       if (lv.f > kNdSmallFront) {
-        cb = std::max(cb, (int64_t)lv.count * lv.f * kNdPanel);
-        pv = std::max(pv, (int64_t)lv.count * kNdPanel * kNdPanel);
-        sw = std::max(sw, (int64_t)lv.count * (1 + 4 * kNdPanel));
+        nf = std::max(nf, (int64_t)lv.count);
+        cu = std::max(cu, (int64_t)lv.count * lv.s);
+        dg = std::max(dg, (int64_t)lv.count * (nd_tc_bytes_w(lv.f) + nd_tc_bytes_u(lv.f)));
+        ex = std::max(ex, (int64_t)lv.count * 2 * lv.f);
+        vs = std::max(vs, (int64_t)lv.count * lv.f * kNdStep);
         if (lv.s > kNdPanelRegRows) ps = std::max(ps, (int64_t)lv.count * lv.s * (kNdPanel + 1));
       }
       max_sr = std::max(max_sr, std::max(lv.s, lv.r));
@@ -178,23 +178,19 @@ lsp_status lsp_nd_factor(lsp_ctx* c, const lsp_nd_opts* opts) {
         !ensure(c, S.perm, sizeof(int32_t) * P.perm_ints) ||
         !ensure(c, S.z, sizeof(double) * P.z_doubles) ||
         !ensure(c, S.u, sizeof(double) * (P.u_doubles > 0 ? P.u_doubles : 1)) ||
-        !ensure(c, S.cbuf, sizeof(double) * 2 * cb) ||
-        !ensure(c, S.pinv, sizeof(double) * 2 * pv) ||
-        !ensure(c, S.swaps, sizeof(int32_t) * 2 * sw) || !ensure(c, S.err, sizeof(int32_t)) ||
+        !ensure(c, S.cur, sizeof(int32_t) * cu) ||
+        !ensure(c, S.xrow, sizeof(double) * nf * 2 * kNdPanel * kNdStep) ||
+        !ensure(c, S.pinv, sizeof(double) * nf * kNdPanel * kNdPanel) ||
+        !ensure(c, S.swaps, sizeof(int32_t) * nf * kNdSwapInts) ||
+        !ensure(c, S.vst, sizeof(double) * vs) || !ensure(c, S.digits, (size_t)dg) || !ensure(c, S.expo, sizeof(int32_t) * ex) ||
+        !ensure(c, S.err, sizeof(int32_t)) ||
         !ensure(c, S.solve, sizeof(double) * P.solve_doubles) ||
         !ensure(c, S.gsrc, sizeof(int32_t) * 3 * P.z_doubles))
       return sfail(c, LSP_ERR_OOM, "nested dissection buffers: %s", c->err.c_str());
-    S.cbuf_half = cb;
-    S.pinv_half = pv;
-    S.swaps_half = sw;
-    SCUDA(c, cudaMemsetAsync(S.swaps.p, 0, sizeof(int32_t) * 2 * sw, c->stream));
-    if (!S.side) {
-      int least = 0, greatest = 0;
-      SCUDA(c, cudaDeviceGetStreamPriorityRange(&least, &greatest));
-      SCUDA(c, cudaStreamCreateWithPriority(&S.side, cudaStreamNonBlocking, greatest));
-      SCUDA(c, cudaEventCreateWithFlags(&S.ev_cols, cudaEventDisableTiming));
-      SCUDA(c, cudaEventCreateWithFlags(&S.ev_panel, cudaEventDisableTiming));
-    }
+    SCUDA(c, cudaMemsetAsync(S.swaps.p, 0, sizeof(int32_t) * nf * kNdSwapInts, c->stream));
+    SCUDA(c, cudaMemsetAsync(S.cur.p, 0, sizeof(int32_t) * cu, c->stream));
+    SCUDA(c, cudaMemsetAsync(S.vst.p, 0, sizeof(double) * vs, c->stream));
+    SCUDA(c, nd_tc_prepare());
     SCUDA(c, nd_prepare_kernels(max_sr));
     S.have_plan = true;
   }
@@ -210,6 +206,8 @@ lsp_status lsp_nd_factor(lsp_ctx* c, const lsp_nd_opts* opts) {
   int32_t herr = 0;
   SCUDA(c, cudaMemcpyAsync(&herr, S.err.p, sizeof(int32_t), cudaMemcpyDeviceToHost, c->stream));
   SCUDA(c, cudaStreamSynchronize(c->stream));
+  if (herr & kNdErrWait)
+    return sfail(c, LSP_ERR_TIMEOUT, "a wait of the nested dissection's updates gave up");
   if (herr)
     return sfail(c, LSP_ERR_DEGENERATE,
                  "a pivot of the nested dissection vanished (code %d): P is singular", herr);

@@ -32,8 +32,11 @@
 
 namespace lsp {
 
-constexpr int kNdPanel = 16;       // columns eliminated per step in the blocked path
+constexpr int kNdStep = 64;        // pivots per step of the blocked path
+constexpr int kNdPanel = 16;       // pivots chosen at once within a step
+constexpr int kNdSwapInts = 1 + 4 * kNdPanel;  // a panel's row exchanges: count, dst, src
 constexpr int kNdSmallFront = 160; // fronts with f <= this are swept in shared memory
+constexpr int kNdErrWait = 1 << 16; // err bit: a wait of k_nd_gemm gave up
 constexpr int kNdMaxN = 1024;      // 2D: the cross has 2n - 1 points
 constexpr int kNdMaxN3 = 64;       // 3D: the slab fronts have 2 (n/2 - 1) n + 2 n^2 points (12 160 at 64)
 constexpr int kNdPanelRegRows = 8 * 256;  // panels up to this many rows keep them in registers
@@ -76,13 +79,12 @@ struct NdState {
   bool factored = false;
   int64_t factored_gen = -1;  // ctx->build_gen of the rows that were factored
   int refine_steps = 0;       // iterative-refinement steps after every solve
-  DevBuf fronts, E, R, inv, asm_dst, asm_src, perm, z, u, cbuf, pinv, swaps, err;
+  DevBuf fronts, E, R, inv, asm_dst, asm_src, perm, z, u, err;
+  DevBuf cur, xrow, pinv, swaps;  // a step's row positions, exchanged rows, pivot blocks
+  DevBuf vst, digits, expo;       // a step's V; the digits and exponents of its W and V
   DevBuf solve, gsrc;         // the blocks a solve reads, transposed; right-hand side sources
   DevBuf ry, rd;              // refinement scratch: a copy of y, the correction
   DevBuf pscratch;            // FP32 pivot-ranking rows of panels over 2048 rows
-  int64_t cbuf_half = 0, pinv_half = 0, swaps_half = 0;  // the two copies of the step buffers
-  cudaStream_t side = nullptr;  // look-ahead panels (high priority)
-  cudaEvent_t ev_cols = nullptr, ev_panel = nullptr;
   // GMRES workspace
   DevBuf V, w, b, x, tmp, gs, fvec;
   double* h_gs = nullptr;  // pinned mirror of the scalars the host loop reads
@@ -97,6 +99,13 @@ void nd_free(NdState* s);
 // ---- launchers (k_nd.cu) ----
 cudaError_t launch_nd_assemble(lsp_ctx* c, int depth, const double* rows);
 cudaError_t launch_nd_sweep(lsp_ctx* c, int depth);
+cudaError_t launch_nd_panel(lsp_ctx* c, int depth, int k, int nb, int k0, int sb);
+const char* nd_timer_name(int kind, int depth);  // 4: sub-steps and splits, 5: updates
+// ---- blocked steps on the tensor cores (k_nd_tc.cu) ----
+cudaError_t launch_nd_blocked(lsp_ctx* c, int depth);
+cudaError_t nd_tc_prepare();
+int64_t nd_tc_bytes_w(int f);  // digit bytes of one front's W and V
+int64_t nd_tc_bytes_u(int f);
 cudaError_t launch_nd_store(lsp_ctx* c, int depth);
 cudaError_t launch_nd_solve(lsp_ctx* c, const double* y, double* x);
 // y = rows u, or sub - rows u when sub is given (y may be sub)
