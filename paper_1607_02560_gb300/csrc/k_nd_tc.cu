@@ -27,7 +27,7 @@
 // operands in shared memory), then about 80 integer operations and one FP64 addition per entry to
 // take the sums out, against 262e3 cycles of the FP64 pipe.
 // Measured against rank-16 updates of the whole front on the FP64 pipe: the updates of 3D n = 32
-// about 100 -> 10 ms, the whole factorisation 118 -> 27.5 ms, of 2D n = 512 28.4 -> 15.4 ms; the
+// about 100 -> 8 ms, the whole factorisation 118 -> 25 ms, of 2D n = 512 28.4 -> 15.1 ms; the
 // unrefined backward error is smaller (3D) or equal (2D).
 #include <cuda_fp16.h>
 #include <math.h>
@@ -343,133 +343,166 @@ __device__ __forceinline__ double sum_of(const int (&a)[kLevels], int ex) {
 
 // The update. One block per SM takes a run of the 128 x 64 tiles (columns j x rows i) of all fronts,
 // rows fastest: the seven W digit tiles stay in shared memory while the columns stay the same, the
-// next V digit tiles are copied while the sums of a tile are taken out. Per tile one thread issues
-// the 28 digit products, weight l = t + t' into accumulator columns 64 l; sixteen warps then take
-// the sums out (eight left the latency of the integer chains exposed).
-constexpr int kGemmThreads = 512;
-constexpr size_t kGemmSmem = (size_t)kDigits * (kBytesW + kBytesU);
+// V digit tiles have two buffers. One thread of the last warp copies the tiles and issues the 28
+// digit products, weight l = t + t' into accumulator columns 64 l (unrolled, descriptors by one
+// addition: a loop took 109 cycles a product to issue, this takes 57). The other sixteen warps take
+// the sums out, 16 rows each in two groups; the accumulators are free for the next tile once the
+// second group is in registers. Cycles a tile: products 6.4e3, sums 9.8e3; with one after the other
+// and the copies exposed the updates of 3D n = 32 took 10.4 ms, with the overlap 7.8 ms.
+constexpr int kSumWarps = 16, kGemmThreads = 32 * (kSumWarps + 1);
+constexpr size_t kGemmSmem = (size_t)kDigits * (kBytesW + 2 * kBytesU);
 __global__ void __launch_bounds__(kGemmThreads, 1) k_nd_gemm(
     double* __restrict__ fronts, int f, int k0, int sb, int64_t total,
     const uint8_t* __restrict__ dW, const int32_t* __restrict__ eW,
     const uint8_t* __restrict__ dV, const int32_t* __restrict__ eV, int32_t* __restrict__ err) {
   extern __shared__ __align__(1024) uint8_t smem[];
-  __shared__ __align__(8) uint64_t bar_w, bar_v, bar_mma;
+  __shared__ __align__(8) uint64_t bar_w, bar_v[2], bar_mma, bar_free;
   __shared__ uint32_t tslot;
-  __shared__ int s_abort;
-  __shared__ int ei[kTileI];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int ni = (f + kTileI - 1) / kTileI, nj = (f + kTileJ - 1) / kTileJ;
   const int64_t g0 = total * blockIdx.x / gridDim.x, g1 = total * (blockIdx.x + 1) / gridDim.x;
-  uint8_t* sW = smem;
-  uint8_t* sV = smem + kDigits * kBytesW;
   if (tid == 0) {
     tc::mbar_init(&bar_w, 1);
-    tc::mbar_init(&bar_v, 1);
+    tc::mbar_init(&bar_v[0], 1);
+    tc::mbar_init(&bar_v[1], 1);
     tc::mbar_init(&bar_mma, 1);
-    s_abort = 0;
+    tc::mbar_init(&bar_free, kSumWarps);
   }
   if (warp == 0) tc::tmem_alloc(&tslot, 512);
   tc::fence_before();
   __syncthreads();
   tc::fence_after();
   const uint32_t tmem = tslot;
-  volatile int* abort_flag = &s_abort;
   chain_start();
-  // thread 0: copies of W and V started, tiles whose products were committed
-  int loads_w = 0, loads_v = 0, tiles = 0;
-  auto load = [&](int64_t g) {
-    const int64_t grp = g / ni, fid = grp / nj;
-    if (g == g0 || g % ni == 0) {
-      tc::mbar_expect_tx(&bar_w, kDigits * kBytesW);
-      tc::bulk_g2s(sW, dW + grp * (kDigits * kBytesW), kDigits * kBytesW, &bar_w);
-      ++loads_w;
-    }
-    tc::mbar_expect_tx(&bar_v, kDigits * kBytesU);
-    tc::bulk_g2s(sV, dV + (fid * ni + g % ni) * (kDigits * kBytesU), kDigits * kBytesU, &bar_v);
-    ++loads_v;
-  };
-  if (tid == 0 && g0 < g1) load(g0);
-  const int ksteps = (sb + 15) / 16;
-  for (int64_t g = g0; g < g1; ++g) {
-    const int64_t grp = g / ni, fid = grp / nj;
-    const int i0 = (int)(g % ni) * kTileI, j0 = (int)(grp % nj) * kTileJ;
-    if (tid < kTileI) ei[tid] = i0 + tid < f ? eV[fid * f + i0 + tid] : kExpNone;
-    if (tid == 0) {
-      // every copy counted is waited for; a phase passed already returns at once
-      if (!tc::mbar_wait(&bar_w, (uint32_t)(loads_w - 1) & 1u, err, kNdErrWait) ||
-          !tc::mbar_wait(&bar_v, (uint32_t)(loads_v - 1) & 1u, err, kNdErrWait))
-        *abort_flag = 1;
-      if (!*abort_flag) {
+  if (warp == kSumWarps) {
+    if (lane == 0 && g0 < g1) {
+      uint8_t* sW = smem;
+      uint8_t* sV = smem + kDigits * kBytesW;
+      int loads_w = 0, loads_v = 0, tiles = 0;
+      auto load_w = [&](int64_t grp) {
+        tc::mbar_expect_tx(&bar_w, kDigits * kBytesW);
+        tc::bulk_g2s(sW, dW + grp * (kDigits * kBytesW), kDigits * kBytesW, &bar_w);
+        ++loads_w;
+      };
+      auto load_v = [&](int64_t g) {
+        const int b = loads_v++ & 1;
+        tc::mbar_expect_tx(&bar_v[b], kDigits * kBytesU);
+        tc::bulk_g2s(sV + b * (kDigits * kBytesU),
+                     dV + (g / ni / nj * ni + g % ni) * (kDigits * kBytesU), kDigits * kBytesU,
+                     &bar_v[b]);
+      };
+      const int ksteps = (sb + 15) / 16;
+      constexpr uint32_t sbo = (SB / 8) * 128;
+      constexpr uint32_t idesc = tc::idesc_f16(kTileJ, kTileI);
+      const uint64_t da = tc::desc_kmajor(tc::smem_u32(sW), 128, sbo);
+      load_w(g0 / ni);
+      load_v(g0);
+      bool ok = true;
+      for (int64_t g = g0; ok && g < g1; ++g) {
+        const int t = (int)(g - g0);
+        // the sums of the tile before are out, so its products have completed
+        if (t > 0) ok = tc::mbar_wait(&bar_free, (uint32_t)(t - 1) & 1u, err, kNdErrWait);
+        if (!ok) break;
+        if (t > 0 && g % ni == 0) load_w(g / ni);
+        if (g + 1 < g1) load_v(g + 1);
+        // (a phase of W passed already returns at once)
+        ok = tc::mbar_wait(&bar_w, (uint32_t)(loads_w - 1) & 1u, err, kNdErrWait) &&
+             tc::mbar_wait(&bar_v[t & 1], (uint32_t)(t >> 1) & 1u, err, kNdErrWait);
+        if (!ok) break;
         tc::fence_after();
-        const uint32_t aw = tc::smem_u32(sW), av = tc::smem_u32(sV);
-        constexpr uint32_t sbo = (SB / 8) * 128;
-        const uint32_t idesc = tc::idesc_f16(kTileJ, kTileI);
-        for (int a = 0; a < kDigits; ++a)
-          for (int b = 0; a + b < kLevels; ++b) {
-            const uint64_t da = tc::desc_kmajor(aw + a * kBytesW, 128, sbo);
-            const uint64_t db = tc::desc_kmajor(av + b * kBytesU, 128, sbo);
-            for (int q = 0; q < ksteps; ++q)
-              tc::mma_bf16(tmem + (uint32_t)((a + b) * kTileI), da + (uint64_t)(16 * q),
-                           db + (uint64_t)(16 * q), idesc, (a > 0 || q > 0) ? 1u : 0u);
-          }
+        const uint64_t db =
+            tc::desc_kmajor(tc::smem_u32(sV + (t & 1) * (kDigits * kBytesU)), 128, sbo);
+        if (ksteps == SB / 16) {
+#pragma unroll
+          for (int a = 0; a < kDigits; ++a)
+#pragma unroll
+            for (int b = 0; a + b < kLevels; ++b)
+#pragma unroll
+              for (int q = 0; q < SB / 16; ++q)
+                tc::mma_bf16(tmem + (uint32_t)((a + b) * kTileI),
+                             da + (uint64_t)(a * kBytesW / 16 + 16 * q),
+                             db + (uint64_t)(b * kBytesU / 16 + 16 * q), idesc,
+                             (a > 0 || q > 0) ? 1u : 0u);
+        } else {
+          for (int a = 0; a < kDigits; ++a)
+            for (int b = 0; a + b < kLevels; ++b)
+              for (int q = 0; q < ksteps; ++q)
+                tc::mma_bf16(tmem + (uint32_t)((a + b) * kTileI),
+                             da + (uint64_t)(a * kBytesW / 16 + 16 * q),
+                             db + (uint64_t)(b * kBytesU / 16 + 16 * q), idesc,
+                             (a > 0 || q > 0) ? 1u : 0u);
+        }
+        tc::commit(&bar_mma);
+        ++tiles;
       }
-      tc::commit(&bar_mma);
-      ++tiles;
+      // before leaving (after a wait that gave up as well): copies and products in flight
+      tc::mbar_wait(&bar_w, (uint32_t)(loads_w - 1) & 1u, err, 0);
+      for (int b = 0; b < 2; ++b) {
+        const int uses = loads_v / 2 + (b < loads_v % 2 ? 1 : 0);
+        if (uses) tc::mbar_wait(&bar_v[b], (uint32_t)(uses - 1) & 1u, err, 0);
+      }
+      if (tiles) tc::mbar_wait(&bar_mma, (uint32_t)(tiles - 1) & 1u, err, 0);
     }
-    const int j = j0 + (warp & 3) * 32 + lane, ib0 = i0 + (warp >> 2) * 16;
-    const bool jl = j < f;
-    const int ej = jl ? eW[fid * f + j] : kExpNone;
-    double* Fj = fronts + fid * f * f + (jl ? j : 0);
+  } else {
     // rows below zlo and from zhi on keep their entry: the pivot rows of sub-steps after the
     // column's own (all of K for a column outside K) are replaced
-    const int zlo = jl && j >= k0 && j < k0 + sb ? k0 + ((j - k0) / NP + 1) * NP : k0,
-              zhi = k0 + sb;
-    // entries to update: the first group is loaded while the products run
-    auto fetch = [&](int c0, double (&old)[8]) {
+    const int zhi = k0 + sb;
+    bool ok = true;
+    for (int64_t g = g0; ok && g < g1; ++g) {
+      const int64_t grp = g / ni, fid = grp / nj;
+      const int j = (int)(grp % nj) * kTileJ + (warp & 3) * 32 + lane;
+      const int ib = (int)(g % ni) * kTileI + (warp >> 2) * 16;
+      const bool jl = j < f;
+      const int ej = (jl ? eW[fid * f + j] : kExpNone) - 16;
+      const int32_t* er = eV + fid * f;
+      double* Fj = fronts + fid * f * f + (jl ? j : 0);
+      const int zlo = jl && j >= k0 && j < zhi ? k0 + ((j - k0) / NP + 1) * NP : k0;
+      double old[8];
+      auto fetch = [&](int c0) {
 #pragma unroll
-      for (int q = 0; q < 8; ++q) {
-        const int i = ib0 + c0 + q;
-        old[q] = jl && i < f && (i < zlo || i >= zhi) ? Fj[(int64_t)i * f] : 0.0;
-      }
-    };
-    double old[8];
-    fetch(0, old);
-    if (lane == 0 && !tc::mbar_wait(&bar_mma, (uint32_t)(g - g0) & 1u, err, kNdErrWait))
-      *abort_flag = 1;
-    __syncthreads();
-    if (*abort_flag) break;
-    tc::fence_after();
-    if (tid == 0 && g + 1 < g1) load(g + 1);  // the products have read the tiles
-    const uint32_t taddr =
-        tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)((warp >> 2) * 16);
+        for (int q = 0; q < 8; ++q) {
+          const int i = ib + c0 + q;
+          old[q] = jl && i < f && (i < zlo || i >= zhi) ? Fj[(int64_t)i * f] : 0.0;
+        }
+      };
+      fetch(0);
+      // (one lane asks, the others follow its answer)
+      const bool got =
+          lane == 0 ? tc::mbar_wait(&bar_mma, (uint32_t)(g - g0) & 1u, err, kNdErrWait) : true;
+      ok = __all_sync(0xffffffffu, got);
+      if (!ok) break;
+      tc::fence_after();
+      const uint32_t taddr =
+          tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)((warp >> 2) * 16);
 #pragma unroll
-    for (int c0 = 0; c0 < 16; c0 += 8) {
-      uint32_t r[kLevels][8];
+      for (int c0 = 0; c0 < 16; c0 += 8) {
+        uint32_t r[kLevels][8];
 #pragma unroll
-      for (int l = 0; l < kLevels; ++l) tmem_ld8(taddr + (uint32_t)(l * kTileI + c0), r[l]);
-      if (c0) fetch(c0, old);
-      tc::ld_wait();
+        for (int l = 0; l < kLevels; ++l) tmem_ld8(taddr + (uint32_t)(l * kTileI + c0), r[l]);
+        if (c0) fetch(c0);
+        tc::ld_wait();
+        if (c0) {
+          tc::fence_before();
+          __syncwarp();
+          if (lane == 0) tc::mbar_arrive(&bar_free);
+        }
 #pragma unroll
-      for (int q = 0; q < 8; ++q) {
-        int a[kLevels];
+        for (int q = 0; q < 8; ++q) {
+          int a[kLevels];
 #pragma unroll
-        for (int l = 0; l < kLevels; ++l) a[l] = __float2int_rn(__uint_as_float(r[l][q]));
-        const int i = ib0 + c0 + q;
-        const double v = sum_of(a, ei[i - i0] + ej - 16);
-        if (jl && i < f) Fj[(int64_t)i * f] = old[q] + v;
+          for (int l = 0; l < kLevels; ++l) a[l] = __float2int_rn(__uint_as_float(r[l][q]));
+          const int i = ib + c0 + q;
+          if (i < f) {
+            const double v = sum_of(a, er[i] + ej);
+            if (jl) Fj[(int64_t)i * f] = old[q] + v;
+          }
+        }
       }
     }
-    tc::fence_before();
-    __syncthreads();  // the accumulators and ei are free again
-    tc::fence_after();
   }
-  // after an abort: the copies in flight land, and the products issued complete, before leaving
-  if (tid == 0 && *abort_flag) {
-    if (loads_w) tc::mbar_wait(&bar_w, (uint32_t)(loads_w - 1) & 1u, err, 0);
-    if (loads_v) tc::mbar_wait(&bar_v, (uint32_t)(loads_v - 1) & 1u, err, 0);
-    if (tiles) tc::mbar_wait(&bar_mma, (uint32_t)(tiles - 1) & 1u, err, 0);
-  }
+  tc::fence_before();
   __syncthreads();
+  tc::fence_after();
   if (warp == 0) tc::tmem_dealloc(tmem, 512);
 }
 
