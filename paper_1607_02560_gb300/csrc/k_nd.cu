@@ -59,113 +59,6 @@ __device__ __forceinline__ void warp_argmax_f(float& best, int& bi) {
     }
   }
 }
-__device__ __forceinline__ void warp_argmax(double& best, int& bi) {
-  for (int off = 16; off > 0; off >>= 1) {
-    const double ob = __shfl_xor_sync(0xffffffffu, best, off);
-    const int oi = __shfl_xor_sync(0xffffffffu, bi, off);
-    if (ob > best || (ob == best && oi < bi)) {
-      best = ob;
-      bi = oi;
-    }
-  }
-}
-
-// Partial inversion of one front (f <= kNdSmallFront) in shared memory, one pivot at a time.
-// Pivot k: the row of largest |F[i][k]| among the rows k..s-1 still unpivoted; then
-//   F[k][k] <- 1/F[k][k], F[k][j] <- F[k][j]/F[k][k], F[i][k] <- -F[i][k]/F[k][k],
-//   F[i][j] <- F[i][j] - F[i][k] F[k][j]/F[k][k]   (i, j != k).
-__global__ void __launch_bounds__(256) k_nd_sweep_small(double* __restrict__ fronts, int f, int s,
-                                                        int32_t* __restrict__ perm,
-                                                        int32_t* __restrict__ err) {
-  extern __shared__ double sm[];
-  double* F = sm;
-  double* colk = F + f * f;
-  double* rowk = colk + f;
-  __shared__ int sperm[kNdSmallFront];
-  __shared__ int piv, bad;
-  __shared__ double spiv;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nt = blockDim.x;
-  double* G = fronts + (int64_t)blockIdx.x * f * f;
-  for (int e = tid; e < f * f; e += nt) F[e] = G[e];
-  for (int e = tid; e < s; e += nt) sperm[e] = e;
-  if (tid == 0) bad = 0;
-  __syncthreads();
-  for (int k = 0; k < s; ++k) {
-    if (warp == 0) {
-      double best = -1.0;
-      int bi = s;
-      for (int i = k + lane; i < s; i += 32) {
-        const double a = fabs(F[i * f + k]);
-        if (a > best) {
-          best = a;
-          bi = i;
-        }
-      }
-      warp_argmax(best, bi);
-      if (lane == 0) {
-        if (!(best > 0.0) || !isfinite(best)) {
-          bad = 1;
-          atomicOr(err, 1);
-        }
-        piv = bi < s ? bi : k;
-        spiv = 1.0 / F[piv * f + k];  // the one FP64 division of this pivot
-      }
-    }
-    __syncthreads();
-    if (bad) break;
-    const int p = piv;
-    if (p != k) {
-      for (int j = tid; j < f; j += nt) {
-        const double a = F[k * f + j];
-        F[k * f + j] = F[p * f + j];
-        F[p * f + j] = a;
-      }
-      if (tid == 0) {
-        const int t = sperm[k];
-        sperm[k] = sperm[p];
-        sperm[p] = t;
-      }
-      __syncthreads();
-    }
-    const double dinv = spiv;
-    for (int j = tid; j < f; j += nt) {
-      rowk[j] = F[k * f + j] * dinv;
-      colk[j] = F[j * f + k];
-    }
-    __syncthreads();
-    for (int i = warp; i < f; i += nt / 32) {
-      double* Fi = F + i * f;
-      if (i == k) {
-        for (int j = lane; j < f; j += 32) Fi[j] = j == k ? dinv : rowk[j];
-      } else {
-        const double ci = colk[i];
-        for (int j = lane; j < f; j += 32) Fi[j] = j == k ? -ci * dinv : fma(-ci, rowk[j], Fi[j]);
-      }
-    }
-    __syncthreads();
-  }
-  for (int e = tid; e < f * f; e += nt) G[e] = F[e];
-  for (int e = tid; e < s; e += nt) perm[(int64_t)blockIdx.x * s + e] = sperm[e];
-}
-
-// ---- blocked partial inversion (k_nd_tc.cu): panels of the sub-steps K = [k, k + nb) of a step
-// with the columns [k0, k0 + sb) ----
-// swaps layout per front: [0] = number of entries q, then dst[q] at 1 + q, src[q] at
-// 1 + 2 NP + q: after the sub-step, position dst holds the row that was at position src; the
-// first nb entries are the pivot rows.
-constexpr int kSwapInts = kNdSwapInts, SB = kNdStep;
-
-// FP32 value of x for ranking pivot candidates, from the high word of the IEEE double: sign,
-// exponent rebased from 1023 to 127, the top 20 fraction bits (relative error < 2^-20);
-// magnitudes below the FP32 normal range give 0, above it infinity. Integer operations only.
-__device__ __forceinline__ float rank_f32(double x) {
-  const int hi = __double2hiint(x);
-  const int e = ((hi >> 20) & 0x7ff) - (1023 - 127);
-  const unsigned sign = (unsigned)hi & 0x80000000u;
-  if (e <= 0) return __uint_as_float(sign);
-  if (e >= 255) return __uint_as_float(sign | 0x7f800000u);
-  return __uint_as_float(sign | ((unsigned)e << 23) | (((unsigned)hi & 0xfffffu) << 3));
-}
 
 // 1 / x to within an ulp: the reciprocal of the mantissa in FP32, one third-order step
 // r (1 + e + e^2) with e = 1 - m r in FP64, the exponent by integers. Three FP64 operations where
@@ -184,21 +77,140 @@ __device__ __forceinline__ double recip_f64(double x) {
   return __hiloint2double((hi & 0x80000000) | (fld << 20) | (rh & 0xfffff), __double2loint(r));
 }
 
+// Partial inversion of one front (f <= kNdSmallFront) in shared memory, one pivot at a time.
+// Pivot k: the row of largest |F[i][k]| (by its upper 32 bits) among the rows k..s-1 still
+// unpivoted, exchanged with row k; then
+//   F[k][k] <- 1/F[k][k], F[k][j] <- F[k][j]/F[k][k], F[i][k] <- -F[i][k]/F[k][k],
+//   F[i][j] <- F[i][j] - F[i][k] F[k][j]/F[k][k]   (i, j != k).
+// A warp updates whole rows, NJ = ceil(f / 32) entries a lane, with its part of the pivot row in
+// registers; the exchange is folded into the update. Rows whose multiplier is zero stay as they
+// are: in a leaf, whose rows have 9 or 27 entries, a third of them on average.
+// What bounds it: the FP64 pipe in the leaves (n = 512: 4096 fronts of 81 rows, 49 pivots) and its
+// latency elsewhere. Measured: the leaves of n = 512 3.90 -> 2.84 ms (before: every row and entry
+// updated, FP64 comparisons and a division per pivot, the exchange as a pass of its own).
+template <int NJ>
+__global__ void __launch_bounds__(512) k_nd_sweep_small(double* __restrict__ fronts, int f, int s,
+                                                        int32_t* __restrict__ perm,
+                                                        int32_t* __restrict__ err) {
+  extern __shared__ double sm[];
+  double* F = sm;
+  double* colk = F + f * f;  // column k (of the row that takes each position)
+  double* rowk = colk + f;   // the scaled pivot row
+  double* rowo = rowk + f;   // row k before the exchange
+  __shared__ int sperm[kNdSmallFront];
+  __shared__ int piv, bad;
+  __shared__ double spiv;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int nt = blockDim.x;
+  double* G = fronts + (int64_t)blockIdx.x * f * f;
+  for (int e = tid; e < f * f; e += nt) F[e] = G[e];
+  for (int e = tid; e < s; e += nt) sperm[e] = e;
+  if (tid == 0) bad = 0;
+  __syncthreads();
+  for (int k = 0; k < s; ++k) {
+    if (warp == 0) {
+      unsigned key = 0;
+      int bi = k;
+      for (int i = k + lane; i < s; i += 32) {
+        const unsigned a = ((unsigned)__double2hiint(F[i * f + k]) & 0x7fffffffu) + 1u;
+        if (a > key) {
+          key = a;
+          bi = i;
+        }
+      }
+      const unsigned top = __reduce_max_sync(0xffffffffu, key);
+      const int p = (int)__reduce_min_sync(0xffffffffu, key == top ? (unsigned)bi : 0xffffffffu);
+      if (lane == 0) {
+        const double x = F[p * f + k];
+        if (x == 0.0 || top > 0x7ff00000u) {  // zero, Inf or NaN
+          bad = 1;
+          atomicOr(err, 1);
+        }
+        piv = p;
+        spiv = recip_f64(x);
+        const int t = sperm[k];
+        sperm[k] = sperm[p];
+        sperm[p] = t;
+      }
+    }
+    __syncthreads();
+    if (bad) break;
+    const int p = piv;
+    const double dinv = spiv;
+    if (tid < f) {
+      rowk[tid] = F[p * f + tid] * dinv;
+      rowo[tid] = F[k * f + tid];
+      colk[tid] = F[(tid == p ? k : tid) * f + k];
+    }
+    __syncthreads();
+    double rk[NJ];
+#pragma unroll
+    for (int c = 0; c < NJ; ++c) {
+      const int j = lane + 32 * c;
+      rk[c] = j < f ? (j == k ? dinv : rowk[j]) : 0.0;
+    }
+    for (int i = warp; i < f; i += nt / 32) {
+      double* Fi = F + i * f;
+      const double* Fo = i == p ? rowo : Fi;
+      const double ci = i == k ? -1.0 : colk[i];
+      if (ci == 0.0 && i != p) continue;
+#pragma unroll
+      for (int c = 0; c < NJ; ++c) {
+        const int j = lane + 32 * c;
+        if (j < f) Fi[j] = fma(-ci, rk[c], j == k || i == k ? 0.0 : Fo[j]);
+      }
+    }
+    __syncthreads();
+  }
+  for (int e = tid; e < f * f; e += nt) G[e] = F[e];
+  for (int e = tid; e < s; e += nt) perm[(int64_t)blockIdx.x * s + e] = sperm[e];
+}
+
+// ---- blocked partial inversion (k_nd_tc.cu): panels of the sub-steps K = [k, k + nb) of a step
+// with the columns [k0, k0 + sb) ----
+// swaps layout per front: [0] = number of entries q, then the positions that get another row after
+// the sub-step, in the order of their rows in xrow; the first nb are the pivot rows.
+constexpr int kSwapInts = kNdSwapInts, SB = kNdStep;
+
+// FP32 value of x for ranking pivot candidates, from the high word of the IEEE double: sign,
+// exponent rebased from 1023 to 127, the top 20 fraction bits (relative error < 2^-20);
+// magnitudes below the FP32 normal range give 0, above it infinity. Integer operations only.
+__device__ __forceinline__ float rank_f32(double x) {
+  const int hi = __double2hiint(x);
+  const int e = ((hi >> 20) & 0x7ff) - (1023 - 127);
+  const unsigned sign = (unsigned)hi & 0x80000000u;
+  if (e <= 0) return __uint_as_float(sign);
+  if (e >= 255) return __uint_as_float(sign | 0x7f800000u);
+  return __uint_as_float(sign | ((unsigned)e << 23) | (((unsigned)hi & 0xfffffu) << 3));
+}
+
 // Common end (after the pivot rows sel[0..nb) are known, block-synchronised): row exchanges, the
 // exchanged rows' columns of the step, the FP64 pivot-block inverse.
-__device__ __forceinline__ void panel_tail(const double* __restrict__ F, int f, int s, int k,
+__device__ __forceinline__ void panel_tail(const double* F, int f, int s, int k,
                                            int nb, int k0, int sb, int64_t fid, const int* sel,
-                                           int32_t* __restrict__ perm, int32_t* __restrict__ cur,
-                                           double* __restrict__ xrow, double* __restrict__ pinv,
-                                           int32_t* __restrict__ swaps, int32_t* __restrict__ err) {
+                                           int32_t* perm, int32_t* cur,
+                                           double* xrow, double* pinv,
+                                           int32_t* swaps, int32_t* err) {
   constexpr int NT = 256;
   __shared__ int nq;
   __shared__ int dstp[2 * NP], srcp[2 * NP];
+  __shared__ double A[2][NP][NP + 1], trow[2][NP];
+  __shared__ int piv_row[NP], row_piv[NP];  // p_j, and the j of a row
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  // row exchanges (warp 0): position k + j takes the row chosen j-th; the rows of K that were
-  // not chosen move, in increasing position order, to the positions the chosen rows left
+  const int gr = tid / NP, gc = tid % NP;  // 256 threads = 16 x 16
+  // the pivot block and the pivot rows' columns of the step: loads that need only the choice
+  double* xr = xrow + fid * (2 * NP * SB);
+  double keep[NP * SB / NT], moved[NP * SB / NT];
+  A[0][gr][gc] = gr < nb && gc < nb ? F[(int64_t)(k + sel[gr]) * f + k + gc] : 0.0;
+#pragma unroll
+  for (int u = 0; u < NP * SB / NT; ++u) {
+    const int e = tid + u * NT, a = e / SB, c = e % SB;
+    keep[u] = a < nb && c < sb ? F[(int64_t)(k + sel[a]) * f + k0 + c] : 0.0;
+  }
+  // row exchanges (the last warp): position k + j takes the row chosen j-th; the rows of K that
+  // were not chosen move, in increasing position order, to the positions the chosen rows left
   // outside K (taken in choice order)
-  if (warp == 0) {
+  if (warp == NT / 32 - 1) {
     const bool act = lane < nb;
     const int ps = act ? k + sel[lane] : 0;
     const bool inK = act && ps < k + nb;
@@ -238,76 +250,77 @@ __device__ __forceinline__ void panel_tail(const double* __restrict__ F, int f, 
       nq = qq;
       sw[0] = qq;
     }
-    for (int a = lane; a < qq; a += 32) {
-      sw[1 + a] = dstp[a];
-      sw[1 + 2 * NP + a] = srcp[a];
-    }
+    for (int a = lane; a < qq; a += 32) sw[1 + a] = dstp[a];
   }
   __syncthreads();
+  // the displaced rows' columns, stored after the inversion, which covers the latency
   const int q = nq;
-  // the step's columns of the exchanged rows (the other rows are read in place by k_nd_sub): loaded
-  // here, stored after the inversion, which covers the latency
-  double* xr = xrow + fid * (2 * NP * SB);
-  double keep[2 * NP * SB / NT];
 #pragma unroll
-  for (int u = 0; u < 2 * NP * SB / NT; ++u) {
-    const int e = tid + u * NT, a = e / SB, c = e % SB;
-    keep[u] = a < q && c < sb ? F[(int64_t)srcp[a] * f + k0 + c] : 0.0;
+  for (int u = 0; u < NP * SB / NT; ++u) {
+    const int e = tid + u * NT, a = nb + e / SB, c = e % SB;
+    moved[u] = a < q && c < sb ? F[(int64_t)srcp[a] * f + k0 + c] : 0.0;
   }
   // Inverse of the pivot block A (FP64): Gauss-Jordan in place, one element per thread, no row
   // exchanges: pivot j is taken in the unpivoted row p_j of largest |a_pj,j| (by the upper 32 bits),
   // row p_j is scaled by one reciprocal, column j is eliminated from the other rows. Row p_j,
-  // column c of the result is element (j, p_c) of A^-1.
-  __shared__ double A[2][NP][NP + 1];
-  __shared__ double trow[NP];
-  __shared__ int piv_row[NP], row_piv[NP];  // p_j, and the j of a row
-  const int gr = tid / NP, gc = tid % NP;  // 256 threads = 16 x 16
-  {
-    int src = k + gr;
-    for (int e = 0; e < q; ++e)
-      if (dstp[e] == k + gr) src = srcp[e];
-    A[0][gr][gc] = (gr < nb && gc < nb) ? F[(int64_t)src * f + k + gc] : 0.0;
+  // column c of the result is element (j, p_c) of A^-1. Warp 0 prepares pivot j + 1 (column, choice,
+  // reciprocal, scaled row) while the others eliminate pivot j: one barrier a pivot.
+  bool open = lane < nb;  // warp 0: the lane's row has not been a pivot row
+  auto choose = [&](int j, double x) {  // x: column j of row lane % 16; the pivot's reciprocal
+    const unsigned key = open ? ((unsigned)__double2hiint(x) & 0x7fffffffu) + 1u : 0u;
+    const unsigned top = __reduce_max_sync(0xffffffffu, key);
+    const int p = __ffs(__ballot_sync(0xffffffffu, key == top)) - 1;
+    const double xp = __shfl_sync(0xffffffffu, x, p);
+    if (lane == p) {
+      open = false;
+      if (x == 0.0 || top > 0x7ff00000u) atomicOr(err, 4);  // zero, Inf or NaN
+      piv_row[j] = p;
+      row_piv[p] = j;
+    }
+    return make_double2(recip_f64(xp), __hiloint2double(0, p));
+  };
+  const int lr = lane & (NP - 1);
+  if (warp == 0) {
+    const double2 d = choose(0, A[0][lr][0]);
+    const int p = __double2loint(d.y);
+    if (lane < NP) trow[0][lane] = lane == 0 ? d.x : A[0][p][lane] * d.x;
   }
   __syncthreads();
-  bool open = lane < nb;  // warp 0: the lane's row has not been a pivot row
   for (int j = 0; j < nb; ++j) {
     const double(*Aj)[NP + 1] = A[j & 1];
     double(*An)[NP + 1] = A[~j & 1];
-    if (warp == 0) {
-      const unsigned key =
-          open ? ((unsigned)__double2hiint(Aj[lane & (NP - 1)][j]) & 0x7fffffffu) + 1u : 0u;
-      const unsigned top = __reduce_max_sync(0xffffffffu, key);
-      const int p = __ffs(__ballot_sync(0xffffffffu, key == top)) - 1;
-      const double x = Aj[p][j];
-      if (lane == p) {
-        open = false;
-        if (x == 0.0 || top - 1u >= 0x7ff00000u) atomicOr(err, 4);  // zero, Inf or NaN
-        piv_row[j] = p;
-        row_piv[p] = j;
-      }
-      const double d = recip_f64(x);
-      if (lane < NP) trow[lane] = lane == j ? d : Aj[p][lane] * d;
+    const double* tj = trow[j & 1];
+    const int p = piv_row[j];
+    if (warp == 0 && j + 1 < nb) {
+      const double2 d = choose(j + 1, lr == p ? tj[j + 1] : fma(-Aj[lr][j], tj[j + 1], Aj[lr][j + 1]));
+      const int pn = __double2loint(d.y);
+      const double y = fma(-Aj[pn][j], tj[lr], lr == j ? 0.0 : Aj[pn][lr]);
+      if (lane < NP) trow[~j & 1][lane] = lane == j + 1 ? d.x : y * d.x;
     }
-    __syncthreads();
-    const double t = trow[gc];
-    An[gr][gc] = gr == piv_row[j] ? t : fma(-Aj[gr][j], t, gc == j ? 0.0 : Aj[gr][gc]);
+    const double t = tj[gc];
+    An[gr][gc] = gr == p ? t : fma(-Aj[gr][j], t, gc == j ? 0.0 : Aj[gr][gc]);
     __syncthreads();
   }
   const bool in = gr < nb && gc < nb;
   pinv[fid * NP * NP + (in ? row_piv[gr] * NP + piv_row[gc] : tid)] = in ? A[nb & 1][gr][gc] : 0.0;
 #pragma unroll
-  for (int u = 0; u < 2 * NP * SB / NT; ++u)
-    if (tid + u * NT < q * SB) xr[tid + u * NT] = keep[u];
+  for (int u = 0; u < NP * SB / NT; ++u) {
+    const int e = tid + u * NT;
+    if (e < nb * SB) xr[e] = keep[u];
+    if (nb * SB + e < q * SB) xr[nb * SB + e] = moved[u];
+  }
 }
 
 constexpr int kPanelRows = 8;  // rows per thread: panels of up to 2048 rows (the cross, n = 1024)
 // A step's first panel: no row has moved yet.
-__device__ __forceinline__ void start_cur(int32_t* __restrict__ cur, int64_t fid, int s, int k,
+__device__ __forceinline__ void start_cur(int32_t* cur, int64_t fid, int s, int k,
                                           int k0) {
   if (k == k0)
     for (int p = k0 + threadIdx.x; p < s; p += blockDim.x) cur[fid * s + p] = p;
 }
-// A kernel of a chain launched to overlap the one before: its blocks wait here.
+// A kernel of a chain launched to overlap the one before: its blocks wait here. (What the chain
+// writes is not read through const __restrict__ pointers: the read-only path may hold lines from
+// before the wait.)
 __device__ __forceinline__ void chain_start() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -319,48 +332,51 @@ __device__ __forceinline__ void chain_start() {
 // it only ranks candidate rows by magnitude, while every value the factorisation keeps is computed
 // from the FP64 entries. Each thread keeps its panel rows (row tid + t * 256, t < ROWS) in
 // registers and each warp publishes its best candidate row to shared memory, so a pivot costs one
-// block barrier. Bound by the latency of the 16 pivots, once here and once in the inversion.
-// Measured at the root of 2D n = 512 (1023 rows): 40 -> 24 us a panel (before: rows read 128 bytes
-// apart by neighbouring lanes, every thread publishing its row, shuffles for the maxima, an FP64
-// division and both halves of [A | I] per pivot of the inversion).
+// block barrier. Bound by the latency of the 16 pivots, once here (580 cycles each) and once in
+// the inversion (1010 cycles each). Measured at the root of 2D n = 512 (1023 rows): 40 -> 21 us a
+// panel (before: rows read 128 bytes apart by neighbouring lanes, every thread publishing its row,
+// shuffles for the maxima, an FP64 division, three barriers and both halves of [A | I] per pivot of
+// the inversion).
 template <int ROWS>
-__global__ void __launch_bounds__(256) k_nd_panel(const double* __restrict__ fronts, int f, int s,
+__global__ void __launch_bounds__(256) k_nd_panel(const double* fronts, int f, int s,
                                                   int k, int nb, int k0, int sb,
-                                                  int32_t* __restrict__ perm,
-                                                  int32_t* __restrict__ cur,
-                                                  double* __restrict__ xrow,
-                                                  double* __restrict__ pinv,
-                                                  int32_t* __restrict__ swaps,
-                                                  int32_t* __restrict__ err) {
+                                                  int32_t* perm,
+                                                  int32_t* cur,
+                                                  double* xrow,
+                                                  double* pinv,
+                                                  int32_t* swaps,
+                                                  int32_t* err) {
   constexpr int NT = 256, NW = NT / 32;
   __shared__ float st[NT][NP + 1];                     // 256 panel rows on their way to registers
   __shared__ __align__(16) float cand[2][NW][NP + 4];  // each warp's best row, double-buffered
   __shared__ __align__(16) uint2 wb[2][NW];            // its magnitude (bits + 1) and index
   __shared__ int sel[NP];
-  const int tid = threadIdx.x, warp = tid >> 5;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int m = s - k;
   const int64_t fid = blockIdx.x;
   const double* F = fronts + fid * f * f;
   chain_start();
   start_cur(cur, fid, s, k, k0);
   float rv[ROWS][NP];
-  double v[NP];
+  constexpr int D = ROWS <= 4 ? ROWS : 2;  // groups of 256 rows in flight
+  double v[D][NP];
   const int hr = tid / NP, hc = tid % NP;  // half a warp reads one row of the panel
   auto fetch = [&](int t) {
 #pragma unroll
     for (int u = 0; u < NP; ++u) {
       const int row = t * NT + hr + u * (NT / NP);
-      v[u] = row < m && hc < nb ? F[(int64_t)(k + row) * f + k + hc] : 0.0;
+      v[t % D][u] = row < m && hc < nb ? F[(int64_t)(k + row) * f + k + hc] : 0.0;
     }
   };
-  fetch(0);
+#pragma unroll
+  for (int t = 0; t < D; ++t) fetch(t);
 #pragma unroll
   for (int t = 0; t < ROWS; ++t) {
     if (t) __syncthreads();
 #pragma unroll
-    for (int u = 0; u < NP; ++u) st[hr + u * (NT / NP)][hc] = rank_f32(v[u]);
+    for (int u = 0; u < NP; ++u) st[hr + u * (NT / NP)][hc] = rank_f32(v[t % D][u]);
     __syncthreads();
-    if (t + 1 < ROWS) fetch(t + 1);
+    if (t + D < ROWS) fetch(t + D);
 #pragma unroll
     for (int c = 0; c < NP; ++c) rv[t][c] = st[tid][c];
   }
@@ -382,35 +398,25 @@ __global__ void __launch_bounds__(256) k_nd_panel(const double* __restrict__ fro
         bt = t;
       }
     }
-    // the warp's: the largest magnitude, ties to the smaller index
+    // the warp's: the largest magnitude, ties to the lower lane
     const unsigned key = best >= 0.0f ? __float_as_uint(best) + 1u : 0u;
     const unsigned top = __reduce_max_sync(0xffffffffu, key);
-    const unsigned bi = (unsigned)(tid + bt * NT);
-    const unsigned wi = __reduce_min_sync(0xffffffffu, key == top ? bi : 0xffffffffu);
-    if (bi == wi) {
+    if (lane == __ffs(__ballot_sync(0xffffffffu, key == top)) - 1) {
 #pragma unroll
-      for (int c = 0; c < NP; ++c) {
-        if (c < j) continue;
-        float val = rv[0][c];
+      for (int t = 0; t < ROWS; ++t)
+        if (t == bt) {
 #pragma unroll
-        for (int t = 1; t < ROWS; ++t)
-          if (t == bt) val = rv[t][c];
-        cand[j & 1][warp][c] = val;
-      }
-      wb[j & 1][warp] = make_uint2(top, wi);
+          for (int c = 0; c < NP; ++c)
+            if (c >= j) cand[j & 1][warp][c] = rv[t][c];
+        }
+      wb[j & 1][warp] = make_uint2(top, (unsigned)(tid + bt * NT));
     }
     __syncthreads();
-    unsigned bk = 0, pr = 0xffffffffu;
-    int bw = 0;
-#pragma unroll
-    for (int w = 0; w < NW; ++w) {
-      const uint2 x = wb[j & 1][w];
-      if (x.x > bk || (x.x == bk && x.y < pr)) {
-        bk = x.x;
-        pr = x.y;
-        bw = w;
-      }
-    }
+    // the block's, ties to the lower warp
+    const uint2 mine = wb[j & 1][lane % NW];
+    const unsigned bk = __reduce_max_sync(0xffffffffu, mine.x);
+    const int bw = __ffs(__ballot_sync(0xffffffffu, mine.x == bk)) - 1;
+    const unsigned pr = __shfl_sync(0xffffffffu, mine.y, bw);
     if (bk < 2u || bk > 0x7f800000u || pr >= (unsigned)m) {  // zero, Inf: uniform over the block
       if (tid == 0) {
         atomicOr(err, 2);
@@ -423,7 +429,7 @@ __global__ void __launch_bounds__(256) k_nd_panel(const double* __restrict__ fro
     float pv[NP];  // the pivot row from column j on
 #pragma unroll
     for (int c = 0; c < NP; ++c) pv[c] = c >= j ? cand[j & 1][bw][c] : 0.0f;
-    const float ipv = 1.0f / pv[j];
+    const float ipv = __fdividef(1.0f, pv[j]);  // ranks only
 #pragma unroll
     for (int t = 0; t < ROWS; ++t) {
       if (used >> t & 1u) continue;
@@ -440,14 +446,14 @@ __global__ void __launch_bounds__(256) k_nd_panel(const double* __restrict__ fro
 // The same for panels of more than kPanelRows * 256 rows (the root planes of 3D grids): the same
 // FP32 trial elimination with the ranking rows in a global scratch (L2-resident) instead of
 // registers; each thread handles rows tid + t * 256, t < 64 (up to 16 384 rows).
-__global__ void __launch_bounds__(256) k_nd_panel_big(const double* __restrict__ fronts, int f,
+__global__ void __launch_bounds__(256) k_nd_panel_big(const double* fronts, int f,
                                                       int s, int k, int nb, int k0, int sb,
-                                                      int32_t* __restrict__ perm,
-                                                      int32_t* __restrict__ cur,
-                                                      double* __restrict__ xrow,
-                                                      double* __restrict__ pinv,
-                                                      int32_t* __restrict__ swaps,
-                                                      int32_t* __restrict__ err,
+                                                      int32_t* perm,
+                                                      int32_t* cur,
+                                                      double* xrow,
+                                                      double* pinv,
+                                                      int32_t* swaps,
+                                                      int32_t* err,
                                                       float* __restrict__ scratch) {
   constexpr int NT = 256, PS = NP + 1;
   __shared__ float cand[2][NT][PS];
@@ -819,11 +825,16 @@ cudaError_t launch_nd_sweep(lsp_ctx* c, int depth) {
   if (lv.s == 0) return cudaSuccess;
   int t = timer_begin(c, level_name("nd_sweep", depth));
   if (lv.f <= kNdSmallFront) {
-    const size_t smem = sizeof(double) * ((size_t)lv.f * lv.f + 2 * lv.f);
-    cudaError_t e = cudaFuncSetAttribute(k_nd_sweep_small,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const size_t smem = sizeof(double) * ((size_t)lv.f * lv.f + 3 * lv.f);
+    auto kern = lv.f <= 32   ? k_nd_sweep_small<1>
+                : lv.f <= 64 ? k_nd_sweep_small<2>
+                : lv.f <= 96 ? k_nd_sweep_small<3>
+                : lv.f <= 128 ? k_nd_sweep_small<4> : k_nd_sweep_small<5>;
+    cudaError_t e =
+        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    k_nd_sweep_small<<<lv.count, 256, smem, c->stream>>>(F, lv.f, lv.s, perm, err);
+    // from 113 rows on a front has the SM's shared memory to itself
+    kern<<<lv.count, lv.f > 112 ? 512 : 256, smem, c->stream>>>(F, lv.f, lv.s, perm, err);
     timer_end(c, t);
     return cudaGetLastError();
   }

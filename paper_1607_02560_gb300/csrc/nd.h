@@ -34,7 +34,7 @@ namespace lsp {
 
 constexpr int kNdStep = 64;        // pivots per step of the blocked path
 constexpr int kNdPanel = 16;       // pivots chosen at once within a step
-constexpr int kNdSwapInts = 1 + 4 * kNdPanel;  // a panel's row exchanges: count, dst, src
+constexpr int kNdSwapInts = 1 + 2 * kNdPanel;  // a panel's row exchanges: count, positions
 constexpr int kNdSmallFront = 160; // fronts with f <= this are swept in shared memory
 constexpr int kNdErrWait = 1 << 16; // err bit: a wait of k_nd_gemm gave up
 constexpr int kNdMaxN = 1024;      // 2D: the cross has 2n - 1 points
