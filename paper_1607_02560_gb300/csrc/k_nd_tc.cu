@@ -23,11 +23,11 @@
 // of the largest of their row and column are not rounded at all by the split. With digits for
 // 55 bits the solution lost a digit in 3D, where rows and columns decay.
 //
-// What bounds it: per 128 x 64 tile 112 products of 128 x 64 x 16 (about 60 cycles each with both
-// operands in shared memory), then about 80 integer operations and one FP64 addition per entry to
-// take the sums out, against 262e3 cycles of the FP64 pipe.
+// What bounds it: per 128 x 64 tile 224 products of 128 x 32 x 16 (47 cycles each with both operands
+// in shared memory) beside about 80 integer operations and one FP64 addition per entry to take the
+// sums out: 14e3 cycles, against 262e3 of the FP64 pipe.
 // Measured against rank-16 updates of the whole front on the FP64 pipe: the updates of 3D n = 32
-// about 100 -> 8 ms, the whole factorisation 118 -> 25 ms, of 2D n = 512 28.4 -> 15.1 ms; the
+// about 100 -> 6 ms, the whole factorisation 118 -> 23 ms, of 2D n = 512 28.4 -> 13.4 ms; the
 // unrefined backward error is smaller (3D) or equal (2D).
 #include <cuda_fp16.h>
 #include <math.h>
@@ -46,13 +46,16 @@ constexpr int kTileJ = 128, kTileI = 64;  // columns (tensor-memory lanes) x row
 constexpr int kBytesW = kTileJ * SB * 2, kBytesU = kTileI * SB * 2;  // one digit of a tile
 constexpr int kExpNone = -100000, kExpBad = 1000000;  // all zero; Inf or NaN inside
 
-__device__ __forceinline__ void chain_start() {  // one kernel of a chain launched to overlap
+// One kernel of a chain launched to overlap. What an earlier kernel of the chain writes is read
+// through plain pointers: a const __restrict__ one allows loads through the read-only path, whose
+// lines may date from before the wait.
+__device__ __forceinline__ void chain_start() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
 // Position, before the step, of the row that is at position x now (only positions in [k0, s) move).
-__device__ __forceinline__ int row_id(const int32_t* __restrict__ cu, int x, int k0, int s) {
+__device__ __forceinline__ int row_id(const int32_t* cu, int x, int k0, int s) {
   return x >= k0 && x < s ? cu[x] : x;
 }
 
@@ -65,10 +68,10 @@ __device__ __forceinline__ int row_id(const int32_t* __restrict__ cu, int x, int
 constexpr int kSubRows = 8;
 __global__ void __launch_bounds__(128) k_nd_sub(double* __restrict__ fronts, int f, int s, int k,
                                                 int nb, int k0, int sb,
-                                                const double* __restrict__ xrow,
-                                                const double* __restrict__ pinv,
-                                                const int32_t* __restrict__ swaps,
-                                                const int32_t* __restrict__ cur,
+                                                const double* xrow,
+                                                const double* pinv,
+                                                const int32_t* swaps,
+                                                const int32_t* cur,
                                                 double* __restrict__ vst) {
   __shared__ double C[kSubRows][SB + 1], W[NP][SB], V[kSubRows][NP + 1], pi[NP][NP];
   __shared__ int from[kSubRows];  // index in xrow, or -1: the row is where it was
@@ -185,8 +188,8 @@ __device__ __forceinline__ void store_digits(const double (&v)[8], int e, uint8_
 // overwrites).
 constexpr int kSplitCols = 8;
 __global__ void __launch_bounds__(128) k_nd_wsplit(double* __restrict__ fronts, int f, int s, int k0,
-                                                   int sb, int nj, const int32_t* __restrict__ cur,
-                                                   const double* __restrict__ vst,
+                                                   int sb, int nj, const int32_t* cur,
+                                                   const double* vst,
                                                    uint8_t* __restrict__ digits,
                                                    int32_t* __restrict__ expo) {
   __shared__ double W[SB][kSplitCols + 1], L[SB - NP][SB - NP + 1];  // L[a - 16][c] = V_p[row a]
@@ -265,8 +268,8 @@ __global__ void __launch_bounds__(128) k_nd_wsplit(double* __restrict__ fronts, 
 
 // V: 64 rows per block, four threads per row (one per sub-step).
 __global__ void __launch_bounds__(256) k_nd_vsplit(int f, int s, int k0, int sb,
-                                                   const int32_t* __restrict__ cur,
-                                                   const double* __restrict__ vst,
+                                                   const int32_t* cur,
+                                                   const double* vst,
                                                    uint8_t* __restrict__ digits,
                                                    int32_t* __restrict__ expo) {
   chain_start();
@@ -295,13 +298,11 @@ __global__ void __launch_bounds__(256) k_nd_vsplit(int f, int s, int k0, int sb,
   if (part == 0 && i < f) expo[fid * f + i] = e;
 }
 
-// 8 consecutive FP32 columns of this thread's tensor-memory lane, without waiting.
-__device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t (&r)[8]) {
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
-        "=r"(r[7])
-      : "r"(taddr));
+// 4 consecutive FP32 columns of this thread's tensor-memory lane, without waiting.
+__device__ __forceinline__ void tmem_ld4(uint32_t taddr, uint32_t (&r)[4]) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+               : "r"(taddr));
 }
 
 // sum_l a[l] 2^(-9 l) times 2^ex as a double, |a[l]| < 2^25 integers: put together exactly as one
@@ -343,30 +344,35 @@ __device__ __forceinline__ double sum_of(const int (&a)[kLevels], int ex) {
 
 // The update. One block per SM takes a run of the 128 x 64 tiles (columns j x rows i) of all fronts,
 // rows fastest: the seven W digit tiles stay in shared memory while the columns stay the same, the
-// V digit tiles have two buffers. One thread of the last warp copies the tiles and issues the 28
-// digit products, weight l = t + t' into accumulator columns 64 l (unrolled, descriptors by one
-// addition: a loop took 109 cycles a product to issue, this takes 57). The other sixteen warps take
-// the sums out, 16 rows each in two groups; the accumulators are free for the next tile once the
-// second group is in registers. Cycles a tile: products 6.4e3, sums 9.8e3; with one after the other
-// and the copies exposed the updates of 3D n = 32 took 10.4 ms, with the overlap 7.8 ms.
+// V digit tiles have two buffers. The last warp copies the tiles and issues the 28 digit products
+// of one half of the rows at a time, weight l = t + t' into accumulator columns 256 half + 32 l
+// (unrolled, descriptors by one addition: a loop took 109 cycles a product to issue; from one lane
+// of a branch, without uniform registers, 57 to 79). The other sixteen warps take the sums of one
+// half out (8 rows each, the entries to update loaded a half ahead) while the products of the other
+// run. Cycles a half: products 5.3e3 (47 each: shared-memory reads of the operands), sums 4e3 and
+// 2e3 of loads; the two sides meet at about 7e3. The products one after the other with the sums,
+// 64 rows at a time: 25e3 a tile.
 constexpr int kSumWarps = 16, kGemmThreads = 32 * (kSumWarps + 1);
+constexpr int kHalf = kTileI / 2, kWarpRows = kHalf / (kSumWarps / 4);
 constexpr size_t kGemmSmem = (size_t)kDigits * (kBytesW + 2 * kBytesU);
 __global__ void __launch_bounds__(kGemmThreads, 1) k_nd_gemm(
-    double* __restrict__ fronts, int f, int k0, int sb, int64_t total,
-    const uint8_t* __restrict__ dW, const int32_t* __restrict__ eW,
-    const uint8_t* __restrict__ dV, const int32_t* __restrict__ eV, int32_t* __restrict__ err) {
+    double* __restrict__ fronts, int f, int k0, int sb, int64_t total, const uint8_t* dW,
+    const int32_t* eW, const uint8_t* dV, const int32_t* eV, int32_t* __restrict__ err) {
   extern __shared__ __align__(1024) uint8_t smem[];
-  __shared__ __align__(8) uint64_t bar_w, bar_v[2], bar_mma, bar_free;
+  __shared__ __align__(8) uint64_t bar_w, bar_v[2], bar_mma[2], bar_free[2];
   __shared__ uint32_t tslot;
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
   const int ni = (f + kTileI - 1) / kTileI, nj = (f + kTileJ - 1) / kTileJ;
   const int64_t g0 = total * blockIdx.x / gridDim.x, g1 = total * (blockIdx.x + 1) / gridDim.x;
+  const int nt = (int)(g1 - g0);
   if (tid == 0) {
     tc::mbar_init(&bar_w, 1);
-    tc::mbar_init(&bar_v[0], 1);
-    tc::mbar_init(&bar_v[1], 1);
-    tc::mbar_init(&bar_mma, 1);
-    tc::mbar_init(&bar_free, kSumWarps);
+    for (int h = 0; h < 2; ++h) {
+      tc::mbar_init(&bar_v[h], 1);
+      tc::mbar_init(&bar_mma[h], 1);
+      tc::mbar_init(&bar_free[h], kSumWarps);
+    }
   }
   if (warp == 0) tc::tmem_alloc(&tslot, 512);
   tc::fence_before();
@@ -374,130 +380,170 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_nd_gemm(
   tc::fence_after();
   const uint32_t tmem = tslot;
   chain_start();
+  // a tile's place: row tile, column tile, front
+  int ti = (int)(g0 % ni), tj = (int)(g0 / ni % nj);
+  int64_t fid = g0 / ni / nj;
+  auto advance = [&]() {
+    if (++ti == ni) {
+      ti = 0;
+      if (++tj == nj) {
+        tj = 0;
+        ++fid;
+      }
+    }
+  };
   if (warp == kSumWarps) {
-    if (lane == 0 && g0 < g1) {
+    if (nt > 0) {
       uint8_t* sW = smem;
       uint8_t* sV = smem + kDigits * kBytesW;
-      int loads_w = 0, loads_v = 0, tiles = 0;
-      auto load_w = [&](int64_t grp) {
-        tc::mbar_expect_tx(&bar_w, kDigits * kBytesW);
-        tc::bulk_g2s(sW, dW + grp * (kDigits * kBytesW), kDigits * kBytesW, &bar_w);
+      int loads_w = 0, loads_v = 0, sets = 0;
+      auto load_w = [&]() {
+        if (lane == 0) {
+          tc::mbar_expect_tx(&bar_w, kDigits * kBytesW);
+          tc::bulk_g2s(sW, dW + (fid * nj + tj) * (kDigits * kBytesW), kDigits * kBytesW, &bar_w);
+        }
+        __syncwarp();
         ++loads_w;
       };
-      auto load_v = [&](int64_t g) {
+      auto load_v = [&]() {
         const int b = loads_v++ & 1;
-        tc::mbar_expect_tx(&bar_v[b], kDigits * kBytesU);
-        tc::bulk_g2s(sV + b * (kDigits * kBytesU),
-                     dV + (g / ni / nj * ni + g % ni) * (kDigits * kBytesU), kDigits * kBytesU,
-                     &bar_v[b]);
+        if (lane == 0) {
+          tc::mbar_expect_tx(&bar_v[b], kDigits * kBytesU);
+          tc::bulk_g2s(sV + b * (kDigits * kBytesU), dV + (fid * ni + ti) * (kDigits * kBytesU),
+                       kDigits * kBytesU, &bar_v[b]);
+        }
+        __syncwarp();
+      };
+      auto wait = [&](uint64_t* bar, uint32_t phase) {  // every lane asks
+        return __all_sync(0xffffffffu, tc::mbar_wait(bar, phase, err, kNdErrWait)) != 0;
       };
       const int ksteps = (sb + 15) / 16;
       constexpr uint32_t sbo = (SB / 8) * 128;
-      constexpr uint32_t idesc = tc::idesc_f16(kTileJ, kTileI);
+      constexpr uint32_t idesc = tc::idesc_f16(kTileJ, kHalf);
       const uint64_t da = tc::desc_kmajor(tc::smem_u32(sW), 128, sbo);
-      load_w(g0 / ni);
-      load_v(g0);
+      load_w();
+      load_v();
       bool ok = true;
-      for (int64_t g = g0; ok && g < g1; ++g) {
-        const int t = (int)(g - g0);
-        // the sums of the tile before are out, so its products have completed
-        if (t > 0) ok = tc::mbar_wait(&bar_free, (uint32_t)(t - 1) & 1u, err, kNdErrWait);
-        if (!ok) break;
-        if (t > 0 && g % ni == 0) load_w(g / ni);
-        if (g + 1 < g1) load_v(g + 1);
-        // (a phase of W passed already returns at once)
-        ok = tc::mbar_wait(&bar_w, (uint32_t)(loads_w - 1) & 1u, err, kNdErrWait) &&
-             tc::mbar_wait(&bar_v[t & 1], (uint32_t)(t >> 1) & 1u, err, kNdErrWait);
-        if (!ok) break;
-        tc::fence_after();
-        const uint64_t db =
+      for (int t = 0; ok && t < nt; ++t) {
+        const uint64_t dv =
             tc::desc_kmajor(tc::smem_u32(sV + (t & 1) * (kDigits * kBytesU)), 128, sbo);
-        if (ksteps == SB / 16) {
+        const uint32_t before = (uint32_t)(t - 1) & 1u;  // the tile before's phase of bar_free
+        for (int h = 0; ok && h < 2; ++h) {
+          // once the sums of the half before in these accumulators are out, its products are done
+          if (t > 0) ok = wait(&bar_free[h], before);
+          if (h == 0) {
+            if (ok && t > 0 && ti == 0) {  // other columns: all products on W must be done
+              ok = wait(&bar_free[1], before);
+              if (ok) load_w();
+            }
+            // (a phase of W passed already returns at once)
+            ok = ok && wait(&bar_w, (uint32_t)(loads_w - 1) & 1u) &&
+                 wait(&bar_v[t & 1], (uint32_t)(t >> 1) & 1u);
+          }
+          if (!ok) break;
+          if (h == 1) {  // the tile before is done with the other V buffer
+            advance();
+            if (t + 1 < nt) load_v();
+          }
+          tc::fence_after();
+          const uint64_t db = dv + (uint64_t)(h * (kHalf / 8) * sbo / 16);
+          const uint32_t acc = tmem + (uint32_t)(h * 256);
+          if (ksteps == SB / 16) {
 #pragma unroll
-          for (int a = 0; a < kDigits; ++a)
+            for (int a = 0; a < kDigits; ++a)
 #pragma unroll
-            for (int b = 0; a + b < kLevels; ++b)
+              for (int b = 0; a + b < kLevels; ++b)
 #pragma unroll
-              for (int q = 0; q < SB / 16; ++q)
-                tc::mma_bf16(tmem + (uint32_t)((a + b) * kTileI),
-                             da + (uint64_t)(a * kBytesW / 16 + 16 * q),
-                             db + (uint64_t)(b * kBytesU / 16 + 16 * q), idesc,
-                             (a > 0 || q > 0) ? 1u : 0u);
-        } else {
-          for (int a = 0; a < kDigits; ++a)
-            for (int b = 0; a + b < kLevels; ++b)
-              for (int q = 0; q < ksteps; ++q)
-                tc::mma_bf16(tmem + (uint32_t)((a + b) * kTileI),
-                             da + (uint64_t)(a * kBytesW / 16 + 16 * q),
-                             db + (uint64_t)(b * kBytesU / 16 + 16 * q), idesc,
-                             (a > 0 || q > 0) ? 1u : 0u);
+                for (int q = 0; q < SB / 16; ++q)
+                  tc::mma_bf16_warp(acc + (uint32_t)((a + b) * kHalf),
+                                    da + (uint64_t)(a * kBytesW / 16 + 16 * q),
+                                    db + (uint64_t)(b * kBytesU / 16 + 16 * q), idesc,
+                                    (a > 0 || q > 0) ? 1u : 0u);
+          } else {
+            for (int a = 0; a < kDigits; ++a)
+              for (int b = 0; a + b < kLevels; ++b)
+                for (int q = 0; q < ksteps; ++q)
+                  tc::mma_bf16_warp(acc + (uint32_t)((a + b) * kHalf),
+                                    da + (uint64_t)(a * kBytesW / 16 + 16 * q),
+                                    db + (uint64_t)(b * kBytesU / 16 + 16 * q), idesc,
+                                    (a > 0 || q > 0) ? 1u : 0u);
+          }
+          tc::commit_warp(&bar_mma[h]);
+          ++sets;
         }
-        tc::commit(&bar_mma);
-        ++tiles;
       }
       // before leaving (after a wait that gave up as well): copies and products in flight
       tc::mbar_wait(&bar_w, (uint32_t)(loads_w - 1) & 1u, err, 0);
       for (int b = 0; b < 2; ++b) {
         const int uses = loads_v / 2 + (b < loads_v % 2 ? 1 : 0);
         if (uses) tc::mbar_wait(&bar_v[b], (uint32_t)(uses - 1) & 1u, err, 0);
+        const int n = sets / 2 + (b < sets % 2 ? 1 : 0);
+        if (n) tc::mbar_wait(&bar_mma[b], (uint32_t)(n - 1) & 1u, err, 0);
       }
-      if (tiles) tc::mbar_wait(&bar_mma, (uint32_t)(tiles - 1) & 1u, err, 0);
     }
-  } else {
-    // rows below zlo and from zhi on keep their entry: the pivot rows of sub-steps after the
-    // column's own (all of K for a column outside K) are replaced
-    const int zhi = k0 + sb;
-    bool ok = true;
-    for (int64_t g = g0; ok && g < g1; ++g) {
-      const int64_t grp = g / ni, fid = grp / nj;
-      const int j = (int)(grp % nj) * kTileJ + (warp & 3) * 32 + lane;
-      const int ib = (int)(g % ni) * kTileI + (warp >> 2) * 16;
+  } else if (nt > 0) {
+    const int zhi = k0 + sb, cj = (warp & 3) * 32 + lane, ci = (warp >> 2) * kWarpRows;
+    // Entries to update of half h of the tile (ti, tj, fid), and its exponents. Rows below zlo and
+    // from zhi on keep their entry: the pivot rows of sub-steps after the column's own (all of K
+    // for a column outside K) are replaced.
+    double old[kWarpRows], nxt[kWarpRows];
+    int ej = 0, er = 0;  // exponent of the column; of row lane % 8
+    auto fetch = [&](int h, double (&o)[kWarpRows], int& ec, int& ex) {
+      const int j = tj * kTileJ + cj, ib = ti * kTileI + h * kHalf + ci;
       const bool jl = j < f;
-      const int ej = (jl ? eW[fid * f + j] : kExpNone) - 16;
-      const int32_t* er = eV + fid * f;
-      double* Fj = fronts + fid * f * f + (jl ? j : 0);
       const int zlo = jl && j >= k0 && j < zhi ? k0 + ((j - k0) / NP + 1) * NP : k0;
-      double old[8];
-      auto fetch = [&](int c0) {
+      const double* Fj = fronts + (fid * f + ib) * f + j;
 #pragma unroll
-        for (int q = 0; q < 8; ++q) {
-          const int i = ib + c0 + q;
-          old[q] = jl && i < f && (i < zlo || i >= zhi) ? Fj[(int64_t)i * f] : 0.0;
-        }
-      };
-      fetch(0);
+      for (int q = 0; q < kWarpRows; ++q) {
+        const int i = ib + q;
+        o[q] = jl && i < f && (i < zlo || i >= zhi) ? Fj[(int64_t)q * f] : 0.0;
+      }
+      ec = jl ? eW[fid * f + j] : kExpNone;
+      ex = ib + (lane & 7) < f ? eV[fid * f + ib + (lane & 7)] : kExpNone;
+    };
+    const uint32_t taddr = tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)ci;
+    bool ok = true;
+    fetch(0, old, ej, er);
+    for (int u = 0; u < 2 * nt; ++u) {
+      const int h = u & 1, j = tj * kTileJ + cj, ib = ti * kTileI + h * kHalf + ci;
+      double* Fj = fronts + (fid * f + ib) * f + j;
+      const int rows = j < f ? f - ib : 0;  // that exist
       // (one lane asks, the others follow its answer)
       const bool got =
-          lane == 0 ? tc::mbar_wait(&bar_mma, (uint32_t)(g - g0) & 1u, err, kNdErrWait) : true;
+          lane == 0 ? tc::mbar_wait(&bar_mma[h], (uint32_t)(u >> 1) & 1u, err, kNdErrWait) : true;
       ok = __all_sync(0xffffffffu, got);
       if (!ok) break;
       tc::fence_after();
-      const uint32_t taddr =
-          tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)((warp >> 2) * 16);
+      int ejn = 0, ern = 0;
 #pragma unroll
-      for (int c0 = 0; c0 < 16; c0 += 8) {
-        uint32_t r[kLevels][8];
+      for (int c0 = 0; c0 < kWarpRows; c0 += 4) {
+        uint32_t r[kLevels][4];
 #pragma unroll
-        for (int l = 0; l < kLevels; ++l) tmem_ld8(taddr + (uint32_t)(l * kTileI + c0), r[l]);
-        if (c0) fetch(c0);
+        for (int l = 0; l < kLevels; ++l)
+          tmem_ld4(taddr + (uint32_t)(h * 256 + l * kHalf + c0), r[l]);
+        if (c0 == 0) {
+          if (h == 1) advance();
+          if (u + 1 < 2 * nt) fetch(h ^ 1, nxt, ejn, ern);
+        }
         tc::ld_wait();
-        if (c0) {
+        if (c0 + 4 == kWarpRows) {
           tc::fence_before();
           __syncwarp();
-          if (lane == 0) tc::mbar_arrive(&bar_free);
+          if (lane == 0) tc::mbar_arrive(&bar_free[h]);
         }
 #pragma unroll
-        for (int q = 0; q < 8; ++q) {
+        for (int q = 0; q < 4; ++q) {
           int a[kLevels];
 #pragma unroll
           for (int l = 0; l < kLevels; ++l) a[l] = __float2int_rn(__uint_as_float(r[l][q]));
-          const int i = ib + c0 + q;
-          if (i < f) {
-            const double v = sum_of(a, er[i] + ej);
-            if (jl) Fj[(int64_t)i * f] = old[q] + v;
-          }
+          const double v = sum_of(a, __shfl_sync(0xffffffffu, er, c0 + q) + ej - 16);
+          if (c0 + q < rows) Fj[(int64_t)(c0 + q) * f] = old[c0 + q] + v;
         }
       }
+#pragma unroll
+      for (int q = 0; q < kWarpRows; ++q) old[q] = nxt[q];
+      ej = ejn;
+      er = ern;
     }
   }
   tc::fence_before();
