@@ -26,6 +26,7 @@
 #include <string>
 #include <vector>
 
+#include "snap.cuh"
 #include "lsp_internal.h"
 #include "tc_common.cuh"
 
@@ -123,14 +124,6 @@ ChunkPlan plan_for(const Dims& m) {
   }
   p.total_bytes = off;
   return p;
-}
-
-__device__ __forceinline__ int64_t snap_m(double x) {
-  const double yf = fma(x, kQuarterInvPi2, -0.5);
-  const double r = rint(yf);
-  if (0.5 - fabs(yf - r) > 1e-14 * fabs(yf) + 1e-14) return (int64_t)r;
-  const double y = __dmul_rn(__dsub_rn(__ddiv_rn(x, kPi2), 2.0), 0.25);
-  return (int64_t)round(y);
 }
 
 // Linear index of j + o (periodic) for an offset o with components in [-R, R], given as
@@ -1372,7 +1365,7 @@ __global__ void k_point_features(const double* __restrict__ v, int64_t N, float 
     const double s = __dmul_rn((double)(4 * snap_m(x) + 2), kPi2);
     const float sf = (float)s;
     xb[j] = __float2bfloat16((xf * h2f - mu_x) * isig_x);
-    sb[j] = __float2bfloat16(((float)(s * (double)h2f) - mu_x) * isig_x);
+    sb[j] = __float2bfloat16((sf * h2f - mu_x) * isig_x);  // h^2 is a power of two
     vh[j] = xf;
     vl[j] = (float)(x - (double)xf);
     sh[j] = sf;

@@ -8,21 +8,13 @@
 // 256 consecutive points, whose rows form one contiguous span of every output array, so
 // consecutive threads store consecutive doubles (fully coalesced, streaming stores).
 #include "lsp_internal.h"
+#include "snap.cuh"
 
 namespace lsp {
 namespace {
 
 constexpr int kThreads = 256;
 
-__device__ __forceinline__ int64_t snap_m(double x) {
-  // Fast path: fma(x, 1/(4 pi^2), -1/2) is within a few ulp of the exact (x/pi^2 - 2)/4, so
-  // its nearest integer is the exact one unless it lies next to a half-integer.
-  const double yf = fma(x, kQuarterInvPi2, -0.5);
-  const double r = rint(yf);
-  if (0.5 - fabs(yf - r) > 1e-14 * fabs(yf) + 1e-14) return (int64_t)r;
-  const double y = __dmul_rn(__dsub_rn(__ddiv_rn(x, kPi2), 2.0), 0.25);
-  return (int64_t)round(y);
-}
 __device__ __forceinline__ double shift_of(int64_t m) { return lattice_shift(m); }
 
 // Index in the sorted list S (given by lattice indices) of the shift nearest to x; ties go to

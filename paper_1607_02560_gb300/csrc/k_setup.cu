@@ -7,6 +7,7 @@
 #include <float.h>
 
 #include "lsp_internal.h"
+#include "snap.cuh"
 
 namespace lsp {
 namespace {
@@ -14,152 +15,113 @@ namespace {
 constexpr int kThreads = 256;
 constexpr int kTileFlags = kThreads * 16;  // flags per compaction tile (one uint4 per thread)
 
-__device__ __forceinline__ double warp_min(double x) {
-  for (int o = 16; o > 0; o >>= 1) x = fmin(x, __shfl_xor_sync(0xffffffffu, x, o));
-  return x;
+// ---- potential statistics ----
+// Minimum and maximum as order-preserving 64-bit integers, reduced by warp instructions on their
+// halves; the sum is the only FP64 operation. The FP64 pipe is narrow and its latency long: with
+// FP64 shuffles for all four the reductions alone took about 5 us of a launch.
+constexpr int kStatThreads = 1024, kStatLoads = 4;
+
+__device__ __forceinline__ unsigned long long order_key(double x) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+  return b ^ ((unsigned long long)((long long)b >> 63) | (1ULL << 63));
 }
-__device__ __forceinline__ double warp_max(double x) {
-  for (int o = 16; o > 0; o >>= 1) x = fmax(x, __shfl_xor_sync(0xffffffffu, x, o));
-  return x;
+__device__ __forceinline__ double key_value(unsigned long long k) {
+  return __longlong_as_double((long long)(k ^ (k >> 63 ? 1ULL << 63 : ~0ULL)));
 }
-__device__ __forceinline__ double warp_sum(double x) {
-  for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-  return x;
+__device__ __forceinline__ unsigned long long warp_max_key(unsigned long long k) {
+  const unsigned hi = __reduce_max_sync(0xffffffffu, (unsigned)(k >> 32));
+  const unsigned lo =
+      __reduce_max_sync(0xffffffffu, (unsigned)(k >> 32) == hi ? (unsigned)k : 0u);
+  return ((unsigned long long)hi << 32) | lo;
 }
 
-// Per-block partial min / max / sum / count of non-finite values, 4 doubles per block. With
-// vcopy, v is also stored there (v read from page-locked host memory over the host link, so
-// the upload and the statistics take one pass and no copy engine).
-__device__ void stats_partial(const double* __restrict__ v, int64_t N, double* __restrict__ part,
-                              double* __restrict__ vcopy) {
-  double mn = DBL_MAX, mx = -DBL_MAX, sm = 0.0, bad = 0.0;
-  for (int64_t j = (int64_t)blockIdx.x * kThreads + threadIdx.x; j < N;
-       j += (int64_t)gridDim.x * kThreads) {
-    const double x = v[j];
-    if (vcopy) vcopy[j] = x;
-    if (!isfinite(x)) {
-      bad += 1.0;
-      continue;
-    }
-    mn = fmin(mn, x);
-    mx = fmax(mx, x);
-    sm += x;
-  }
-  __shared__ double red[4][kThreads / 32];
-  mn = warp_min(mn);
-  mx = warp_max(mx);
-  sm = warp_sum(sm);
-  bad = warp_sum(bad);
-  int w = threadIdx.x >> 5, l = threadIdx.x & 31;
-  if (l == 0) {
-    red[0][w] = mn;
-    red[1][w] = mx;
-    red[2][w] = sm;
-    red[3][w] = bad;
-  }
+struct Stats {
+  unsigned long long mn, mx;  // keys
+  double sum;
+  unsigned bad;  // non-finite values
+};
+__device__ __forceinline__ Stats empty_stats() {
+  return {order_key(DBL_MAX), order_key(-DBL_MAX), 0.0, 0u};
+}
+__device__ __forceinline__ Stats warp_stats(Stats s) {
+  s.mn = ~warp_max_key(~s.mn);
+  s.mx = warp_max_key(s.mx);
+  s.bad = __reduce_add_sync(0xffffffffu, s.bad);
+  for (int o = 16; o > 0; o >>= 1) s.sum += __shfl_xor_sync(0xffffffffu, s.sum, o);
+  return s;
+}
+// Over the block; the result is valid in warp 0.
+__device__ __forceinline__ Stats block_stats(Stats s) {
+  __shared__ Stats red[kStatThreads / 32];
+  const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
+  s = warp_stats(s);
+  if (l == 0) red[w] = s;
   __syncthreads();
-  if (w == 0) {
-    mn = l < kThreads / 32 ? red[0][l] : DBL_MAX;
-    mx = l < kThreads / 32 ? red[1][l] : -DBL_MAX;
-    sm = l < kThreads / 32 ? red[2][l] : 0.0;
-    bad = l < kThreads / 32 ? red[3][l] : 0.0;
-    mn = warp_min(mn);
-    mx = warp_max(mx);
-    sm = warp_sum(sm);
-    bad = warp_sum(bad);
-    if (l == 0) {
-      part[4 * blockIdx.x + 0] = mn;
-      part[4 * blockIdx.x + 1] = mx;
-      part[4 * blockIdx.x + 2] = sm;
-      part[4 * blockIdx.x + 3] = bad;
-    }
-  }
+  if (w == 0) s = warp_stats(red[l]);  // 32 warps
+  return s;
 }
 
-// Reduces the partials to (min, max, sum, non-finite count) in out[0..3], and also in
-// host_out[0..3] (page-locked host memory, device address) when given, so that the host reads
-// them without a copy. The partials are taken in block order, so the sum does not depend on
-// which block finished last.
-__device__ void stats_final(const double* part, int nb, double* out, double* host_out) {
-  double mn = DBL_MAX, mx = -DBL_MAX, sm = 0.0, bad = 0.0;
-  for (int b = threadIdx.x; b < nb; b += kThreads) {
-    mn = fmin(mn, part[4 * b + 0]);
-    mx = fmax(mx, part[4 * b + 1]);
-    sm += part[4 * b + 2];
-    bad += part[4 * b + 3];
-  }
-  __shared__ double red[4][kThreads / 32];
-  mn = warp_min(mn);
-  mx = warp_max(mx);
-  sm = warp_sum(sm);
-  bad = warp_sum(bad);
-  int w = threadIdx.x >> 5, l = threadIdx.x & 31;
-  if (l == 0) {
-    red[0][w] = mn;
-    red[1][w] = mx;
-    red[2][w] = sm;
-    red[3][w] = bad;
-  }
-  __syncthreads();
-  if (w == 0) {
-    mn = l < kThreads / 32 ? red[0][l] : DBL_MAX;
-    mx = l < kThreads / 32 ? red[1][l] : -DBL_MAX;
-    sm = l < kThreads / 32 ? red[2][l] : 0.0;
-    bad = l < kThreads / 32 ? red[3][l] : 0.0;
-    mn = warp_min(mn);
-    mx = warp_max(mx);
-    sm = warp_sum(sm);
-    bad = warp_sum(bad);
-    if (l == 0) {
-      out[0] = mn;
-      out[1] = mx;
-      out[2] = sm;
-      out[3] = bad;
-      if (host_out) {
-        host_out[0] = mn;
-        host_out[1] = mx;
-        host_out[2] = sm;
-        host_out[3] = bad;
+// min, max, sum and count of non-finite values of v into out[0..3], and also into host_out[0..3]
+// (page-locked host memory, device address) when given, so that the host reads them without a copy.
+// With vcopy, v is also stored there (v read from page-locked host memory over the host link, so
+// the upload and the statistics take one pass and no copy engine). Every block writes its partial,
+// and the block that finishes last (a ticket counter, reset by that block for the next call)
+// reduces them, in block order, so the sum does not depend on which block that is.
+// Bound by the latency of two reductions; 2^20 points 24 -> 13 us (before: 256 threads a block with
+// one load in flight each), 2^10 points 12.7 -> 8.5 us.
+__global__ void __launch_bounds__(kStatThreads) k_stats(const double* __restrict__ v, int64_t N,
+                                                        Stats* part, double* __restrict__ vcopy,
+                                                        double* __restrict__ out,
+                                                        double* __restrict__ host_out,
+                                                        unsigned int* __restrict__ ticket) {
+  Stats s = empty_stats();
+  const int64_t step = (int64_t)gridDim.x * kStatThreads;
+  for (int64_t j0 = (int64_t)blockIdx.x * kStatThreads + threadIdx.x; j0 < N;
+       j0 += kStatLoads * step) {
+    double x[kStatLoads];
+#pragma unroll
+    for (int u = 0; u < kStatLoads; ++u) x[u] = j0 + u * step < N ? v[j0 + u * step] : 0.0;
+#pragma unroll
+    for (int u = 0; u < kStatLoads; ++u) {
+      if (j0 + u * step >= N) break;
+      if (vcopy) vcopy[j0 + u * step] = x[u];
+      if (((unsigned)__double2hiint(x[u]) & 0x7ff00000u) == 0x7ff00000u) {
+        ++s.bad;
+        continue;
       }
+      const unsigned long long k = order_key(x[u]);
+      s.mn = min(s.mn, k);
+      s.mx = max(s.mx, k);
+      s.sum += x[u];
     }
   }
-}
-
-// One launch: every block writes its partial, and the block that finishes last (a ticket
-// counter, reset by that block for the next call) reduces them all.
-__global__ void __launch_bounds__(kThreads) k_stats(const double* __restrict__ v, int64_t N,
-                                                    double* __restrict__ part,
-                                                    double* __restrict__ vcopy,
-                                                    double* __restrict__ out,
-                                                    double* __restrict__ host_out,
-                                                    unsigned int* __restrict__ ticket) {
-  stats_partial(v, N, part, vcopy);
-  __shared__ bool last;
-  __threadfence();  // this block's partial is visible before its ticket is taken
-  __syncthreads();
-  if (threadIdx.x == 0) last = atomicAdd(ticket, 1u) == gridDim.x - 1;
-  __syncthreads();
-  if (!last) return;
-  __threadfence();
-  stats_final(part, gridDim.x, out, host_out);
-  if (threadIdx.x == 0) *ticket = 0u;
-}
-
-// Lattice index of the resonance-free shift (4m+2) pi^2 nearest to x (Sec. 4.1); halves away
-// from zero. Explicit round-to-nearest intrinsics keep the decision identical to a plain
-// IEEE evaluation of (x / pi^2 - 2) / 4 (no contraction into fused operations).
-__device__ __forceinline__ int64_t snap_m(double x) {
-  // Fast path: fma(x, 1/(4 pi^2), -1/2) is within a few ulp of the exact (x/pi^2 - 2)/4, so
-  // its nearest integer is the exact one unless it lies next to a half-integer.
-  const double yf = fma(x, kQuarterInvPi2, -0.5);
-  const double r = rint(yf);
-  if (0.5 - fabs(yf - r) > 1e-14 * fabs(yf) + 1e-14) return (int64_t)r;
-  const double y = __dmul_rn(__dsub_rn(__ddiv_rn(x, kPi2), 2.0), 0.25);
-  return (int64_t)round(y);
+  s = block_stats(s);
+  if (gridDim.x > 1) {
+    __shared__ bool last;
+    if (threadIdx.x == 0) {
+      part[blockIdx.x] = s;
+      __threadfence();  // this block's partial is visible before its ticket is taken
+      last = atomicAdd(ticket, 1u) == gridDim.x - 1;
+    }
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    s = threadIdx.x < gridDim.x ? part[threadIdx.x] : empty_stats();
+    s = block_stats(s);
+    if (threadIdx.x == 0) *ticket = 0u;
+  }
+  if (threadIdx.x == 0) {
+    const double r[4] = {key_value(s.mn), key_value(s.mx), s.sum, (double)s.bad};
+    for (int q = 0; q < 4; ++q) out[q] = r[q];
+    if (host_out)
+      for (int q = 0; q < 4; ++q) host_out[q] = r[q];
+  }
 }
 
 // The host derived [mlo, mlo + R) from snap(v_min) and snap(v_max) with the same IEEE
-// operations; an index outside it would mean the two disagree, and is recorded in *err.
+// operations; an index outside it would mean the two disagree, and is recorded in *err. Bound by
+// the scattered byte stores (2^20 points, 31 us; a look at the flag before the store makes it
+// 117 us: the two halves of the L2 pass the written lines back and forth).
 __global__ void __launch_bounds__(kThreads) k_mark_local(const double* __restrict__ v, int64_t N,
                                                          int64_t mlo, int64_t R,
                                                          uint8_t* __restrict__ flag,
@@ -409,13 +371,20 @@ __global__ void __launch_bounds__(kThreads) k_copy_f64(const double* __restrict_
 
 }  // namespace
 
-cudaError_t launch_stats(lsp_ctx* c, int nblocks, const double* src) {
+// One load of every thread in flight per block and SM, and a single block (no ticket) for small grids.
+int stats_blocks(int64_t N) {
+  const int64_t b = (N + kStatThreads * kStatLoads - 1) / (kStatThreads * kStatLoads);
+  return (int)(b < 152 ? b : 152);
+}
+size_t stats_part_bytes(int64_t N) { return sizeof(Stats) * stats_blocks(N); }
+
+cudaError_t launch_stats(lsp_ctx* c, const double* src) {
   int t = timer_begin(c, "stats");
   double* vd = (double*)c->v.p;
   double* st = (double*)c->stats.p;
-  k_stats<<<nblocks, kThreads, 0, c->stream>>>(src, c->geo.N, (double*)c->stats_part.p,
-                                               src == vd ? nullptr : vd, st, c->h_stats_dev,
-                                               (unsigned int*)(st + 4));
+  k_stats<<<stats_blocks(c->geo.N), kStatThreads, 0, c->stream>>>(
+      src, c->geo.N, (Stats*)c->stats_part.p, src == vd ? nullptr : vd, st, c->h_stats_dev,
+      (unsigned int*)(st + 4));
   timer_end(c, t);
   return cudaGetLastError();
 }

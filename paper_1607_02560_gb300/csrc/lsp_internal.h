@@ -258,7 +258,8 @@ void timer_end(lsp_ctx* ctx, int slot);
 // src: c->v itself, or page-locked host memory (device address) that is copied into c->v
 // v_min, v_max, sum and the count of non-finite values of v in stats[0..3] (one launch; the
 // ticket of its last block lives in stats[4] and is zero between calls).
-cudaError_t launch_stats(lsp_ctx* c, int nblocks, const double* src);
+size_t stats_part_bytes(int64_t N);
+cudaError_t launch_stats(lsp_ctx* c, const double* src);
 // bytes / 4 words of p set to zero (bytes a multiple of 4, p 4-byte aligned)
 cudaError_t launch_zero(lsp_ctx* c, void* p, size_t bytes);
 // the same for up to three ranges in one launch
