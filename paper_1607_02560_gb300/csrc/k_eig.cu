@@ -15,6 +15,8 @@
 #include <float.h>
 #include <string.h>
 
+#include <algorithm>
+
 #include "lsp_internal.h"
 
 namespace lsp {
@@ -857,27 +859,31 @@ __global__ void __launch_bounds__(WARPS * 32) k_eig3d(const double* __restrict__
   }
 }
 
-// ---- 2D, t = 2: one warp per shift, blocks of mu_0^2 formed from the class values ----------
+// ---- 2D, t = 2: three warps per shift, blocks of mu_0^2 formed from the class values ----------
 // mu_0^2 is the 5 x 5 neighbourhood; its symmetry blocks (host-built basis, see build_sym_t2)
 // are A1 (6 x 6), E (6 x 6, two partners), B1 (3 x 3), B2 (3 x 3) and A2 (1 x 1). As in 3D,
 // G maps every block's span into itself, so B_b = U_b^T A1 U_b - G_b G_b with both terms linear
 // in the 15 class values through one coefficient table (55 entries). The 6 x 6 blocks are
-// solved one after the other on the whole warp as 8 x 8 matrices (two entries per lane, the
+// solved side by side on a warp each as 8 x 8 matrices (two entries per lane, the
 // padding decoupled on the diagonal above the block's spectrum): LDL^T of B + delta I column by
 // column, the inverse by lanes 0-7 (one column each), seven scaled squarings, Rayleigh quotient
 // and residual; the next eigenvalue from three squarings of the deflated inverse. The 3 x 3
-// blocks run side by side on the two half-warps (4 x 4 padded, as in 3D); A2 is 1 x 1.
-constexpr int kT2Ent = 55;
+// blocks run on the two halves of the third warp (4 x 4 padded, as in 3D); A2 is 1 x 1.
+// Bound by the latency of one block's chain: with the blocks one after the other on one warp 13
+// shifts took 85 us, now 44 us.
+constexpr int kT2Ent = 55, kT2Threads = 96;
 __constant__ double c_coef2[kT2Ent][kMaxCls];
 __constant__ int8_t c_ent2[kT2Ent][3];
 __constant__ SymBasis c_sym2;
 
-struct EigT2Warp {
+struct EigT2Scratch {  // of one 6 x 6 block
+  double L[64], dd[8], dinv[8];
+  double M[64], M0[64];
+};
+struct EigT2Shift {
   double g[2 * 15];
   double Gb[5][64];   // 8 x 8 padded blocks (row stride 8)
   double B[5][64];
-  double L[64], dd[8], dinv[8];
-  double M[64], M0[64];
   double M4[2][16];   // the two half-warps' 4 x 4 matrices
   double v[5][8];     // eigenvector (block coordinates) of each block's smallest eigenvalue
   double lam[5][2];
@@ -887,8 +893,8 @@ struct EigT2Warp {
 
 // Smallest eigenpair (and next eigenvalue) of the block b (dim <= 6) held in sm.B[b], on the
 // whole warp. Writes sm.v[b], sm.lam[b], sm.tr[b], sm.conv[b].
-__device__ void warp_block_eig8(EigT2Warp& sm, int b, int dim, int lane) {
-  const double* Bb = sm.B[b];
+__device__ void warp_block_eig8(EigT2Shift& sh, EigT2Scratch& sm, int b, int dim, int lane) {
+  const double* Bb = sh.B[b];
   const int r0 = lane >> 3, r1 = r0 + 4, cc = lane & 7;
   // scale and trace of the block
   double sc = fmax(fabs(Bb[r0 * 8 + cc]), fabs(Bb[r1 * 8 + cc]));
@@ -1018,18 +1024,17 @@ __device__ void warp_block_eig8(EigT2Warp& sm, int b, int dim, int lane) {
                    v2[4] != 0.0 || v2[5] != 0.0))
     lam2 = lam1;
   if (lane == 0) {
-    sm.lam[b][0] = lam1;
-    sm.lam[b][1] = lam2;
-    sm.tr[b] = tr;
-    sm.conv[b] = conv;
+    sh.lam[b][0] = lam1;
+    sh.lam[b][1] = lam2;
+    sh.tr[b] = tr;
+    sh.conv[b] = conv;
 #pragma unroll
-    for (int q = 0; q < 8; ++q) sm.v[b][q] = v1[q];
+    for (int q = 0; q < 8; ++q) sh.v[b][q] = v1[q];
   }
   __syncwarp();
 }
 
-template <int WARPS>
-__global__ void __launch_bounds__(WARPS * 32) k_eig2d_t2(const double* __restrict__ gvals,
+__global__ void __launch_bounds__(kT2Threads) k_eig2d_t2(const double* __restrict__ gvals,
                                                          int64_t cap,
                                                          const int32_t* __restrict__ count,
                                                          double* __restrict__ alpha_out,
@@ -1040,61 +1045,51 @@ __global__ void __launch_bounds__(WARPS * 32) k_eig2d_t2(const double* __restric
   __shared__ double s_coef[kT2Ent][NCLS];
   __shared__ double s_u[kMaxSymVec][MU];
   __shared__ int8_t s_ent[kT2Ent][3];
-  __shared__ EigT2Warp sw[WARPS];
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  for (int e = threadIdx.x; e < kT2Ent * NCLS; e += WARPS * 32)
+  __shared__ EigT2Shift sm;
+  __shared__ EigT2Scratch scratch[2];
+  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+  for (int e = threadIdx.x; e < kT2Ent * NCLS; e += kT2Threads)
     s_coef[e / NCLS][e % NCLS] = c_coef2[e / NCLS][e % NCLS];
-  for (int e = threadIdx.x; e < kMaxSymVec * MU; e += WARPS * 32)
+  for (int e = threadIdx.x; e < kMaxSymVec * MU; e += kT2Threads)
     s_u[e / MU][e % MU] = c_sym2.u[e / MU][e % MU];
-  for (int e = threadIdx.x; e < kT2Ent * 3; e += WARPS * 32) s_ent[e / 3][e % 3] = c_ent2[e / 3][e % 3];
+  for (int e = threadIdx.x; e < kT2Ent * 3; e += kT2Threads) s_ent[e / 3][e % 3] = c_ent2[e / 3][e % 3];
   __syncthreads();
-  EigT2Warp& sm = sw[w];
   const int64_t cnt = *count;
   const int h = lane >> 4, q = lane & 15, r = q >> 2, cc = q & 3;
-  for (int64_t i = (int64_t)blockIdx.x * WARPS + w; i < cnt; i += (int64_t)gridDim.x * WARPS) {
-    if (lane < 2 * NCLS) sm.g[lane] = gvals[(int64_t)lane * cap + i];
-    for (int e = lane; e < 5 * 64; e += 32) {
+  for (int64_t i = blockIdx.x; i < cnt; i += gridDim.x) {
+    if (tid < 2 * NCLS) sm.g[tid] = gvals[(int64_t)tid * cap + i];
+    for (int e = tid; e < 5 * 64; e += kT2Threads) {
       (&sm.Gb[0][0])[e] = 0.0;
       (&sm.B[0][0])[e] = 0.0;
     }
-    __syncwarp();
-    // ---- a4: G_b and U_b^T A1 U_b, then B_b = U_b^T A1 U_b - G_b G_b (entries e, e + 32) ----
-    double a1v[2] = {0.0, 0.0};
+    __syncthreads();
+    // ---- a4: G_b and U_b^T A1 U_b, then B_b = U_b^T A1 U_b - G_b G_b (entry tid) ----
+    const int eb = tid < kT2Ent ? s_ent[tid][0] : 0, ei = tid < kT2Ent ? s_ent[tid][1] : 0,
+              ej = tid < kT2Ent ? s_ent[tid][2] : 0;
+    double a1v = 0.0;
+    if (tid < kT2Ent) {
+      double gg = 0.0;
 #pragma unroll
-    for (int pass = 0; pass < 2; ++pass) {
-      const int e = lane + 32 * pass;
-      if (e < kT2Ent) {
-        const int eb = s_ent[e][0], ei = s_ent[e][1], ej = s_ent[e][2];
-        double gg = 0.0, aa = 0.0;
-#pragma unroll
-        for (int k = 0; k < NCLS; ++k) {
-          gg = fma(s_coef[e][k], sm.g[2 * k], gg);
-          aa = fma(s_coef[e][k], sm.g[2 * k + 1], aa);
-        }
-        sm.Gb[eb][ei * 8 + ej] = gg;
-        sm.Gb[eb][ej * 8 + ei] = gg;
-        a1v[pass] = aa;
+      for (int k = 0; k < NCLS; ++k) {
+        gg = fma(s_coef[tid][k], sm.g[2 * k], gg);
+        a1v = fma(s_coef[tid][k], sm.g[2 * k + 1], a1v);
       }
+      sm.Gb[eb][ei * 8 + ej] = gg;
+      sm.Gb[eb][ej * 8 + ei] = gg;
     }
-    __syncwarp();
+    __syncthreads();
+    if (tid < kT2Ent) {
 #pragma unroll
-    for (int pass = 0; pass < 2; ++pass) {
-      const int e = lane + 32 * pass;
-      if (e < kT2Ent) {
-        const int eb = s_ent[e][0], ei = s_ent[e][1], ej = s_ent[e][2];
-        double sv = a1v[pass];
-#pragma unroll
-        for (int k = 0; k < 8; ++k) sv = fma(-sm.Gb[eb][ei * 8 + k], sm.Gb[eb][k * 8 + ej], sv);
-        sm.B[eb][ei * 8 + ej] = sv;
-        sm.B[eb][ej * 8 + ei] = sv;
-      }
+      for (int k = 0; k < 8; ++k) a1v = fma(-sm.Gb[eb][ei * 8 + k], sm.Gb[eb][k * 8 + ej], a1v);
+      sm.B[eb][ei * 8 + ej] = a1v;
+      sm.B[eb][ej * 8 + ei] = a1v;
     }
-    __syncwarp();
-    // ---- a5: the two 6 x 6 blocks (A1, E) on the whole warp ----
-    warp_block_eig8(sm, 0, 6, lane);
-    warp_block_eig8(sm, 1, 6, lane);
-    // ---- the 3 x 3 blocks (B1, B2) on the two half-warps, padded to 4 x 4 ----
-    {
+    __syncthreads();
+    // ---- a5: the two 6 x 6 blocks (A1, E) on a warp each; the 3 x 3 blocks (B1, B2) on the two
+    // halves of the third, padded to 4 x 4 ----
+    if (w < 2) {
+      warp_block_eig8(sm, scratch[w], w, 6, lane);
+    } else {
       const int bb = 2 + h;
       double b4[4][4], scale = 0.0, tr = 0.0;
 #pragma unroll
@@ -1192,7 +1187,7 @@ __global__ void __launch_bounds__(WARPS * 32) k_eig2d_t2(const double* __restric
       }
     }
     // ---- A2 (1 x 1) ----
-    if (lane == 0) {
+    if (tid == 64) {
       sm.lam[4][0] = sm.B[4][0];
       sm.lam[4][1] = DBL_MAX;
       sm.tr[4] = sm.B[4][0];
@@ -1200,8 +1195,12 @@ __global__ void __launch_bounds__(WARPS * 32) k_eig2d_t2(const double* __restric
 #pragma unroll
       for (int x = 0; x < 8; ++x) sm.v[4][x] = x == 0 ? 1.0 : 0.0;
     }
-    __syncwarp();
+    __syncthreads();
     // ---- fallback: cyclic Jacobi for a block whose residual check failed (one lane each) ----
+    if (w > 0) {
+      __syncthreads();  // the next shift
+      continue;
+    }
     if (lane < 4 && !sm.conv[lane]) {
       const int dim = lane < 2 ? 6 : 3;
       double a[8][8], vv[8][8];
@@ -1278,7 +1277,7 @@ __global__ void __launch_bounds__(WARPS * 32) k_eig2d_t2(const double* __restric
       lam_out[2 * i + 1] = lam2;
       flags_out[i] = flags;
     }
-    __syncwarp();
+    __syncthreads();  // the next shift
   }
 }
 
@@ -1729,13 +1728,10 @@ cudaError_t upload_sym(lsp_ctx* c) {
   return cudaMemcpyToSymbol(c_B2f, B2f, sizeof B2f);
 }
 
-cudaError_t launch_eig_t2(lsp_ctx* c, const int32_t* count, int64_t cap) {
+cudaError_t launch_eig_t2(lsp_ctx* c, const int32_t* count, int64_t cap, cudaStream_t stream) {
   int t = timer_begin(c, "eig_t2");
-  constexpr int kW = 2;
-  int64_t b = (cap + kW - 1) / kW;
-  if (b > 152 * 8) b = 152 * 8;
-  if (b < 1) b = 1;
-  k_eig2d_t2<kW><<<(int)b, kW * 32, 0, c->stream>>>(
+  const int64_t b = std::min<int64_t>(std::max<int64_t>(cap, 1), 152 * 8);
+  k_eig2d_t2<<<(int)b, kT2Threads, 0, stream>>>(
       (const double*)c->gvals.p, cap, count, (double*)c->alpha2.p, (double*)c->cst2.p,
       (double*)c->lam2.p, (int32_t*)c->sflags2.p);
   timer_end(c, t);

@@ -496,12 +496,24 @@ lsp_status issue_build(lsp_ctx* c, const lsp_stencil_opts& o, int64_t cap_s, boo
   }
   // t = 1 stencils read the first classes of a t = 2 table (same row stride cap_s)
   // the eigen kernels also write ap = alpha - c s per shift for the P rows
+  // Both widths of a 2D t = 2 build with a leaf: their eigen kernels only read the class values,
+  // and for short lists each is one latency chain, so they run side by side.
+  const bool beside = o.t == 2 && o.nd_leaf > 0 && d == 2 && c->eig_stream && !c->timing;
+  if (beside) {
+    CUDA_OK(c, cudaEventRecord(c->ev_eig[0], c->stream));
+    CUDA_OK(c, cudaStreamWaitEvent(c->eig_stream, c->ev_eig[0], 0));
+    CUDA_OK(c, launch_eig_t2(c, counts + 0, cap_s, c->eig_stream));
+    CUDA_OK(c, cudaEventRecord(c->ev_eig[1], c->eig_stream));
+  }
+  cudaError_t e1 = cudaSuccess;
   if (o.t == 1 || o.nd_leaf > 0)
-    CUDA_OK(c, launch_eig(c, counts + 0, cap_s, o.eig_method, o.refine_steps, fp32));
+    e1 = launch_eig(c, counts + 0, cap_s, o.eig_method, o.refine_steps, fp32);
+  if (beside) CUDA_OK(c, cudaStreamWaitEvent(c->stream, c->ev_eig[1], 0));  // also when e1 failed
+  CUDA_OK(c, e1);
   if (o.t == 2) {
-    if (d == 2)
-      CUDA_OK(c, launch_eig_t2(c, counts + 0, cap_s));
-    else
+    if (d == 2 && !beside)
+      CUDA_OK(c, launch_eig_t2(c, counts + 0, cap_s, c->stream));
+    else if (d == 3)
       CUDA_OK(c, launch_eig_dense3(c, counts + 0, cap_s));
     CUDA_OK(c, launch_rows_t2(c, o.policy, counts + 0, o.nd_leaf));
   } else if (rows) {
@@ -659,6 +671,12 @@ lsp_status lsp_create(int d, int n, void* cuda_stream, lsp_ctx** out) {
 lsp_status lsp_destroy(lsp_ctx* c) {
   if (!c) return LSP_OK;
   cudaStreamSynchronize(c->stream);
+  if (c->eig_stream) {
+    cudaStreamSynchronize(c->eig_stream);
+    cudaStreamDestroy(c->eig_stream);
+  }
+  for (cudaEvent_t e : c->ev_eig)
+    if (e) cudaEventDestroy(e);
   if (c->copy_stream) {
     cudaStreamSynchronize(c->copy_stream);
     cudaStreamDestroy(c->copy_stream);
@@ -922,6 +940,11 @@ lsp_status lsp_build_stencils(lsp_ctx* c, const lsp_stencil_opts* opts) {
   }
   c->ns_host = o.policy == LSP_SHIFT_LOCAL ? -1 : cap_s;
   c->last_policy = o.policy;
+  if (o.t == 2 && o.nd_leaf > 0 && d == 2 && !c->eig_stream) {
+    for (cudaEvent_t& e : c->ev_eig)
+      if (!e) CUDA_OK(c, cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
+    CUDA_OK(c, cudaStreamCreateWithFlags(&c->eig_stream, cudaStreamNonBlocking));
+  }
 
   // w depends only on its index range and precision: refreshed (outside any graph) only when
   // those change, so a replayed graph always finds the table it was recorded with.

@@ -215,6 +215,8 @@ struct lsp_ctx {
   // (Q, C, P), taken on the context stream, is sent to the host on copy_stream, so that the next
   // build may overwrite the rows while the host copy is still in flight
   lsp::DevBuf stage[3];
+  cudaStream_t eig_stream = nullptr;  // the t = 2 eigen kernel beside the t = 1 one
+  cudaEvent_t ev_eig[2] = {nullptr, nullptr};  // fork, join
   cudaStream_t copy_stream = nullptr;
   cudaEvent_t ev_staged[3] = {nullptr, nullptr, nullptr};
   cudaEvent_t ev_copied[3] = {nullptr, nullptr, nullptr};
@@ -290,7 +292,7 @@ FmmTree fmm_tree(const lsp_ctx* c);
 cudaError_t launch_fmm_mark(lsp_ctx* c, const int32_t* list, const int32_t* count, int64_t cap);
 cudaError_t launch_fmm(lsp_ctx* c, const int32_t* list, const int32_t* count, int64_t cap);
 void fmm_free(FmmPlan& p);
-cudaError_t launch_eig_t2(lsp_ctx* c, const int32_t* count, int64_t cap);
+cudaError_t launch_eig_t2(lsp_ctx* c, const int32_t* count, int64_t cap, cudaStream_t stream);
 cudaError_t launch_eig_dense3(lsp_ctx* c, const int32_t* count, int64_t cap);
 cudaError_t upload_cls125(const Geometry& g);
 cudaError_t launch_rows_t2(lsp_ctx* c, int policy, const int32_t* count, int leaf);
