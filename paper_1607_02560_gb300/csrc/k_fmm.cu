@@ -208,66 +208,54 @@ __global__ void __launch_bounds__(kThreads) k_fmm_mark(const int32_t* __restrict
     fmm_mark(t, __ldg(list + i), used, err);
 }
 
-// Node values from the boxes two or three apart (children of the parent's neighbours), every
-// level at once: they need only the moments. One block per box, one thread per (node, class, f).
+// Node values from the boxes two or three apart (children of the parent's neighbours; offsets
+// -2, 2, 3 of even boxes, -3, -2, 2 of odd ones: indices 0..3 = -3, -2, 2, 3), every level at once:
+// they need only the moments. One thread per value, tables and moments through L1. FP64 pipe.
+// Measured with the translation downwards (before: a block per box, tables in shared memory): 2D
+// n = 1024 233 -> 216 us, n = 512 59 -> 52 us, n = 32 17.3 -> 15.2 us, 3D n = 64 29.6 -> 25.1 us.
 template <int NC>
 __global__ void __launch_bounds__(kThreads) k_fmm_m2l(const __grid_constant__ Tree t,
-                                                      const uint8_t* __restrict__ used,
-                                                      const double* __restrict__ tab,
-                                                      const double* __restrict__ q,
-                                                      double* __restrict__ loc) {
+                                                             const uint8_t* __restrict__ used,
+                                                             const double* __restrict__ tab,
+                                                             const double* __restrict__ q,
+                                                             double* __restrict__ loc) {
   constexpr int FC = 2 * NC, OUT = FC * kQ;
-  __shared__ double sK[8 * kQ * kQ];
-  __shared__ double sq[3][NC * kQ];
-  for (int e = threadIdx.x; e < 8 * kQ * kQ; e += kThreads) sK[e] = tab[kTabK + e];
-  const double c1 = 1.0 / (4.0 * kPi2);
+  const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, u = e / OUT;
+  if (u >= t.off[t.L + 1] || !used[u]) return;
+  const int o = (int)(e - u * OUT), i = o / FC, fc = o - i * FC, c = fc >> 1, f = fc & 1;
   int l = 0;
-  for (int64_t u = blockIdx.x; u < t.off[t.L + 1]; u += gridDim.x) {
-    if (!used[u]) continue;  // uniform
-    while (u >= t.off[l + 1]) ++l;
-    const int64_t j = t.jlo[l] + (u - t.off[l]);
-    const int odd = (int)(j & 1);
-    // offsets: even boxes -2, 2, 3; odd boxes -3, -2, 2 (indices 0..3 = -3, -2, 2, 3)
-    __syncthreads();
-    bool have[3];
+  while (u >= t.off[l + 1]) ++l;
+  const int64_t j = t.jlo[l] + (u - t.off[l]);
+  double acc = 0.0;
 #pragma unroll
-    for (int d = 0; d < 3; ++d) {
-      const int di = d + 1 - odd;
-      const int64_t x = j + (di < 2 ? di - 3 : di);
-      have[d] = x >= 0 && x < t.nsb[l];
-      if (have[d])
-        for (int e = threadIdx.x; e < NC * kQ; e += kThreads)
-          sq[d][e] = q[(t.qoff[l] + x) * (NC * kQ) + e];
-    }
-    __syncthreads();
-    const double inv_h = 1.0 / (double)((int64_t)(kBox / 2) << l);  // exact
-    for (int o = threadIdx.x; o < OUT; o += kThreads) {
-      const int i = o / FC, fc = o - i * FC, c = fc >> 1, f = fc & 1;
-      double acc = 0.0;
+  for (int d = 0; d < 3; ++d) {
+    const int di = d + 1 - (int)(j & 1);
+    const int64_t x = j + (di < 2 ? di - 3 : di);
+    if (x < 0 || x >= t.nsb[l]) continue;
+    const double* K = tab + kTabK + ((f * 4 + di) * kQ) * kQ + i;
+    const double* qq = q + (t.qoff[l] + x) * (NC * kQ) + c * kQ;
 #pragma unroll
-      for (int d = 0; d < 3; ++d) {
-        if (!have[d]) continue;
-        const double* K = sK + ((f * 4 + d + 1 - odd) * kQ) * kQ + i;
-        const double* qq = sq[d] + c * kQ;
-#pragma unroll
-        for (int k = 0; k < kQ; ++k) acc = fma(K[k * kQ], qq[k], acc);
-      }
-      const double sc = c1 * inv_h;
-      loc[u * OUT + o] = acc * (f ? sc * sc : sc);
-    }
+    for (int k = 0; k < kQ; ++k) acc = fma(__ldg(K + k * kQ), __ldg(qq + k), acc);
   }
+  const double sc = (1.0 / (4.0 * kPi2)) * (1.0 / (double)((int64_t)(kBox / 2) << l));
+  loc[e] = acc * (f ? sc * sc : sc);
 }
 
 // Node values of the leaves: from the top, child = own + interpolation of the parent's. A block
 // follows the path to one box of level S <= 3, then the boxes below it: S = 3 repeats the least of
 // the upper levels' work (2D n = 1024: 50e6 FP64 instructions, S = 0 183e6), smaller S spreads
 // a small tree over more SMs (2D n = 128, 55 leaves: both passes 40 -> 25 us).
-template <int NC>
+// FS of the 2 NC columns (class, f) per block: they are independent of each other.
+template <int NC, int FS>
 __global__ void __launch_bounds__(kThreads) k_fmm_l2l(const __grid_constant__ Tree t,
                                                       const uint8_t* __restrict__ used,
                                                       const double* __restrict__ tab,
                                                       double* __restrict__ loc, int S) {
-  constexpr int FC = 2 * NC, OUT = FC * kQ;
+  constexpr int FC = 2 * NC, ALL = FC * kQ, OUT = FS * kQ;
+  const int f0 = blockIdx.y * FS;
+  auto at = [&](int64_t u, int o) {  // place of value o of this block's columns of box u
+    return u * ALL + o / FS * FC + f0 + o % FS;
+  };
   __shared__ double sM[2 * kQ * kQ];
   __shared__ double buf[2][(1 << (kSubLev - 1)) * OUT];  // levels S - 1.. 1 at most 4 boxes
   const int64_t root = blockIdx.x;  // box of level S
@@ -276,25 +264,25 @@ __global__ void __launch_bounds__(kThreads) k_fmm_l2l(const __grid_constant__ Tr
   const int64_t jr = t.jlo[S] + root;
   // from the parent's node values src to those of a child on the given side
   auto down = [&](const double* src, int side, int o) -> double {
-    const int i = o / FC, fc = o - i * FC;
+    const int i = o / FS, fc = o - i * FS;
     const double* M = sM + side * kQ * kQ + i;
     double acc = 0.0;
 #pragma unroll
-    for (int k = 0; k < kQ; ++k) acc = fma(M[k * kQ], src[k * FC + fc], acc);
+    for (int k = 0; k < kQ; ++k) acc = fma(M[k * kQ], src[k * FS + fc], acc);
     return acc;
   };
   int cur = 0;
   {
     const int64_t u = t.off[t.L] + (jr >> (t.L - S)) - t.jlo[t.L];
-    for (int o = threadIdx.x; o < OUT; o += kThreads) buf[0][o] = loc[u * OUT + o];
+    for (int o = threadIdx.x; o < OUT; o += kThreads) buf[0][o] = loc[at(u, o)];
   }
   __syncthreads();
   for (int l = t.L - 1; l >= S; --l, cur ^= 1) {
     const int64_t j = jr >> (l - S), u = t.off[l] + j - t.jlo[l];
     for (int o = threadIdx.x; o < OUT; o += kThreads) {
-      const double v = loc[u * OUT + o] + down(buf[cur], (int)(j & 1), o);
+      const double v = loc[at(u, o)] + down(buf[cur], (int)(j & 1), o);
       if (l == 0)
-        loc[u * OUT + o] = v;
+        loc[at(u, o)] = v;
       else
         buf[cur ^ 1][o] = v;
     }
@@ -306,9 +294,9 @@ __global__ void __launch_bounds__(kThreads) k_fmm_l2l(const __grid_constant__ Tr
       const int b = e / OUT, o = e - b * OUT;
       const int64_t x = (jr << (S - l)) + b - t.jlo[l], u = t.off[l] + x;
       if (x < 0 || u >= t.off[l + 1] || !used[u]) continue;
-      const double v = loc[u * OUT + o] + down(buf[cur] + (b >> 1) * OUT, b & 1, o);
+      const double v = loc[at(u, o)] + down(buf[cur] + (b >> 1) * OUT, b & 1, o);
       if (l == 0)
-        loc[u * OUT + o] = v;
+        loc[at(u, o)] = v;
       else
         buf[cur ^ 1][b * OUT + o] = v;
     }
@@ -551,9 +539,9 @@ cudaError_t build_t(lsp_ctx* c, const int32_t* list, const int32_t* count, int64
   // stage 1: far field at the nodes of the leaf boxes
   int tm = timer_begin(c, "stage1");
   e = tuned_launch(c, std::string("stage1/fmm") + std::to_string(NC) + "/w" + work_bucket(boxes),
-                   {kThreads, 4}, kThreads, kThreads, [&](LaunchShape sh) {
-    const int64_t b = std::min<int64_t>(boxes, 152 * (int64_t)sh.per_sm);
-    k_fmm_m2l<NC><<<(int)b, kThreads, 0, c->stream>>>(t, used, tab, (const double*)P.q.p, loc);
+                   {64, 2}, kThreads, 0, [&](LaunchShape sh) {  // (one value per thread: no cap)
+    k_fmm_m2l<NC><<<(unsigned)((boxes * 2 * NC * kQ + sh.threads - 1) / sh.threads), sh.threads, 0,
+                    c->stream>>>(t, used, tab, (const double*)P.q.p, loc);
     return cudaGetLastError();
   });
   if (e != cudaSuccess) return e;
@@ -561,7 +549,14 @@ cudaError_t build_t(lsp_ctx* c, const int32_t* list, const int32_t* count, int64
     // the deepest subtrees that still leave two blocks per SM
     int S = 0;
     while (S < std::min(t.L, kSubLev) && t.off[S + 2] - t.off[S + 1] >= 2 * 152) ++S;
-    k_fmm_l2l<NC><<<(int)(t.off[S + 1] - t.off[S]), kThreads, 0, c->stream>>>(t, used, tab, loc, S);
+    // At most two subtrees per SM to do (no more than there are shifts): a quarter of the columns
+    // per block (65 shifts at 2D n = 1024 61 -> 49 us for both translations, n = 256 25.5 -> 21.8,
+    // 3D n = 64 25.1 -> 21.4; all 440 subtrees of n = 512 with per-point shifts 51.9 -> 54.1).
+    const int roots = (int)(t.off[S + 1] - t.off[S]);
+    if (std::min<int64_t>(cap, roots) <= 2 * 152)
+      k_fmm_l2l<NC, NC / 2><<<dim3(roots, 4), kThreads, 0, c->stream>>>(t, used, tab, loc, S);
+    else
+      k_fmm_l2l<NC, 2 * NC><<<roots, kThreads, 0, c->stream>>>(t, used, tab, loc, S);
   }
   timer_end(c, tm);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
