@@ -22,6 +22,29 @@ __device__ __forceinline__ double shift_of(int64_t m) { return lattice_shift(m);
 // insertion point can win.
 __device__ __forceinline__ int nearest_shift(const int32_t* __restrict__ m, int ns, double x) {
   int lo = 0, hi = ns;
+  int64_t f;
+  if (lattice_fixed(x, &f)) {
+    // the same search and choice in integers, unless a comparison is closer than they resolve
+    // (rows of 2^20 points from 65 shifts 76 -> 39 us: each step took four FP64 operations)
+    bool close = false;
+    while (lo < hi) {
+      const int mid = (lo + hi) >> 1;
+      const int64_t d = f - ((int64_t)__ldg(m + mid) << 20);
+      close |= d <= kFixedGuard && d >= -kFixedGuard;
+      if (d > 0)
+        lo = mid + 1;
+      else
+        hi = mid;
+    }
+    if (!close) {
+      if (lo == 0) return 0;
+      if (lo == ns) return ns - 1;
+      const int64_t e = 2 * f - (((int64_t)__ldg(m + lo - 1) + __ldg(m + lo)) << 20);
+      if (e > 2 * kFixedGuard || e < -2 * kFixedGuard) return e < 0 ? lo - 1 : lo;
+    }
+    lo = 0;
+    hi = ns;
+  }
   while (lo < hi) {
     const int mid = (lo + hi) >> 1;
     if (shift_of(__ldg(m + mid)) < x)
@@ -91,7 +114,10 @@ __global__ void __launch_bounds__(kThreads) k_rows(
     __syncthreads();
     if (ROWS) {
       const int64_t obase = j0 * MU;
-      for (int e = t; e < npts * MU; e += kThreads) {
+#pragma unroll 3
+      for (int it = 0; it < MU; ++it) {  // three entries' loads in flight
+        const int e = t + it * kThreads;
+        if (e >= npts * MU) break;
         const int p = e / MU, o = e - p * MU;
         const int idx = s_idx[p];
         const double a = __ldg(alpha + (int64_t)idx * MU + o);

@@ -56,3 +56,27 @@ def test_statistics_refuse_non_finite_values(n):
         with pytest.raises(LspError):
             ctx.set_potential(v.reshape(n, n))
     ctx.set_potential(rng.standard_normal((n, n)))
+
+
+@pytest.mark.parametrize("n,ns,spread", [(8, 1, 0), (64, 2, 1), (64, 3, 5000), (128, 64, 1000)])
+def test_nearest_of_a_shift_list(n, ns, spread):
+    """Every point takes the listed shift nearest to its value, ties to the smaller: the oracle's
+    assignment, with values on the shifts, half-way between neighbours and next to both."""
+    import torch
+    from paper_1607_02560_gb300 import Context
+    rng = np.random.default_rng(n + ns)
+    N = n * n
+    m = np.sort(rng.choice(np.arange(0, max(spread, ns) + 1), size=ns, replace=False)) + 3
+    s = np.asarray(O.shift_value(m))
+    k = rng.integers(0, ns, size=N)
+    near = 10.0 ** rng.uniform(-16, 0, size=N) * np.sign(rng.uniform(-1, 1, size=N))
+    mid = 0.5 * (s[k] + s[np.minimum(k + 1, ns - 1)])
+    v = np.where(rng.random(N) < 0.5, s[k], mid) * np.where(rng.random(N) < 0.2, 1.0, 1.0 + near)
+    v = np.where(rng.random(N) < 0.3, rng.uniform(s[0] - 100, s[-1] + 100, size=N), v)
+    want = np.asarray(O.assign_shifts(v, m)).reshape(-1)
+    ctx = Context(2, n, stream=torch.cuda.Stream())
+    ctx.set_potential(v.reshape(n, n))
+    ctx.build_stencils(policy="list", shifts=s)
+    t = ctx.get_shift_table()
+    assert np.array_equal(t["s"], s)
+    assert np.array_equal(t["s_idx"], want)
