@@ -17,16 +17,16 @@
 //
 // What bounds it: the FP64 pipe. The sums stage by stage cost 1.5e9 FP64 instructions in stage 1
 // and 0.6e9 in stage 2 at 2D n = 1024 with per-point shifts (93 491 of them); here it is 2e8:
-// moments depend on n only and are made once per context; 19 200 per box (6900 boxes) for the
-// translations, 970 per shift at the end. Fewer nodes or smaller boxes trade these against each
-// other: boxes of 64 cost 266e6 + 56e6, of 256 67e6 + 158e6, of 128 133e6 + 90e6.
+// moments depend on n only and are made once per context; 19 200 per box (6900 boxes; 12 000 where
+// mirrored nodes share the work, see k_fmm_m2l_box and k_fmm_l2l) for the translations, 970 per
+// shift at the end. Fewer nodes or smaller boxes trade these against each other: without the
+// mirroring boxes of 64 cost 266e6 + 56e6, of 256 67e6 + 158e6, of 128 133e6 + 90e6.
 // Accuracy against extended precision, 2D n = 1024, largest error relative to the largest g of the
 // shift: f = 1 1.9e-15 (stages 1.3e-15), f = 2 5e-16 (stages 1e-15); rms 2.6e-16 and 0.9e-16
 // (stages 2.4e-16 and 2e-16).
-// Measured (both stages, GB300): 2D n = 1024 per-point shifts 3.68 -> 0.48 ms, 65 shifts 0.39 ->
-// 0.08 ms, n = 512 0.49 -> 0.13 ms, n = 256 0.155 -> 0.057 ms, n = 128 0.052 -> 0.045 ms, 3D
-// n = 64 0.047 -> 0.041 ms (and two launches fewer for the stage lists). The translations run at
-// 0.8 of the FP64 rate, the final sums at 0.6.
+// Measured (both stages, GB300; stage by stage before): 2D n = 1024 per-point shifts 3.68 -> 0.42 ms,
+// 65 shifts 0.39 -> 0.06 ms, n = 512 0.49 -> 0.13 ms, n = 256 0.155 -> 0.051 ms, n = 128 0.052 ->
+// 0.039 ms, 3D n = 64 0.047 -> 0.033 ms (and two launches fewer for the stage lists).
 #include <math.h>
 
 #include <algorithm>
@@ -43,10 +43,14 @@ constexpr int kThreads = 256;
 constexpr int kSubLev = 3;                 // a block of the downward pass ends in 2^3 leaf boxes
 
 // Device tables of the plan (doubles): P2M [128][20], M2M [2][20][20], M2L [2][4][20][20]
-// (f = 1, 2; offsets -3, -2, 2, 3), L2P [20][128], near w [512][2].
+// (f = 1, 2; offsets -3, -2, 2, 3), L2P [20][128], near w [512][2], and for the symmetric pairs (see
+// k_fmm_m2l_box and k_fmm_l2l) the half sums and half differences of M2L [2][2][20][10] at offset 2
+// and of the interpolation to the lower child [2][10][20].
+constexpr int kH = kQ / 2;
 constexpr int kTabP = 0, kTabM = kTabP + kBox * kQ, kTabK = kTabM + 2 * kQ * kQ,
               kTabE = kTabK + 8 * kQ * kQ, kTabW = kTabE + kQ * kBox,
-              kTabSize = kTabW + 4 * kBox * 2;
+              kTabKS = kTabW + 4 * kBox * 2, kTabMS = kTabKS + 4 * kQ * kH,
+              kTabSize = kTabMS + 2 * kH * kQ;
 static_assert(kTabW % 2 == 0, "16-byte aligned");
 
 template <int D>
@@ -241,6 +245,56 @@ __global__ void __launch_bounds__(kThreads) k_fmm_m2l(const __grid_constant__ Tr
   loc[e] = acc * (f ? sc * sc : sc);
 }
 
+// The same, a block per box and a thread per pair of mirrored nodes (i, 19 - i). With R the moments
+// of the box at offset 2 and L those at -2 in reverse order, K_-2[k][i] = -+K_2[19 - k][19 - i] (f = 1,
+// 2) gives
+//   out[i] + out[19 - i] = sum_k (K_2[k][i] + K_2[k][19 - i]) (R -+ L)[k],
+//   out[i] - out[19 - i] = sum_k (K_2[k][i] - K_2[k][19 - i]) (R +- L)[k],
+// 80 instead of 120 multiply-adds a pair with the third offset. Measured with the translation
+// downwards: 2D n = 1024 208 -> 175 us, n = 512 53.7 -> 50.0 us, n = 128 20.5 -> 18.7 us.
+template <int NC>
+__global__ void __launch_bounds__(NC * kQ) k_fmm_m2l_box(const __grid_constant__ Tree t,
+                                                         const uint8_t* __restrict__ used,
+                                                         const double* __restrict__ tab,
+                                                         const double* __restrict__ q,
+                                                         double* __restrict__ loc) {
+  constexpr int FC = 2 * NC, OUT = FC * kQ;
+  __shared__ double sa[2][NC][kQ], s3[NC][kQ];  // R + L, R - L; the moments at offset 3 or -3
+  const int64_t u = blockIdx.x;
+  if (!used[u]) return;
+  int l = 0;
+  while (u >= t.off[l + 1]) ++l;
+  const int64_t j = t.jlo[l] + (u - t.off[l]);
+  const int odd = (int)(j & 1);
+  {
+    const int c = threadIdx.x / kQ, k = threadIdx.x % kQ;
+    auto moment = [&](int64_t x, int kk) {
+      return x >= 0 && x < t.nsb[l] ? __ldg(q + (t.qoff[l] + x) * (NC * kQ) + c * kQ + kk) : 0.0;
+    };
+    const double r = moment(j + 2, k), m = moment(j - 2, kQ - 1 - k);
+    sa[0][c][k] = r + m;
+    sa[1][c][k] = r - m;
+    s3[c][k] = moment(odd ? j - 3 : j + 3, k);
+  }
+  __syncthreads();
+  const int i = threadIdx.x / FC, fc = threadIdx.x - i * FC, c = fc >> 1, f = fc & 1;
+  const double* KS = tab + kTabKS + 2 * f * kQ * kH + i;
+  const double* K3 = tab + kTabK + ((f * 4 + (odd ? 0 : 3)) * kQ) * kQ + i;
+  const double *ps = sa[1 - f][c], *pd = sa[f][c], *p3 = s3[c];
+  double sum = 0.0, dif = 0.0, lo = 0.0, hi = 0.0;
+#pragma unroll
+  for (int k = 0; k < kQ; ++k) {
+    sum = fma(__ldg(KS + k * kH), ps[k], sum);
+    dif = fma(__ldg(KS + (kQ + k) * kH), pd[k], dif);
+    lo = fma(__ldg(K3 + k * kQ), p3[k], lo);
+    hi = fma(__ldg(K3 + k * kQ + kQ - 1 - 2 * i), p3[k], hi);
+  }
+  const double sc1 = (1.0 / (4.0 * kPi2)) * (1.0 / (double)((int64_t)(kBox / 2) << l));
+  const double sc = f ? sc1 * sc1 : sc1;
+  loc[u * OUT + i * FC + fc] = (lo + (sum + dif)) * sc;
+  loc[u * OUT + (kQ - 1 - i) * FC + fc] = (hi + (sum - dif)) * sc;
+}
+
 // Node values of the leaves: from the top, child = own + interpolation of the parent's. A block
 // follows the path to one box of level S <= 3, then the boxes below it: S = 3 repeats the least of
 // the upper levels' work (2D n = 1024: 50e6 FP64 instructions, S = 0 183e6), smaller S spreads
@@ -256,11 +310,12 @@ __global__ void __launch_bounds__(kThreads) k_fmm_l2l(const __grid_constant__ Tr
   auto at = [&](int64_t u, int o) {  // place of value o of this block's columns of box u
     return u * ALL + o / FS * FC + f0 + o % FS;
   };
-  __shared__ double sM[2 * kQ * kQ];
+  __shared__ double sM[2 * kQ * kQ], sS[2 * kH * kQ];
   __shared__ double buf[2][(1 << (kSubLev - 1)) * OUT];  // levels S - 1.. 1 at most 4 boxes
   const int64_t root = blockIdx.x;  // box of level S
   if (t.L == 0 || !used[t.off[S] + root]) return;
   for (int e = threadIdx.x; e < 2 * kQ * kQ; e += kThreads) sM[e] = tab[kTabM + e];
+  for (int e = threadIdx.x; e < 2 * kH * kQ; e += kThreads) sS[e] = tab[kTabMS + e];
   const int64_t jr = t.jlo[S] + root;
   // from the parent's node values src to those of a child on the given side
   auto down = [&](const double* src, int side, int o) -> double {
@@ -288,17 +343,68 @@ __global__ void __launch_bounds__(kThreads) k_fmm_l2l(const __grid_constant__ Tr
     }
     __syncthreads();
   }
+  if constexpr (FS < FC) {
+    for (int l = S - 1; l >= 0; --l, cur ^= 1) {
+      const int nb = 1 << (S - l);  // boxes of this level under the root
+      for (int e = threadIdx.x; e < nb * OUT; e += kThreads) {
+        const int b = e / OUT, o = e - b * OUT;
+        const int64_t x = (jr << (S - l)) + b - t.jlo[l], u = t.off[l] + x;
+        if (x < 0 || u >= t.off[l + 1] || !used[u]) continue;
+        const double v = loc[at(u, o)] + down(buf[cur] + (b >> 1) * OUT, b & 1, o);
+        if (l == 0)
+          loc[at(u, o)] = v;
+        else
+          buf[cur ^ 1][b * OUT + o] = v;
+      }
+      __syncthreads();
+    }
+    return;
+  }
+  // All columns: both children of a parent together. With e, o the sums and differences of its values
+  // at mirrored nodes, node i of the lower child is E + O and node 19 - i of the upper one E - O,
+  // E = sum_k<10 Ms[k][i] e[k], O = sum Md[k][i] o[k]: half the multiply-adds for one more barrier a
+  // level (2D n = 1024, both translations 216 -> 208 us; with few subtrees the barrier costs more:
+  // 3D n = 64 21.4 -> 23.5 us).
   for (int l = S - 1; l >= 0; --l, cur ^= 1) {
-    const int nb = 1 << (S - l);  // boxes of this level under the root
-    for (int e = threadIdx.x; e < nb * OUT; e += kThreads) {
-      const int b = e / OUT, o = e - b * OUT;
-      const int64_t x = (jr << (S - l)) + b - t.jlo[l], u = t.off[l] + x;
-      if (x < 0 || u >= t.off[l + 1] || !used[u]) continue;
-      const double v = loc[at(u, o)] + down(buf[cur] + (b >> 1) * OUT, b & 1, o);
-      if (l == 0)
-        loc[at(u, o)] = v;
-      else
-        buf[cur ^ 1][b * OUT + o] = v;
+    const int np = 1 << (S - 1 - l);  // parents under the root
+    double* par = buf[cur];
+    for (int e = threadIdx.x; e < np * kH * FS; e += kThreads) {
+      const int b = e / (kH * FS), o = e - b * (kH * FS), kk = o / FS, fc = o - kk * FS;
+      double* x = par + b * OUT + kk * FS + fc;
+      double* y = par + b * OUT + (kQ - 1 - kk) * FS + fc;
+      const double vx = *x, vy = *y;
+      *x = vx + vy;
+      *y = vx - vy;
+    }
+    __syncthreads();
+    for (int e = threadIdx.x; e < np * OUT; e += kThreads) {
+      const int b = e / OUT, o = e - b * OUT, i = o / FS, fc = o - i * FS;
+      const int64_t x = (jr << (S - l)) + 2 * b - t.jlo[l], u = t.off[l] + x;  // the lower child
+      const bool lower = x >= 0 && u < t.off[l + 1] && used[u];
+      const bool upper = x + 1 >= 0 && u + 1 < t.off[l + 1] && used[u + 1];
+      if (!lower && !upper) continue;
+      const double* src = par + b * OUT + fc;
+      double E = 0.0, O = 0.0;
+#pragma unroll
+      for (int k = 0; k < kH; ++k) {
+        E = fma(sS[k * kQ + i], src[k * FS], E);
+        O = fma(sS[(kH + k) * kQ + i], src[(kQ - 1 - k) * FS], O);
+      }
+      const int om = (kQ - 1 - i) * FS + fc;  // the mirrored node
+      if (lower) {
+        const double v = loc[at(u, o)] + (E + O);
+        if (l == 0)
+          loc[at(u, o)] = v;
+        else
+          buf[cur ^ 1][2 * b * OUT + o] = v;
+      }
+      if (upper) {
+        const double v = loc[at(u + 1, om)] + (E - O);
+        if (l == 0)
+          loc[at(u + 1, om)] = v;
+        else
+          buf[cur ^ 1][(2 * b + 1) * OUT + om] = v;
+      }
     }
     __syncthreads();
   }
@@ -456,6 +562,21 @@ std::vector<double> make_tables() {
         t[kTabK + (d * kQ + k) * kQ + i] = (double)x;
         t[kTabK + ((4 + d) * kQ + k) * kQ + i] = (double)(x * x);
       }
+  for (int f = 0; f < 2; ++f)
+    for (int k = 0; k < kQ; ++k)
+      for (int i = 0; i < kH; ++i) {
+        const R x = 1 / (4 + node[k] - node[i]), y = 1 / (4 + node[k] + node[i]);
+        const R a = f ? x * x : x, b2 = f ? y * y : y;
+        t[kTabKS + ((2 * f) * kQ + k) * kH + i] = (double)((a + b2) / 2);
+        t[kTabKS + ((2 * f + 1) * kQ + k) * kH + i] = (double)((a - b2) / 2);
+      }
+  for (int i = 0; i < kQ; ++i) {
+    basis((node[i] - 1) / 2, b);
+    for (int k = 0; k < kH; ++k) {
+      t[kTabMS + k * kQ + i] = (double)((b[k] + b[kQ - 1 - k]) / 2);
+      t[kTabMS + (kH + k) * kQ + i] = (double)((b[k] - b[kQ - 1 - k]) / 2);
+    }
+  }
   for (int l = 0; l < 4 * kBox; ++l) {  // w(l - 256) and its square, as the stages' table
     const double w = 1.0 / (kPi2 * (double)(4 * (l - 2 * kBox) + 2));
     t[kTabW + 2 * l] = w;
@@ -538,10 +659,16 @@ cudaError_t build_t(lsp_ctx* c, const int32_t* list, const int32_t* count, int64
   cudaError_t e;
   // stage 1: far field at the nodes of the leaf boxes
   int tm = timer_begin(c, "stage1");
+  // (a tree of 4 boxes, 3D n = 64: 21.4 us a value per thread, 23.3 a pair per thread)
+  const bool few = boxes <= 32;
   e = tuned_launch(c, std::string("stage1/fmm") + std::to_string(NC) + "/w" + work_bucket(boxes),
-                   {64, 2}, kThreads, 0, [&](LaunchShape sh) {  // (one value per thread: no cap)
-    k_fmm_m2l<NC><<<(unsigned)((boxes * 2 * NC * kQ + sh.threads - 1) / sh.threads), sh.threads, 0,
-                    c->stream>>>(t, used, tab, (const double*)P.q.p, loc);
+                   {64, 2}, kThreads, 0, [&](LaunchShape sh) {
+    if (few)  // (one value per thread: no cap)
+      k_fmm_m2l<NC><<<(unsigned)((boxes * 2 * NC * kQ + sh.threads - 1) / sh.threads), sh.threads,
+                      0, c->stream>>>(t, used, tab, (const double*)P.q.p, loc);
+    else
+      k_fmm_m2l_box<NC><<<(unsigned)boxes, NC * kQ, 0, c->stream>>>(t, used, tab,
+                                                                    (const double*)P.q.p, loc);
     return cudaGetLastError();
   });
   if (e != cudaSuccess) return e;
