@@ -181,8 +181,10 @@ def lattice_domain_sizes(m_list: np.ndarray, n: int, d: int) -> list[int]:
 def fmm_flops(m_list: np.ndarray, n: int, d: int) -> dict:
     """FP64 flops of the fast multipole evaluation of the kernel vectors (t = 1, 2D and 3D): 20
     nodes per box of 128 integers, classes x 2 functions; "stage1" the node-to-node products of
-    every box that holds a shift (up to three sources each) and one interpolation from its
-    parent, "stage2" the interpolation to the shifts and their near sources (three boxes)."""
+    every box that holds a shift (the sources two boxes away on either side share one product by
+    the nodes' symmetry, the third has its own) and the interpolation from its parent (half of one
+    in the three lowest levels, where two children share it), "stage2" the interpolation to the
+    shifts and their near sources (three boxes)."""
     half, nq, box = n // 2, 20, 128
     fc = 2 * {2: 6, 3: 10}[d]
     p2 = np.arange(half + 1, dtype=np.int64) ** 2
@@ -191,16 +193,16 @@ def fmm_flops(m_list: np.ndarray, n: int, d: int) -> dict:
         r = np.unique(r[:, None] + p2[None, :])
     x = -np.asarray(m_list, dtype=np.int64)
     lo, hi = min(int(x.min()), 0), max(int(x.max()), int(r.max()))
-    prods = 0
+    prods = 0.0
     level = 0
     while True:
         width = box << level
         j = np.unique(x // width)
         top = (hi // (2 * width)) - (lo // (2 * width)) <= 1
-        for odd, offs in ((0, (-2, 2, 3)), (1, (-3, -2, 2))):
-            sel = j[j % 2 == odd]
-            prods += sum(int(((sel + o >= 0) & (sel + o <= r.max() // width)).sum()) for o in offs)
-        prods += 0 if top else len(j)
+        has = lambda x: (x >= 0) & (x <= r.max() // width)  # noqa: E731
+        prods += int((has(j - 2) | has(j + 2)).sum())
+        prods += int(has(np.where(j % 2 == 0, j + 3, j - 3)).sum())
+        prods += 0 if top else (0.5 if level < 3 else 1.0) * len(j)
         if top:
             break
         level += 1
@@ -848,7 +850,9 @@ def solve_variant(torch, n: int, policy: str = "paper", fp64_peak: float | None 
         ach = info["flops_lu"] / setup_s / 1e12
         out["setup_roofline"] = {"bound": "fp64", "achieved": ach, "peak": fp64_peak,
                                  "unit": "TFLOP/s", "frac": ach / fp64_peak,
-                                 "work": "multifrontal LU count 2/3 s^3 + 2 s^2 r + 2 s r^2 per front"}
+                                 "work": "multifrontal LU count 2/3 s^3 + 2 s^2 r + 2 s r^2 per front "
+                                         "(the large fronts' updates run on the tensor cores: "
+                                         "above the FP64 rate)"}
     if hbm_peak:
         ach = info["solve_bytes"] / (app_ms * 1e-3) / 1e9
         out["solve_roofline"] = {"bound": "hbm", "achieved": ach, "peak": hbm_peak,

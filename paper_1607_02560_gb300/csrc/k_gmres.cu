@@ -162,9 +162,9 @@ __global__ void k_gmres_givens(double* gs, int col, int ld, int restart) {
 // registers from the first projection to the last, so a projection reads v_k once (and the next
 // one while the blocks exchange their partial sums) instead of w twice and v_k twice, and the
 // blocks meet once per projection instead of ending a kernel. Bound by the FP64 pipe (2 N
-// products a projection, 3.3 us at N = 2^20) and the meeting (about 2 us): 18 us a projection with
-// one kernel each, now 8 us. Every block adds all partial sums in block order, so all have
-// the same h and the result is deterministic. The wait for the others is bounded (1 s); when it
+// products a projection, 3.3 us at N = 2^20) and the meeting (about 2 us): 9.1 us a projection, where
+// one kernel each took 14.4 us and the gap to the next launch. Every block adds all partial sums in
+// block order, so all have the same h and the result is deterministic. The wait for the others is bounded (1 s); when it
 // runs out, gs[kGsFail] is set and every block leaves.
 constexpr int kArnThreads = 1024, kArnPer = 8;
 __device__ __forceinline__ bool meet(unsigned* bar, unsigned target, bool ok) {
