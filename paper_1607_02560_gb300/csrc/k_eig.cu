@@ -22,11 +22,17 @@
 namespace lsp {
 namespace {
 
-__constant__ uint8_t c_cls[kMaxMu][kMaxMu];
-__constant__ SymBasis c_sym;
+// Tables of the t = 1 neighbourhood, one set per dimension (index d - 1): they depend on d only, so
+// contexts of different dimensions have their own and those of one dimension write the same bytes.
+__constant__ uint8_t c_cls[kMaxD][kMaxMu][kMaxMu];
+__constant__ SymBasis c_sym[kMaxD];
 // Projection entries (block, i, j), i <= j, for the symmetric method.
-__constant__ int8_t c_ent[64][3];
-__constant__ int c_nent;
+__constant__ int8_t c_ent[kMaxD][64][3];
+__constant__ int c_nent[kMaxD];
+template <int MU>
+__host__ __device__ constexpr int dim_index() {  // MU = 3^d
+  return MU == 3 ? 0 : MU == 9 ? 1 : 2;
+}
 
 // Cyclic Jacobi on a small symmetric matrix held by one thread. a is dim x dim (row-major,
 // leading dimension 4) and is overwritten; v receives the eigenvectors as columns.
@@ -382,14 +388,15 @@ __global__ void __launch_bounds__(WARPS * 32) k_eig(const double* __restrict__ g
                                                     int32_t* __restrict__ flags_out,
                                                     const int32_t* __restrict__ shift_m,
                                                     double* __restrict__ ap_out) {
+  constexpr int kD = dim_index<MU>();
   extern __shared__ __align__(16) unsigned char smraw[];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   BlockTables<MU>& tb = *reinterpret_cast<BlockTables<MU>*>(smraw);
   WarpSmem<MU>& sm =
       reinterpret_cast<WarpSmem<MU>*>(smraw + ((sizeof(BlockTables<MU>) + 15) / 16) * 16)[w];
   for (int e = threadIdx.x; e < kMaxSymVec * MU; e += WARPS * 32)
-    tb.u[e / MU][e % MU] = c_sym.u[e / MU][e % MU];
-  for (int e = threadIdx.x; e < MU * MU; e += WARPS * 32) tb.cls[e / MU][e % MU] = c_cls[e / MU][e % MU];
+    tb.u[e / MU][e % MU] = c_sym[kD].u[e / MU][e % MU];
+  for (int e = threadIdx.x; e < MU * MU; e += WARPS * 32) tb.cls[e / MU][e % MU] = c_cls[kD][e / MU][e % MU];
   __syncthreads();
   const int64_t cnt = *count;
   const int centre = MU / 2;
@@ -424,10 +431,10 @@ __global__ void __launch_bounds__(WARPS * 32) k_eig(const double* __restrict__ g
       }
     } else {
       // projections B_b[i][j] = u_i^T A u_j
-      for (int ent = lane; ent < c_nent; ent += 32) {
-        const int b = c_ent[ent][0], ii = c_ent[ent][1], jj = c_ent[ent][2];
-        const double* ui = tb.u[c_sym.first[b] + ii];
-        const double* uj = tb.u[c_sym.first[b] + jj];
+      for (int ent = lane; ent < c_nent[kD]; ent += 32) {
+        const int b = c_ent[kD][ent][0], ii = c_ent[kD][ent][1], jj = c_ent[kD][ent][2];
+        const double* ui = tb.u[c_sym[kD].first[b] + ii];
+        const double* uj = tb.u[c_sym[kD].first[b] + jj];
         double s = 0.0;
         for (int a = 0; a < MU; ++a) {
           if (ui[a] == 0.0) continue;
@@ -440,8 +447,8 @@ __global__ void __launch_bounds__(WARPS * 32) k_eig(const double* __restrict__ g
         sm.B[b][jj * 4 + ii] = s;
       }
       __syncwarp();
-      if (lane < c_sym.nblk) {
-        const int dim = c_sym.dim[lane];
+      if (lane < c_sym[kD].nblk) {
+        const int dim = c_sym[kD].dim[lane];
         double a[4][4], y[4], lmin, l2;
         for (int r = 0; r < 4; ++r)
           for (int q = 0; q < 4; ++q) a[r][q] = (r < dim && q < dim) ? sm.B[lane][r * 4 + q] : 0.0;
@@ -478,15 +485,15 @@ __global__ void __launch_bounds__(WARPS * 32) k_eig(const double* __restrict__ g
       __syncwarp();
       if (lane == 0) {
         int bstar = 0;
-        for (int b = 1; b < c_sym.nblk; ++b)
+        for (int b = 1; b < c_sym[kD].nblk; ++b)
           if (sm.lam[b][0] < sm.lam[bstar][0]) bstar = b;
         lam1 = sm.lam[bstar][0];
         lam2 = DBL_MAX;
-        for (int b = 0; b < c_sym.nblk; ++b) lmax = fmax(lmax, fabs(sm.work[b]));
-        for (int b = 0; b < c_sym.nblk; ++b) {
-          for (int r = 0; r < c_sym.dim[b] && r < 2; ++r) {
+        for (int b = 0; b < c_sym[kD].nblk; ++b) lmax = fmax(lmax, fabs(sm.work[b]));
+        for (int b = 0; b < c_sym[kD].nblk; ++b) {
+          for (int r = 0; r < c_sym[kD].dim[b] && r < 2; ++r) {
             if (b == bstar && r == 0) {
-              if (c_sym.copies[b] > 1) lam2 = fmin(lam2, sm.lam[b][r]);
+              if (c_sym[kD].copies[b] > 1) lam2 = fmin(lam2, sm.lam[b][r]);
               continue;
             }
             lam2 = fmin(lam2, sm.lam[b][r]);
@@ -496,8 +503,8 @@ __global__ void __launch_bounds__(WARPS * 32) k_eig(const double* __restrict__ g
         if (bstar != 0) flags |= LSP_FLAG_NONSYMMETRIC;
         for (int a = 0; a < MU; ++a) {
           double s = 0.0;
-          for (int r = 0; r < c_sym.dim[bstar]; ++r)
-            s = fma(sm.y[bstar][r], tb.u[c_sym.first[bstar] + r][a], s);
+          for (int r = 0; r < c_sym[kD].dim[bstar]; ++r)
+            s = fma(sm.y[bstar][r], tb.u[c_sym[kD].first[bstar] + r][a], s);
           sm.alpha[a] = s;
         }
       }
@@ -607,8 +614,8 @@ __global__ void __launch_bounds__(WARPS * 32) k_eig3d(const double* __restrict__
   for (int e = threadIdx.x; e < NENT * NCLS; e += WARPS * 32)
     s_coef[e / NCLS][e % NCLS] = c_coef3[e / NCLS][e % NCLS];
   for (int e = threadIdx.x; e < kMaxSymVec * MU; e += WARPS * 32)
-    s_u[e / MU][e % MU] = c_sym.u[e / MU][e % MU];
-  for (int e = threadIdx.x; e < NENT * 3; e += WARPS * 32) s_ent[e / 3][e % 3] = c_ent[e / 3][e % 3];
+    s_u[e / MU][e % MU] = c_sym[2].u[e / MU][e % MU];
+  for (int e = threadIdx.x; e < NENT * 3; e += WARPS * 32) s_ent[e / 3][e % 3] = c_ent[2][e / 3][e % 3];
   __syncthreads();
   Eig3Warp& sm = sw[w];
   const int64_t cnt = *count;
@@ -806,7 +813,7 @@ __global__ void __launch_bounds__(WARPS * 32) k_eig3d(const double* __restrict__
       lmax = fmax(lmax, fabs(sm.tr[bb]));
       if (bb == bstar) {
         lam2 = fmin(lam2, sm.lam[bb][1]);
-        if (c_sym.copies[bb] > 1) lam2 = fmin(lam2, sm.lam[bb][0]);
+        if (c_sym[2].copies[bb] > 1) lam2 = fmin(lam2, sm.lam[bb][0]);
       } else {
         lam2 = fmin(lam2, sm.lam[bb][0]);
       }
@@ -816,7 +823,7 @@ __global__ void __launch_bounds__(WARPS * 32) k_eig3d(const double* __restrict__
     if (bstar != 0) flags |= LSP_FLAG_NONSYMMETRIC;
     if (lam2 - lam1 < 1e-8 * lmax) flags |= LSP_FLAG_DEGENERATE;
     // ---- alpha = U_b y and (a6) c = G alpha = U_b (G_b y) ----
-    const int first = c_sym.first[bstar];
+    const int first = c_sym[2].first[bstar];
     double y[4], gy[4];
 #pragma unroll
     for (int x = 0; x < 4; ++x) y[x] = sm.v[bstar][x];
@@ -828,7 +835,7 @@ __global__ void __launch_bounds__(WARPS * 32) k_eig3d(const double* __restrict__
     }
     double av = 0.0, cv = 0.0;
     if (lane < MU) {
-      const int dimb = c_sym.dim[bstar];
+      const int dimb = c_sym[2].dim[bstar];
 #pragma unroll
       for (int x = 0; x < 4; ++x)
         if (x < dimb) {
@@ -1540,7 +1547,7 @@ __global__ void __launch_bounds__(128) k_eig2d(const double* __restrict__ gvals,
       if constexpr (sizeof(GT) == 4) {
 #pragma unroll
         for (int a = 0; a < 9; ++a) {
-          al[a] = y[0] * c_sym.u[0][a] + y[1] * c_sym.u[1][a] + y[2] * c_sym.u[2][a];
+          al[a] = y[0] * c_sym[1].u[0][a] + y[1] * c_sym[1].u[1][a] + y[2] * c_sym[1].u[2][a];
           cv[a] = y[0] * w0[a] + y[1] * w1[a] + y[2] * w2[a];
         }
       } else {  // c = U_b (G_b y): one value per orbit
@@ -1558,7 +1565,7 @@ __global__ void __launch_bounds__(128) k_eig2d(const double* __restrict__ gvals,
     } else if (win == 1 || win == 2) {
       const int vi = win == 1 ? 3 : 4;
 #pragma unroll
-      for (int a = 0; a < 9; ++a) al[a] = c_sym.u[vi][a];
+      for (int a = 0; a < 9; ++a) al[a] = c_sym[1].u[vi][a];
       if constexpr (sizeof(GT) == 4) {
         GT u[9];
         if (win == 1) w_vec<3>(g, u); else w_vec<4>(g, u);
@@ -1581,7 +1588,7 @@ __global__ void __launch_bounds__(128) k_eig2d(const double* __restrict__ gvals,
       p /= nr;
       q /= nr;
 #pragma unroll
-      for (int a = 0; a < 9; ++a) al[a] = p * c_sym.u[5][a] + q * c_sym.u[6][a];
+      for (int a = 0; a < 9; ++a) al[a] = p * c_sym[1].u[5][a] + q * c_sym[1].u[6][a];
       if constexpr (sizeof(GT) == 4) {
         GT u[9], v[9];
         w_vec<5>(g, u);
@@ -1591,7 +1598,7 @@ __global__ void __launch_bounds__(128) k_eig2d(const double* __restrict__ gvals,
       } else {
         const double zp = fma(h00, p, h01 * q), zq = fma(h01, p, h11 * q);
 #pragma unroll
-        for (int a = 0; a < 9; ++a) cv[a] = zp * c_sym.u[5][a] + zq * c_sym.u[6][a];
+        for (int a = 0; a < 9; ++a) cv[a] = zp * c_sym[1].u[5][a] + zq * c_sym[1].u[6][a];
       }
     }
     // sign: alpha[centre] > 0, else the first entry above 1e-12 in magnitude
@@ -1642,11 +1649,12 @@ cudaError_t upload_sym(lsp_ctx* c) {
   uint8_t cls[kMaxMu][kMaxMu];  // the t = 1 classes (the geometry holds up to 125 offsets)
   for (int a = 0; a < kMaxMu; ++a)
     for (int b = 0; b < kMaxMu; ++b) cls[a][b] = c->geo.cls_of[a][b];
-  cudaError_t e = cudaMemcpyToSymbol(c_cls, cls, sizeof cls);
+  const size_t di = (size_t)c->geo.d - 1;
+  cudaError_t e = cudaMemcpyToSymbol(c_cls, cls, sizeof cls, di * sizeof cls);
   if (e != cudaSuccess) return e;
-  e = cudaMemcpyToSymbol(c_sym, &c->sym, sizeof(SymBasis));
+  e = cudaMemcpyToSymbol(c_sym, &c->sym, sizeof(SymBasis), di * sizeof(SymBasis));
   if (e != cudaSuccess) return e;
-  int8_t ent[64][3];
+  int8_t ent[64][3] = {};
   int n = 0;
   for (int b = 0; b < c->sym.nblk; ++b)
     for (int i = 0; i < c->sym.dim[b]; ++i)
@@ -1656,14 +1664,13 @@ cudaError_t upload_sym(lsp_ctx* c) {
         ent[n][2] = (int8_t)j;
         ++n;
       }
-  e = cudaMemcpyToSymbol(c_ent, ent, sizeof(ent));
+  e = cudaMemcpyToSymbol(c_ent, ent, sizeof(ent), di * sizeof(ent));
   if (e != cudaSuccess) return e;
-  e = cudaMemcpyToSymbol(c_nent, &n, sizeof(int));
+  e = cudaMemcpyToSymbol(c_nent, &n, sizeof(int), di * sizeof(int));
   if (e != cudaSuccess) return e;
   if (c->geo.d == 3) {
     // coef[e][k] = sum of u_i[a] u_j[b] over the pairs (a, b) of class k, e = (block, i, j)
-    static double coef[24][kMaxCls];
-    memset(coef, 0, sizeof coef);
+    double coef[24][kMaxCls] = {};
     if (n != 24) return cudaErrorInvalidValue;
     for (int q = 0; q < n; ++q) {
       const int b = ent[q][0], i = ent[q][1], j = ent[q][2];
@@ -1676,9 +1683,7 @@ cudaError_t upload_sym(lsp_ctx* c) {
   }
   if (c->geo.d != 2) return cudaSuccess;  // the tables below are for the 2D kernels
   // W_i[k] = sum_a G[k, a] u_i[a] = sum_a g[cls(k, a)] u_i[a];  u_i^T A1 u_j = sum g2[cls(a,b)] u_i[a] u_j[b]
-  static double W2[7][9][6], B2[7][7][6];
-  memset(W2, 0, sizeof W2);
-  memset(B2, 0, sizeof B2);
+  double W2[7][9][6] = {}, B2[7][7][6] = {};
   for (int i = 0; i < 7; ++i)
     for (int k = 0; k < 9; ++k)
       for (int a = 0; a < 9; ++a) W2[i][k][c->geo.cls_of[k][a]] += c->sym.u[i][a];
@@ -1687,7 +1692,7 @@ cudaError_t upload_sym(lsp_ctx* c) {
       for (int a = 0; a < 9; ++a)
         for (int b = 0; b < 9; ++b)
           B2[i][j][c->geo.cls_of[a][b]] += c->sym.u[i][a] * c->sym.u[j][b];
-  static float W2f[7][9][6], B2f[7][7][6];
+  float W2f[7][9][6], B2f[7][7][6];
   for (int i = 0; i < 7; ++i)
     for (int k = 0; k < 9; ++k)
       for (int q = 0; q < 6; ++q) W2f[i][k][q] = (float)W2[i][k][q];
@@ -1698,9 +1703,8 @@ cudaError_t upload_sym(lsp_ctx* c) {
     // t = 2 (2D): block entries (b, i <= j) of mu_0^2 and their class coefficients
     const SymBasis& s2 = c->sym2;
     const Geometry& g2 = c->geo2;
-    static double coef2[kT2Ent][kMaxCls];
+    double coef2[kT2Ent][kMaxCls] = {};
     int8_t ent2[kT2Ent][3];
-    memset(coef2, 0, sizeof coef2);
     int q = 0;
     for (int b = 0; b < s2.nblk; ++b)
       for (int i = 0; i < s2.dim[b]; ++i)

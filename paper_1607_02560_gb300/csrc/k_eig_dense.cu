@@ -223,7 +223,7 @@ __global__ void __launch_bounds__(kT) k_eig_dense3(const double* __restrict__ gv
 }  // namespace
 
 cudaError_t upload_cls125(const Geometry& g) {
-  static uint8_t t[kM * kM];
+  uint8_t t[kM * kM];
   for (int a = 0; a < kM; ++a)
     for (int b = 0; b < kM; ++b) t[a * kM + b] = g.cls_of[a][b];
   return cudaMemcpyToSymbol(c_cls125, t, sizeof t);
