@@ -579,14 +579,18 @@ __global__ void __launch_bounds__(256) k_nd_store(const double* __restrict__ fro
                                                   double* __restrict__ BT,
                                                   int32_t* __restrict__ gsrc) {
   __shared__ double t[kTile][kTile + 1];
-  const int64_t p = blockIdx.y;
-  const double* F = fronts + p * f * f;
   const int ti = (f + kTile - 1) / kTile, tm = (s + kTile - 1) / kTile;  // tiles of FT
   const int bi = (s + kTile - 1) / kTile, bm = (r + kTile - 1) / kTile;  // tiles of BT
-  int q = blockIdx.x;
+  // one grid dimension for both: fronts (leaves of 2D n = 1024: 65 536) as well as tiles (3D n = 64:
+  // 78 864) can exceed the 65 535 blocks of a second one
+  const int per = ti * tm + bi * bm + 1;
+  const int64_t p = blockIdx.x / per;
+  const double* F = fronts + p * f * f;
+  const int q0 = blockIdx.x % per;
+  int q = q0;
   const int x = threadIdx.x & 31, y = threadIdx.x >> 5;
   if (q < ti * tm || (q -= ti * tm) < bi * bm) {
-    const bool fwd = (int)blockIdx.x < ti * tm;
+    const bool fwd = q0 < ti * tm;
     const int nr = fwd ? f : s, nm = fwd ? s : r, c0 = fwd ? 0 : s, tr = fwd ? ti : bi;
     const int i0 = (q % tr) * kTile, m0 = (q / tr) * kTile;
     for (int k = y; k < kTile; k += 8)
@@ -637,8 +641,8 @@ __global__ void __launch_bounds__(1024) k_nd_mv(MvArgs a) {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   constexpr int NP = 8;  // values in flight per thread
   const int tid = threadIdx.x, nt = a.ib * a.mg;
-  const int ti = tid % a.ib, tm = tid / a.ib, i = blockIdx.x * a.ib + ti;
-  const int64_t p = blockIdx.y;
+  const int ti = tid % a.ib, tm = tid / a.ib, i = blockIdx.y * a.ib + ti;
+  const int64_t p = blockIdx.x;  // (a second grid dimension holds 65 535 blocks: too few fronts)
   const double* M = a.M + p * a.nr * a.nm + (i < a.nr ? i : 0);
   const bool live = __any_sync(0xffffffffu, i < a.nr);  // else the warp only helps to gather
   const int nm = live ? a.nm : 0;
@@ -892,7 +896,7 @@ cudaError_t launch_nd_store(lsp_ctx* c, int depth) {
   const int tf = (lv.f + kTile - 1) / kTile, ts = (lv.s + kTile - 1) / kTile;
   const int tr = (lv.r + kTile - 1) / kTile;
   int t = timer_begin(c, level_name("nd_asm", depth));
-  k_nd_store<<<dim3(tf * ts + ts * tr + 1, lv.count), 256, 0, c->stream>>>(
+  k_nd_store<<<(unsigned)((int64_t)lv.count * (tf * ts + ts * tr + 1)), 256, 0, c->stream>>>(
       (const double*)S.fronts.p + lv.front_off, lv.f, lv.s, lv.r,
       (const int32_t*)S.E.p + lv.E_off, (const int32_t*)S.perm.p + lv.perm_off,
       lv.nchild ? (const int32_t*)S.inv.p + lv.inv_off : nullptr, lv.nchild,
@@ -925,7 +929,7 @@ cudaError_t launch_nd_solve(lsp_ctx* c, const double* y, double* x) {
            blocks() * a.ib * a.mg < (int64_t)152 * 512)
       a.mg <<= 1;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((a.nr + a.ib - 1) / a.ib, count);
+    cfg.gridDim = dim3(count, (a.nr + a.ib - 1) / a.ib);
     cfg.blockDim = dim3(a.ib * a.mg);
     cfg.dynamicSmemBytes = sizeof(double) * ((size_t)a.nm + (a.mg > 1 ? a.ib * a.mg : 0));
     cfg.stream = c->stream;

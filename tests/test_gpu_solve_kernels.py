@@ -83,3 +83,22 @@ def test_arnoldi_columns(d, n, steps):
     assert abs(res["resid_true"] - rel) <= max(tol, 1e-9)
     u2, _ = ctx.gmres(f.ravel(), rtol=1e-30, restart=steps, max_cycles=1, precond=False)
     assert np.array_equal(u, u2)
+
+
+@pytest.mark.parametrize("n,leaf", [(1024, 4), (256, 4)])
+def test_more_fronts_than_a_second_grid_dimension_holds(n, leaf):
+    """The smallest leaves of the largest grid: 65 536 fronts at one depth. One refinement step
+    leaves the rounding of a residual of nine products: backward error below 1e-15 of
+    9 max|P| max|x| + max|y|."""
+    import torch
+    ctx = context(2, n, make_workload("helm2d_n256", n=n))
+    ctx.build_stencils(policy="paper")
+    ctx.nd_factor(leaf=leaf, refine_steps=1)
+    y = torch.from_numpy(np.random.default_rng(n).standard_normal(n * n)).cuda()
+    x, r = torch.empty_like(y), torch.empty_like(y)
+    torch.cuda.synchronize()
+    ctx.nd_solve(y, x)
+    ctx.apply_rows("P", x, r)
+    rows = ctx.get_rows("P")
+    scale = 9 * np.abs(rows).max() * x.abs().max().item() + y.abs().max().item()
+    assert (r - y).abs().max().item() <= 1e-15 * scale
