@@ -111,9 +111,13 @@ struct DevBuf {
   size_t bytes = 0;
 };
 
+// Levels of the tree over the integers, leaf boxes of 2^kFmmLog. The points (32-bit lattice indices,
+// whatever the list of shifts) and |p|^2 lie within +-2^31, and two boxes of 2^31 at the level above
+// the top one hold them all, so that the top level's boxes interact within their parents.
+constexpr int kFmmLog = 7, kFmmLevels = 26;
+static_assert(kFmmLog + kFmmLevels - 1 > 31, "a level above the top one for every 32-bit index");
 // Plan and workspace of the fast multipole evaluation of a3 (k_fmm.cu): charges, leaf lists and
 // moments depend on the grid only and are made once per context; used and loc belong to a build.
-constexpr int kFmmLevels = 24;  // boxes of 128 * 2^23 integers hold any shift range and |p|^2
 // Shifts at most (a bound known on the host) for one block per shift, and for eight lanes a shift
 // instead of two.
 constexpr int64_t kFmmBlockShifts = 152 * 8, kFmmLaneShifts = 152 * 256;
@@ -127,7 +131,6 @@ struct FmmPlan {
 };
 // Boxes of the tree over the points -m - 1/2 of a shift range, level 0 the leaves: box j of level l
 // covers the integers [128 2^l j, 128 2^l (j + 1)) of -m (points half an integer below).
-constexpr int kFmmLog = 7;
 struct FmmTree {
   int L;                          // top level: its parents are all neighbours
   int64_t jlo[kFmmLevels];        // first box of a level

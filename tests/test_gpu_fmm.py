@@ -75,3 +75,28 @@ def test_shifts_beyond_the_frequencies_and_at_box_edges(d, n):
     for part in (m, m[:1]):
         ctx.build_stencils(policy="list", shifts=shifts[:len(part)])
         check_shift_table(ctx.get_shift_table(), v, "list", m_list=part)
+
+
+@pytest.mark.parametrize("d,n", [(2, 8), (2, 64), (3, 16)])
+def test_shifts_up_to_the_largest_index(d, n):
+    """Listed shifts far beyond the frequencies, up to the largest lattice index a build takes.
+    There the sums are almost w(m) times the identity: G has the eigenvalues w(m + r) of a
+    projection of functions of |p|^2 = r <= r_max, so |G - w(m)| <= w(m) r_max / (|m| - r_max) in the
+    spectral norm, and |c - w(m) alpha| is at most that for the unit vector alpha. (alpha itself is
+    not determined to any digit.) Rounding: at most 1e-12 of w(m)."""
+    import torch
+    from paper_1607_02560_gb300 import Context
+    r_max = d * (n // 2) ** 2
+    ctx = Context(d, n, stream=torch.cuda.Stream())
+    ctx.set_potential(make_workload("helm2d_n256" if d == 2 else "schr3d_n64", n=n))
+    big = 2147483000 - 4 * r_max
+    for ms in ((2 ** 29 + 5,), (2 ** 30 - 1, 2 ** 30, 2 ** 30 + 1, 2 ** 30 + 300), (1100000000,),
+               (big - 200, big), (-2 ** 30 - 1, -2 ** 30), (-big,)):
+        shifts = (4.0 * np.array(ms) + 2.0) * PI2
+        ctx.build_stencils(policy="list", shifts=shifts)
+        t = ctx.get_shift_table(with_sidx=False)
+        assert len(t["s"]) == len(ms)
+        for m, s, alpha, c in zip(ms, t["s"], t["alpha"], t["c"]):
+            assert abs(np.linalg.norm(alpha) - 1.0) <= 1e-12, m
+            tol = r_max / (abs(m) - r_max) + 1e-12
+            assert np.linalg.norm(c * s - alpha) <= tol, (m, np.linalg.norm(c * s - alpha))
