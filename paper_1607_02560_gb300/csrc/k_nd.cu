@@ -834,9 +834,6 @@ cudaError_t launch_nd_sweep(lsp_ctx* c, int depth) {
                 : lv.f <= 64 ? k_nd_sweep_small<2>
                 : lv.f <= 96 ? k_nd_sweep_small<3>
                 : lv.f <= 128 ? k_nd_sweep_small<4> : k_nd_sweep_small<5>;
-    cudaError_t e =
-        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
     // from 113 rows on a front has the SM's shared memory to itself
     kern<<<lv.count, lv.f > 112 ? 512 : 256, smem, c->stream>>>(F, lv.f, lv.s, perm, err);
     timer_end(c, t);
@@ -992,12 +989,29 @@ cudaError_t launch_nd_solve(lsp_ctx* c, const double* y, double* x) {
   return cudaGetLastError();
 }
 
-cudaError_t nd_prepare_kernels(int max_cols) {
-  const int smem = (int)sizeof(double) * (max_cols + 1024);
-  cudaError_t e = cudaFuncSetAttribute(k_nd_mv<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       smem);
-  if (e != cudaSuccess) return e;
-  return cudaFuncSetAttribute(k_nd_mv<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+// Dynamic shared memory up to what a block can have, for the kernels whose need varies with the
+// plan. The limit belongs to the kernel, not to a context: one set to a plan's need would be lowered
+// by the next, smaller plan of another context, whose launches are then refused.
+cudaError_t nd_prepare_kernels() {
+  int dev = 0, most = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess)
+    e = cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  auto allow = [&](auto kern) {
+    cudaFuncAttributes at;
+    if (e == cudaSuccess) e = cudaFuncGetAttributes(&at, kern);
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               most - (int)at.sharedSizeBytes);
+  };
+  allow(k_nd_mv<true>);
+  allow(k_nd_mv<false>);
+  allow(k_nd_sweep_small<1>);
+  allow(k_nd_sweep_small<2>);
+  allow(k_nd_sweep_small<3>);
+  allow(k_nd_sweep_small<4>);
+  allow(k_nd_sweep_small<5>);
+  return e;
 }
 
 cudaError_t launch_apply_rows(lsp_ctx* c, const double* rows, int mu, int t, const double* u,

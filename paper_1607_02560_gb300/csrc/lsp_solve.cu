@@ -104,7 +104,7 @@ void nd_free(NdState* s) {
   delete s;
 }
 
-cudaError_t nd_prepare_kernels(int max_cols);
+cudaError_t nd_prepare_kernels();
 
 }  // namespace lsp
 
@@ -160,7 +160,6 @@ lsp_status lsp_nd_factor(lsp_ctx* c, const lsp_nd_opts* opts) {
     if ((st = upload(c, S.asm_src, S.plan.asm_src)) != LSP_OK) return st;
     const NdPlan& P = S.plan;
     int64_t nf = 1, cu = 1, dg = 16, ex = 1, vs = 1, ps = 0;
-    int max_sr = 1;
     for (const NdLevel& lv : P.lv) {
       if (lv.f > kNdSmallFront) {
         nf = std::max(nf, (int64_t)lv.count);
@@ -170,7 +169,6 @@ lsp_status lsp_nd_factor(lsp_ctx* c, const lsp_nd_opts* opts) {
         vs = std::max(vs, (int64_t)lv.count * lv.f * kNdStep);
         if (lv.s > kNdPanelRegRows) ps = std::max(ps, (int64_t)lv.count * lv.s * (kNdPanel + 1));
       }
-      max_sr = std::max(max_sr, std::max(lv.s, lv.r));
     }
     if (ps > 0 && !ensure(c, S.pscratch, sizeof(float) * ps))
       return sfail(c, LSP_ERR_OOM, "nested dissection buffers: %s", c->err.c_str());
@@ -191,7 +189,7 @@ lsp_status lsp_nd_factor(lsp_ctx* c, const lsp_nd_opts* opts) {
     SCUDA(c, cudaMemsetAsync(S.cur.p, 0, sizeof(int32_t) * cu, c->stream));
     SCUDA(c, cudaMemsetAsync(S.vst.p, 0, sizeof(double) * vs, c->stream));
     SCUDA(c, nd_tc_prepare());
-    SCUDA(c, nd_prepare_kernels(max_sr));
+    SCUDA(c, nd_prepare_kernels());
     S.have_plan = true;
   }
   S.factored = false;
