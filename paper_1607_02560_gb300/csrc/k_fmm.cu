@@ -598,8 +598,8 @@ cudaError_t plan_t(lsp_ctx* c) {
       !need(P.start, flag_bytes) || !need(c->counts, sizeof(int32_t) * (16 + nr / 4096 + 32)))
     return cudaErrorMemoryAllocation;
   static const std::vector<double> t = make_tables();  // constants: once per process
-  if ((e = cudaMemcpy(P.tab.p, t.data(), sizeof(double) * kTabSize, cudaMemcpyHostToDevice)) !=
-      cudaSuccess)
+  if ((e = cudaMemcpyAsync(P.tab.p, t.data(), sizeof(double) * kTabSize, cudaMemcpyHostToDevice,
+                           c->stream)) != cudaSuccess)
     return e;
   // distinct |p|^2, sorted (the flags live in the buffer of the leaf lists)
   uint8_t* flag = (uint8_t*)P.start.p;

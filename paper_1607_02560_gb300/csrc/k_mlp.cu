@@ -2241,7 +2241,9 @@ lsp_status lsp_mlp_create(int d, uint64_t seed, void* cuda_stream, lsp_mlp** out
       cudaMemset(m->adam_m.p, 0, sizeof(float) * P) != cudaSuccess ||
       cudaMemset(m->adam_v.p, 0, sizeof(float) * P) != cudaSuccess ||
       cudaMemset(m->tiles.p, 0, m->plan.total_bytes) != cudaSuccess ||
-      cudaMemset(m->errflag.p, 0, 64) != cudaSuccess)
+      cudaMemset(m->errflag.p, 0, 64) != cudaSuccess ||
+      // the legacy stream's copies and fills land before m->stream writes the weight tiles
+      cudaStreamSynchronize(cudaStreamLegacy) != cudaSuccess)
     st = LSP_ERR_CUDA;
   if (st == LSP_OK) st = retile(m);
   if (st == LSP_OK && cudaStreamSynchronize(m->stream) != cudaSuccess) st = LSP_ERR_CUDA;

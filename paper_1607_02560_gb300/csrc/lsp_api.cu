@@ -659,6 +659,13 @@ lsp_status lsp_create(int d, int n, void* cuda_stream, lsp_ctx** out) {
       st = LSP_ERR_CUDA;
       break;
     }
+    // The copies above went through the legacy stream, and from pageable memory a copy may return
+    // before it has landed: a context stream that does not wait for the legacy one reads the
+    // tables only after this.
+    if (cudaStreamSynchronize(cudaStreamLegacy) != cudaSuccess) {
+      st = LSP_ERR_CUDA;
+      break;
+    }
   } while (0);
   if (st != LSP_OK) {
     lsp_destroy(c);
