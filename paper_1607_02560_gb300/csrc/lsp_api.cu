@@ -623,6 +623,12 @@ lsp_status lsp_create(int d, int n, void* cuda_stream, lsp_ctx** out) {
       tw[2 * (size_t)n + j] = 4.0 * kPi2 * (k * k) / (double)n;
     }
     std::vector<float> X32(X.begin(), X.end());
+    // and what the doubles of a = 0, 1, 2 leave of them (the multipole plan's charges)
+    for (int a = 0; a < 3; ++a)
+      for (int p = 0; p < P; ++p) {
+        const long double x = ((p == 0 || p == n / 2) ? 1.0L : 2.0L) * cos_r(a * p);
+        X.push_back((double)(x - (long double)X[a * P + p]));
+      }
     // double words of the same values, split from the extended-precision cosines
     std::vector<float> Xdw(2 * 5 * P);
     for (int a = 0; a < 5; ++a)

@@ -126,7 +126,7 @@ struct FmmPlan {
   int32_t ns = 0;                 // sources: distinct |p|^2
   int64_t nsb[kFmmLevels] = {0};  // source boxes of a level
   int64_t qoff[kFmmLevels] = {0}; // boxes of the levels below it in q
-  DevBuf tab, pos, wgt, start, q, used, loc;
+  DevBuf tab, pos, wgt, rank, q, q0, used, loc;
   size_t used_bytes = 0;  // of the last build's tree, a multiple of 4
 };
 // Boxes of the tree over the points -m - 1/2 of a shift range, level 0 the leaves: box j of level l
