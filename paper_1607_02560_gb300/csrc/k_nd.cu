@@ -11,6 +11,7 @@
 #include <stdio.h>
 
 #include "nd.h"
+#include "recip.cuh"
 
 namespace lsp {
 namespace {
@@ -58,23 +59,6 @@ __device__ __forceinline__ void warp_argmax_f(float& best, int& bi) {
       bi = oi;
     }
   }
-}
-
-// 1 / x to within an ulp: the reciprocal of the mantissa in FP32, one third-order step
-// r (1 + e + e^2) with e = 1 - m r in FP64, the exponent by integers. Three FP64 operations where
-// the FP64 division takes several times that, on a pipe that is serial for one warp.
-__device__ __forceinline__ double recip_f64(double x) {
-  const int hi = __double2hiint(x), lo = __double2loint(x);
-  const int ef = (hi >> 20) & 0x7ff;
-  const double m = __hiloint2double((hi & 0xfffff) | 0x3ff00000, lo);  // in [1, 2)
-  const unsigned rb = __float_as_uint(
-      1.0f / __uint_as_float(0x3f800000u | ((unsigned)(hi & 0xfffff) << 3) | ((unsigned)lo >> 29)));
-  const double r0 = __hiloint2double((int)((rb >> 3) + (896u << 20)), (int)(rb << 29));
-  const double e = fma(-m, r0, 1.0);
-  const double r = fma(r0, fma(e, e, e), r0);  // in [1/2, 1]
-  const int rh = __double2hiint(r), fld = (rh >> 20) - (ef - 1023);
-  if (ef == 0 || ef == 0x7ff || fld < 1 || fld > 2046) return 1.0 / x;
-  return __hiloint2double((hi & 0x80000000) | (fld << 20) | (rh & 0xfffff), __double2loint(r));
 }
 
 // Partial inversion of one front (f <= kNdSmallFront) in shared memory, one pivot at a time.

@@ -1,5 +1,6 @@
-"""Device functions that stand in for FP64 arithmetic, on their own: the digits of the error-free split
-and the sum of its levels against exact integers."""
+"""Device functions that stand in for FP64 arithmetic, on their own: the pivots' reciprocal against
+CUDA's correctly rounded division, the digits of the error-free split and the sum of its levels
+against exact integers."""
 
 import ctypes
 import os
@@ -13,7 +14,15 @@ pytestmark = pytest.mark.gpu
 
 SOURCE = r"""
 #include <stdint.h>
+#include "recip.cuh"
 #include "digits.cuh"
+__global__ void k_recip(const double* x, double* r, double* q, int n) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < n) {
+    r[i] = lsp::recip_f64(x[i]);
+    q[i] = 1.0 / x[i];
+  }
+}
 __global__ void k_digits(const double* x, const int* e, int* d, int* ex, int n) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n) {
@@ -33,6 +42,7 @@ __global__ void k_sum(const int* a, const int* ex, double* s, int n) {
 }
 extern "C" int run(int which, const void* a, const void* b, void* c, void* d, int n) {
   const int g = (n + 255) / 256;
+  if (which == 0) k_recip<<<g, 256>>>((const double*)a, (double*)c, (double*)d, n);
   if (which == 1) k_digits<<<g, 256>>>((const double*)a, (const int*)b, (int*)c, (int*)d, n);
   if (which == 2) k_sum<<<g, 256>>>((const int*)a, (const int*)b, (double*)c, n);
   return (int)cudaDeviceSynchronize();
@@ -59,6 +69,37 @@ def run(tmp_path_factory):
         return [t.cpu().numpy() for t in dev[2:]]
 
     return call
+
+
+def patterns(rng, n):
+    """Doubles of every exponent, with random mantissas and with mantissas next to powers of two."""
+    mant = rng.integers(0, 1 << 52, n, dtype=np.uint64)
+    edge = rng.integers(0, 3, n)
+    near = rng.integers(0, 4, n).astype(np.uint64)
+    mant = np.where(edge == 1, near, np.where(edge == 2, np.uint64((1 << 52) - 1) - near, mant))
+    expo = rng.integers(0, 2048, n).astype(np.uint64)
+    sign = rng.integers(0, 2, n).astype(np.uint64)
+    return ((sign << np.uint64(63)) | (expo << np.uint64(52)) | mant).view(np.float64)
+
+
+def test_reciprocal_of_a_pivot(run):
+    """Less than 0.51 ulp off the exact value, so at most one representable number away from the
+    correctly rounded division (and mostly the same); zeros, subnormals, infinities, NaN and results
+    that are not normal are the division's."""
+    x = patterns(np.random.default_rng(0), 1 << 20)
+    x[:8] = [0.0, -0.0, np.inf, -np.inf, np.nan, 5e-324, 2.0 ** -1022, 1.7976931348623157e308]
+    r, q = run(0, x, x, np.empty_like(x), np.empty_like(x))
+    normal = np.isfinite(x) & (np.abs(x) >= 2.0 ** -1022) & (np.abs(q) >= 2.0 ** -1022) \
+        & np.isfinite(q)
+    assert np.array_equal(r[~normal].view(np.int64)[~np.isnan(r[~normal])],
+                          q[~normal].view(np.int64)[~np.isnan(q[~normal])])
+    apart = np.abs(r[normal].view(np.int64) - q[normal].view(np.int64))
+    assert apart.max() <= 1
+    some = np.flatnonzero(normal)[:20000]
+    for i in some[apart[:20000] > 0]:
+        exact = 1 / Fraction(x[i])
+        ulp = Fraction(float(np.spacing(np.abs(r[i]))))
+        assert abs(Fraction(r[i]) - exact) < Fraction(51, 100) * ulp
 
 
 def test_digits_of_values_far_below_the_largest(run):
