@@ -911,18 +911,17 @@ cudaError_t build_t(lsp_ctx* c, const int32_t* list, const int32_t* count, int64
   // stage 1: far field at the nodes of the leaf boxes
   int tm = timer_begin(c, "stage1");
   // (a tree of 4 boxes, 3D n = 64: 21.4 us a value per thread, 23.3 a pair per thread)
-  if (boxes <= 32) {
-    e = tuned_launch(c, std::string("stage1/fmm") + std::to_string(NC) + "/w" + work_bucket(boxes),
-                     {64, 2}, kThreads, 0, [&](LaunchShape sh) {  // (one value per thread: no cap)
+  const bool few = boxes <= 32;
+  e = tuned_launch(c, std::string("stage1/fmm") + std::to_string(NC) + "/w" + work_bucket(boxes),
+                   {64, 2}, kThreads, 0, [&](LaunchShape sh) {
+    if (few)  // (one value per thread: no cap)
       k_fmm_m2l<NC><<<(unsigned)((boxes * 2 * NC * kQ1 + sh.threads - 1) / sh.threads), sh.threads,
                       0, c->stream>>>(t, used, tab, (const double*)P.q.p, q0, loc);
-      return cudaGetLastError();
-    });
-  } else {  // (a block per box: nothing to tune)
-    k_fmm_m2l_box<NC><<<(unsigned)boxes, m2l_threads<NC>(), 0, c->stream>>>(
-        t, used, tab, (const double*)P.q.p, q0, loc);
-    e = cudaGetLastError();
-  }
+    else
+      k_fmm_m2l_box<NC><<<(unsigned)boxes, m2l_threads<NC>(), 0, c->stream>>>(
+          t, used, tab, (const double*)P.q.p, q0, loc);
+    return cudaGetLastError();
+  });
   if (e != cudaSuccess) return e;
   if (t.L > 0) {
     // the deepest subtrees that still leave two blocks per SM to do (no more than there are shifts)

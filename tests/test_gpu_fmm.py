@@ -140,17 +140,3 @@ def test_kernel_vectors_as_accurate_as_direct_sums(d, n, more):
         off.append((c[i] - g[diff] @ alpha[i]) / (np.abs(g).max() * R(2) ** -53))
     rms = float(np.sqrt(np.mean(np.array(off, dtype=float) ** 2)))
     assert rms <= (1.5 if d == 2 else 1.0), rms
-
-
-@pytest.mark.parametrize("n,tuned", [(16, True), (256, False)])
-def test_only_launches_with_a_choice_are_tuned(n, tuned):
-    """Trees of at most 32 boxes take a thread per value and any block size; larger ones a block
-    per box, whose shape is fixed."""
-    import torch
-    from paper_1607_02560_gb300 import Context
-    ctx = Context(2, n, stream=torch.cuda.Stream())
-    ctx.set_autotune(True)
-    ctx.set_potential(make_workload("helm2d_n256", n=n))
-    ctx.build_stencils(policy="local")
-    ctx.synchronize()
-    assert any(k.startswith("stage1/fmm") for k in ctx.tuning()) == tuned
