@@ -315,90 +315,94 @@ __global__ void __launch_bounds__(kThreads) k_fmm_m2l(const __grid_constant__ Tr
   }
 }
 
+constexpr int kBoxThreads = 256;
 // The same, a block per box and a thread per pair of mirrored nodes (i, 19 - i). With R the moments
 // of the box at offset 2 and L those at -2 in reverse order, K_-2[k][i] = -+K_2[19 - k][19 - i] (f = 1,
 // 2) gives
 //   out[i] + out[19 - i] = sum_k (K_2[k][i] + K_2[k][19 - i]) (R -+ L)[k],
 //   out[i] - out[19 - i] = sum_k (K_2[k][i] - K_2[k][19 - i]) (R +- L)[k],
-// 80 instead of 120 multiply-adds a pair with the third offset. The values at the centre by one more
-// warp, in 2D on two lanes a column (offsets +-2 and 3): an FP64 instruction of a warp takes 64 cycles
-// of its quarter of the SM, which a pair's warp shares.
-// Measured with the translation downwards, plain node values: 2D n = 1024 208 -> 175 us,
-// n = 512 53.7 -> 50.0 us, n = 128 20.5 -> 18.7 us.
+// 80 instead of 120 multiply-adds a pair with the third offset. The values at the centre by a warp of
+// their own where the block has one to spare (any block size will do), in 2D on two lanes a column
+// (offsets +-2 and 3): an FP64 instruction of a warp takes 64 cycles of its quarter of the SM, which a
+// pair's warp shares. Measured with the translation downwards, plain node values: 2D n = 1024 208 ->
+// 175 us, n = 512 53.7 -> 50.0 us, n = 128 20.5 -> 18.7 us.
 template <int NC>
-constexpr int m2l_threads() {
-  return (NC * kQ + 31) / 32 * 32 + 32;
-}
-template <int NC>
-__global__ void __launch_bounds__(m2l_threads<NC>()) k_fmm_m2l_box(
+__global__ void __launch_bounds__(kThreads) k_fmm_m2l_box(
     const __grid_constant__ Tree t, const uint8_t* __restrict__ used,
     const double* __restrict__ tab, const double* __restrict__ q, const double* __restrict__ q0,
     double* __restrict__ loc) {
-  constexpr int FC = 2 * NC, BASE = m2l_threads<NC>() - 32;
+  constexpr int FC = 2 * NC, PAIRS = FC * kH;
   __shared__ double sa[2][NC][kQ], s3[NC][kQ];  // R + L, R - L; the moments at offset 3 or -3
-  const int64_t u = blockIdx.x;
-  if (!used[u]) return;
+  const int64_t boxes = t.off[t.L + 1];
+  const int spare = (PAIRS + 31) / 32, warps = blockDim.x >> 5;
   int l = 0;
-  while (u >= t.off[l + 1]) ++l;
-  const int64_t j = t.jlo[l] + (u - t.off[l]);
-  const int odd = (int)(j & 1);
-  auto inside = [&](int64_t x) { return x >= 0 && x < t.nsb[l]; };
-  if (threadIdx.x < NC * kQ) {
-    const int c = threadIdx.x / kQ, k = threadIdx.x % kQ;
-    auto moment = [&](int64_t x, int kk) {
-      return inside(x) ? __ldg(q + (t.qoff[l] + x) * (NC * kQ) + c * kQ + kk) : 0.0;
-    };
-    const double r = moment(j + 2, k), m = moment(j - 2, kQ - 1 - k);
-    sa[0][c][k] = r + m;
-    sa[1][c][k] = r - m;
-    s3[c][k] = moment(odd ? j - 3 : j + 3, k);
-  }
-  __syncthreads();
-  double* out = loc + u * (FC * kRows);
-  if (threadIdx.x < BASE) {
-    if (threadIdx.x >= FC * kH) return;
-    const int i = threadIdx.x / FC, fc = threadIdx.x - i * FC, c = fc >> 1, f = fc & 1;
-    const double* KS = tab + kTabKS + 2 * f * kQ * kH + i;
-    const double* K3 = tab + kTabK + ((f * 4 + (odd ? 0 : 3)) * kQ) * kQ1 + i;
-    const double *ps = sa[1 - f][c], *pd = sa[f][c], *p3 = s3[c];
-    double sum = 0.0, dif = 0.0, lo = 0.0, hi = 0.0;
-#pragma unroll
-    for (int k = 0; k < kQ; ++k) {
-      sum = fma(__ldg(KS + k * kH), ps[k], sum);
-      dif = fma(__ldg(KS + (kQ + k) * kH), pd[k], dif);
-      lo = fma(__ldg(K3 + k * kQ1), p3[k], lo);
-      hi = fma(__ldg(K3 + k * kQ1 + kQ - 1 - 2 * i), p3[k], hi);
+  for (int64_t u = blockIdx.x; u < boxes; u += gridDim.x) {
+    if (!used[u]) continue;
+    while (u >= t.off[l + 1]) ++l;
+    const int64_t j = t.jlo[l] + (u - t.off[l]);
+    const int odd = (int)(j & 1);
+    auto inside = [&](int64_t x) { return x >= 0 && x < t.nsb[l]; };
+    for (int e = threadIdx.x; e < NC * kQ; e += blockDim.x) {
+      const int c = e / kQ, k = e % kQ;
+      auto moment = [&](int64_t x, int kk) {
+        return inside(x) ? __ldg(q + (t.qoff[l] + x) * (NC * kQ) + c * kQ + kk) : 0.0;
+      };
+      const double r = moment(j + 2, k), m = moment(j - 2, kQ - 1 - k);
+      sa[0][c][k] = r + m;
+      sa[1][c][k] = r - m;
+      s3[c][k] = moment(odd ? j - 3 : j + 3, k);
     }
-    const double sc = level_scale(tab, f, l);
-    out[i * FC + fc] = (lo + (sum + dif)) * sc;
-    out[(kQ - 1 - i) * FC + fc] = (hi + (sum - dif)) * sc;
-    return;
-  }
-  constexpr bool SPLIT = 2 * FC <= 32;
-  const int lane = threadIdx.x & 31, fc = lane % FC, c = fc >> 1, f = fc & 1;
-  auto total = [&](int64_t x) { return inside(x) ? __ldg(q0 + (t.qoff[l] + x) * NC + c) : 0.0; };
-  const double ql = total(j - 2), q2 = total(j + 2) + (f ? ql : -ql);  // c at -2 is -+ c at 2
-  const double q3 = total(odd ? j - 3 : j + 3);
-  const double* K2 = tab + kTabK + ((f * 4 + 2) * kQ) * kQ1 + kQ;
-  const double* K3 = tab + kTabK + ((f * 4 + (odd ? 0 : 3)) * kQ) * kQ1 + kQ;
-  const double *ps = sa[1 - f][c], *p3 = s3[c];
-  double dif = 0.0;
-  if (SPLIT) {
-    const double *K = lane < FC ? K2 : K3, *p = lane < FC ? ps : p3;
+    __syncthreads();
+    double* out = loc + u * (FC * kRows);
+    for (int e = threadIdx.x; e < PAIRS; e += blockDim.x) {
+      const int i = e / FC, fc = e - i * FC, c = fc >> 1, f = fc & 1;
+      const double* KS = tab + kTabKS + 2 * f * kQ * kH + i;
+      const double* K3 = tab + kTabK + ((f * 4 + (odd ? 0 : 3)) * kQ) * kQ1 + i;
+      const double *ps = sa[1 - f][c], *pd = sa[f][c], *p3 = s3[c];
+      double sum = 0.0, dif = 0.0, lo = 0.0, hi = 0.0;
 #pragma unroll
-    for (int k = 0; k < kQ; ++k) dif = fma(__ldg(K + k * kQ1), p[k], dif);
-    dif += __shfl_down_sync(0xffffffffu, dif, FC);
-  } else {
+      for (int k = 0; k < kQ; ++k) {
+        sum = fma(__ldg(KS + k * kH), ps[k], sum);
+        dif = fma(__ldg(KS + (kQ + k) * kH), pd[k], dif);
+        lo = fma(__ldg(K3 + k * kQ1), p3[k], lo);
+        hi = fma(__ldg(K3 + k * kQ1 + kQ - 1 - 2 * i), p3[k], hi);
+      }
+      const double sc = level_scale(tab, f, l);
+      out[i * FC + fc] = (lo + (sum + dif)) * sc;
+      out[(kQ - 1 - i) * FC + fc] = (hi + (sum - dif)) * sc;
+    }
+    if ((int)(threadIdx.x >> 5) == (warps > spare ? spare : (int)(u % warps))) {
+      constexpr bool SPLIT = 2 * FC <= 32;
+      const int lane = threadIdx.x & 31, fc = lane % FC, c = fc >> 1, f = fc & 1;
+      auto total = [&](int64_t x) {
+        return inside(x) ? __ldg(q0 + (t.qoff[l] + x) * NC + c) : 0.0;
+      };
+      const double ql = total(j - 2), q2 = total(j + 2) + (f ? ql : -ql);  // c at -2 is -+ c at 2
+      const double q3 = total(odd ? j - 3 : j + 3);
+      const double* K2 = tab + kTabK + ((f * 4 + 2) * kQ) * kQ1 + kQ;
+      const double* K3 = tab + kTabK + ((f * 4 + (odd ? 0 : 3)) * kQ) * kQ1 + kQ;
+      const double *ps = sa[1 - f][c], *p3 = s3[c];
+      double dif = 0.0;
+      if (SPLIT) {
+        const double *K = lane < FC ? K2 : K3, *p = lane < FC ? ps : p3;
 #pragma unroll
-    for (int k = 0; k < kQ; ++k)
-      dif = fma(__ldg(K3 + k * kQ1), p3[k], fma(__ldg(K2 + k * kQ1), ps[k], dif));
+        for (int k = 0; k < kQ; ++k) dif = fma(__ldg(K + k * kQ1), p[k], dif);
+        dif += __shfl_down_sync(0xffffffffu, dif, FC);
+      } else {
+#pragma unroll
+        for (int k = 0; k < kQ; ++k)
+          dif = fma(__ldg(K3 + k * kQ1), p3[k], fma(__ldg(K2 + k * kQ1), ps[k], dif));
+      }
+      if (lane < FC) {
+        const double sc = level_scale(tab, f, l);
+        const double tot = fma(__ldg(tab + kTabC + f * 4 + (odd ? 0 : 3)), q3,
+                               __ldg(tab + kTabC + f * 4 + 2) * q2);
+        out[kQ * FC + fc] = tot * sc;
+        out[kQ1 * FC + fc] = dif * sc;
+      }
+    }
+    __syncthreads();  // the next box
   }
-  if (lane >= FC) return;
-  const double sc = level_scale(tab, f, l);
-  const double tot = fma(__ldg(tab + kTabC + f * 4 + (odd ? 0 : 3)), q3,
-                         __ldg(tab + kTabC + f * 4 + 2) * q2);
-  out[kQ * FC + fc] = tot * sc;
-  out[kQ1 * FC + fc] = dif * sc;
 }
 
 // Values of the leaves: from the top, child = own + interpolation of the parent's (the centre as one
@@ -913,13 +917,14 @@ cudaError_t build_t(lsp_ctx* c, const int32_t* list, const int32_t* count, int64
   // (a tree of 4 boxes, 3D n = 64: 21.4 us a value per thread, 23.3 a pair per thread)
   const bool few = boxes <= 32;
   e = tuned_launch(c, std::string("stage1/fmm") + std::to_string(NC) + "/w" + work_bucket(boxes),
-                   {64, 2}, kThreads, 0, [&](LaunchShape sh) {
+                   few ? LaunchShape{64, 2} : LaunchShape{kBoxThreads, 32}, kThreads, 0,
+                   [&](LaunchShape sh) {
     if (few)  // (one value per thread: no cap)
       k_fmm_m2l<NC><<<(unsigned)((boxes * 2 * NC * kQ1 + sh.threads - 1) / sh.threads), sh.threads,
                       0, c->stream>>>(t, used, tab, (const double*)P.q.p, q0, loc);
     else
-      k_fmm_m2l_box<NC><<<(unsigned)boxes, m2l_threads<NC>(), 0, c->stream>>>(
-          t, used, tab, (const double*)P.q.p, q0, loc);
+      k_fmm_m2l_box<NC><<<(unsigned)std::min<int64_t>(boxes, 152 * (int64_t)sh.per_sm), sh.threads,
+                          0, c->stream>>>(t, used, tab, (const double*)P.q.p, q0, loc);
     return cudaGetLastError();
   });
   if (e != cudaSuccess) return e;
