@@ -234,6 +234,10 @@ def kernel_work(name: str, n: int, d: int, N: int, mu: int, sizes, mode: str = "
         k = int(name[-1])
         # stage k runs over E_k; sizes lists E_d, E_{d-1}, ..., so E_k = sizes[d - k]
         count = sizes[d - k]
+        if mode == "dword" and d == 1:
+            # double-word stage (1D only): FP32 operations as written (a double-word multiply-add
+            # is 10, a double-word add or subtract 11, a renormalisation 3, every fourth step)
+            return count * ((n // 4) * (4 * 11 + 6 * 10 + 6 * 3 / 4) + 2 * 3 * 10), "fp32_op"
         if mode == "mixed":
             # FP32 stages, counted in FP32 operations as written: stage 1 per mirror pair two
             # squarings, four additions and six fused multiply-adds; later stages one fused

@@ -7,6 +7,9 @@ import os
 import subprocess
 import sys
 
+import numpy as np
+import pytest
+
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 
 
@@ -118,3 +121,15 @@ def test_cpu_oracle_sample_reports_the_processes_it_used():
     j = json.loads([ln for ln in p.stdout.splitlines() if ln.startswith("{")][-1])
     assert j["cores"] == 2 and j["kind"] == "oracle" and j["value"] > 0
     assert "2 process(es)" in j["sample"]
+
+
+@pytest.mark.parametrize("d,mode,kind", [(1, "dword", "fp32_op"), (1, "fp64", "flop"),
+                                         (2, "dword", "flop"), (2, "mixed", "fp32_op")])
+def test_stage_work_is_counted_in_the_arithmetic_that_runs(d, mode, kind):
+    """Double words run in 1D; in 2D that mode's sums are FP64."""
+    sys.path.insert(0, ROOT)
+    import bench
+
+    n = 64
+    sizes = bench.stage_work(np.arange(-40, -10), n, d, mode)
+    assert bench.kernel_work("stage1", n, d, n ** d, 3 ** d, sizes, mode)[1] == kind
