@@ -37,3 +37,33 @@ def test_step_remainders(d, n, leaf):
     assert backward_error(P, x, y) <= 1e-15
     ref = O.solve_p(P, y)
     assert np.abs(x - ref).max() <= 256 * U * kappa_1(P) * np.abs(ref).max()
+
+
+@pytest.mark.parametrize("d,n,leaf", [(2, 64, 32), (3, 16, 8)])
+@pytest.mark.parametrize("kind", ["blocks", "log"])
+def test_rows_of_very_different_scales(d, n, leaf, kind):
+    """One listed shift for a potential of nine (blocks of rows) to eleven (every row) orders of
+    magnitude: rows of P up to 1e5 times larger than others inside one step of 64 pivots, whose
+    digits are taken relative to the largest entry of a row or column. Each row by itself: the plain
+    solve contracts (1e-7) and one refinement step leaves the rounding of a residual of mu products,
+    (mu + 2) u of sum |P| |x| + |y|."""
+    rng = np.random.default_rng(n)
+    N = n ** d
+    s0 = 18 * O.PI2
+    f, sign = rng.random((n,) * d), rng.choice([-1.0, 1.0], (n,) * d)
+    if kind == "log":
+        v = s0 + 10.0 ** (11 * f - 3) * sign
+    else:
+        v = np.where(np.indices((n,) * d)[0] % 7 < 2, 1e9 * (0.5 + 0.5 * f), s0 + 100 * f * sign)
+    ctx = ctx_for(v)
+    ctx.set_potential(v)
+    ctx.build_stencils(policy="list", shifts=np.array([s0]))
+    P = csr(ctx, "P", N)
+    rows = abs(P).max(axis=1).toarray()
+    assert rows.max() > 1e3 * rows.min()
+    y = P @ rng.standard_normal(N)
+    for steps, tol in ((0, 1e-7), (1, (3 ** d + 2) * U)):
+        ctx.nd_factor(leaf=leaf, refine_steps=steps)
+        x = gpu_solve(ctx, y)
+        err = np.abs(P @ x - y) / (abs(P) @ np.abs(x) + np.abs(y))
+        assert err.max() <= tol, (steps, err.max())
