@@ -378,7 +378,10 @@ typedef struct {
   int max_front;        /* largest front |E| + |R|                                            */
   int factored;         /* 1 when a factorisation of the current stencils is held             */
   int64_t fronts;       /* number of fronts                                                   */
-  int64_t front_bytes;  /* device bytes of the fronts (sum of (|E| + |R|)^2 * 8)              */
+  int64_t front_bytes;  /* device bytes of the fronts (sum of (|E| + |R|)^2 * 8). Beside them a */
+                        /* factor holds solve_bytes once more (the blocks a solve reads,      */
+                        /* transposed) and the scratch of one depth's updates (2.3 KiB per row */
+                        /* of its fronts above 160 rows, at the depth with most of them)      */
   int64_t solve_bytes;  /* front bytes one solve reads (sum of (|E| + |R|) |E| + |E| |R|, x 8) */
   double flops;         /* FP64 flops of the factorisation as run: 2 |E| (|E| + |R|)^2 a front  */
   double flops_lu;      /* the multifrontal LU count 2/3 |E|^3 + 2 |E|^2 |R| + 2 |E| |R|^2    */
