@@ -588,14 +588,9 @@ lsp_status lsp_create(int d, int n, void* cuda_stream, lsp_ctx** out) {
     const int P = c->geo.P;
     std::vector<double> X(5 * P);
     const long double two_pi = 6.283185307179586476925286766559005768L;
-    auto cos_r = [&](int r) -> long double {  // cos(2 pi r / n), r in [0, n)
-      r %= n;
-      int sign = 1;
-      if (r > n / 2) r = n - r;            // cos(2 pi - t) = cos t
-      if (r > n / 4) {                     // cos(pi - t) = -cos t
-        r = n / 2 - r;
-        sign = -1;
-      }
+    // (each angle evaluated once: extended precision is slow where the host has it in software)
+    std::vector<long double> cosines(n);
+    for (int r = 0; r <= n / 4; ++r) {
       long double val;
       if (r == 0)
         val = 1.0L;
@@ -605,8 +600,11 @@ lsp_status lsp_create(int d, int n, void* cuda_stream, lsp_ctx** out) {
         val = sinl(two_pi * (long double)(n / 4 - r) / (long double)n);
       else
         val = cosl(two_pi * (long double)r / (long double)n);
-      return sign * val;
-    };
+      cosines[r] = val;
+      cosines[n / 2 - r] = r == n / 4 ? val : -val;  // cos(pi - t) = -cos t
+    }
+    for (int r = n / 2 + 1; r < n; ++r) cosines[r] = cosines[n - r];  // cos(2 pi - t) = cos t
+    auto cos_r = [&](int r) { return cosines[r % n]; };  // cos(2 pi r / n)
     for (int a = 0; a < 5; ++a)
       for (int p = 0; p < P; ++p) {
         const long double wgt = (p == 0 || p == n / 2) ? 1.0L : 2.0L;
